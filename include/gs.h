@@ -311,6 +311,22 @@ gs_status gs_iso_crossings(gs_ctx* ctx, const float* volume, int32_t nx, int32_t
                            const float* origin /* host [3] */, const float* spacing /* host [3] */, float* points,
                            float* normals, int64_t capacity, int64_t* count);
 
+/* gs_iso_crossings in two steps, for callers that size the outputs by the
+ * count without a second pass over the volume.  gs_iso_count fills the
+ * caller's workspace (device, 8-byte aligned, gs_iso_workspace_bytes(nx, ny,
+ * nz) bytes; 0 for a dimension below 1) and sets *count (host; synchronises
+ * the stream); gs_iso_emit, given the same volume, level and workspace,
+ * writes the crossings (points, normals: device, float [capacity][3]) on the
+ * context's stream; a capacity below the count is reported by the next
+ * gs_sync as GS_ECAPACITY.  gs_iso_count ends the context's current batch.
+ * Errors: GS_EINVAL, GS_ECUDA. */
+int64_t gs_iso_workspace_bytes(int32_t nx, int32_t ny, int32_t nz);
+gs_status gs_iso_count(gs_ctx* ctx, const float* volume, int32_t nx, int32_t ny, int32_t nz, float iso,
+                       void* workspace, int64_t* count);
+gs_status gs_iso_emit(gs_ctx* ctx, const float* volume, int32_t nx, int32_t ny, int32_t nz, float iso,
+                      const float* origin /* host [3] */, const float* spacing /* host [3] */,
+                      const void* workspace, float* points, float* normals, int64_t capacity);
+
 /* Initial Gaussians from a point cloud (device, float [m][3] points and unit
  * normals): the n points select[0..n) (device int64 indices into the m, or
  * select == NULL with n == m) become out's n Gaussians: mean = point,

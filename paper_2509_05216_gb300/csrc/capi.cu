@@ -87,7 +87,7 @@ struct gs_ctx {
       target_slot, host_tgt0, host_tgt1, pair_stats, cells, vismask, ssim_table, ssim_partials, ssim_sums,
       init_pts, init_scales, knn_part, knn_table, ord_keys0, ord_keys1, ord_vals0, ord_vals1, ord_total, ord_hist,
       ord_hist_scan, ord_lookback, ord_counters, ord_views, tile_order, vis_sums, vis_offsets, dtotal, dkeys0,
-      dkeys1, dvals0, dvals1, dhist, dhist_scan, dlookback, elookback, dorder, torder;
+      dkeys1, dvals0, dvals1, dhist, dhist_scan, dlookback, elookback, dorder, torder, iso_work;
 
   // launch accounting and optional per-kernel event timing
   struct KStat {
@@ -435,7 +435,7 @@ void gs_destroy(gs_ctx* c) {
                     &c->ord_vals0, &c->ord_vals1, &c->ord_total, &c->ord_hist, &c->ord_hist_scan, &c->ord_lookback,
                     &c->ord_counters, &c->ord_views, &c->tile_order, &c->vis_sums, &c->vis_offsets, &c->dtotal,
                     &c->dkeys0, &c->dkeys1, &c->dvals0, &c->dvals1, &c->dhist, &c->dhist_scan, &c->dlookback,
-                    &c->elookback, &c->dorder, &c->torder};
+                    &c->elookback, &c->dorder, &c->torder, &c->iso_work};
   for (DevBuf* b : bufs)
     if (b->p) cudaFree(b->p);
   for (const auto& p : c->pending) {
@@ -1185,6 +1185,79 @@ static gs_status sort_pairs(gs_ctx* c, int64_t n, int bits, int* which) {
   return GS_OK;
 }
 
+// Workspace of the crossings: scan totals (total, view total, two segment
+// words; 32 bytes), block counts, block offsets, side words.
+static IsoArgs iso_args(const float* volume, int32_t nx, int32_t ny, int32_t nz, float iso, void* workspace) {
+  IsoArgs a{};
+  a.vol = volume;
+  a.nx = nx;
+  a.ny = ny;
+  a.nz = nz;
+  a.nverts = (int64_t)nx * ny * nz;
+  a.nwords = iso_words(a.nverts);
+  a.iso = iso;
+  a.block_counts = static_cast<uint32_t*>(workspace) + 8;
+  a.block_offsets = a.block_counts + iso_blocks(a.nverts);
+  a.sides = a.block_counts + 2 * iso_blocks(a.nverts);
+  return a;
+}
+
+int64_t gs_iso_workspace_bytes(int32_t nx, int32_t ny, int32_t nz) {
+  if (nx < 1 || ny < 1 || nz < 1) return 0;
+  const int64_t nverts = (int64_t)nx * ny * nz;
+  return (int64_t)sizeof(uint32_t) * (8 + 2 * iso_blocks(nverts) + iso_words(nverts));
+}
+
+gs_status gs_iso_count(gs_ctx* c, const float* volume, int32_t nx, int32_t ny, int32_t nz, float iso, void* workspace,
+                       int64_t* count) {
+  if (!c) return GS_EINVAL;
+  if (!volume || !workspace || !count) return fail(c, GS_EINVAL, "NULL argument");
+  if (nx < 1 || ny < 1 || nz < 1) return fail(c, GS_EINVAL, "volume dimensions must be >= 1");
+  if (reinterpret_cast<uintptr_t>(workspace) % 8 != 0) return fail(c, GS_EINVAL, "workspace not 8-byte aligned");
+  set_device(c);
+  c->projected = c->sorted = c->rastered = c->cells_ready = false;
+  IsoArgs a = iso_args(volume, nx, ny, nz, iso, workspace);
+  uint64_t* total = static_cast<uint64_t*>(workspace);
+  {
+    LaunchScope ls(c, "iso_crossings", 2);
+    launch_iso_count(a, c->stream);
+  }
+  {
+    LaunchScope ls(c, "scan_block_sums", 2);
+    launch_scan_block_sums(a.block_counts, iso_blocks(a.nverts), 1, const_cast<uint32_t*>(a.block_offsets), total + 1,
+                           reinterpret_cast<uint32_t*>(total + 2), total, c->stream);
+  }
+  GS_CHECK_LAUNCH(c);
+  GS_CUDA(c, cudaMemcpyAsync(c->pinned, total, sizeof(uint64_t), cudaMemcpyDeviceToHost, c->stream));
+  GS_CUDA(c, cudaStreamSynchronize(c->stream));
+  *count = (int64_t)c->pinned[0];
+  return GS_OK;
+}
+
+gs_status gs_iso_emit(gs_ctx* c, const float* volume, int32_t nx, int32_t ny, int32_t nz, float iso,
+                      const float* origin, const float* spacing, const void* workspace, float* points, float* normals,
+                      int64_t capacity) {
+  if (!c) return GS_EINVAL;
+  if (!volume || !origin || !spacing || !workspace || !points || !normals) return fail(c, GS_EINVAL, "NULL argument");
+  if (nx < 1 || ny < 1 || nz < 1) return fail(c, GS_EINVAL, "volume dimensions must be >= 1");
+  set_device(c);
+  IsoArgs a = iso_args(volume, nx, ny, nz, iso, const_cast<void*>(workspace));
+  for (int d = 0; d < 3; d++) {
+    a.origin[d] = origin[d];
+    a.h[d] = spacing[d];
+  }
+  a.status = c->status_d;
+  a.points = points;
+  a.normals = normals;
+  a.capacity = capacity;
+  {
+    LaunchScope ls(c, "iso_crossings");
+    launch_iso_emit(a, c->stream);
+  }
+  GS_CHECK_LAUNCH(c);
+  return GS_OK;
+}
+
 gs_status gs_iso_crossings(gs_ctx* c, const float* volume, int32_t nx, int32_t ny, int32_t nz, float iso,
                            const float* origin, const float* spacing, float* points, float* normals, int64_t capacity,
                            int64_t* count) {
@@ -1194,51 +1267,13 @@ gs_status gs_iso_crossings(gs_ctx* c, const float* volume, int32_t nx, int32_t n
   if ((points == nullptr) != (normals == nullptr)) return fail(c, GS_EINVAL, "points and normals go together");
   set_device(c);
   c->projected = c->sorted = c->rastered = c->cells_ready = false;
-  IsoArgs a{};
-  a.vol = volume;
-  a.nx = nx;
-  a.ny = ny;
-  a.nz = nz;
-  a.nverts = (int64_t)nx * ny * nz;
-  a.iso = iso;
-  for (int d = 0; d < 3; d++) {
-    a.origin[d] = origin[d];
-    a.h[d] = spacing[d];
-  }
-  const int64_t nb = (a.nverts + 255) / 256;
-  GS_TRY(ensure(c, c->block_sums, sizeof(uint32_t) * nb));
-  GS_TRY(ensure(c, c->block_offsets, sizeof(uint32_t) * nb));
-  GS_TRY(ensure(c, c->total, sizeof(uint64_t) * (1 + kMaxViews) +
-                                 sizeof(uint32_t) * (2 * (kMaxViews + 1) + 16 + 8 * kMaxViews)));
-  a.block_counts = P<uint32_t>(c->block_sums);
-  a.block_offsets = P<uint32_t>(c->block_offsets);
-  a.status = c->status_d;
-  uint64_t* total = P<uint64_t>(c->total);
-  {
-    LaunchScope ls(c, "iso_crossings");
-    launch_iso(a, false, c->stream);
-  }
-  {
-    LaunchScope ls(c, "scan_block_sums", 2);
-    launch_scan_block_sums(P<uint32_t>(c->block_sums), nb, 1, P<uint32_t>(c->block_offsets), total + 1,
-                           reinterpret_cast<uint32_t*>(total + 1 + kMaxViews), total, c->stream);
-  }
-  GS_CHECK_LAUNCH(c);
-  uint64_t m = 0;
-  GS_CUDA(c, cudaMemcpyAsync(&m, total, sizeof(m), cudaMemcpyDeviceToHost, c->stream));
-  GS_CUDA(c, cudaStreamSynchronize(c->stream));
-  *count = (int64_t)m;
+  GS_TRY(ensure(c, c->iso_work, (size_t)gs_iso_workspace_bytes(nx, ny, nz)));
+  int64_t m = 0;
+  GS_TRY(gs_iso_count(c, volume, nx, ny, nz, iso, c->iso_work.p, &m));
+  *count = m;
   if (!points) return GS_OK;
-  if ((int64_t)m > capacity) return fail(c, GS_ECAPACITY, "%llu crossings exceed the capacity", (unsigned long long)m);
-  a.points = points;
-  a.normals = normals;
-  a.capacity = capacity;
-  {
-    LaunchScope ls(c, "iso_crossings");
-    launch_iso(a, true, c->stream);
-  }
-  GS_CHECK_LAUNCH(c);
-  return GS_OK;
+  if (m > capacity) return fail(c, GS_ECAPACITY, "%lld crossings exceed the capacity", (long long)m);
+  return gs_iso_emit(c, volume, nx, ny, nz, iso, origin, spacing, c->iso_work.p, points, normals, capacity);
 }
 
 gs_status gs_init_gaussians(gs_ctx* c, const float* points, const float* normals, int64_t m, const int64_t* select,

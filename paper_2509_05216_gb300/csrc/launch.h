@@ -207,17 +207,21 @@ void launch_ssim(const SsimArgs& a, int blocks, bool backward, double* out_view,
 struct IsoArgs {
   const float* vol;  // [nz][ny][nx]
   int nx, ny, nz;
-  int64_t nverts;
+  int64_t nverts, nwords;
   float iso;
   float origin[3], h[3];
-  uint32_t* block_counts;         // count pass: crossings per block of 256 vertices
+  uint32_t* sides;                // [nwords] bit b of word w: sample 32 w + b >= iso
+  uint32_t* block_counts;         // [iso_blocks] crossings per block of 1,024 words
   const uint32_t* block_offsets;  // emit pass: exclusive scan of block_counts
   float* points;                  // [capacity][3]
   float* normals;                 // [capacity][3]
   int64_t capacity;
   int* status;
 };
-void launch_iso(const IsoArgs& a, bool emit, cudaStream_t s);
+int64_t iso_words(int64_t nverts);
+int64_t iso_blocks(int64_t nverts);
+void launch_iso_count(const IsoArgs& a, cudaStream_t s);  // sides and block_counts
+void launch_iso_emit(const IsoArgs& a, cudaStream_t s);
 
 struct KnnArgs {
   const float* pts;  // [n][3]

@@ -93,7 +93,7 @@ EXPORTS = ["gs_raster_fwd_l1", "gs_train_graph_capture", "gs_train_graph_launch"
            "gs_serve_stats", "gs_set_option", "gs_get_option", "gs_l1_loss_noalloc", "gs_profile_enable", "gs_profile_read", "gs_profile_reset", "gs_create", "gs_destroy", "gs_last_error", "gs_set_stream", "gs_sync", "gs_project",
            "gs_bin_sort", "gs_raster_fwd", "gs_raster_bwd", "gs_l1_loss", "gs_adam", "gs_get_buffer",
            "gs_get_counts", "gs_pair_stats", "gs_serve_timeline", "gs_ssim_loss",
-           "gs_image_metrics", "gs_iso_crossings", "gs_init_gaussians",
+           "gs_image_metrics", "gs_iso_crossings", "gs_iso_workspace_bytes", "gs_iso_count", "gs_iso_emit", "gs_init_gaussians",
            "gs_set_densify_stats", "gs_densify"]
 
 
@@ -146,6 +146,11 @@ def load(path: str | None = None):
                              P(gs_params), P(gs_params), P(gs_params), P(i64)]
     L.gs_iso_crossings.argtypes = [vp, vp, i32, i32, i32, ctypes.c_float, P(ctypes.c_float), P(ctypes.c_float),
                                    vp, vp, i64, P(i64)]
+    L.gs_iso_workspace_bytes.argtypes = [i32, i32, i32]
+    L.gs_iso_workspace_bytes.restype = i64
+    L.gs_iso_count.argtypes = [vp, vp, i32, i32, i32, ctypes.c_float, vp, P(i64)]
+    L.gs_iso_emit.argtypes = [vp, vp, i32, i32, i32, ctypes.c_float, P(ctypes.c_float), P(ctypes.c_float), vp, vp, vp,
+                              i64]
     L.gs_init_gaussians.argtypes = [vp, vp, vp, i64, vp, i64, ctypes.c_float, ctypes.c_float, P(gs_params)]
     L.gs_image_metrics.argtypes = [vp, vp, vp, P(ctypes.c_double), P(ctypes.c_double)]
     L.gs_serve_timeline.argtypes = [vp, P(ctypes.c_double), i32, P(i32), P(i64)]
@@ -331,15 +336,16 @@ class Context:
         nz, ny, nx = volume.shape
         o = (ctypes.c_float * 3)(*[float(x) for x in origin])
         h = (ctypes.c_float * 3)(*[float(x) for x in spacing])
-        cnt = ctypes.c_int64()
-        self._check(self.L.gs_iso_crossings(self.h, ctypes.c_void_p(volume.data_ptr()), nx, ny, nz, float(iso), o, h,
-                                            None, None, 0, ctypes.byref(cnt)), "gs_iso_crossings")
+        vol, cnt = ctypes.c_void_p(volume.data_ptr()), ctypes.c_int64()
+        work = torch.empty(self.L.gs_iso_workspace_bytes(nx, ny, nz), device=volume.device, dtype=torch.uint8)
+        wp = ctypes.c_void_p(work.data_ptr())
+        self._check(self.L.gs_iso_count(self.h, vol, nx, ny, nz, float(iso), wp, ctypes.byref(cnt)),
+                    "gs_iso_crossings")
         m = cnt.value
         pts = torch.empty((max(m, 1), 3), device=volume.device, dtype=torch.float32)
         nrm = torch.empty_like(pts)
-        self._check(self.L.gs_iso_crossings(self.h, ctypes.c_void_p(volume.data_ptr()), nx, ny, nz, float(iso), o, h,
-                                            ctypes.c_void_p(pts.data_ptr()), ctypes.c_void_p(nrm.data_ptr()), m,
-                                            ctypes.byref(cnt)), "gs_iso_crossings")
+        self._check(self.L.gs_iso_emit(self.h, vol, nx, ny, nz, float(iso), o, h, wp, ctypes.c_void_p(pts.data_ptr()),
+                                       ctypes.c_void_p(nrm.data_ptr()), m), "gs_iso_crossings")
         return pts[:m], nrm[:m]
 
     def gs_init_gaussians(self, points: torch.Tensor, normals: torch.Tensor, out: torch.Tensor, n: int, deg: int,
