@@ -87,7 +87,7 @@ struct gs_ctx {
       target_slot, host_tgt0, host_tgt1, pair_stats, cells, vismask, ssim_table, ssim_partials, ssim_sums,
       init_pts, init_scales, knn_part, knn_table, ord_keys0, ord_keys1, ord_vals0, ord_vals1, ord_total, ord_hist,
       ord_hist_scan, ord_lookback, ord_counters, ord_views, tile_order, vis_sums, vis_offsets, dtotal, dkeys0,
-      dkeys1, dvals0, dvals1, dhist, dhist_scan, dlookback, elookback, dorder, torder, iso_work;
+      dkeys1, dvals0, dvals1, dhist, dhist_scan, dlookback, elookback, dorder, torder, iso_work, densify_source;
 
   // launch accounting and optional per-kernel event timing
   struct KStat {
@@ -435,7 +435,7 @@ void gs_destroy(gs_ctx* c) {
                     &c->ord_vals0, &c->ord_vals1, &c->ord_total, &c->ord_hist, &c->ord_hist_scan, &c->ord_lookback,
                     &c->ord_counters, &c->ord_views, &c->tile_order, &c->vis_sums, &c->vis_offsets, &c->dtotal,
                     &c->dkeys0, &c->dkeys1, &c->dvals0, &c->dvals1, &c->dhist, &c->dhist_scan, &c->dlookback,
-                    &c->elookback, &c->dorder, &c->torder, &c->iso_work};
+                    &c->elookback, &c->dorder, &c->torder, &c->iso_work, &c->densify_source};
   for (DevBuf* b : bufs)
     if (b->p) cudaFree(b->p);
   for (const auto& p : c->pending) {
@@ -1416,7 +1416,7 @@ gs_status gs_densify(gs_ctx* c, const gs_params* p, const gs_params* m, const gs
   if (m_out->stride != p_out->stride || v_out->stride != p_out->stride)
     return fail(c, GS_EINVAL, "p_out, m_out, v_out must share the stride");
   set_device(c);
-  const int64_t nb = (p->n + 255) / 256;
+  const int64_t nb = densify_blocks(p->n);
   GS_TRY(ensure(c, c->block_sums, sizeof(uint32_t) * nb));
   GS_TRY(ensure(c, c->block_offsets, sizeof(uint32_t) * nb));
   GS_TRY(ensure(c, c->total, sizeof(uint64_t) * (1 + kMaxViews) +
@@ -1441,7 +1441,7 @@ gs_status gs_densify(gs_ctx* c, const gs_params* p, const gs_params* m, const gs
   uint64_t* total = P<uint64_t>(c->total);
   {
     LaunchScope ls(c, "densify");
-    launch_densify(a, false, c->stream);
+    launch_densify_count(a, c->stream);
   }
   {
     LaunchScope ls(c, "scan_block_sums", 2);
@@ -1460,9 +1460,11 @@ gs_status gs_densify(gs_ctx* c, const gs_params* p, const gs_params* m, const gs
   a.mo = m_out->data;
   a.vo = v_out->data;
   a.out_stride = p_out->stride;
+  GS_TRY(ensure(c, c->densify_source, sizeof(uint32_t) * cnt));
+  a.source = P<uint32_t>(c->densify_source);
   {
-    LaunchScope ls(c, "densify");
-    launch_densify(a, true, c->stream);
+    LaunchScope ls(c, "densify", cnt > 0 ? 2 : 0);
+    launch_densify_emit(a, (int64_t)cnt, c->stream);
   }
   GS_CHECK_LAUNCH(c);
   c->projected = c->sorted = c->rastered = c->cells_ready = false;

@@ -272,8 +272,12 @@ struct DensifyArgs {
   float* mo;
   float* vo;
   int64_t out_stride;
+  uint32_t* source;  // [outputs] input Gaussian of each output and what it takes from it
 };
-void launch_densify(const DensifyArgs& a, bool emit, cudaStream_t s);
+int64_t densify_blocks(int64_t n);
+void launch_densify_count(const DensifyArgs& a, cudaStream_t s);
+// 2 kernels (none for n_out == 0)
+void launch_densify_emit(const DensifyArgs& a, int64_t n_out, cudaStream_t s);
 
 struct AdamArgs {
   float* p;

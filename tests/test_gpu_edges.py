@@ -56,3 +56,33 @@ def test_crossings_of_ragged_volumes(shape):
         cos = np.sum(nrm.cpu().numpy().astype(np.float64) * rn, axis=1)
         assert cos.min() > 1 - 1e-5
     ctx.close()
+
+
+@pytest.mark.parametrize("n,split_n,opacity", [(1, 2, 2.0), (1023, 1, None), (1024, 3, None), (1025, 4, None),
+                                               (2500, 2, -9.0), (2049, 2, None)])
+def test_densify_blocks_and_sample_counts(n, split_n, opacity):
+    rng = np.random.default_rng(n + split_n)
+    deg, stride = 1, n + (-n) % 4
+    P = 11 + 3 * (deg + 1) ** 2
+    p = rng.normal(size=(P, stride)).astype(np.float32)
+    p[3:6] = rng.uniform(-6.0, -3.0, (3, stride))
+    p[10] = opacity if opacity is not None else rng.uniform(-7.0, 3.0, stride)
+    m, v = (rng.normal(size=(P, stride)).astype(np.float32) for _ in range(2))
+    avg = np.where(rng.uniform(size=n) < 0.6, rng.uniform(3e-4, 1e-3, n), rng.uniform(0.0, 1e-4, n))
+    cnt = rng.integers(0, 5, n).astype(np.float32)
+    grad = (avg * cnt).astype(np.float32)
+    noise = rng.normal(size=(n, split_n, 3)).astype(np.float32)
+    f64 = [a.astype(np.float64) for a in (p[:, :n], m[:, :n], v[:, :n], grad, cnt, noise)]
+    rp, rm, rv, _ = OD.densify(*f64, tau=2e-4, dense=0.01, extent=2.0, min_opacity=0.005, split_n=split_n)
+    outs = [torch.full((P, 4 * stride), float("nan"), device="cuda") for _ in range(3)]
+    ctx = gs.Context(0)
+    nout = ctx.gs_densify(dev(p), dev(m), dev(v), n, deg, dev(grad), dev(cnt), dev(noise),
+                          dict(scene_extent=2.0, split_n=split_n), *outs)
+    ctx.gs_sync()
+    assert nout == rp.shape[1]
+    po, mo, vo = (o[:, :nout].cpu().numpy().astype(np.float64) for o in outs)
+    np.testing.assert_allclose(po, rp, rtol=1e-6, atol=2e-6)
+    np.testing.assert_array_equal(mo, rm)
+    np.testing.assert_array_equal(vo, rv)
+    assert all(bool(torch.isnan(o[:, nout:]).all()) for o in outs)  # nothing past the outputs
+    ctx.close()
