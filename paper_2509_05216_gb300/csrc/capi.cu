@@ -63,7 +63,7 @@ struct gs_ctx {
   cudaEvent_t tgt_free[2] = {nullptr, nullptr};
   int64_t host_launches = 0;
   int raster_fwd = 2;  // compositing variants (pixels per thread; 8 = one warp per tile)
-  int raster_bwd = 2;
+  int raster_bwd = 4;
   int bwd_direct = 2;  // per-lane gradient atomics when at most this many lanes contribute
   int sort_passes = 0;  // LSD passes of the last tile sort
   int sort_items = 16;  // keys per thread of a sort partition

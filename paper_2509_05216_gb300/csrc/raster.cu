@@ -830,12 +830,403 @@ __global__ void __launch_bounds__(Geo<PPT>::THREADS, PPT == 2 ? 8 : 1) raster_bw
   }
 }
 
+__device__ __forceinline__ uint32_t bit_of(int j) {  // 1 << j, 0 for j = -1
+  uint32_t b;
+  asm("shl.b32 %0, 1, %1;" : "=r"(b) : "r"(j));
+  return b;
+}
+
+// Forward of one pixel pair by the walk of contribution cells.  T is the
+// transmittance, negative once the pixel has stopped: a stopped pixel's
+// product with 1 - alpha is negative too, so it fails the same test that
+// stops a live one and needs no flag of its own.  mx, my collect the
+// contributing entries' bits.
+__device__ __forceinline__ void fwd_cell_pair(const float2& cC, const float2& a1, const float2& a0, const float2& op,
+                                              const float2& r, const float2& g, const float2& b, float2 dy,
+                                              uint32_t jbit, float2& T, float2 (&C)[3], uint32_t& mx, uint32_t& my) {
+  const float2 p2 = __ffma2_rn(__ffma2_rn(cC, dy, a1), dy, a0);
+  const float2 raw = __fmul2_rn(op, make_float2(ex2_approx(p2.x), ex2_approx(p2.y)));
+  const float ax = fminf(kAlphaClamp, raw.x), ay = fminf(kAlphaClamp, raw.y);
+  const float2 Tn = __fmul2_rn(T, __fadd2_rn(bc2(1.f), make_float2(-ax, -ay)));
+  const bool okx = !(p2.x > 0.f) && !(ax < kAlphaSkip);
+  const bool oky = !(p2.y > 0.f) && !(ay < kAlphaSkip);
+  const bool accx = okx && !(Tn.x < kTStop), accy = oky && !(Tn.y < kTStop);
+  const float2 aT = __fmul2_rn(make_float2(ax, ay), T);
+  const float2 w = make_float2(accx ? aT.x : 0.f, accy ? aT.y : 0.f);
+  C[0] = __ffma2_rn(r, w, C[0]);
+  C[1] = __ffma2_rn(g, w, C[1]);
+  C[2] = __ffma2_rn(b, w, C[2]);
+  if (okx) T.x = accx ? Tn.x : -fabsf(T.x);
+  if (oky) T.y = accy ? Tn.y : -fabsf(T.y);
+  if (accx) mx |= jbit;
+  if (accy) my |= jbit;
+}
+
+// One step of the transposition of a 32 x 32 bit matrix held as one row per
+// lane: lanes that differ in bit s exchange the halves of their rows' bits
+// whose index differs in bit s.
+template <int S>
+__device__ __forceinline__ uint32_t transpose_step(uint32_t x, int lane) {
+  constexpr uint32_t kLow = S == 16 ? 0x0000ffffu : S == 8 ? 0x00ff00ffu : S == 4 ? 0x0f0f0f0fu : S == 2 ? 0x33333333u : 0x55555555u;
+  const uint32_t y = __shfl_xor_sync(0xffffffffu, x, S);
+  const bool up = (lane & S) != 0;
+  const uint32_t keep = up ? ~kLow : kLow;
+  const uint32_t rot = __funnelshift_l(y, y, up ? 32 - S : S);
+  return (x & keep) | (rot & ~keep);
+}
+__device__ __forceinline__ uint32_t transpose32(uint32_t x, int lane) {
+  x = transpose_step<16>(x, lane);
+  x = transpose_step<8>(x, lane);
+  x = transpose_step<4>(x, lane);
+  x = transpose_step<2>(x, lane);
+  return transpose_step<1>(x, lane);
+}
+
+// Forward with 2 NP pixels per thread (NP = 1: 4 warps per tile, 8 x 8 pixels
+// each; NP = 2: 2 warps, 16 x 8).  The warp's pixels are 2 x 4 cells, 4 / NP
+// lanes each; every cell walks the entries whose alpha >= 1/255 box reaches
+// it (the box test only removes pairs that the per-pixel test would skip; the
+// exact ellipse test on top of it costs more than the walk steps it saves).
+template <int NP>
+struct FwdCells {
+  static constexpr int LPC = 4 / NP, NC = 32 / LPC, NCX = NP == 1 ? 4 : 8;  // lanes per cell, cells, cells per row
+  static constexpr int NW = 32 / NC;                                        // warps per tile
+};
+
+template <int NP>
+__global__ void __launch_bounds__(32 * FwdCells<NP>::NW) raster_fwd_cells_kernel(RasterArgs a) {
+  using G = FwdCells<NP>;
+  constexpr int PPT = 2 * NP;
+  // slot 0: a neutral record (opacity 0) that an idle cell evaluates without effect
+  __shared__ float4 s0[G::NW][33], s1[G::NW][33];
+  __shared__ float s2[G::NW][33];
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t bin = a.tile_order ? a.tile_order[blockIdx.x] : (int64_t)blockIdx.x;
+  const int v = view_of_bin(a.views, a.B, (int)bin);
+  const ViewRec& V = a.views[v];
+  const int tile = (int)bin - V.tile_offset;
+  // the warp's first cell column and row in the tile, and the lane's cell
+  const int wcx = NP == 1 ? 4 * (w & 1) : 0, wcy = NP == 1 ? 2 * (w >> 1) : 2 * w;
+  const int c = lane / G::LPC;
+  const int cx = wcx + c % G::NCX, cy = wcy + c / G::NCX;
+  const int tx0 = (tile % V.gw) * kTile, ty0 = (tile / V.gw) * kTile;
+  const int px = tx0 + 2 * cx + (lane & 1);
+  const int py0 = ty0 + 4 * cy + (NP == 1 ? (lane & 2) : 0);
+  const float wx0 = (float)(tx0 + 2 * wcx), wy0 = (float)(ty0 + 4 * wcy);
+  const uint2 rg = a.ranges[bin];
+  const int n = (int)(rg.y - rg.x);
+  const uint32_t* __restrict__ vals = *a.vals;
+  float2 T2[NP], C2[NP][3];
+  uint32_t last[PPT];
+#pragma unroll
+  for (int j = 0; j < NP; j++) {
+    // a pixel outside the image is a stopped one
+    T2[j] = make_float2(px < V.W && py0 + 2 * j < V.H ? 1.f : -1.f, px < V.W && py0 + 2 * j + 1 < V.H ? 1.f : -1.f);
+    C2[j][0] = C2[j][1] = C2[j][2] = bc2(0.f);
+    last[2 * j] = last[2 * j + 1] = 0;
+  }
+  if (lane == 0) {
+    s0[w][0] = s1[w][0] = make_float4(0.f, 0.f, 0.f, 0.f);
+    s2[w][0] = 0.f;
+  }
+  const float fpx = (float)px, nfy = -(float)py0;
+  const uint32_t cell_lanes = ((1u << G::LPC) - 1u) << (lane & ~(G::LPC - 1));
+  const bool owner = (lane & (G::LPC - 1)) == 0;
+  uint32_t* const cells = a.cells ? a.cells + cells_offset(rg.x, bin) + cx + 8 * cy : nullptr;
+  int b0 = 0;
+  // software pipeline over the batches: the record of batch k + 1 and the
+  // index of batch k + 2 are loaded while batch k is walked
+  uint32_t g_next = lane < n ? vals[rg.x + lane] : 0u;
+  uint32_t g_after = 32 + lane < n ? vals[rg.x + 32 + lane] : 0u;
+  float4 p0 = make_float4(0.f, 0.f, 0.f, 0.f), p1 = p0, p2 = p0;
+  if (lane < n) stage_one(a, v, g_next, p0, p1, p2);
+  for (; b0 < n; b0 += 32) {
+    bool live = false;
+#pragma unroll
+    for (int j = 0; j < NP; j++) live |= T2[j].x > 0.f || T2[j].y > 0.f;
+    const uint32_t alive = __ballot_sync(0xffffffffu, live);
+    if (alive == 0u) break;
+    const int i = b0 + lane;
+    // bit l: the record's box reaches the cell of lane l
+    uint32_t hits = 0;
+    if (i < n) {
+      s0[w][1 + lane] = p0;
+      s1[w][1 + lane] = p1;
+      s2[w][1 + lane] = p2.x;
+      const float lox = p0.x - p2.y, hix = p0.x + p2.y, loy = p0.y - p2.z, hiy = p0.y + p2.z;
+#pragma unroll
+      for (int q = 0; q < G::NCX; q++)
+        hits |= hix >= wx0 + (float)(2 * q) && lox <= wx0 + (float)(2 * q + 1) ? ((1u << G::LPC) - 1u) << (q * G::LPC) : 0u;
+      const bool top = hiy >= wy0 && loy <= wy0 + 3.f, bottom = hiy >= wy0 + 4.f && loy <= wy0 + 7.f;
+      hits = (top ? hits : 0u) | (bottom ? hits << 16 : 0u);
+    }
+    {
+      const int i1 = i + 32, i2 = i + 64;
+      if (i1 < n) stage_one(a, v, g_after, p0, p1, p2);
+      g_after = i2 < n ? vals[rg.x + i2] : 0u;
+    }
+    // the entries that reach the lane's cell; none once its pixels have stopped
+    uint32_t mask = transpose32(hits, lane);
+    if ((alive & cell_lanes) == 0u) mask = 0u;
+    const int iters = (int)__reduce_max_sync(0xffffffffu, (uint32_t)__popc(mask));
+    uint32_t m[PPT];
+#pragma unroll
+    for (int k = 0; k < PPT; k++) m[k] = 0u;
+    __syncwarp();
+    for (int it = 0; it < iters; it++) {
+      const int slot = __ffs((int)mask);  // 0: the neutral record
+      mask &= mask - 1u;
+      const float4 q0 = s0[w][slot];
+      const float4 q1 = s1[w][slot];
+      const float blue = s2[w][slot];
+      const uint32_t jbit = bit_of(slot - 1);
+      const float dx = __fsub_rn(q0.x, fpx);
+      const float a0 = __fmul_rn(q0.z, __fmul_rn(dx, dx));
+      const float a1 = __fmul_rn(q0.w, dx);
+      const float2 cC = bc2(q1.x), A1 = bc2(a1), A0 = bc2(a0), op = bc2(q1.y);
+      const float2 r = bc2(q1.z), g = bc2(q1.w), b = bc2(blue), qy = bc2(q0.y);
+#pragma unroll
+      for (int j = 0; j < NP; j++)
+        fwd_cell_pair(cC, A1, A0, op, r, g, b,
+                      __fadd2_rn(qy, make_float2(nfy - (float)(2 * j), nfy - (float)(2 * j + 1))), jbit, T2[j], C2[j],
+                      m[2 * j], m[2 * j + 1]);
+    }
+    __syncwarp();
+    uint32_t e = 0;
+#pragma unroll
+    for (int k = 0; k < PPT; k++) {
+      if (m[k]) last[k] = (uint32_t)(b0 + 32 - __clz((int)m[k]));
+      e |= m[k];
+    }
+    // the batch's contribution masks: per cell, the OR of its lanes' masks
+    if (cells) {
+#pragma unroll
+      for (int x = 1; x < G::LPC; x <<= 1) e |= __shfl_xor_sync(0xffffffffu, e, x);
+      if (owner) cells[b0] = e;
+    }
+  }
+  // batches after the warp's pixels all stopped: nothing contributed
+  if (cells && owner)
+    for (; b0 < n; b0 += 32) cells[b0] = 0u;
+  const int64_t plane = (int64_t)V.W * V.H;
+  float* img = a.image ? a.image + 3 * V.pix_offset : nullptr;
+  const float* tgt = a.target_slot ? *a.target_slot : a.target;
+  const bool l1 = tgt != nullptr;
+  // the targets are loaded before any store (the stores could alias them,
+  // which would serialise each load behind the stores before it)
+  float tv[PPT][3];
+#pragma unroll
+  for (int k = 0; k < PPT; k++) {
+    const bool in = l1 && px < V.W && py0 + k < V.H;
+    const int64_t p = (int64_t)(py0 + k) * V.W + px;
+#pragma unroll
+    for (int ch = 0; ch < 3; ch++) tv[k][ch] = in ? __ldg(tgt + 3 * V.pix_offset + ch * plane + p) : 0.f;
+  }
+  float l1sum = 0.f;
+#pragma unroll
+  for (int k = 0; k < PPT; k++) {
+    if (px >= V.W || py0 + k >= V.H) continue;
+    const int64_t p = (int64_t)(py0 + k) * V.W + px;
+    const float T = fabsf(k % 2 ? T2[k / 2].y : T2[k / 2].x);
+    float cc[3];
+#pragma unroll
+    for (int ch = 0; ch < 3; ch++) {
+      cc[ch] = fmaf(T, V.bg[ch], k % 2 ? C2[k / 2][ch].y : C2[k / 2][ch].x);
+      if (img) img[ch * plane + p] = cc[ch];
+    }
+    a.tfinal[V.pix_offset + p] = T;
+    a.nlast[V.pix_offset + p] = last[k];
+    if (l1) {
+      // L1 loss mean |C - target| and its gradient sign(C - target) / count
+      float* gd = a.l1_grad + 3 * V.pix_offset;
+#pragma unroll
+      for (int ch = 0; ch < 3; ch++) {
+        const float d = cc[ch] - tv[k][ch];
+        l1sum += fabsf(d);
+        gd[ch * plane + p] = d > 0.f ? a.inv_count : (d < 0.f ? -a.inv_count : 0.f);
+      }
+    }
+  }
+  if (l1) {
+    // one partial sum per warp (fixed order: deterministic)
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) l1sum += __shfl_down_sync(0xffffffffu, l1sum, off);
+    // indexed by tile, so the loss does not depend on the tile order
+    if (lane == 0) a.l1_partial[bin * G::NW + w] = l1sum;
+  }
+}
+
+// Backward with 4 pixels per thread: a warp owns the upper or lower 16 x 8
+// pixels of its tile, 16 contribution cells; a pair of lanes owns a cell, each
+// lane one column of 4 pixels (two packed row pairs).  Against 2 pixels per
+// thread, a walked entry's set-up and its reduction (one exchange between the
+// two lanes instead of two levels and a gather over four) serve twice the
+// pixels.
+//
+// The warp pays for the pair of lanes with the most entries, so the pairs may
+// run ahead: two batches are staged, a pair that has finished the older one
+// goes on with the newer, and the warp moves on when every pair has finished
+// the older.
+struct Bwd4Smem {
+  // two halves of a neutral record (opacity 0: an idle pair evaluates it
+  // without effect) and 32 records
+  float4 s0[2 * 33], s1[2 * 33];
+  float2 sx[2 * 33];  // blue, bits of the Gaussian
+};
+
+__global__ void __launch_bounds__(64, 10) raster_bwd4_kernel(RasterArgs a, int64_t bins) {
+  __shared__ Bwd4Smem smem[2];
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  Bwd4Smem& sm = smem[w];
+  const int64_t bin = a.tile_order ? a.tile_order[blockIdx.x] : (int64_t)blockIdx.x;
+  const int v = view_of_bin(a.views, a.B, (int)bin);
+  const ViewRec& V = a.views[v];
+  const int tile = (int)bin - V.tile_offset;
+  const int cell = 16 * w + (lane >> 1);
+  const int px = (tile % V.gw) * kTile + 2 * (cell & 7) + (lane & 1);
+  const int py0 = (tile / V.gw) * kTile + 4 * (cell >> 3);
+  const uint2 rg = a.ranges[bin];
+  const uint32_t* __restrict__ vals = *a.vals;
+  const int64_t plane = (int64_t)V.W * V.H;
+  const float* dimg = a.dimage + 3 * V.pix_offset;
+
+  // per pixel: T (running, from T_final backwards), dL/dC, sum_c dC_c S_c
+  // (S = colour behind), T_final * sum_c dC_c bg_c, and n_last
+  float2 T2[2], dC2[2][3], dCS2[2], bgd2[2];
+  uint32_t nl[4], mymax = 0;
+  {
+    float T[4], dC[4][3], bgd[4];
+#pragma unroll
+    for (int k = 0; k < 4; k++) {
+      const bool in = px < V.W && py0 + k < V.H;
+      const int64_t p = (int64_t)(py0 + k) * V.W + px;
+      T[k] = in ? a.tfinal[V.pix_offset + p] : 1.f;
+      nl[k] = in ? a.nlast[V.pix_offset + p] : 0u;
+#pragma unroll
+      for (int c = 0; c < 3; c++) dC[k][c] = in ? dimg[c * plane + p] : 0.f;
+      bgd[k] = T[k] * (dC[k][0] * V.bg[0] + dC[k][1] * V.bg[1] + dC[k][2] * V.bg[2]);
+      mymax = max(mymax, nl[k]);
+    }
+#pragma unroll
+    for (int j = 0; j < 2; j++) {
+      T2[j] = make_float2(T[2 * j], T[2 * j + 1]);
+#pragma unroll
+      for (int c = 0; c < 3; c++) dC2[j][c] = make_float2(dC[2 * j][c], dC[2 * j + 1][c]);
+      dCS2[j] = bc2(0.f);
+      bgd2[j] = make_float2(bgd[2 * j], bgd[2 * j + 1]);
+    }
+  }
+  const int total = (int)__reduce_max_sync(0xffffffffu, mymax);
+  if (total == 0) return;
+  if (lane < 2) {
+    sm.s0[33 * lane] = sm.s1[33 * lane] = make_float4(0.f, 0.f, 0.f, 0.f);
+    sm.sx[33 * lane] = make_float2(0.f, 0.f);
+  }
+  const float fpx = (float)px, nfy = -(float)py0;
+  const uint32_t* __restrict__ cells = a.cells + cells_offset(rg.x, bin) + cell;
+  float* const geo = a.g2d + kG2dGeo * (int64_t)v * a.stride;
+  float* const col = a.g2d + kG2dGeo * (int64_t)a.B * a.stride + kG2dCol * (int64_t)v * a.stride;
+  const bool odd = lane & 1;
+  const uint32_t pair = 3u << (lane & 30);
+
+  int b = ((total - 1) >> 5) << 5;  // next batch to stage
+  uint32_t cm_next = cells[b];
+  // the older and the newer staged batch: entries left in the pair's cell,
+  // list position of the first entry, slot before the first record
+  uint32_t mo = 0, mn = 0;
+  int so = 0, sn = 0, po = 0, pn = 33;
+  while (true) {
+    // the next batch in which an entry contributed to a pixel of the warp
+    uint32_t any = 0;
+    mn = 0;
+    for (; b >= 0 && any == 0u; b -= 32) {
+      const int nb = total - b;
+      mn = nb >= 32 ? cm_next : cm_next & ((1u << nb) - 1u);
+      if (b >= 32) cm_next = cells[b - 32];
+      any = __reduce_or_sync(0xffffffffu, mn);
+      sn = b;
+    }
+    if (any) {
+      if ((any >> lane) & 1u) {
+        const uint32_t g = vals[rg.x + sn + lane];
+        float4 n0, n1, n2;
+        stage_one(a, v, g, n0, n1, n2);
+        sm.s0[pn + 1 + lane] = n0;
+        sm.s1[pn + 1 + lane] = n1;
+        sm.sx[pn + 1 + lane] = make_float2(n2.x, __uint_as_float(g));
+      }
+      __syncwarp();
+    }
+    const int iters = (int)__reduce_max_sync(0xffffffffu, (uint32_t)__popc(mo));
+    for (int it = 0; it < iters; it++) {  // back to front
+      const bool older = mo != 0u;
+      const uint32_t m = older ? mo : mn;
+      const int j = 31 - __clz(m);  // -1: the neutral record
+      const uint32_t left = m ^ bit_of(j);
+      mo = older ? left : 0u;
+      mn = older ? mn : left;
+      const int slot = (older ? po : pn) + 1 + j;
+      const uint32_t idx = (uint32_t)((older ? so : sn) + j);
+      const float4 q0 = sm.s0[slot];
+      const float4 q1 = sm.s1[slot];
+      const float2 qx = sm.sx[slot];
+      const float dx = __fsub_rn(q0.x, fpx);
+      const float dx2 = __fmul_rn(dx, dx);
+      const float a0 = __fmul_rn(q0.z, dx2);
+      const float a1 = __fmul_rn(q0.w, dx);
+      const float2 cC = bc2(q1.x), A1 = bc2(a1), A0 = bc2(a0), op = bc2(q1.y);
+      const float2 r = bc2(q1.z), g = bc2(q1.w), bl = bc2(qx.x), qy = bc2(q0.y);
+      float2 racc[3] = {bc2(0.f), bc2(0.f), bc2(0.f)}, oacc = bc2(0.f);
+      float2 S0 = bc2(0.f), S1 = bc2(0.f), S2 = bc2(0.f);
+      bool on = false;
+#pragma unroll
+      for (int jp = 0; jp < 2; jp++) {
+        const float2 ny = make_float2(nfy - (float)(2 * jp), nfy - (float)(2 * jp + 1));
+        on |= bwd_pair2(idx < nl[2 * jp], idx < nl[2 * jp + 1], cC, A1, A0, op, r, g, bl, __fadd2_rn(qy, ny), T2[jp],
+                        dCS2[jp], dC2[jp], bgd2[jp], racc, oacc, S0, S1, S2);
+      }
+      // mean and conic gradients of p2 from the moments of dL/dp2
+      const float m0 = S0.x + S0.y, m1 = S1.x + S1.y;
+      const float g0 = fmaf(q0.w, m1, 2.f * q0.z * dx * m0);  // sum dp (cB dy + 2 cA dx)
+      const float g1 = fmaf(2.f * q1.x, m1, a1 * m0);         // sum dp (2 cC dy + cB dx)
+      const float g2 = dx2 * m0, g3 = dx * m1, g4 = S2.x + S2.y, g5 = oacc.x + oacc.y;
+      const float c0 = racc[0].x + racc[0].y, c1 = racc[1].x + racc[1].y, c2 = racc[2].x + racc[2].y;
+      // the pair's sums: the even lane takes the geometry record's first four
+      // values, the odd lane the other five
+      const float x0 = __shfl_xor_sync(0xffffffffu, odd ? g0 : g4, 1);
+      const float x1 = __shfl_xor_sync(0xffffffffu, odd ? g1 : g5, 1);
+      const float x2 = __shfl_xor_sync(0xffffffffu, odd ? g2 : c0, 1);
+      const float x3 = __shfl_xor_sync(0xffffffffu, odd ? g3 : c1, 1);
+      const float x4 = __shfl_xor_sync(0xffffffffu, c2, 1);
+      if (__ballot_sync(0xffffffffu, on) & pair) {
+        const int64_t gi = (int64_t)__float_as_uint(qx.y);
+        const float y0 = x0 + (odd ? g4 : g0), y1 = x1 + (odd ? g5 : g1);
+        const float y2 = x2 + (odd ? c0 : g2), y3 = x3 + (odd ? c1 : g3);
+        if (!odd) {
+          red_v4(geo + kG2dGeo * gi, y0 * grad_scale(0), y1 * grad_scale(1), y2 * grad_scale(2), y3 * grad_scale(3));
+        } else {
+          red_v2(geo + kG2dGeo * gi + 4, y0 * grad_scale(4), y1 * grad_scale(5));
+          red_v4(col + kG2dCol * gi, y2, y3, x4 + c2, 0.f);
+        }
+      }
+    }
+    if (!any) break;
+    // the newer batch becomes the older; its half is kept, the other is free
+    mo = mn;
+    so = sn;
+    const int t = po;
+    po = pn;
+    pn = t;
+    __syncwarp();
+  }
+}
+
 template <int PPT>
 void launch_shape(bool fwd, const RasterArgs& a, int64_t bins, cudaStream_t s) {
   using G = Geo<PPT>;
   const unsigned blocks = (unsigned)((bins + G::TPB - 1) / G::TPB);
-  if (fwd) raster_fwd_kernel<PPT><<<blocks, G::THREADS, 0, s>>>(a, bins);
-  else raster_bwd_kernel<PPT><<<blocks, G::THREADS, 0, s>>>(a, bins);
+  if constexpr (PPT != 2 && PPT != 4) if (fwd) raster_fwd_kernel<PPT><<<blocks, G::THREADS, 0, s>>>(a, bins);
+  if constexpr (PPT != 4) if (!fwd) raster_bwd_kernel<PPT><<<blocks, G::THREADS, 0, s>>>(a, bins);
 }
 
 int64_t raster_fwd_warps(int64_t bins, int ppt) {
@@ -945,9 +1336,9 @@ void launch_raster_fwd(const RasterArgs& a, int64_t bins, int ppt, cudaStream_t 
   if (bins == 0) return;
   switch (ppt) {
     case 1: launch_shape<1>(true, a, bins, s); break;
-    case 4: launch_shape<4>(true, a, bins, s); break;
+    case 4: raster_fwd_cells_kernel<2><<<(unsigned)bins, 64, 0, s>>>(a); break;
     case 8: launch_shape<8>(true, a, bins, s); break;
-    default: launch_shape<2>(true, a, bins, s); break;
+    default: raster_fwd_cells_kernel<1><<<(unsigned)bins, 128, 0, s>>>(a); break;
   }
 }
 
@@ -955,7 +1346,7 @@ void launch_raster_bwd(const RasterArgs& a, int64_t bins, int ppt, cudaStream_t 
   if (bins == 0) return;
   switch (ppt) {
     case 1: launch_shape<1>(false, a, bins, s); break;
-    case 4: launch_shape<4>(false, a, bins, s); break;
+    case 4: raster_bwd4_kernel<<<(unsigned)bins, 64, 0, s>>>(a, bins); break;
     case 8: launch_shape<8>(false, a, bins, s); break;
     default: launch_shape<2>(false, a, bins, s); break;
   }
