@@ -26,23 +26,25 @@ namespace gs {
 
 // ---------------------------------------------------------------- scan
 
-// Exclusive scan of the projection's per-(view, block) instance counts: block
-// v of the grid scans view v's nb counts (1024 threads looping over chunks)
-// and writes the view's total.
-__global__ void __launch_bounds__(1024) scan_block_sums_kernel(const uint32_t* __restrict__ sums,
-                                                                int64_t nb, uint32_t* __restrict__ offsets,
-                                                                uint64_t* __restrict__ view_total) {
+// Exclusive scan of per-(view, block) counts, of one or two kinds (the
+// projection's instances and visible pairs; blockIdx.y): block v of the grid
+// scans view v's nb counts (1024 threads looping over chunks) and writes the
+// view's total.  The last block to finish turns the view totals into segment
+// offsets: seg[v] = first of view v, seg[B] = *total.
+__global__ void __launch_bounds__(1024) scan_block_sums_kernel(ScanArgs a, uint32_t* ticket) {
   __shared__ uint64_t warp_tot[32];
   __shared__ uint64_t carry;
+  __shared__ bool s_last;
   const int v = blockIdx.x;
-  sums += (int64_t)v * nb;
-  offsets += (int64_t)v * nb;
+  const ScanArgs::Kind& k = a.kind[blockIdx.y];
+  const uint32_t* sums = k.sums + (int64_t)v * a.nb;
+  uint32_t* offsets = k.offsets + (int64_t)v * a.nb;
   if (threadIdx.x == 0) carry = 0;
   __syncthreads();
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  for (int64_t base = 0; base < nb; base += 1024) {
+  for (int64_t base = 0; base < a.nb; base += 1024) {
     const int64_t i = base + threadIdx.x;
-    uint64_t x = i < nb ? sums[i] : 0;
+    uint64_t x = i < a.nb ? sums[i] : 0;
     uint64_t inc = x;
 #pragma unroll
     for (int off = 1; off < 32; off <<= 1) {
@@ -63,31 +65,42 @@ __global__ void __launch_bounds__(1024) scan_block_sums_kernel(const uint32_t* _
     }
     __syncthreads();
     const uint64_t excl = carry + warp_tot[wid] + inc - x;
-    if (i < nb) offsets[i] = (uint32_t)excl;
+    if (i < a.nb) offsets[i] = (uint32_t)excl;
     __syncthreads();
     if (threadIdx.x == 1023) carry = excl + x;
     __syncthreads();
   }
-  if (threadIdx.x == 0) view_total[v] = carry;
-}
-
-// Segment offsets: seg[v] = first instance of view v, seg[B] = *total.
-__global__ void segment_offsets_kernel(const uint64_t* __restrict__ view_total, int B, uint32_t* __restrict__ seg,
-                                       uint64_t* __restrict__ total) {
-  if (threadIdx.x != 0) return;
-  uint64_t run = 0;
-  for (int v = 0; v < B; v++) {
-    seg[v] = (uint32_t)min(run, (uint64_t)0xffffffffu);
-    run += view_total[v];
+  if (threadIdx.x == 0) {
+    k.view_total[v] = carry;
+    __threadfence();
+    // (the ticket wraps to 0 with the last block)
+    const uint32_t blocks = gridDim.x * gridDim.y;
+    s_last = atomicInc(ticket, blocks - 1) == blocks - 1;
   }
-  seg[B] = (uint32_t)min(run, (uint64_t)0xffffffffu);
-  *total = run;
+  __syncthreads();
+  if (!s_last || wid >= (int)gridDim.y) return;
+  __threadfence();
+  const ScanArgs::Kind& q = a.kind[wid];
+  uint64_t run = 0;
+  for (int v0 = 0; v0 < a.B; v0 += 32) {
+    const uint64_t x = v0 + lane < a.B ? __ldcg(q.view_total + v0 + lane) : 0;
+    uint64_t inc = x;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+      const uint64_t y = __shfl_up_sync(0xffffffffu, inc, off);
+      if (lane >= off) inc += y;
+    }
+    if (v0 + lane < a.B) q.seg[v0 + lane] = (uint32_t)min(run + inc - x, (uint64_t)0xffffffffu);
+    run += __shfl_sync(0xffffffffu, inc, 31);
+  }
+  if (lane == 0) {
+    q.seg[a.B] = (uint32_t)min(run, (uint64_t)0xffffffffu);
+    *q.total = run;
+  }
 }
 
-void launch_scan_block_sums(const uint32_t* sums, int64_t nb, int B, uint32_t* offsets, uint64_t* view_total,
-                            uint32_t* seg, uint64_t* total, cudaStream_t s) {
-  scan_block_sums_kernel<<<B, 1024, 0, s>>>(sums, nb, offsets, view_total);
-  segment_offsets_kernel<<<1, 32, 0, s>>>(view_total, B, seg, total);
+void launch_scan_block_sums(const ScanArgs& a, int kinds, uint32_t* ticket, cudaStream_t s) {
+  scan_block_sums_kernel<<<dim3(a.B, kinds), 1024, 0, s>>>(a, ticket);
 }
 
 // ---------------------------------------------------------------- compaction
@@ -156,6 +169,25 @@ int64_t sort_partitions(int64_t count, int items, int segments) {
 size_t sort_lookback_bytes(int64_t count, int items, int segments) {
   const int64_t parts = sort_partitions(count, items, segments);
   return (size_t)(parts > 0 ? parts : 1) * kRadix * sizeof(uint32_t);
+}
+
+// Keys per thread of a sort of `capacity` keys in `segments` segments: the
+// configured ones, fewer for short segments.  A pass there is one round of
+// blocks, whose time is the chain of one block -- a ranking step per key of a
+// thread, then look-back rounds over the segment's partitions -- so the two
+// are balanced (4 keys up to 65,536 per segment, 8 up to 262,144): 10,000 Gaussians in one
+// view, the four depth passes 56 -> 38 us.
+int sort_items_for(int64_t capacity, int items, int segments) {
+  const int64_t per = capacity / segments;
+  return per <= 65536 ? 4 : per <= 262144 ? 8 : items;
+}
+
+// Partitions that sorts of up to `capacity` keys in up to `segments` segments
+// need at most, whatever the keys per thread.
+int64_t sort_partitions_reserve(int64_t capacity, int items, int segments) {
+  int64_t most = sort_partitions(capacity, items, segments);
+  most = std::max(most, sort_partitions(std::min<int64_t>(capacity, (int64_t)65537 * segments), 4, segments));
+  return std::max(most, sort_partitions(std::min<int64_t>(capacity, (int64_t)262145 * segments), 8, segments));
 }
 
 // Largest u in [0, B) with off[u] <= i (off nondecreasing): for i below
@@ -307,7 +339,7 @@ __global__ void __launch_bounds__(kSortThreads, MIN_BLOCKS) onesweep_pass_kernel
   const uint32_t nparts = a.part_off[a.B];
   if (tid == 0) {
     const uint32_t t = atomicAdd(a.counters + pass, 1u);
-    const uint32_t part = t < nparts ? (a.part_order ? a.part_order[t] : t) : nparts;  // status slot
+    const uint32_t part = t < nparts ? (a.part_order && a.B > 1 ? a.part_order[t] : t) : nparts;  // status slot
     sm.part = part;
     sm.timed_out = 0;
     if (part < nparts) {
@@ -511,6 +543,8 @@ static void launch_pass(const SortArgs& a, int pass, int64_t grid, cudaStream_t 
 template <typename KeyT>
 static void launch_pass_items(const SortArgs& a, int pass, int items, int64_t grid, cudaStream_t s) {
   switch (items) {
+    case 4: launch_pass<KeyT, 4, 4>(a, pass, grid, s); break;
+    case 8: launch_pass<KeyT, 8, 4>(a, pass, grid, s); break;
     case 12: launch_pass<KeyT, 12, 4>(a, pass, grid, s); break;
     case 20: launch_pass<KeyT, 20, 3>(a, pass, grid, s); break;
     case 24: launch_pass<KeyT, 24, 2>(a, pass, grid, s); break;
@@ -526,9 +560,12 @@ void launch_onesweep_pass(const SortArgs& a, int pass, int items, cudaStream_t s
 }
 
 // Exclusive scan of each (view, pass)'s 256 digit counts (block v of the
-// grid: view v), and whether the view's keys share one digit in the pass.
-__global__ void __launch_bounds__(kRadix) digit_scan_kernel(SortArgs a) {
+// grid: view v), and whether the view's keys share one digit in the pass.  The
+// last block to finish writes the pass control words and the first partition
+// of every view's segment (B <= 64 views, npass <= 8).
+__global__ void __launch_bounds__(kRadix) digit_scan_kernel(SortArgs a, int items, uint32_t* ticket) {
   __shared__ uint32_t wsum[kRadix / 32];
+  __shared__ bool s_last;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const int v = blockIdx.x;
   const uint32_t cap = (uint32_t)min(a.capacity, (int64_t)0xffffffff);
@@ -551,35 +588,45 @@ __global__ void __launch_bounds__(kRadix) digit_scan_kernel(SortArgs a) {
     if (tid == 0) a.single[v * 8 + p] = single ? 1u : 0u;
     __syncthreads();
   }
-}
-
-// Pass control words and the first partition of every view's segment (one
-// thread; B <= 64 views, npass <= 8).
-__global__ void sort_control_kernel(SortArgs a, int items) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  uint32_t parity = 0;
-  for (int p = 0; p < a.npass; p++) {
-    bool trivial = true;
-    for (int v = 0; v < a.B; v++) trivial &= a.single[v * 8 + p] != 0;
-    a.ctrl[p] = parity | (trivial ? kCtrlTrivial : 0u);
-    if (!trivial) parity ^= 1u;
+  if (tid == 0) {
+    __threadfence();
+    s_last = atomicInc(ticket, gridDim.x - 1) == gridDim.x - 1;  // (wraps to 0 with the last block)
   }
-  a.ctrl[a.npass] = parity;
-  const uint32_t cap = (uint32_t)min(a.capacity, (int64_t)0xffffffff);
+  __syncthreads();
+  if (!s_last || wid != 0) return;
+  __threadfence();
+  // lane p < npass: is pass p the same digit in every view
+  bool trivial = true;
+  if (lane < a.npass)
+    for (int u = 0; u < a.B; u++) trivial &= __ldcg(a.single + u * 8 + lane) != 0;
+  const uint32_t skip = __ballot_sync(0xffffffffu, trivial);
+  if (lane <= a.npass) {
+    const uint32_t parity = (uint32_t)__popc(~skip & ((1u << lane) - 1u)) & 1u;  // executed passes before it
+    a.ctrl[lane] = parity | (lane < a.npass && trivial ? kCtrlTrivial : 0u);
+  }
   const uint32_t tile = (uint32_t)(kSortThreads * items);
   uint32_t run = 0;
-  for (int v = 0; v < a.B; v++) {
-    a.part_off[v] = run;
-    const uint32_t cnt = min(a.seg[v + 1], cap) - min(a.seg[v], cap);
-    run += (cnt + tile - 1) / tile;
+  for (int v0 = 0; v0 < a.B; v0 += 32) {
+    uint32_t x = 0;
+    if (v0 + lane < a.B) x = (min(a.seg[v0 + lane + 1], cap) - min(a.seg[v0 + lane], cap) + tile - 1) / tile;
+    uint32_t inc = x;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, inc, off);
+      if (lane >= off) inc += y;
+    }
+    if (v0 + lane < a.B) a.part_off[v0 + lane] = run + inc - x;
+    run += __shfl_sync(0xffffffffu, inc, 31);
   }
-  a.part_off[a.B] = run;
+  if (lane == 0) a.part_off[a.B] = run;
 }
 
-void launch_digit_scan(const SortArgs& a, int items, cudaStream_t s) {
-  digit_scan_kernel<<<a.B, kRadix, 0, s>>>(a);
-  sort_control_kernel<<<1, 32, 0, s>>>(a, items);
-  if (a.part_order) {
+// Kernels of launch_digit_scan: one view takes its partitions in ticket order.
+int digit_scan_kernels(const SortArgs& a) { return a.part_order && a.B > 1 ? 2 : 1; }
+
+void launch_digit_scan(const SortArgs& a, int items, uint32_t* ticket, cudaStream_t s) {
+  digit_scan_kernel<<<a.B, kRadix, 0, s>>>(a, items, ticket);
+  if (a.part_order && a.B > 1) {
     const int64_t slots = sort_partitions(a.capacity, items, a.B);
     const int64_t blocks = std::min<int64_t>((slots + 255) / 256, (int64_t)sm_count() * 4);
     partition_order_kernel<<<(unsigned)std::max<int64_t>(blocks, 1), 256, 0, s>>>(a.part_off, a.B, a.part_order,
@@ -587,15 +634,18 @@ void launch_digit_scan(const SortArgs& a, int items, cudaStream_t s) {
   }
 }
 
-void launch_digit_histogram(const SortArgs& a, int64_t grid_hint, int items, cudaStream_t s) {
+void launch_digit_histogram(const SortArgs& a, int64_t grid_hint, int items, uint32_t* ticket, cudaStream_t s) {
   const int sms = sm_count();
-  // about 8 blocks per SM over all views, at least one per view
-  int64_t want = (grid_hint + 4095) / 4096;
+  // 512 keys per block, up to about 8 blocks per SM over all views, at least
+  // one per view (a block's rounds are a chain of shared-memory atomics:
+  // 111,000 keys in 3 views, counts and scans: 32 us with 4,096 keys per
+  // block, 22 us with 512)
+  int64_t want = (grid_hint + 511) / 512;
   want = want < 1 ? 1 : (want > (int64_t)sms * 8 ? (int64_t)sms * 8 : want);
   const unsigned per_view = (unsigned)std::max<int64_t>(1, want / a.B);
   if (a.key_bytes == 4) digit_histogram_kernel<uint32_t><<<dim3(per_view, a.B), 256, 0, s>>>(a);
   else digit_histogram_kernel<uint64_t><<<dim3(per_view, a.B), 256, 0, s>>>(a);
-  launch_digit_scan(a, items, s);
+  launch_digit_scan(a, items, ticket, s);
 }
 
 // ---------------------------------------------------------------- emission
@@ -608,13 +658,19 @@ constexpr uint64_t kEmitPrefix = 2ull << 62;
 constexpr uint64_t kEmitFailed = 3ull << 62;
 constexpr uint64_t kEmitValue = (1ull << 62) - 1;
 constexpr int kEmitThreads = 256;
-constexpr int kEmitItems = 16;  // visible pairs per thread
 constexpr int kEmitWarps = kEmitThreads / 32;
-constexpr int kEmitTile = kEmitThreads * kEmitItems;
-constexpr int kEmitChunkLane = kEmitWarps * kEmitItems / 32;  // chunks per lane in the block's chunk scan
-static_assert(kEmitWarps * kEmitItems % 32 == 0, "the chunk scan takes whole chunks per lane");
 
-int64_t emit_partitions(int64_t pairs, int segments) { return (pairs + kEmitTile - 1) / kEmitTile + segments; }
+// Visible pairs per thread: 16, or 4 where partitions of 4,096 pairs would
+// leave SMs without one (37,001 Gaussians in 3 views: 37 -> 17 us).
+constexpr int kEmitMany = 16, kEmitFew = 4;
+static int emit_items(int64_t pairs) {
+  return pairs >= (int64_t)kEmitThreads * kEmitMany * sm_count() * 2 ? kEmitMany : kEmitFew;
+}
+
+static int64_t emit_partitions(int64_t pairs, int segments) {
+  const int tile = kEmitThreads * emit_items(pairs);
+  return (pairs + tile - 1) / tile + segments;
+}
 
 __device__ __forceinline__ uint64_t warp_sum_u64(uint64_t x) {
 #pragma unroll
@@ -622,7 +678,7 @@ __device__ __forceinline__ uint64_t warp_sum_u64(uint64_t x) {
   return x;
 }
 
-// One partition of kEmitTile depth-sorted visible pairs of one view per
+// One partition of 256 kEmitItems depth-sorted visible pairs of one view per
 // block (partitions taken by ticket, so every earlier partition is running
 // or done).  Warp w holds chunks of 32 consecutive pairs; each pair's tile
 // rect comes from its (view, Gaussian) entry.  The block scans the chunks'
@@ -631,7 +687,11 @@ __device__ __forceinline__ uint64_t warp_sum_u64(uint64_t x) {
 // and each lane writes its pair's (tile, Gaussian) instances, tiles of a
 // rect in row-major order.  The tile digits of the following sort are
 // counted on the way (shared memory, one flush per block).
+template <int kEmitItems>
 __global__ void __launch_bounds__(kEmitThreads) emit_kernel(EmitArgs a) {
+  constexpr int kEmitTile = kEmitThreads * kEmitItems;
+  constexpr int kEmitChunkLane = kEmitWarps * kEmitItems / 32;  // chunks per lane in the block's chunk scan
+  static_assert(kEmitWarps * kEmitItems % 32 == 0, "the chunk scan takes whole chunks per lane");
   __shared__ uint32_t s_part[kMaxViews + 1];
   __shared__ uint32_t s_chunk[kEmitWarps * kEmitItems];
   __shared__ uint32_t s_hist[4][kRadix];
@@ -836,11 +896,18 @@ __global__ void __launch_bounds__(kEmitThreads) emit_kernel(EmitArgs a) {
 void launch_emit(const EmitArgs& a, int64_t pair_capacity, cudaStream_t s) {
   const int64_t grid = emit_partitions(pair_capacity, a.B);
   if (grid <= 0) return;
-  emit_kernel<<<(unsigned)grid, kEmitThreads, 0, s>>>(a);
+  if (emit_items(pair_capacity) == kEmitMany) emit_kernel<kEmitMany><<<(unsigned)grid, kEmitThreads, 0, s>>>(a);
+  else emit_kernel<kEmitFew><<<(unsigned)grid, kEmitThreads, 0, s>>>(a);
 }
 
 size_t emit_lookback_bytes(int64_t pair_capacity, int segments) {
   return (size_t)emit_partitions(pair_capacity, segments) * sizeof(uint64_t);
+}
+
+// Most bytes that emissions of up to this many pairs need.
+size_t emit_lookback_reserve(int64_t pair_capacity, int segments) {
+  const int64_t few = std::min<int64_t>(pair_capacity, (int64_t)kEmitThreads * kEmitMany * sm_count() * 2 - 1);
+  return std::max(emit_lookback_bytes(pair_capacity, segments), emit_lookback_bytes(few, segments));
 }
 
 // ---------------------------------------------------------------- tile ranges

@@ -34,7 +34,7 @@ struct gs_ctx {
   cudaStream_t stream = nullptr;
   gs_config cfg{};
   std::string err;
-  int* status_d = nullptr;
+  int* status_d = nullptr;     // status word, then the ticket of the scans' last block (0 between launches)
   int* status_h = nullptr;     // pinned
   uint64_t* pinned = nullptr;  // pinned scratch for small read-backs (16 KB)
   // pinned staging of the per-step constants (cameras, Adam constants) read by
@@ -81,13 +81,14 @@ struct gs_ctx {
   int64_t n = 0, stride = 0, bins = 0, pixels = 0, instances = 0, nblocks = 0;
   bool projected = false, sorted = false, rastered = false;
   std::vector<ViewRec> views_h;
+  uint2* ranges = nullptr;  // tile ranges of the last sort (in `zeroed`)
 
   DevBuf views, rec, rec3, tiles, block_sums, block_offsets, total, keys0, keys1, vals0, vals1,
-      hist, hist_scan, lookback, counters, ranges, tfinal, nlast, g2d, l1_partial, sorted_slots, adam_consts,
+      zeroed, hist_scan, tfinal, nlast, g2d, l1_partial, sorted_slots, adam_consts,
       target_slot, host_tgt0, host_tgt1, pair_stats, cells, vismask, ssim_table, ssim_partials, ssim_sums,
       init_pts, init_scales, knn_part, knn_table, ord_keys0, ord_keys1, ord_vals0, ord_vals1, ord_total, ord_hist,
       ord_hist_scan, ord_lookback, ord_counters, ord_views, tile_order, vis_sums, vis_offsets, dtotal, dkeys0,
-      dkeys1, dvals0, dvals1, dhist, dhist_scan, dlookback, elookback, dorder, torder, iso_work, densify_source;
+      dkeys1, dvals0, dvals1, dhist_scan, dorder, torder, iso_work, densify_source;
 
   // launch accounting and optional per-kernel event timing
   struct KStat {
@@ -295,6 +296,8 @@ struct SortWords {
   uint32_t* single;
 };
 
+static uint32_t* scan_ticket(gs_ctx* c) { return reinterpret_cast<uint32_t*>(c->status_d) + 1; }
+
 static size_t sort_words_bytes() {
   return sizeof(uint64_t) * (1 + kMaxViews) + sizeof(uint32_t) * (2 * (kMaxViews + 1) + 16 + 8 * kMaxViews);
 }
@@ -312,6 +315,36 @@ static SortWords sort_words(DevBuf& b) {
 
 constexpr int kDepthPasses = 4;  // 32 depth bits
 constexpr int kSortCounters = 24;  // tickets: [0, 8) tile sort, [8, 16) depth sort, [16] emission
+
+// What a binning zeroes first, in one buffer (one clear instead of seven):
+// tickets, digit counts and look-back statuses of both sorts and the emission,
+// tile ranges.
+struct BinZeroed {
+  uint32_t *counters, *dhist, *hist;
+  uint64_t* elookback;
+  uint32_t *dlookback, *lookback;
+  uint2* ranges;
+};
+
+static size_t bin_zeroed_layout(void* base, int B, int tpass, size_t elb, size_t dlb, size_t lb, int64_t bins,
+                                BinZeroed* z) {
+  size_t off = 0;
+  auto take = [&](size_t bytes) {
+    unsigned char* p = static_cast<unsigned char*>(base) + off;
+    off += (bytes + 15) / 16 * 16;
+    return static_cast<void*>(p);
+  };
+  BinZeroed q;
+  q.counters = static_cast<uint32_t*>(take(sizeof(uint32_t) * kSortCounters));
+  q.dhist = static_cast<uint32_t*>(take(sizeof(uint32_t) * (size_t)B * kDepthPasses * 256));
+  q.hist = static_cast<uint32_t*>(take(sizeof(uint32_t) * (size_t)B * tpass * 256));
+  q.elookback = static_cast<uint64_t*>(take(elb));
+  q.dlookback = static_cast<uint32_t*>(take(dlb * kDepthPasses));
+  q.lookback = static_cast<uint32_t*>(take(lb * tpass));
+  q.ranges = static_cast<uint2*>(take(sizeof(uint2) * bins));
+  if (z) *z = q;
+  return off;
+}
 
 // LSD passes of the tile sort: the bits of the largest tile index inside a view.
 static int tile_passes(int64_t view_tiles) {
@@ -351,17 +384,15 @@ gs_status ctx_reserve(gs_ctx* c, int64_t stride, int B, int64_t bins, int64_t pi
   GS_TRY(ensure_exact(c, c->dkeys1, sizeof(uint32_t) * pc));
   GS_TRY(ensure_exact(c, c->dvals0, sizeof(uint32_t) * pc));
   GS_TRY(ensure_exact(c, c->dvals1, sizeof(uint32_t) * pc));
-  GS_TRY(ensure_exact(c, c->ranges, sizeof(uint2) * bins));
-  GS_TRY(ensure_exact(c, c->hist, sizeof(uint32_t) * (size_t)B * 8 * 256));
   GS_TRY(ensure_exact(c, c->hist_scan, sizeof(uint32_t) * (size_t)B * 8 * 256));
-  GS_TRY(ensure_exact(c, c->dhist, sizeof(uint32_t) * (size_t)B * 8 * 256));
   GS_TRY(ensure_exact(c, c->dhist_scan, sizeof(uint32_t) * (size_t)B * 8 * 256));
-  GS_TRY(ensure_exact(c, c->lookback, sort_lookback_bytes(cap, c->sort_items, B) * tpass));
-  GS_TRY(ensure_exact(c, c->dlookback, sort_lookback_bytes(pc, c->sort_items, B) * kDepthPasses));
-  GS_TRY(ensure_exact(c, c->elookback, emit_lookback_bytes(pc, B)));
-  GS_TRY(ensure_exact(c, c->torder, sizeof(uint32_t) * sort_partitions(cap, c->sort_items, B)));
-  GS_TRY(ensure_exact(c, c->dorder, sizeof(uint32_t) * sort_partitions(pc, c->sort_items, B)));
-  GS_TRY(ensure_exact(c, c->counters, sizeof(uint32_t) * kSortCounters));
+  const int64_t tparts = sort_partitions_reserve(cap, c->sort_items, B);
+  const int64_t dparts = sort_partitions_reserve(pc, c->sort_items, B);
+  GS_TRY(ensure_exact(c, c->zeroed,
+                      bin_zeroed_layout(nullptr, B, tpass, emit_lookback_reserve(pc, B), sizeof(uint32_t) * 256 * dparts,
+                                        sizeof(uint32_t) * 256 * tparts, bins, nullptr)));
+  GS_TRY(ensure_exact(c, c->torder, sizeof(uint32_t) * tparts));
+  GS_TRY(ensure_exact(c, c->dorder, sizeof(uint32_t) * dparts));
   GS_TRY(ensure_exact(c, c->sorted_slots, 2 * sizeof(void*)));
   GS_TRY(ensure_exact(c, c->tfinal, sizeof(float) * pixels));
   GS_TRY(ensure_exact(c, c->nlast, sizeof(uint32_t) * pixels));
@@ -407,8 +438,8 @@ gs_status gs_create(gs_ctx** out, int device, const gs_config* cfg) {
   gs_ctx* c = new gs_ctx();
   c->device = device;
   c->cfg = conf;
-  if (cudaSetDevice(device) != cudaSuccess || cudaMalloc(&c->status_d, sizeof(int)) != cudaSuccess ||
-      cudaMemset(c->status_d, 0, sizeof(int)) != cudaSuccess ||
+  if (cudaSetDevice(device) != cudaSuccess || cudaMalloc(&c->status_d, 2 * sizeof(int)) != cudaSuccess ||
+      cudaMemset(c->status_d, 0, 2 * sizeof(int)) != cudaSuccess ||
       cudaMallocHost(&c->status_h, sizeof(int)) != cudaSuccess ||
       cudaMallocHost(&c->pinned, 16384) != cudaSuccess ||
       cudaMallocHost(&c->staging, kStagingBytes) != cudaSuccess ||
@@ -427,15 +458,13 @@ void gs_destroy(gs_ctx* c) {
   if (c->stream) cudaStreamSynchronize(c->stream);
   else cudaDeviceSynchronize();
   DevBuf* bufs[] = {&c->views, &c->rec, &c->rec3, &c->tiles, &c->block_sums, &c->block_offsets,
-                    &c->total, &c->keys0, &c->keys1, &c->vals0, &c->vals1, &c->hist, &c->hist_scan,
-                    &c->lookback, &c->counters, &c->ranges, &c->tfinal, &c->nlast, &c->g2d, &c->l1_partial,
+                    &c->total, &c->keys0, &c->keys1, &c->vals0, &c->vals1, &c->zeroed, &c->hist_scan, &c->tfinal, &c->nlast, &c->g2d, &c->l1_partial,
                     &c->sorted_slots, &c->adam_consts, &c->target_slot, &c->host_tgt0, &c->host_tgt1,
                     &c->pair_stats, &c->cells, &c->vismask, &c->ssim_table, &c->ssim_partials, &c->ssim_sums,
                     &c->init_pts, &c->init_scales, &c->knn_part, &c->knn_table, &c->ord_keys0, &c->ord_keys1,
                     &c->ord_vals0, &c->ord_vals1, &c->ord_total, &c->ord_hist, &c->ord_hist_scan, &c->ord_lookback,
                     &c->ord_counters, &c->ord_views, &c->tile_order, &c->vis_sums, &c->vis_offsets, &c->dtotal,
-                    &c->dkeys0, &c->dkeys1, &c->dvals0, &c->dvals1, &c->dhist, &c->dhist_scan, &c->dlookback,
-                    &c->elookback, &c->dorder, &c->torder, &c->iso_work, &c->densify_source};
+                    &c->dkeys0, &c->dkeys1, &c->dvals0, &c->dvals1, &c->dhist_scan, &c->dorder, &c->torder, &c->iso_work, &c->densify_source};
   for (DevBuf* b : bufs)
     if (b->p) cudaFree(b->p);
   for (const auto& p : c->pending) {
@@ -503,7 +532,9 @@ gs_status gs_project(gs_ctx* c, const gs_params* params, const gs_camera* cams, 
   GS_TRY(ensure(c, c->block_sums, sizeof(uint32_t) * B * nb));
   GS_TRY(ensure(c, c->vis_sums, sizeof(uint32_t) * B * nb));
   GS_TRY(ensure(c, c->vismask, sizeof(uint64_t) * stride));
-  GS_CUDA(c, cudaMemsetAsync(c->vismask.p, 0, sizeof(uint64_t) * stride, c->stream));
+  // (the kernel writes the first n)
+  if (stride > n)
+    GS_CUDA(c, cudaMemsetAsync(P<uint64_t>(c->vismask) + n, 0, sizeof(uint64_t) * (stride - n), c->stream));
   if (c->capturing) {
     // a captured step copies the cameras from the pinned staging area at its start
   } else {
@@ -555,11 +586,11 @@ gs_status gs_bin_sort(gs_ctx* c) {
   const SortWords iw = sort_words(c->total);   // instances (tile sort)
   const SortWords dw = sort_words(c->dtotal);  // visible pairs (depth sort)
   {
-    LaunchScope ls(c, "scan_block_sums", 4);
-    launch_scan_block_sums(P<uint32_t>(c->block_sums), c->nblocks, B, P<uint32_t>(c->block_offsets),
-                           iw.view_total, iw.seg, iw.total, c->stream);
-    launch_scan_block_sums(P<uint32_t>(c->vis_sums), c->nblocks, B, P<uint32_t>(c->vis_offsets), dw.view_total,
-                           dw.seg, dw.total, c->stream);
+    LaunchScope ls(c, "scan_block_sums");
+    const ScanArgs sc{c->nblocks, B,
+                      {{P<uint32_t>(c->block_sums), P<uint32_t>(c->block_offsets), iw.view_total, iw.seg, iw.total},
+                       {P<uint32_t>(c->vis_sums), P<uint32_t>(c->vis_offsets), dw.view_total, dw.seg, dw.total}}};
+    launch_scan_block_sums(sc, 2, scan_ticket(c), c->stream);
   }
   GS_CHECK_LAUNCH(c);
   // capacity: the exact count (grow-on-demand contexts read it, one stream
@@ -586,36 +617,29 @@ gs_status gs_bin_sort(gs_ctx* c) {
   GS_TRY(ensure(c, c->dkeys1, sizeof(uint32_t) * pc));
   GS_TRY(ensure(c, c->dvals0, sizeof(uint32_t) * pc));
   GS_TRY(ensure(c, c->dvals1, sizeof(uint32_t) * pc));
-  GS_TRY(ensure(c, c->ranges, sizeof(uint2) * c->bins));
   // each view is sorted on its own: the tile sort on the bits of the
   // largest tile index inside a view
   int64_t most_tiles = 1;
   for (int v = 0; v < B; v++) most_tiles = std::max<int64_t>(most_tiles, (int64_t)c->views_h[v].gw * c->views_h[v].gh);
   const int tpass = tile_passes(most_tiles);
   c->sort_passes = tpass;
-  const size_t lb = sort_lookback_bytes(cap, c->sort_items, B);
-  const size_t dlb = sort_lookback_bytes(pc, c->sort_items, B);
+  const int titems = sort_items_for(cap, c->sort_items, B), ditems = sort_items_for(pc, c->sort_items, B);
+  const size_t lb = sort_lookback_bytes(cap, titems, B);
+  const size_t dlb = sort_lookback_bytes(pc, ditems, B);
   const size_t elb = emit_lookback_bytes(pc, B);
-  GS_TRY(ensure(c, c->hist, sizeof(uint32_t) * (size_t)B * 8 * 256));
   GS_TRY(ensure(c, c->hist_scan, sizeof(uint32_t) * (size_t)B * 8 * 256));
-  GS_TRY(ensure(c, c->dhist, sizeof(uint32_t) * (size_t)B * 8 * 256));
   GS_TRY(ensure(c, c->dhist_scan, sizeof(uint32_t) * (size_t)B * 8 * 256));
-  GS_TRY(ensure(c, c->lookback, lb * tpass));
-  GS_TRY(ensure(c, c->dlookback, dlb * kDepthPasses));
-  GS_TRY(ensure(c, c->elookback, elb));
-  GS_TRY(ensure(c, c->torder, sizeof(uint32_t) * sort_partitions(cap, c->sort_items, B)));
-  GS_TRY(ensure(c, c->dorder, sizeof(uint32_t) * sort_partitions(pc, c->sort_items, B)));
-  GS_TRY(ensure(c, c->counters, sizeof(uint32_t) * kSortCounters));
+  const size_t zeroed_bytes = bin_zeroed_layout(nullptr, B, tpass, elb, dlb, lb, c->bins, nullptr);
+  GS_TRY(ensure(c, c->zeroed, zeroed_bytes));
+  BinZeroed z;
+  bin_zeroed_layout(c->zeroed.p, B, tpass, elb, dlb, lb, c->bins, &z);
+  c->ranges = z.ranges;
+  GS_TRY(ensure(c, c->torder, sizeof(uint32_t) * sort_partitions(cap, titems, B)));
+  GS_TRY(ensure(c, c->dorder, sizeof(uint32_t) * sort_partitions(pc, ditems, B)));
   GS_TRY(ensure(c, c->sorted_slots, 2 * sizeof(void*)));
   // contribution masks: every tile's region padded to whole batches of 32
   if (!c->forward_only) GS_TRY(ensure(c, c->cells, sizeof(uint32_t) * (cap + 32 * c->bins)));
-  uint32_t* counters = P<uint32_t>(c->counters);
-  GS_CUDA(c, cudaMemsetAsync(c->counters.p, 0, sizeof(uint32_t) * kSortCounters, c->stream));
-  GS_CUDA(c, cudaMemsetAsync(c->dhist.p, 0, sizeof(uint32_t) * (size_t)B * kDepthPasses * 256, c->stream));
-  GS_CUDA(c, cudaMemsetAsync(c->hist.p, 0, sizeof(uint32_t) * (size_t)B * tpass * 256, c->stream));
-  GS_CUDA(c, cudaMemsetAsync(c->dlookback.p, 0, dlb * kDepthPasses, c->stream));
-  GS_CUDA(c, cudaMemsetAsync(c->elookback.p, 0, elb, c->stream));
-  GS_CUDA(c, cudaMemsetAsync(c->lookback.p, 0, lb * tpass, c->stream));
+  GS_CUDA(c, cudaMemsetAsync(c->zeroed.p, 0, zeroed_bytes, c->stream));
 
   // 1. visible pairs -> (depth bits, Gaussian), view by view in Gaussian order
   CompactArgs ca{};
@@ -649,24 +673,24 @@ gs_status gs_bin_sort(gs_ctx* c) {
   ds.seg = dw.seg;
   ds.part_off = dw.part_off;
   ds.part_order = P<uint32_t>(c->dorder);
-  ds.hist = P<uint32_t>(c->dhist);
+  ds.hist = z.dhist;
   ds.hist_scan = P<uint32_t>(c->dhist_scan);
   ds.ctrl = dw.ctrl;
   ds.single = dw.single;
-  ds.lookback = P<uint32_t>(c->dlookback);
+  ds.lookback = z.dlookback;
   ds.lookback_stride = dlb / sizeof(uint32_t);
-  ds.counters = counters + 8;
+  ds.counters = z.counters + 8;
   ds.npass = kDepthPasses;
   ds.wait_rounds = c->sort_wait;
   ds.status = c->status_d;
   {
-    LaunchScope ls(c, "depth_histogram", 4);
-    launch_digit_histogram(ds, pc, c->sort_items, c->stream);
+    LaunchScope ls(c, "depth_histogram", 1 + digit_scan_kernels(ds));
+    launch_digit_histogram(ds, pc, ditems, scan_ticket(c), c->stream);
   }
   GS_CHECK_LAUNCH(c);
   for (int p = 0; p < kDepthPasses; p++) {
     LaunchScope ls(c, "depth_pass");
-    launch_onesweep_pass(ds, p, c->sort_items, c->stream);
+    launch_onesweep_pass(ds, p, ditems, c->stream);
   }
   GS_CHECK_LAUNCH(c);
 
@@ -686,9 +710,9 @@ gs_status gs_bin_sort(gs_ctx* c) {
   ea.keys = P<uint32_t>(c->keys0);
   ea.vals = P<uint32_t>(c->vals0);
   ea.capacity = cap;
-  ea.lookback = P<uint64_t>(c->elookback);
-  ea.counter = counters + 16;
-  ea.hist = P<uint32_t>(c->hist);
+  ea.lookback = z.elookback;
+  ea.counter = z.counters + 16;
+  ea.hist = z.hist;
   ea.tpass = tpass;
   ea.wait_rounds = c->sort_wait;
   ea.status = c->status_d;
@@ -714,33 +738,32 @@ gs_status gs_bin_sort(gs_ctx* c) {
   sa.seg = iw.seg;
   sa.part_off = iw.part_off;
   sa.part_order = P<uint32_t>(c->torder);
-  sa.hist = P<uint32_t>(c->hist);
+  sa.hist = z.hist;
   sa.hist_scan = P<uint32_t>(c->hist_scan);
   sa.ctrl = iw.ctrl;
   sa.single = iw.single;
-  sa.lookback = P<uint32_t>(c->lookback);
+  sa.lookback = z.lookback;
   sa.lookback_stride = lb / sizeof(uint32_t);
-  sa.counters = counters;
+  sa.counters = z.counters;
   sa.npass = tpass;
   sa.wait_rounds = c->sort_wait;
   sa.status = c->status_d;
   sa.sorted_keys = reinterpret_cast<const void**>(c->sorted_slots.p);
   sa.sorted_vals = reinterpret_cast<const uint32_t**>(P<unsigned char>(c->sorted_slots) + sizeof(void*));
   {
-    LaunchScope ls(c, "tile_scan", 3);
-    launch_digit_scan(sa, c->sort_items, c->stream);
+    LaunchScope ls(c, "tile_scan", digit_scan_kernels(sa));
+    launch_digit_scan(sa, titems, scan_ticket(c), c->stream);
   }
   GS_CHECK_LAUNCH(c);
   for (int p = 0; p < tpass; p++) {
     LaunchScope ls(c, "tile_pass");
-    launch_onesweep_pass(sa, p, c->sort_items, c->stream);
+    launch_onesweep_pass(sa, p, titems, c->stream);
   }
   GS_CHECK_LAUNCH(c);
   // 5. per-tile ranges
-  GS_CUDA(c, cudaMemsetAsync(c->ranges.p, 0, sizeof(uint2) * c->bins, c->stream));
   {
     LaunchScope ls(c, "tile_ranges");
-    launch_tile_ranges(sa, cap, P<uint2>(c->ranges), c->stream);
+    launch_tile_ranges(sa, cap, c->ranges, c->stream);
   }
   GS_CHECK_LAUNCH(c);
   c->tile_order_ready = false;
@@ -801,9 +824,9 @@ static gs_status sort_tiles_longest_first(gs_ctx* c) {
   GS_CUDA(c, cudaMemsetAsync(c->ord_counters.p, 0, sizeof(uint32_t) * 8, c->stream));
   GS_CUDA(c, cudaMemsetAsync(c->ord_lookback.p, 0, lb, c->stream));
   {
-    LaunchScope ls(c, "tile_order", 6);
-    launch_tile_order_keys(P<uint2>(c->ranges), bins, P<uint64_t>(c->ord_keys0), sa.vals[0], count, seg, c->stream);
-    launch_digit_histogram(sa, bins, items, c->stream);
+    LaunchScope ls(c, "tile_order", 5);
+    launch_tile_order_keys(c->ranges, bins, P<uint64_t>(c->ord_keys0), sa.vals[0], count, seg, c->stream);
+    launch_digit_histogram(sa, bins, items, scan_ticket(c), c->stream);
     launch_onesweep_pass(sa, 0, items, c->stream);
     launch_tile_order_finish(ctrl, 1, sa.vals[0], sa.vals[1], bins, P<uint32_t>(c->tile_order), c->stream);
   }
@@ -818,7 +841,7 @@ static RasterArgs raster_args(gs_ctx* c) {
   r.B = c->B;
   r.n = c->n;
   r.stride = c->stride;
-  r.ranges = P<uint2>(c->ranges);
+  r.ranges = c->ranges;
   r.vals = reinterpret_cast<const uint32_t* const*>(P<unsigned char>(c->sorted_slots) + sizeof(void*));
   r.rec0 = P<float4>(c->rec);
   r.rec1 = P<float4>(c->rec) + 1;
@@ -923,7 +946,8 @@ gs_status gs_raster_bwd(gs_ctx* c, const gs_params* params, const float* dL_dima
   b.dens_count = c->dens_count;
   if (grads->stride > grads->n) {
     // padding columns are not written by the kernel; keep them zero
-    GS_CUDA(c, cudaMemsetAsync(grads->data, 0, sizeof(float) * n_planes(c->deg) * grads->stride, c->stream));
+    GS_CUDA(c, cudaMemset2DAsync(grads->data + grads->n, sizeof(float) * grads->stride, 0,
+                                 sizeof(float) * (grads->stride - grads->n), n_planes(c->deg), c->stream));
   }
   {
     LaunchScope ls(c, "project_bwd", 2);
@@ -1021,7 +1045,7 @@ gs_status gs_get_buffer(gs_ctx* c, int32_t which, void** ptr, int64_t* count) {
       *count = (int64_t)cnt;
       break;
     }
-    case GS_BUF_RANGES: if (!c->sorted) return GS_ESTATE; *ptr = c->ranges.p; *count = c->bins; break;
+    case GS_BUF_RANGES: if (!c->sorted) return GS_ESTATE; *ptr = c->ranges; *count = c->bins; break;
     case GS_BUF_TFINAL: if (!c->rastered) return GS_ESTATE; *ptr = c->tfinal.p; *count = c->pixels; break;
     case GS_BUF_NLAST: if (!c->rastered) return GS_ESTATE; *ptr = c->nlast.p; *count = c->pixels; break;
     case GS_BUF_G2D: if (!c->g2d.p) return GS_ESTATE; *ptr = c->g2d.p; *count = (kG2dGeo + kG2dCol) * bn; break;
@@ -1128,11 +1152,13 @@ static gs_status sort_pairs(gs_ctx* c, int64_t n, int bits, int* which) {
   const int npass = std::max(1, (bits + 7) / 8);
   GS_TRY(ensure(c, c->views, sizeof(ViewRec)));
   GS_TRY(ensure(c, c->total, sort_words_bytes()));
-  const size_t lb = sort_lookback_bytes(n, c->sort_items, 1);
-  GS_TRY(ensure(c, c->hist, sizeof(uint32_t) * 8 * 256));
+  const int items = sort_items_for(n, c->sort_items, 1);
+  const size_t lb = sort_lookback_bytes(n, items, 1);
   GS_TRY(ensure(c, c->hist_scan, sizeof(uint32_t) * 8 * 256));
-  GS_TRY(ensure(c, c->lookback, lb * npass));
-  GS_TRY(ensure(c, c->counters, sizeof(uint32_t) * 8));
+  // tickets, digit counts, look-back statuses
+  const size_t zeroed_bytes = sizeof(uint32_t) * (8 + npass * 256) + lb * npass;
+  GS_TRY(ensure(c, c->zeroed, zeroed_bytes));
+  uint32_t* counters = P<uint32_t>(c->zeroed);
   uint64_t* total = P<uint64_t>(c->total);
   uint32_t* seg = reinterpret_cast<uint32_t*>(total + 1 + kMaxViews);
   uint32_t* part_off = seg + kMaxViews + 1;
@@ -1156,26 +1182,24 @@ static gs_status sort_pairs(gs_ctx* c, int64_t n, int bits, int* which) {
   sa.views = P<ViewRec>(c->views);
   sa.seg = seg;
   sa.part_off = part_off;
-  sa.hist = P<uint32_t>(c->hist);
+  sa.hist = counters + 8;
   sa.hist_scan = P<uint32_t>(c->hist_scan);
   sa.ctrl = ctrl;
   sa.single = ctrl + 16;
-  sa.lookback = P<uint32_t>(c->lookback);
+  sa.lookback = counters + 8 + npass * 256;
   sa.lookback_stride = lb / sizeof(uint32_t);
-  sa.counters = P<uint32_t>(c->counters);
+  sa.counters = counters;
   sa.npass = npass;
   sa.wait_rounds = c->sort_wait;
   sa.status = c->status_d;
-  GS_CUDA(c, cudaMemsetAsync(c->hist.p, 0, sizeof(uint32_t) * npass * 256, c->stream));
-  GS_CUDA(c, cudaMemsetAsync(c->counters.p, 0, sizeof(uint32_t) * 8, c->stream));
-  GS_CUDA(c, cudaMemsetAsync(c->lookback.p, 0, lb * npass, c->stream));
+  GS_CUDA(c, cudaMemsetAsync(c->zeroed.p, 0, zeroed_bytes, c->stream));
   {
-    LaunchScope ls(c, "digit_histogram", 3);
-    launch_digit_histogram(sa, n, c->sort_items, c->stream);
+    LaunchScope ls(c, "digit_histogram", 2);
+    launch_digit_histogram(sa, n, items, scan_ticket(c), c->stream);
   }
   for (int p = 0; p < npass; p++) {
     LaunchScope ls(c, "onesweep_pass");
-    launch_onesweep_pass(sa, p, c->sort_items, c->stream);
+    launch_onesweep_pass(sa, p, items, c->stream);
   }
   GS_CHECK_LAUNCH(c);
   uint32_t par = 0;
@@ -1223,9 +1247,11 @@ gs_status gs_iso_count(gs_ctx* c, const float* volume, int32_t nx, int32_t ny, i
     launch_iso_count(a, c->stream);
   }
   {
-    LaunchScope ls(c, "scan_block_sums", 2);
-    launch_scan_block_sums(a.block_counts, iso_blocks(a.nverts), 1, const_cast<uint32_t*>(a.block_offsets), total + 1,
-                           reinterpret_cast<uint32_t*>(total + 2), total, c->stream);
+    LaunchScope ls(c, "scan_block_sums");
+    const ScanArgs sc{iso_blocks(a.nverts), 1,
+                      {{a.block_counts, const_cast<uint32_t*>(a.block_offsets), total + 1,
+                        reinterpret_cast<uint32_t*>(total + 2), total}}};
+    launch_scan_block_sums(sc, 1, scan_ticket(c), c->stream);
   }
   GS_CHECK_LAUNCH(c);
   GS_CUDA(c, cudaMemcpyAsync(c->pinned, total, sizeof(uint64_t), cudaMemcpyDeviceToHost, c->stream));
@@ -1444,9 +1470,11 @@ gs_status gs_densify(gs_ctx* c, const gs_params* p, const gs_params* m, const gs
     launch_densify_count(a, c->stream);
   }
   {
-    LaunchScope ls(c, "scan_block_sums", 2);
-    launch_scan_block_sums(P<uint32_t>(c->block_sums), nb, 1, P<uint32_t>(c->block_offsets), total + 1,
-                           reinterpret_cast<uint32_t*>(total + 1 + kMaxViews), total, c->stream);
+    LaunchScope ls(c, "scan_block_sums");
+    const ScanArgs sc{nb, 1,
+                      {{P<uint32_t>(c->block_sums), P<uint32_t>(c->block_offsets), total + 1,
+                        reinterpret_cast<uint32_t*>(total + 1 + kMaxViews), total}}};
+    launch_scan_block_sums(sc, 1, scan_ticket(c), c->stream);
   }
   GS_CHECK_LAUNCH(c);
   uint64_t cnt = 0;

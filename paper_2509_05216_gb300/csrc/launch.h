@@ -60,7 +60,7 @@ struct EmitArgs {
   uint32_t* keys;                 // [capacity] bins
   uint32_t* vals;                 // [capacity] Gaussians
   int64_t capacity;
-  uint64_t* lookback;             // [emit_partitions] status words, zeroed before the launch
+  uint64_t* lookback;             // [emit_lookback_bytes] status words, zeroed before the launch
   uint32_t* counter;              // partition ticket, zeroed before the launch
   uint32_t* hist;                 // [B][tpass][256] tile digit counts (added to; zeroed before)
   int tpass;
@@ -109,13 +109,24 @@ int project_fwd_block();
 void launch_project_fwd(const ProjectArgs& a, int deg, cudaStream_t s);
 void launch_project_bwd(const ProjectBwdArgs& a, int deg, cudaStream_t s);
 
-void launch_scan_block_sums(const uint32_t* sums, int64_t nb, int B, uint32_t* offsets, uint64_t* view_total,
-                            uint32_t* seg, uint64_t* total, cudaStream_t s);
+struct ScanArgs {
+  int64_t nb;  // counts per view
+  int B;
+  struct Kind {
+    const uint32_t* sums;   // [B][nb]
+    uint32_t* offsets;      // [B][nb] exclusive scan within the view
+    uint64_t* view_total;   // [B]
+    uint32_t* seg;          // [B + 1] first of each view, then the total
+    uint64_t* total;
+  } kind[2];
+};
+// ticket: device word, 0 between launches (the kernel leaves it so)
+void launch_scan_block_sums(const ScanArgs& a, int kinds, uint32_t* ticket, cudaStream_t s);
 void launch_compact(const CompactArgs& a, cudaStream_t s);
 // pair_capacity: visible pairs the grid covers (B x stride)
 void launch_emit(const EmitArgs& a, int64_t pair_capacity, cudaStream_t s);
-int64_t emit_partitions(int64_t pairs, int segments);
 size_t emit_lookback_bytes(int64_t pair_capacity, int segments);
+size_t emit_lookback_reserve(int64_t pair_capacity, int segments);
 
 // LSD radix sort of (key, value) pairs on key bits [0, 8 npass), ping-pong
 // between keys[0]/vals[0] (input) and keys[1]/vals[1].  Everything that
@@ -160,11 +171,15 @@ void launch_tile_order_finish(const uint32_t* ctrl, int npass, const uint32_t* v
 
 size_t sort_lookback_bytes(int64_t count, int items, int segments);
 int64_t sort_partitions(int64_t count, int items, int segments);
+int sort_items_for(int64_t capacity, int items, int segments);
+int64_t sort_partitions_reserve(int64_t capacity, int items, int segments);
 // digit counts (into a.hist, zeroed before), their scans and the pass control words
-void launch_digit_histogram(const SortArgs& a, int64_t grid_hint, int items, cudaStream_t s);
+// (ticket: device word, 0 between launches)
+void launch_digit_histogram(const SortArgs& a, int64_t grid_hint, int items, uint32_t* ticket, cudaStream_t s);
 // the scans, control words and partition order only (a.hist counted elsewhere)
-void launch_digit_scan(const SortArgs& a, int items, cudaStream_t s);
-// items: keys per thread (12, 16, 20 or 24); the grid covers a.capacity
+void launch_digit_scan(const SortArgs& a, int items, uint32_t* ticket, cudaStream_t s);
+int digit_scan_kernels(const SortArgs& a);  // kernels of launch_digit_scan
+// items: keys per thread (4, 8, 12, 16, 20 or 24); the grid covers a.capacity
 void launch_onesweep_pass(const SortArgs& a, int pass, int items, cudaStream_t s);
 void launch_tile_ranges(const SortArgs& a, int64_t grid_hint, uint2* ranges, cudaStream_t s);
 

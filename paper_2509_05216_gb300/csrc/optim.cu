@@ -77,7 +77,8 @@ void launch_l1(const float* x, const float* y, const float* const* y_slot, int64
 // rate is uniform across the warp and, in the visible-only variant, the
 // column's visibility is read once: a column of 4 invisible Gaussians reads
 // and writes nothing; otherwise invisible lanes write their values back
-// unchanged.
+// unchanged.  Sets whose columns do not fill the GPU split the planes over
+// blockIdx.y.
 __global__ void __launch_bounds__(256) adam_kernel(AdamArgs a) {
   // step-dependent constants come from device memory, so the launch can be
   // captured once and replayed for any step
@@ -110,7 +111,7 @@ __global__ void __launch_bounds__(256) adam_kernel(AdamArgs a) {
       on[3] = q1.y != 0ull;
       if (!(on[0] || on[1] || on[2] || on[3])) continue;
     }
-    for (int pl = 0; pl < a.planes; pl++) {
+    for (int pl = (int)blockIdx.y; pl < a.planes; pl += (int)gridDim.y) {
       const int64_t i = pl * cols + col;
       const float lr = lr_s[pl];
       const float4 g = g4[i];
@@ -134,7 +135,11 @@ void launch_adam(const AdamArgs& a, cudaStream_t s) {
   const int64_t most = (int64_t)sm_count() * 16;
   if (blocks > most) blocks = most;
   if (blocks < 1) blocks = 1;
-  adam_kernel<<<(unsigned)blocks, 256, 0, s>>>(a);
+  // below 4 blocks per SM a thread's walk over the planes is a chain of loads
+  // with too few others to hide it: more blocks per column
+  int64_t split = 1;
+  while (split * 2 <= a.planes && blocks * split < (int64_t)sm_count() * 4) split *= 2;
+  adam_kernel<<<dim3((unsigned)blocks, (unsigned)split), 256, 0, s>>>(a);
 }
 
 }  // namespace gs
