@@ -1087,17 +1087,19 @@ static gs_status run_ssim(gs_ctx* c, const float* images, const float* targets, 
   set_device(c);
   const int B = c->B;
   std::vector<int> first(B + 1, 0);
-  for (int v = 0; v < B; v++) first[v + 1] = first[v] + ssim_blocks_of_view(c->views_h[v].W, c->views_h[v].H);
+  const int rows = ssim_strip_rows(c->pixels);
+  for (int v = 0; v < B; v++) first[v + 1] = first[v] + ssim_strips_of_view(c->views_h[v].W, c->views_h[v].H, rows);
   const int blocks = first[B];
   const int64_t count = 3 * c->pixels;
   GS_TRY(ensure(c, c->ssim_table, sizeof(int) * (B + 1)));
-  GS_TRY(ensure(c, c->ssim_partials, sizeof(float) * 3 * count));
+  if (dL_dimages) GS_TRY(ensure(c, c->ssim_partials, sizeof(float) * 3 * count));
   GS_TRY(ensure(c, c->ssim_sums, sizeof(double) * (3 * (size_t)blocks + 3 * kMaxViews)));
   GS_CUDA(c, cudaMemcpyAsync(c->ssim_table.p, first.data(), sizeof(int) * (B + 1), cudaMemcpyHostToDevice, c->stream));
   SsimArgs a{};
   a.views = P<ViewRec>(c->views);
   a.B = B;
   a.first_block = P<int>(c->ssim_table);
+  a.rows = rows;
   a.x = images;
   a.y = targets;
   a.count = count;
@@ -1131,7 +1133,8 @@ gs_status gs_image_metrics(gs_ctx* c, const float* images, const float* targets,
   GS_TRY(run_ssim(c, images, targets, 0.f, nullptr, nullptr));
   std::vector<double> sums(3 * (size_t)c->B);
   int blocks = 0;
-  for (int v = 0; v < c->B; v++) blocks += ssim_blocks_of_view(c->views_h[v].W, c->views_h[v].H);
+  const int rows = ssim_strip_rows(c->pixels);
+  for (int v = 0; v < c->B; v++) blocks += ssim_strips_of_view(c->views_h[v].W, c->views_h[v].H, rows);
   GS_CUDA(c, cudaMemcpyAsync(sums.data(), P<double>(c->ssim_sums) + 3 * (size_t)blocks,
                              sizeof(double) * sums.size(), cudaMemcpyDeviceToHost, c->stream));
   GS_CUDA(c, cudaStreamSynchronize(c->stream));

@@ -201,22 +201,24 @@ int l1_parts(int64_t count);
 struct SsimArgs {
   const ViewRec* views;
   int B;
-  const int* first_block;  // [B + 1] first block of each view (3 channels x 32 x 16 tiles)
+  const int* first_block;  // [B + 1] first strip of each view
   const float* x;          // images (batch layout)
   const float* y;          // targets
   int64_t count;           // 3 x pixels of the batch
-  float* partials;         // [3][count]: dSSIM/d(mx), dSSIM/dE[x^2], dSSIM/dE[xy] per pixel
-  double* block_sums;      // [blocks][3]: sums of the SSIM map, |x - y|, (x - y)^2
+  float* partials;         // per pixel dSSIM/d(mx), dSSIM/dE[x^2]: [count][2], then dSSIM/dE[xy]: [count]
+  int rows;                // rows per strip (ssim_strip_rows)
+  double* block_sums;      // [strips][3]: sums of the SSIM map, |x - y|, (x - y)^2
   float* grad;             // dL/dx (backward)
-  float win[11];           // normalised Gaussian window (sigma 1.5)
+  float2 win[11];          // normalised Gaussian window (sigma 1.5), each weight twice
   float w_l1, w_ssim, inv_count;
   double w_l1_d, w_ssim_d;
 };
-int ssim_blocks_of_view(int W, int H);
-void ssim_window(float* w);
+int ssim_strip_rows(int64_t pixels);
+int ssim_strips_of_view(int W, int H, int rows);
+void ssim_window(float2* w);
 // forward (+ per-view sums into out_view[3 B] and the loss) and, if
 // backward, the gradient
-void launch_ssim(const SsimArgs& a, int blocks, bool backward, double* out_view, float* loss, cudaStream_t s);
+void launch_ssim(const SsimArgs& a, int strips, bool backward, double* out_view, float* loss, cudaStream_t s);
 
 // Point-cloud initialisation (init.cu).
 struct IsoArgs {
