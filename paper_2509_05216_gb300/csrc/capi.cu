@@ -86,7 +86,7 @@ struct gs_ctx {
   DevBuf views, rec, rec3, tiles, block_sums, block_offsets, total, keys0, keys1, vals0, vals1,
       zeroed, hist_scan, tfinal, nlast, g2d, l1_partial, sorted_slots, adam_consts,
       target_slot, host_tgt0, host_tgt1, pair_stats, cells, vismask, ssim_table, ssim_partials, ssim_sums,
-      init_pts, init_scales, knn_part, knn_table, ord_keys0, ord_keys1, ord_vals0, ord_vals1, ord_total, ord_hist,
+      init_pts, init_scales, knn_part, knn_table, knn_heads, ord_keys0, ord_keys1, ord_vals0, ord_vals1, ord_total, ord_hist,
       ord_hist_scan, ord_lookback, ord_counters, ord_views, tile_order, vis_sums, vis_offsets, dtotal, dkeys0,
       dkeys1, dvals0, dvals1, dhist_scan, dorder, torder, iso_work, densify_source;
 
@@ -461,7 +461,7 @@ void gs_destroy(gs_ctx* c) {
                     &c->total, &c->keys0, &c->keys1, &c->vals0, &c->vals1, &c->zeroed, &c->hist_scan, &c->tfinal, &c->nlast, &c->g2d, &c->l1_partial,
                     &c->sorted_slots, &c->adam_consts, &c->target_slot, &c->host_tgt0, &c->host_tgt1,
                     &c->pair_stats, &c->cells, &c->vismask, &c->ssim_table, &c->ssim_partials, &c->ssim_sums,
-                    &c->init_pts, &c->init_scales, &c->knn_part, &c->knn_table, &c->ord_keys0, &c->ord_keys1,
+                    &c->init_pts, &c->init_scales, &c->knn_part, &c->knn_table, &c->knn_heads, &c->ord_keys0, &c->ord_keys1,
                     &c->ord_vals0, &c->ord_vals1, &c->ord_total, &c->ord_hist, &c->ord_hist_scan, &c->ord_lookback,
                     &c->ord_counters, &c->ord_views, &c->tile_order, &c->vis_sums, &c->vis_offsets, &c->dtotal,
                     &c->dkeys0, &c->dkeys1, &c->dvals0, &c->dvals1, &c->dhist_scan, &c->dorder, &c->torder, &c->iso_work, &c->densify_source};
@@ -1148,12 +1148,12 @@ gs_status gs_image_metrics(gs_ctx* c, const float* images, const float* targets,
 
 // ---------------------------------------------------------------- initialisation
 
-// Stable LSD sort of n (key, value) pairs on the low `bits` key bits with the
-// binning's onesweep (one segment), in the context's instance buffers;
-// *which = the buffer (0 / 1) holding the result.  Synchronises the stream.
-static gs_status sort_pairs(gs_ctx* c, int64_t n, int bits, int* which) {
+// Stable LSD sort of n (32-bit key, value) pairs on the low `bits` key bits
+// with the binning's onesweep (one segment), in the context's instance
+// buffers; bit 0 of (*ctrl_out)[*npass_out] (device) says which of the two
+// buffers holds the result.
+static gs_status sort_pairs(gs_ctx* c, int64_t n, int bits, const uint32_t** ctrl_out, int* npass_out) {
   const int npass = std::max(1, (bits + 7) / 8);
-  GS_TRY(ensure(c, c->views, sizeof(ViewRec)));
   GS_TRY(ensure(c, c->total, sort_words_bytes()));
   const int items = sort_items_for(n, c->sort_items, 1);
   const size_t lb = sort_lookback_bytes(n, items, 1);
@@ -1168,21 +1168,19 @@ static gs_status sort_pairs(gs_ctx* c, int64_t n, int bits, int* which) {
   uint32_t* ctrl = part_off + kMaxViews + 1;
   const uint64_t cnt = (uint64_t)n;
   const uint32_t segs[2] = {0u, (uint32_t)n};
-  GS_CUDA(c, cudaMemsetAsync(c->views.p, 0, sizeof(ViewRec), c->stream));
   GS_CUDA(c, cudaMemcpyAsync(total, &cnt, sizeof(cnt), cudaMemcpyHostToDevice, c->stream));
   GS_CUDA(c, cudaMemcpyAsync(seg, segs, sizeof(segs), cudaMemcpyHostToDevice, c->stream));
   SortArgs sa{};
   sa.keys[0] = c->keys0.p;
   sa.keys[1] = c->keys1.p;
-  sa.key_bytes = 8;
-  sa.view_shift = 32;
+  sa.key_bytes = 4;
+  sa.view_shift = 0;
   sa.vals[0] = P<uint32_t>(c->vals0);
   sa.vals[1] = P<uint32_t>(c->vals1);
   sa.count = total;
   sa.capacity = n;
   sa.bins = 1;
   sa.B = 1;
-  sa.views = P<ViewRec>(c->views);
   sa.seg = seg;
   sa.part_off = part_off;
   sa.hist = counters + 8;
@@ -1205,10 +1203,8 @@ static gs_status sort_pairs(gs_ctx* c, int64_t n, int bits, int* which) {
     launch_onesweep_pass(sa, p, items, c->stream);
   }
   GS_CHECK_LAUNCH(c);
-  uint32_t par = 0;
-  GS_CUDA(c, cudaMemcpyAsync(&par, ctrl + npass, sizeof(par), cudaMemcpyDeviceToHost, c->stream));
-  GS_CUDA(c, cudaStreamSynchronize(c->stream));
-  *which = (int)(par & 1u);
+  *ctrl_out = ctrl;
+  *npass_out = npass;
   return GS_OK;
 }
 
@@ -1315,77 +1311,63 @@ gs_status gs_init_gaussians(gs_ctx* c, const float* points, const float* normals
   if (!(flatten > 0.f) || n >= ((int64_t)1 << 31)) return fail(c, GS_EINVAL, "bad flatten or n");
   set_device(c);
   c->projected = c->sorted = c->rastered = c->cells_ready = false;
-  // the selected points, contiguous
-  const float* pts = points;
-  if (select) {
-    GS_TRY(ensure(c, c->init_pts, sizeof(float) * 3 * n));
-    launch_init_gather(points, select, n, P<float>(c->init_pts), c->stream);
-    GS_CHECK_LAUNCH(c);
-    pts = P<float>(c->init_pts);
-  }
-  // bounds -> grid of about one point per cell volume
+  // bounds -> finest cells
   const int nparts = (int)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, (int64_t)sm_count() * 8));
   GS_TRY(ensure(c, c->knn_part, sizeof(float) * 6 * (nparts + 1)));
   float* bounds_d = P<float>(c->knn_part) + 6 * nparts;
-  launch_knn_bounds(pts, n, P<float>(c->knn_part), nparts, bounds_d, c->stream);
+  {
+    LaunchScope ls(c, "knn_bounds", 2);
+    launch_knn_bounds(points, select, n, P<float>(c->knn_part), nparts, bounds_d, c->stream);
+  }
   GS_CHECK_LAUNCH(c);
   float bounds[6];
-  GS_CUDA(c, cudaMemcpyAsync(bounds, bounds_d, sizeof(bounds), cudaMemcpyDeviceToHost, c->stream));
+  GS_CUDA(c, cudaMemcpyAsync(c->pinned, bounds_d, sizeof(bounds), cudaMemcpyDeviceToHost, c->stream));
   GS_CUDA(c, cudaStreamSynchronize(c->stream));
+  std::memcpy(bounds, c->pinned, sizeof(bounds));
   KnnArgs k{};
-  k.pts = pts;
+  k.pts = points;
+  k.sel = select;
   k.n = n;
-  k.k = 3;
-  double ext[3], vol = 1.0, emax = 0.0;
+  double emax = 0.0;
   for (int d = 0; d < 3; d++) {
-    ext[d] = (double)bounds[3 + d] - (double)bounds[d];
-    emax = std::max(emax, ext[d]);
-  }
-  if (!(emax > 0.0) || !std::isfinite(emax)) return fail(c, GS_EINVAL, "points must span a finite, nonzero box");
-  for (int d = 0; d < 3; d++) vol *= std::max(ext[d], emax * 1e-3);
-  double cell = std::cbrt(vol / (double)n);
-  int64_t cells = 1;
-  for (int d = 0; d < 3; d++) {
-    int64_t dim = (int64_t)(ext[d] / cell) + 1;
-    while (dim > (1 << 20)) {  // keep every axis within 2^20 cells
-      cell *= 2.0;
-      dim = (int64_t)(ext[d] / cell) + 1;
-    }
-    k.dims[d] = (int)dim;
-  }
-  for (int d = 0; d < 3; d++) {
-    k.dims[d] = (int)((int64_t)(ext[d] / cell) + 1);
-    cells *= k.dims[d];
+    emax = std::max(emax, (double)bounds[3 + d] - (double)bounds[d]);
     k.lo[d] = bounds[d];
   }
+  if (!(emax > 0.0) || !std::isfinite(emax)) return fail(c, GS_EINVAL, "points must span a finite, nonzero box");
+  const int key_bits = knn_key_bits();
+  const double cell = emax / (double)(1 << (key_bits / 3));
   k.cell = (float)cell;
   k.inv_cell = (float)(1.0 / cell);
-  int bits = 1;
-  while (((int64_t)1 << bits) < cells) bits++;
+  // the chosen level has at most n / 2 cells: at most half full
   int tbits = 10;
-  while (((int64_t)1 << tbits) < 2 * n) tbits++;
+  while (((int64_t)1 << tbits) < n) tbits++;
   k.table_bits = tbits;
-  GS_TRY(ensure(c, c->keys0, sizeof(uint64_t) * n));
-  GS_TRY(ensure(c, c->keys1, sizeof(uint64_t) * n));
+  GS_TRY(ensure(c, c->keys0, sizeof(uint32_t) * n));
+  GS_TRY(ensure(c, c->keys1, sizeof(uint32_t) * n));
   GS_TRY(ensure(c, c->vals0, sizeof(uint32_t) * n));
   GS_TRY(ensure(c, c->vals1, sizeof(uint32_t) * n));
-  GS_TRY(ensure(c, c->knn_table, (sizeof(uint64_t) + sizeof(uint32_t)) << tbits));
+  GS_TRY(ensure(c, c->init_pts, sizeof(float4) * n));
+  GS_TRY(ensure(c, c->knn_heads, sizeof(uint32_t) * 16));
+  GS_TRY(ensure(c, c->knn_table, sizeof(uint4) << tbits));
   GS_TRY(ensure(c, c->init_scales, sizeof(float) * n));
+  k.keys[0] = P<uint32_t>(c->keys0);
+  k.keys[1] = P<uint32_t>(c->keys1);
+  k.vals[0] = P<uint32_t>(c->vals0);
+  k.vals[1] = P<uint32_t>(c->vals1);
   {
     LaunchScope ls(c, "knn_cells");
-    launch_knn_keys(k, P<uint64_t>(c->keys0), P<uint32_t>(c->vals0), c->stream);
+    launch_knn_keys(k, c->stream);
   }
   GS_CHECK_LAUNCH(c);
-  int which = 0;
-  GS_TRY(sort_pairs(c, n, bits, &which));
-  k.skeys = which ? P<uint64_t>(c->keys1) : P<uint64_t>(c->keys0);
-  k.svals = which ? P<uint32_t>(c->vals1) : P<uint32_t>(c->vals0);
-  k.table_keys = P<uint64_t>(c->knn_table);
-  k.table_start = reinterpret_cast<uint32_t*>(P<uint64_t>(c->knn_table) + ((size_t)1 << tbits));
+  GS_TRY(sort_pairs(c, n, key_bits, &k.sort_ctrl, &k.sort_passes));
+  k.sorted = P<float4>(c->init_pts);
+  k.heads = P<uint32_t>(c->knn_heads);
+  k.table = P<uint4>(c->knn_table);
   k.out = P<float>(c->init_scales);
-  GS_CUDA(c, cudaMemsetAsync(k.table_keys, 0xff, sizeof(uint64_t) << tbits, c->stream));
+  GS_CUDA(c, cudaMemsetAsync(k.heads, 0, sizeof(uint32_t) * 16, c->stream));
+  GS_CUDA(c, cudaMemsetAsync(k.table, 0xff, sizeof(uint4) << tbits, c->stream));
   {
-    LaunchScope ls(c, "knn_query", 2);
+    LaunchScope ls(c, "knn_query", 4);
     launch_knn_query(k, c->stream);
   }
   GS_CHECK_LAUNCH(c);

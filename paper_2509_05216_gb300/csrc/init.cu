@@ -10,10 +10,14 @@
 // in vertex order (x fastest, then y, then z; per vertex its +x, +y, +z
 // edges).  One pass over the volume keeps a side bit per vertex; counting
 // and placing the crossings works on those bits.  Each Gaussian's initial scale is log sqrt of the mean squared
-// distance to its k nearest other points, found exactly with a uniform grid:
-// points are sorted by cell (the onesweep radix sort), cell starts go into
-// an open-addressing table, and each query examines growing cubes of cells
-// until the k-th distance lies inside the examined radius.
+// distance to its 3 nearest other points, found exactly with a grid: points
+// are sorted by the Morton code of a fine cell (the onesweep radix sort), the
+// level of the grid whose occupied cells hold a few points is picked on the
+// device (points of a surface fill a small part of a volume's cells, so the
+// cell size follows the occupied cells), its cells go into an open-addressing
+// table, and each query examines growing cubes of cells until the third
+// distance lies inside the examined radius.
+#include <algorithm>
 #include <cmath>
 
 #include "gs_internal.cuh"
@@ -261,19 +265,22 @@ void launch_iso_emit(const IsoArgs& a, cudaStream_t s) {
 
 // ---------------------------------------------------------------- k nearest neighbours
 
-// Per-block bounds of the points (6 floats: min xyz, max xyz), then one
-// block combines them.
-__global__ void __launch_bounds__(256) knn_bounds_kernel(const float* __restrict__ pts, int64_t n,
+// Per-block bounds of the (selected) points (6 floats: min xyz, max xyz), then
+// one block combines them.
+__global__ void __launch_bounds__(256) knn_bounds_kernel(const float* __restrict__ pts,
+                                                         const int64_t* __restrict__ sel, int64_t n,
                                                          float* __restrict__ part) {
   __shared__ float red[6][8];
   float b[6] = {3.0e38f, 3.0e38f, 3.0e38f, -3.0e38f, -3.0e38f, -3.0e38f};
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t src = sel ? sel[i] : i;
 #pragma unroll
     for (int d = 0; d < 3; d++) {
-      const float v = pts[3 * i + d];
+      const float v = pts[3 * src + d];
       b[d] = fminf(b[d], v);
       b[3 + d] = fmaxf(b[3 + d], v);
     }
+  }
 #pragma unroll
   for (int d = 0; d < 6; d++) {
 #pragma unroll
@@ -292,140 +299,342 @@ __global__ void __launch_bounds__(256) knn_bounds_kernel(const float* __restrict
   }
 }
 
-__global__ void knn_bounds_finish_kernel(const float* __restrict__ part, int nparts, float* __restrict__ out) {
-  if (threadIdx.x >= 6) return;
-  const int d = threadIdx.x;
+__global__ void __launch_bounds__(192) knn_bounds_finish_kernel(const float* __restrict__ part, int nparts,
+                                                                float* __restrict__ out) {
+  const int d = threadIdx.x >> 5, lane = threadIdx.x & 31;  // a warp per bound
   float v = part[d];
-  for (int b = 1; b < nparts; b++) v = d < 3 ? fminf(v, part[6 * b + d]) : fmaxf(v, part[6 * b + d]);
-  out[d] = v;
+  for (int b = lane; b < nparts; b += 32) v = d < 3 ? fminf(v, part[6 * b + d]) : fmaxf(v, part[6 * b + d]);
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) {
+    const float o = __shfl_down_sync(0xffffffffu, v, off);
+    v = d < 3 ? fminf(v, o) : fmaxf(v, o);
+  }
+  if (lane == 0) out[d] = v;
 }
 
 namespace {
 
-__device__ __forceinline__ void cell_of(const KnnArgs& a, float x, float y, float z, int& cx, int& cy, int& cz) {
-  cx = min(max((int)((x - a.lo[0]) * a.inv_cell), 0), a.dims[0] - 1);
-  cy = min(max((int)((y - a.lo[1]) * a.inv_cell), 0), a.dims[1] - 1);
-  cz = min(max((int)((z - a.lo[2]) * a.inv_cell), 0), a.dims[2] - 1);
+// The finest grid has 2^10 cells along the longest side of the bounding box;
+// a point's key is the Morton code of its finest cell, so that one sort orders
+// the points by cell at every level l (cells of 2^l finest ones: the key
+// without its low 3 l bits), and a cell of any level is a run of the sorted
+// points.
+constexpr int kMortonBits = 10;
+
+__device__ __forceinline__ uint32_t spread3(uint32_t x) {  // bit i -> bit 3 i
+  x &= 0x3ffu;
+  x = (x | (x << 16)) & 0x030000ffu;
+  x = (x | (x << 8)) & 0x0300f00fu;
+  x = (x | (x << 4)) & 0x030c30c3u;
+  x = (x | (x << 2)) & 0x09249249u;
+  return x;
+}
+__device__ __forceinline__ uint32_t gather3(uint32_t x) {  // bit 3 i -> bit i
+  x &= 0x09249249u;
+  x = (x | (x >> 2)) & 0x030c30c3u;
+  x = (x | (x >> 4)) & 0x0300f00fu;
+  x = (x | (x >> 8)) & 0x030000ffu;
+  x = (x | (x >> 16)) & 0x3ffu;
+  return x;
 }
 
-__device__ __forceinline__ uint64_t cell_id(const KnnArgs& a, int cx, int cy, int cz) {
-  return ((uint64_t)cz * (uint64_t)a.dims[1] + (uint64_t)cy) * (uint64_t)a.dims[0] + (uint64_t)cx;
+__device__ __forceinline__ uint32_t fine_cell(float x, float lo, float inv) {
+  return (uint32_t)min(max((int)((x - lo) * inv), 0), (1 << kMortonBits) - 1);
 }
 
-__device__ __forceinline__ uint64_t slot_of(uint64_t key, int bits) {
-  return (key * 0x9E3779B97F4A7C15ull) >> (64 - bits);
+// First slot of a cell: the 8 cells of a cube of the next level share a line.
+__device__ __forceinline__ uint32_t slot_of(uint32_t key, int bits) {
+  return (((key >> 3) * 0x9E3779B1u) >> (35 - bits)) << 3 | (key & 7u);
 }
 
-constexpr uint64_t kEmptySlot = ~0ull;
+constexpr uint32_t kEmptySlot = ~0u;
 
-// First sorted position of a cell, or -1 when no point lies in it.
-__device__ __forceinline__ int64_t cell_start(const KnnArgs& a, uint64_t key) {
-  const uint64_t mask = (1ull << a.table_bits) - 1ull;
-  for (uint64_t s = slot_of(key, a.table_bits), probes = 0; probes <= mask; s = (s + 1) & mask, probes++) {
-    const uint64_t k = a.table_keys[s];
-    if (k == key) return (int64_t)a.table_start[s];
-    if (k == kEmptySlot) return -1;
+// The run of sorted points of a cell (empty when no point lies in it).
+__device__ __forceinline__ uint2 cell_run(const KnnArgs& a, uint32_t key) {
+  const uint32_t mask = (uint32_t)((1ull << a.table_bits) - 1ull);
+  for (uint32_t s = slot_of(key, a.table_bits), probes = 0; probes <= mask; s = (s + 1) & mask, probes++) {
+    const uint4 e = a.table[s];
+    if (e.x == key) return make_uint2(e.y, e.z);
+    if (e.x == kEmptySlot) break;
   }
-  return -1;
+  return make_uint2(0u, 0u);
+}
+
+// The level whose occupied cells hold kCellPoints points or more on average
+// (the finest such one).  heads[l]: sorted points whose cell at level l, but
+// not at l + 1, differs from their predecessor's; a level has one cell more
+// than the heads at it and above.
+constexpr int64_t kCellPoints = 2;
+__device__ __forceinline__ int pick_level(const KnnArgs& a) {
+  int64_t cells = 1;
+  int level = kMortonBits;
+  for (int l = kMortonBits - 1; l >= 0; l--) {
+    cells += a.heads[l];
+    if (cells * kCellPoints <= a.n) level = l; else break;
+  }
+  return level;
+}
+
+__device__ __forceinline__ const uint32_t* sorted_keys(const KnnArgs& a) {
+  return (a.sort_ctrl[a.sort_passes] & 1u) ? a.keys[1] : a.keys[0];
+}
+
+// The sort's other value buffer: free after the sort.
+__device__ __forceinline__ uint32_t* spare_vals(const KnnArgs& a) {
+  return (a.sort_ctrl[a.sort_passes] & 1u) ? a.vals[0] : a.vals[1];
+}
+constexpr int kTodo = 12;  // word of `heads` that counts the points left to the warps
+
+// First sorted position in [lo, n) whose key is at least `key`.
+__device__ __forceinline__ int64_t lower_bound(const uint32_t* keys, int64_t lo, int64_t n, uint64_t key) {
+  int64_t hi = n;
+  while (lo < hi) {
+    const int64_t mid = (lo + hi) >> 1;
+    if ((uint64_t)keys[mid] < key) lo = mid + 1; else hi = mid;
+  }
+  return lo;
+}
+
+// Insert the squared distance of sorted point j into the sorted list of the
+// three smallest.
+__device__ __forceinline__ void near_point(const KnnArgs& a, int64_t j, float px, float py, float pz,
+                                           float (&best)[3]) {
+  const float4 q = a.sorted[j];
+  const float ex = q.x - px, ey = q.y - py, ez = q.z - pz;
+  const float d2 = fmaf(ex, ex, fmaf(ey, ey, ez * ez));
+  if (d2 < best[2]) {
+    best[2] = d2 < best[1] ? best[1] : d2;
+    best[1] = d2 < best[0] ? best[0] : fminf(d2, best[1]);
+    best[0] = fminf(d2, best[0]);
+  }
+}
+
+// One axis of the 3^3 cells around a point's cell c (of dim cells; f: the
+// point's fraction of it): per neighbour the spread coordinate and the squared
+// distance to it (3e38 outside the grid), less a margin for the rounding of f
+// (1e-4 of a finest cell).  *border: distance to the nearer side of the cell.
+struct CellAxis {
+  uint32_t code[3];
+  float gap2[3];
+};
+__device__ __forceinline__ CellAxis cell_axis(int c, int dim, float f, float cell, float* border) {
+  CellAxis x;
+  const float lo = fmaxf(f - 2e-3f, 0.f) * cell, hi = fmaxf(1.f - f - 2e-3f, 0.f) * cell;
+  x.code[0] = spread3((uint32_t)(c - 1));
+  x.code[1] = spread3((uint32_t)c);
+  x.code[2] = spread3((uint32_t)(c + 1));
+  x.gap2[0] = c > 0 ? lo * lo * 0.999f : 3.0e38f;
+  x.gap2[1] = 0.f;
+  x.gap2[2] = c + 1 < dim ? hi * hi * 0.999f : 3.0e38f;
+  *border = fminf(*border, fminf(f, 1.f - f));
+  return x;
 }
 
 }  // namespace
 
-__global__ void __launch_bounds__(256) knn_cell_keys_kernel(KnnArgs a, uint64_t* __restrict__ keys,
-                                                            uint32_t* __restrict__ vals) {
+__global__ void __launch_bounds__(256) knn_keys_kernel(KnnArgs a) {
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < a.n; i += (int64_t)gridDim.x * blockDim.x) {
-    int cx, cy, cz;
-    cell_of(a, a.pts[3 * i], a.pts[3 * i + 1], a.pts[3 * i + 2], cx, cy, cz);
-    keys[i] = cell_id(a, cx, cy, cz);
-    vals[i] = (uint32_t)i;
+    const int64_t src = a.sel ? a.sel[i] : i;
+    const uint32_t x = fine_cell(a.pts[3 * src], a.lo[0], a.inv_cell);
+    const uint32_t y = fine_cell(a.pts[3 * src + 1], a.lo[1], a.inv_cell);
+    const uint32_t z = fine_cell(a.pts[3 * src + 2], a.lo[2], a.inv_cell);
+    a.keys[0][i] = spread3(x) | (spread3(y) << 1) | (spread3(z) << 2);
+    a.vals[0][i] = (uint32_t)i;
   }
 }
 
-// Insert the first sorted position of every cell into the table.
-__global__ void __launch_bounds__(256) knn_cell_table_kernel(KnnArgs a) {
-  const uint64_t mask = (1ull << a.table_bits) - 1ull;
+// The points in sorted order (position and output index in one float4), and
+// the heads per level.
+__global__ void __launch_bounds__(256) knn_sorted_points_kernel(KnnArgs a) {
+  __shared__ uint32_t s_heads[kMortonBits];
+  if (threadIdx.x < kMortonBits) s_heads[threadIdx.x] = 0;
+  __syncthreads();
+  const uint32_t* keys = sorted_keys(a);
+  const uint32_t* vals = keys == a.keys[1] ? a.vals[1] : a.vals[0];
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < a.n; i += (int64_t)gridDim.x * blockDim.x) {
-    const uint64_t key = a.skeys[i];
-    if (i > 0 && a.skeys[i - 1] == key) continue;
-    for (uint64_t s = slot_of(key, a.table_bits), probes = 0; probes <= mask; s = (s + 1) & mask, probes++) {
-      const unsigned long long prev =
-          atomicCAS(reinterpret_cast<unsigned long long*>(a.table_keys + s), (unsigned long long)kEmptySlot,
-                    (unsigned long long)key);
-      if (prev == kEmptySlot) {
-        a.table_start[s] = (uint32_t)i;
+    const uint32_t o = vals[i];
+    if ((int64_t)o >= a.n) continue;  // (only after a sort that gave up)
+    const int64_t src = a.sel ? a.sel[o] : (int64_t)o;
+    a.sorted[i] = make_float4(a.pts[3 * src], a.pts[3 * src + 1], a.pts[3 * src + 2], __uint_as_float(o));
+    const uint32_t diff = i > 0 ? keys[i] ^ keys[i - 1] : 0u;
+    if (diff) atomicAdd(&s_heads[min((31 - __clz(diff)) / 3, kMortonBits - 1)], 1u);
+  }
+  __syncthreads();
+  if (threadIdx.x < kMortonBits && s_heads[threadIdx.x]) atomicAdd(a.heads + threadIdx.x, s_heads[threadIdx.x]);
+}
+
+// Insert every cell of the chosen level with its run of sorted points.  The
+// end of a run is found by doubling steps and bisection, so that a cell of
+// many points does not make one thread walk it.
+__global__ void __launch_bounds__(256) knn_table_kernel(KnnArgs a) {
+  const int sh = 3 * pick_level(a);
+  const uint32_t* keys = sorted_keys(a);
+  const uint32_t mask = (uint32_t)((1ull << a.table_bits) - 1ull);
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < a.n; i += (int64_t)gridDim.x * blockDim.x) {
+    const uint32_t cell = keys[i] >> sh;
+    if (i > 0 && keys[i - 1] >> sh == cell) continue;
+    int64_t step = 1, lo = i + 1;
+    while (i + step < a.n && keys[i + step] >> sh == cell) {
+      lo = i + step + 1;
+      step *= 2;
+    }
+    const int64_t end = lower_bound(keys, lo, min(a.n, i + step), ((uint64_t)cell + 1) << sh);
+    for (uint32_t s = slot_of(cell, a.table_bits), probes = 0; probes <= mask; s = (s + 1) & mask, probes++) {
+      if (atomicCAS(&a.table[s].x, kEmptySlot, cell) == kEmptySlot) {
+        a.table[s].y = (uint32_t)i;
+        a.table[s].z = (uint32_t)end;
         break;
       }
     }
   }
 }
 
-// One thread per point (in cell order): the k smallest squared distances to
-// other points over cubes of (2 r + 1)^3 cells, r = 1, 2, ..., until the
-// k-th lies within r cells (every point closer than r cell widths lies in
-// the cube), then out[point] = 0.5 log(max(1e-14, mean)).
-__global__ void __launch_bounds__(256) knn_query_kernel(KnnArgs a) {
-  constexpr int KMAX = 8;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < a.n; i += (int64_t)gridDim.x * blockDim.x) {
-    const uint32_t me = a.svals[i];
-    const float px = a.pts[3 * me], py = a.pts[3 * me + 1], pz = a.pts[3 * me + 2];
-    int cx, cy, cz;
-    cell_of(a, px, py, pz, cx, cy, cz);
-    float best[KMAX];
+__device__ __forceinline__ void write_scale(const KnnArgs& a, const float4& me, const float (&best)[3]) {
+  float sum = 0.f;
 #pragma unroll
-    for (int k = 0; k < KMAX; k++) best[k] = 3.0e38f;
-    const int maxr = max(a.dims[0], max(a.dims[1], a.dims[2]));
-    for (int r = 1; r <= maxr; r++) {
-      for (int dz = -r; dz <= r; dz++)
-        for (int dy = -r; dy <= r; dy++)
-          for (int dx = -r; dx <= r; dx++) {
-            // only the shell of the cube: the inside was examined with r - 1
-            if (r > 1 && max(abs(dx), max(abs(dy), abs(dz))) < r) continue;
-            const int x = cx + dx, y = cy + dy, z = cz + dz;
-            if (x < 0 || y < 0 || z < 0 || x >= a.dims[0] || y >= a.dims[1] || z >= a.dims[2]) continue;
-            const uint64_t key = cell_id(a, x, y, z);
-            const int64_t s0 = cell_start(a, key);
-            if (s0 < 0) continue;
-            for (int64_t j = s0; j < a.n && a.skeys[j] == key; j++) {
-              const uint32_t o = a.svals[j];
-              if (o == me) continue;
-              const float ex = a.pts[3 * o] - px, ey = a.pts[3 * o + 1] - py, ez = a.pts[3 * o + 2] - pz;
-              float d2 = fmaf(ex, ex, fmaf(ey, ey, ez * ez));
-              // insert into the sorted list of the k best
+  for (int k = 0; k < 3; k++) sum += best[k];
+  const uint32_t o = __float_as_uint(me.w);
+  if ((int64_t)o < a.n) a.out[o] = 0.5f * logf(fmaxf(sum / 3.f, 1e-14f));
+}
+
+// The cells around a sorted point at one level.
+struct CellCube {
+  CellAxis x, y, z;
+  float border;
+  __device__ __forceinline__ CellCube(const KnnArgs& a, const float4& me, uint32_t key, int l) {
+    const int dim = 1 << (kMortonBits - l);
+    const float scale = 1.f / (float)(1 << l), cell = a.cell * (float)(1 << l);
+    const int cx = (int)gather3(key) >> l, cy = (int)gather3(key >> 1) >> l, cz = (int)gather3(key >> 2) >> l;
+    border = 1.f;
+    x = cell_axis(cx, dim, (me.x - a.lo[0]) * a.inv_cell * scale - (float)cx, cell, &border);
+    y = cell_axis(cy, dim, (me.y - a.lo[1]) * a.inv_cell * scale - (float)cy, cell, &border);
+    z = cell_axis(cz, dim, (me.z - a.lo[2]) * a.inv_cell * scale - (float)cz, cell, &border);
+  }
+  // squared distance within which every point lies in the cube
+  __device__ __forceinline__ float reach2(const KnnArgs& a, int l) const {
+    const float r = (1.f + border - 2e-3f) * a.cell * (float)(1 << l) * 0.999f;
+    return r * r;
+  }
+};
+
+// One thread per point, in Morton order: the 3 smallest squared distances to
+// other points, then out[point] = 0.5 log(max(1e-14, mean)).  The points next
+// to it in sorted order bound the third distance; the runs of those of the 3^3
+// cells around it that the bound reaches are listed in shared memory, and one
+// loop goes through all of their points.  (A loop per cell made every warp pay
+// for its fullest cell 27 times.)  A point whose third distance is not inside
+// the cube goes on the list of the next kernel.
+constexpr int kQueryThreads = 128;
+__global__ void __launch_bounds__(kQueryThreads) knn_query_kernel(KnnArgs a) {
+  __shared__ uint2 s_run[27][kQueryThreads];
+  const int64_t i = (int64_t)blockIdx.x * kQueryThreads + threadIdx.x;
+  if (i >= a.n) return;
+  const int level = pick_level(a);
+  const uint32_t* keys = sorted_keys(a);
+  const float4 me = a.sorted[i];
+  float best[3] = {3.0e38f, 3.0e38f, 3.0e38f};
+  for (int64_t j = max((int64_t)0, i - 4); j < min(a.n, i + 5); j++)
+    if (j != i) near_point(a, j, me.x, me.y, me.z, best);
+  const float bound = best[2];
+  const CellCube c(a, me, keys[i], level);
+  int runs = 0;
 #pragma unroll
-              for (int k = 0; k < KMAX; k++) {
-                if (k < a.k && d2 < best[k]) {
-                  const float t = best[k];
-                  best[k] = d2;
-                  d2 = t;
-                }
-              }
-            }
-          }
-      // (with a margin for the rounding of the cell coordinates)
-      const float reach = (float)r * a.cell * 0.999f;
-      if (best[a.k - 1] <= reach * reach) break;
+  for (int q = 0; q < 27; q++) {
+    const int x = q % 3, y = q / 3 % 3, z = q / 9;
+    // (3e38: a cell outside the grid)
+    const float gap2 = c.x.gap2[x] + c.y.gap2[y] + c.z.gap2[z];
+    if (gap2 > bound || gap2 >= 3.0e38f) continue;
+    const uint2 run = cell_run(a, c.x.code[x] | (c.y.code[y] << 1) | (c.z.code[z] << 2));
+    if (run.y > run.x) s_run[runs++][threadIdx.x] = run;
+  }
+  best[0] = best[1] = best[2] = 3.0e38f;  // (the cells hold the neighbours in sorted order too)
+  uint32_t j = 0, end = 0;
+  int r = 0;
+  while (true) {
+    if (j == end) {
+      if (r == runs) break;
+      const uint2 run = s_run[r++][threadIdx.x];
+      j = run.x;
+      end = run.y;
     }
-    float sum = 0.f;
+    if ((int64_t)j != i) near_point(a, j, me.x, me.y, me.z, best);
+    j++;
+  }
+  if (best[2] <= c.reach2(a, level)) write_scale(a, me, best);
+  else spare_vals(a)[atomicAdd(a.heads + kTodo, 1u)] = (uint32_t)i;
+}
+
+// The points left over (a few in a thousand on a surface; isolated ones among
+// them need cubes that hold thousands of others): one warp each, over the
+// cubes of 3^3 cells of coarser and coarser levels until the third distance is
+// inside.  Lanes find the 27 runs by bisection, share the points of the runs,
+// and merge their three best.
+__global__ void __launch_bounds__(256) knn_far_kernel(KnnArgs a) {
+  const int level = pick_level(a), lane = threadIdx.x & 31;
+  const uint32_t* keys = sorted_keys(a);
+  const int64_t todo = min((int64_t)a.heads[kTodo], a.n);
+  const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t t = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; t < todo; t += warps) {
+    const int64_t i = spare_vals(a)[t];
+    const float4 me = a.sorted[i];
+    float third[3] = {3.0e38f, 3.0e38f, 3.0e38f};
+    for (int l = min(level + 1, kMortonBits); l <= kMortonBits; l++) {
+      const CellCube c(a, me, keys[i], l);
+      const int x = lane % 3, y = lane / 3 % 3, z = lane / 9;
+      uint32_t lo = 0, hi = 0;
+      auto pick = [](const float (&g)[3], int k) { return k == 0 ? g[0] : k == 1 ? g[1] : g[2]; };
+      auto code = [](const uint32_t (&g)[3], int k) { return k == 0 ? g[0] : k == 1 ? g[1] : g[2]; };
+      if (lane < 27) {
+        const float gap2 = pick(c.x.gap2, x) + pick(c.y.gap2, y) + pick(c.z.gap2, z);
+        if (!(gap2 > third[2]) && gap2 < 3.0e38f) {
+          const uint64_t k = code(c.x.code, x) | (code(c.y.code, y) << 1) | (code(c.z.code, z) << 2);
+          lo = (uint32_t)lower_bound(keys, 0, a.n, k << (3 * l));
+          hi = (uint32_t)lower_bound(keys, lo, a.n, (k + 1) << (3 * l));
+        }
+      }
+      float best[3] = {3.0e38f, 3.0e38f, 3.0e38f};
+      for (int q = 0; q < 27; q++) {
+        const uint32_t s0 = __shfl_sync(0xffffffffu, lo, q), s1 = __shfl_sync(0xffffffffu, hi, q);
+        for (uint32_t j = s0 + lane; j < s1; j += 32)
+          if ((int64_t)j != i) near_point(a, j, me.x, me.y, me.z, best);
+      }
+      // the three smallest of the lanes' lists (distances order like their bits)
 #pragma unroll
-    for (int k = 0; k < KMAX; k++) sum += k < a.k ? best[k] : 0.f;
-    a.out[me] = 0.5f * logf(fmaxf(sum / (float)a.k, 1e-14f));
+      for (int k = 0; k < 3; k++) {
+        const uint32_t m = __reduce_min_sync(0xffffffffu, __float_as_uint(best[0]));
+        const uint32_t who = __ballot_sync(0xffffffffu, __float_as_uint(best[0]) == m);
+        if (lane == __ffs((int)who) - 1) {
+          best[0] = best[1];
+          best[1] = best[2];
+          best[2] = 3.0e38f;
+        }
+        third[k] = __uint_as_float(m);
+      }
+      if (third[2] <= c.reach2(a, l)) break;
+    }
+    if (lane == 0) write_scale(a, me, third);
   }
 }
 
-void launch_knn_bounds(const float* pts, int64_t n, float* part, int nparts, float* out, cudaStream_t s) {
-  knn_bounds_kernel<<<nparts, 256, 0, s>>>(pts, n, part);
-  knn_bounds_finish_kernel<<<1, 32, 0, s>>>(part, nparts, out);
+void launch_knn_bounds(const float* pts, const int64_t* sel, int64_t n, float* part, int nparts, float* out,
+                       cudaStream_t s) {
+  knn_bounds_kernel<<<nparts, 256, 0, s>>>(pts, sel, n, part);
+  knn_bounds_finish_kernel<<<1, 192, 0, s>>>(part, nparts, out);
 }
 
-void launch_knn_keys(const KnnArgs& a, uint64_t* keys, uint32_t* vals, cudaStream_t s) {
-  const int64_t blocks = std::min<int64_t>((a.n + 255) / 256, (int64_t)sm_count() * 32);
-  knn_cell_keys_kernel<<<(unsigned)std::max<int64_t>(blocks, 1), 256, 0, s>>>(a, keys, vals);
+static unsigned knn_blocks(int64_t n) {
+  return (unsigned)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, (int64_t)sm_count() * 32));
 }
+
+void launch_knn_keys(const KnnArgs& a, cudaStream_t s) { knn_keys_kernel<<<knn_blocks(a.n), 256, 0, s>>>(a); }
+
+int knn_key_bits() { return 3 * kMortonBits; }
 
 void launch_knn_query(const KnnArgs& a, cudaStream_t s) {
-  const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>((a.n + 255) / 256, (int64_t)sm_count() * 32));
-  knn_cell_table_kernel<<<(unsigned)blocks, 256, 0, s>>>(a);
-  knn_query_kernel<<<(unsigned)((a.n + 255) / 256), 256, 0, s>>>(a);
+  knn_sorted_points_kernel<<<knn_blocks(a.n), 256, 0, s>>>(a);
+  knn_table_kernel<<<knn_blocks(a.n), 256, 0, s>>>(a);
+  knn_query_kernel<<<(unsigned)((a.n + kQueryThreads - 1) / kQueryThreads), kQueryThreads, 0, s>>>(a);
+  knn_far_kernel<<<knn_blocks(a.n), 256, 0, s>>>(a);
 }
 
 // ---------------------------------------------------------------- initial parameters
@@ -464,26 +673,9 @@ __global__ void __launch_bounds__(256) init_params_kernel(InitArgs a) {
   for (int k = 0; k < a.planes - 11; k++) P[(11 + k) * S + g] = k < 3 ? dc : 0.f;
 }
 
-// Gather the selected points (for the neighbour search, which runs on the
-// selected set).
-__global__ void __launch_bounds__(256) init_gather_kernel(const float* __restrict__ pts,
-                                                          const int64_t* __restrict__ sel, int64_t n,
-                                                          float* __restrict__ out) {
-  const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (g >= n) return;
-  const int64_t s = sel[g];
-#pragma unroll
-  for (int d = 0; d < 3; d++) out[3 * g + d] = pts[3 * s + d];
-}
-
 void launch_init_params(const InitArgs& a, cudaStream_t s) {
   if (a.n <= 0) return;
   init_params_kernel<<<(unsigned)((a.n + 255) / 256), 256, 0, s>>>(a);
-}
-
-void launch_init_gather(const float* pts, const int64_t* sel, int64_t n, float* out, cudaStream_t s) {
-  if (n <= 0) return;
-  init_gather_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(pts, sel, n, out);
 }
 
 }  // namespace gs

@@ -241,20 +241,26 @@ void launch_iso_count(const IsoArgs& a, cudaStream_t s);  // sides and block_cou
 void launch_iso_emit(const IsoArgs& a, cudaStream_t s);
 
 struct KnnArgs {
-  const float* pts;  // [n][3]
+  const float* pts;      // [m][3]
+  const int64_t* sel;    // [n] the points searched (NULL: the first n)
   int64_t n;
-  int k;             // 1..8 neighbours
-  float lo[3], cell, inv_cell;
-  int dims[3];
-  const uint64_t* skeys;  // cell ids, sorted
-  const uint32_t* svals;  // point of each sorted position
-  uint64_t* table_keys;   // [2^table_bits] cell id (all ones: empty)
-  uint32_t* table_start;  // first sorted position of the cell
+  float lo[3], cell, inv_cell;  // finest cells
+  uint32_t* keys[2];     // [n] Morton codes of the finest cells; the sort's buffers
+  uint32_t* vals[2];     // [n] points
+  const uint32_t* sort_ctrl;  // sort_ctrl[sort_passes] bit 0: which buffer is sorted
+  int sort_passes;
+  float4* sorted;        // [n] points in sorted order: x, y, z, bits of the point's index
+  uint32_t* heads;       // [16], zeroed: sorted points that start a cell, by the coarsest level at which they do;
+                         // [12] the points that the first query leaves over
+  uint4* table;          // [2^table_bits] cell, first and one past the last sorted point (cell all ones: empty)
   int table_bits;
-  float* out;        // [n] log-scales
+  float* out;            // [n] log-scales
 };
-void launch_knn_bounds(const float* pts, int64_t n, float* part, int nparts, float* out, cudaStream_t s);
-void launch_knn_keys(const KnnArgs& a, uint64_t* keys, uint32_t* vals, cudaStream_t s);
+// out: min xyz, max xyz of the points
+void launch_knn_bounds(const float* pts, const int64_t* sel, int64_t n, float* part, int nparts, float* out,
+                       cudaStream_t s);
+int knn_key_bits();
+void launch_knn_keys(const KnnArgs& a, cudaStream_t s);
 void launch_knn_query(const KnnArgs& a, cudaStream_t s);
 
 struct InitArgs {
@@ -269,7 +275,6 @@ struct InitArgs {
   int planes;
 };
 void launch_init_params(const InitArgs& a, cudaStream_t s);
-void launch_init_gather(const float* pts, const int64_t* sel, int64_t n, float* out, cudaStream_t s);
 
 // Adaptive density control (densify.cu).
 struct DensifyArgs {
