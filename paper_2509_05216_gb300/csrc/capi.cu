@@ -88,7 +88,7 @@ struct gs_ctx {
       target_slot, host_tgt0, host_tgt1, pair_stats, cells, vismask, ssim_table, ssim_partials, ssim_sums,
       init_pts, init_scales, knn_part, knn_table, knn_heads, ord_keys0, ord_keys1, ord_vals0, ord_vals1, ord_total, ord_hist,
       ord_hist_scan, ord_lookback, ord_counters, ord_views, tile_order, vis_sums, vis_offsets, dtotal, dkeys0,
-      dkeys1, dvals0, dvals1, dhist_scan, dorder, torder, iso_work, densify_source;
+      dkeys1, dvals0, dvals1, dhist_scan, dorder, torder, iso_work, densify_source, pair_flags, contrib;
 
   // launch accounting and optional per-kernel event timing
   struct KStat {
@@ -464,7 +464,7 @@ void gs_destroy(gs_ctx* c) {
                     &c->init_pts, &c->init_scales, &c->knn_part, &c->knn_table, &c->knn_heads, &c->ord_keys0, &c->ord_keys1,
                     &c->ord_vals0, &c->ord_vals1, &c->ord_total, &c->ord_hist, &c->ord_hist_scan, &c->ord_lookback,
                     &c->ord_counters, &c->ord_views, &c->tile_order, &c->vis_sums, &c->vis_offsets, &c->dtotal,
-                    &c->dkeys0, &c->dkeys1, &c->dvals0, &c->dvals1, &c->dhist_scan, &c->dorder, &c->torder, &c->iso_work, &c->densify_source};
+                    &c->dkeys0, &c->dkeys1, &c->dvals0, &c->dvals1, &c->dhist_scan, &c->dorder, &c->torder, &c->iso_work, &c->densify_source, &c->pair_flags, &c->contrib};
   for (DevBuf* b : bufs)
     if (b->p) cudaFree(b->p);
   for (const auto& p : c->pending) {
@@ -928,9 +928,28 @@ gs_status gs_raster_bwd(gs_ctx* c, const gs_params* params, const float* dL_dima
   r.dimage = dL_dimages;
   r.g2d = P<float>(c->g2d);
   r.direct_max = c->bwd_direct;
+  // The compositing backward can flag the (view, Gaussian) pairs that it adds a
+  // gradient to, so that the projection backward reads only their records.
+  // The reads saved grow with the pairs, the flags' cost with the entries
+  // walked, roughly the pixels: 64M pairs on 67M pixels (4M Gaussians, 16
+  // views of 2048^2) 0.44 ms saved, 0.15 ms spent; 4M pairs on 8.4M pixels
+  // (500,000 Gaussians, 8 views of 1024^2) 16 us saved, 31 us spent; so from
+  // three pairs on four pixels.
+  const bool flagged = c->B > 1 && raster_bwd_flags(c->raster_bwd) && 4 * (int64_t)c->B * c->n >= 3 * c->pixels;
+  if (flagged) {
+    const size_t flag_bytes = (size_t)c->B * c->stride;
+    GS_TRY(ensure(c, c->pair_flags, flag_bytes));
+    GS_TRY(ensure(c, c->contrib, sizeof(uint64_t) * c->stride));
+    GS_CUDA(c, cudaMemsetAsync(c->pair_flags.p, 0, flag_bytes, c->stream));
+    r.pair_flags = P<uint8_t>(c->pair_flags);
+  }
   {
     LaunchScope ls(c, "raster_bwd");
     launch_raster_bwd(r, c->bins, c->raster_bwd, c->stream);
+  }
+  if (flagged) {
+    LaunchScope ls(c, "pair_masks");
+    launch_pair_masks(r.pair_flags, c->stride, c->B, P<uint64_t>(c->contrib), c->stream);
   }
   GS_CHECK_LAUNCH(c);
   ProjectBwdArgs b{};
@@ -941,6 +960,7 @@ gs_status gs_raster_bwd(gs_ctx* c, const gs_params* params, const float* dL_dima
   b.B = c->B;
   b.g2d = P<float>(c->g2d);
   b.grads = grads->data;
+  b.contrib = P<uint64_t>(flagged ? c->contrib : c->vismask);
   b.vismask = P<uint64_t>(c->vismask);
   b.dens_grad = c->dens_grad;
   b.dens_count = c->dens_count;

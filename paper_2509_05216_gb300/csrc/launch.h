@@ -30,7 +30,8 @@ struct ProjectBwdArgs {
   int B;
   const float* g2d;   // [B][stride] geometry records (kG2dGeo floats), then [B][stride] colour records (kG2dCol)
   float* grads;       // [P][stride]
-  const uint64_t* vismask;  // [stride] views where the Gaussian touches a tile (others: zero 2D gradient)
+  const uint64_t* contrib;  // [stride] views whose 2D gradient may be nonzero (the others are not read)
+  const uint64_t* vismask;  // [stride] views where the Gaussian touches a tile
   float* dens_grad;   // densification statistic (NULL: not accumulated): += sum of NDC mean-gradient norms
   float* dens_count;  //   and += the number of views where the Gaussian touches a tile
 };
@@ -91,6 +92,8 @@ struct RasterArgs {
   const uint32_t* tile_order;
   const float* dimage;  // backward only
   float* g2d;           // backward only: [B][stride] geometry records, then [B][stride] colour records
+  uint8_t* pair_flags;  // backward only: [B][stride], set to 1 for the pairs that a gradient is added to (NULL: not kept;
+                        // raster_bwd_flags says which kernels keep them)
   int direct_max;       // backward only: at most this many contributing lanes -> per-lane atomics
   // forward fused with the L1 loss (target non-NULL or read from target_slot):
   // writes dL/dimage = sign(image - target) * inv_count and one partial sum
@@ -108,6 +111,8 @@ int sm_count();
 int project_fwd_block();
 void launch_project_fwd(const ProjectArgs& a, int deg, cudaStream_t s);
 void launch_project_bwd(const ProjectBwdArgs& a, int deg, cudaStream_t s);
+// masks[g] bit v = flags[v][g] (stride a multiple of 4)
+void launch_pair_masks(const uint8_t* flags, int64_t stride, int B, uint64_t* masks, cudaStream_t s);
 
 struct ScanArgs {
   int64_t nb;  // counts per view
@@ -190,6 +195,7 @@ int64_t l1_finish_scratch_bytes();
 void launch_l1_finish(const float* partial, int64_t nparts, double* scratch, double inv_count, float* loss,
                       cudaStream_t s);
 void launch_raster_bwd(const RasterArgs& a, int64_t bins, int ppt, cudaStream_t s);
+bool raster_bwd_flags(int ppt);
 // out[0] += list entries up to each pixel's last contributor, out[1] += contributing pairs
 void launch_pair_stats(const RasterArgs& a, int64_t bins, unsigned long long* out, cudaStream_t s);
 

@@ -328,11 +328,11 @@ __global__ void __launch_bounds__(128, 4) project_bwd_color_kernel(ProjectBwdArg
   if (g >= a.n) return;
   const float* P = a.params;
   const int64_t S = a.stride;
-  // only the views where the Gaussian touches a tile have a nonzero 2D
-  // gradient, and only their records are read; the parameters are loaded
-  // without waiting for the mask (a Gaussian invisible in every view reads
+  // only the views where the Gaussian contributed to a pixel have a nonzero
+  // 2D gradient, and only their records are read; the parameters are loaded
+  // without waiting for the mask (a Gaussian that contributed to none reads
   // them for nothing, but no load of the prologue waits on another)
-  uint64_t vm = a.vismask[g];
+  uint64_t vm = a.contrib[g];
   float mean[3], sh[3][K], gsh[3][K];
 #pragma unroll
   for (int k = 0; k < K; k++)
@@ -411,7 +411,7 @@ __global__ void __launch_bounds__(128, 5) project_bwd_geom_kernel(ProjectBwdArgs
   if (g >= a.n) return;
   const float* P = a.params;
   const int64_t S = a.stride;
-  uint64_t vm = a.vismask[g];
+  uint64_t vm = a.contrib[g];
   float* G = a.grads;
   float mean[3], lsc[3], quat[4];
 #pragma unroll
@@ -421,7 +421,11 @@ __global__ void __launch_bounds__(128, 5) project_bwd_geom_kernel(ProjectBwdArgs
 #pragma unroll
   for (int i = 0; i < 4; i++) quat[i] = __ldg(P + (6 + i) * S + g);
   const float op = __ldg(P + 10 * S + g);  // (loaded before the mask is known, as above)
-  if (!vm) {  // no tile in any view: every gradient of this Gaussian is zero
+  // densification statistic: the screen-space mean gradient in normalised
+  // device coordinates, summed over the views where the Gaussian touches a
+  // tile, and the number of those views
+  if (a.dens_grad) a.dens_count[g] += (float)__popcll(a.vismask[g]);
+  if (!vm) {  // no contribution in any view: every gradient of this Gaussian is zero
     // (the mean planes were written by the colour part)
 #pragma unroll
     for (int i = 3; i < 11; i++) G[i * S + g] = 0.f;
@@ -445,11 +449,8 @@ __global__ void __launch_bounds__(128, 5) project_bwd_geom_kernel(ProjectBwdArgs
   float cur[6], nxt[6];
   int vn = __ffsll((long long)vm) - 1;
   load6(vn, cur);
-  // densification statistic: the screen-space mean gradient in normalised
-  // device coordinates, summed over the views where the Gaussian touches a
-  // tile, and the number of those views
-  float dens_g = 0.f, dens_c = 0.f;
-  while (vn >= 0) {  // the views where the Gaussian touches a tile
+  float dens_g = 0.f;
+  while (vn >= 0) {  // the views where the Gaussian contributed to a pixel
     const int v = vn;
     vm &= vm - 1;
     vn = vm ? __ffsll((long long)vm) - 1 : -1;
@@ -461,7 +462,6 @@ __global__ void __launch_bounds__(128, 5) project_bwd_geom_kernel(ProjectBwdArgs
       const ViewRec& Vd = s_views[v];
       const float nx = gmx * 0.5f * (float)Vd.W, ny = gmy * 0.5f * (float)Vd.H;
       dens_g += sqrtf(fmaf(nx, nx, ny * ny));
-      dens_c += 1.f;
     }
     if (gmx == 0.f && gmy == 0.f && gA == 0.f && gB == 0.f && gC == 0.f && gsig == 0.f) continue;
     const ViewRec& V = s_views[v];
@@ -552,15 +552,39 @@ __global__ void __launch_bounds__(128, 5) project_bwd_geom_kernel(ProjectBwdArgs
   const float dq = gqn[0] * gc.qn[0] + gqn[1] * gc.qn[1] + gqn[2] * gc.qn[2] + gqn[3] * gc.qn[3];
 #pragma unroll
   for (int i = 0; i < 3; i++) G[i * S + g] += gm[i];
-  if (a.dens_grad) {
-    a.dens_grad[g] += dens_g;
-    a.dens_count[g] += dens_c;
-  }
+  if (a.dens_grad) a.dens_grad[g] += dens_g;
 #pragma unroll
   for (int i = 0; i < 3; i++) G[(3 + i) * S + g] = gls[i];
 #pragma unroll
   for (int i = 0; i < 4; i++) G[(6 + i) * S + g] = (gqn[i] - gc.qn[i] * dq) * gc.qinv;
   G[10 * S + g] = gop;
+}
+
+// One mask per Gaussian (bit v) from the flags of the pairs that the
+// compositing backward added a gradient to: 64M pairs, 24 us.  The projection
+// backward reads 48 bytes per pair of the masks instead of per visible pair (4M
+// Gaussians, 16 views: 1.59 -> 1.15 ms).
+__global__ void __launch_bounds__(256) pair_masks_kernel(const uint8_t* __restrict__ flags, int64_t stride, int B,
+                                                         uint64_t* __restrict__ masks) {
+  const int64_t g = 4 * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x);
+  if (g >= stride) return;
+  uint64_t mask[4] = {0, 0, 0, 0};
+  for (int v0 = 0; v0 < B; v0 += 8) {
+    uint32_t f[8];
+#pragma unroll
+    for (int i = 0; i < 8; i++)
+      f[i] = v0 + i < B ? __ldg(reinterpret_cast<const uint32_t*>(flags + (int64_t)(v0 + i) * stride + g)) : 0u;
+#pragma unroll
+    for (int i = 0; i < 8; i++)
+#pragma unroll
+      for (int k = 0; k < 4; k++) mask[k] |= (uint64_t)((f[i] >> (8 * k)) & 1u) << (v0 + i);
+  }
+#pragma unroll
+  for (int k = 0; k < 4; k++) masks[g + k] = mask[k];
+}
+
+void launch_pair_masks(const uint8_t* flags, int64_t stride, int B, uint64_t* masks, cudaStream_t s) {
+  pair_masks_kernel<<<(unsigned)((stride + 1023) / 1024), 256, 0, s>>>(flags, stride, B, masks);
 }
 
 void launch_project_fwd(const ProjectArgs& a, int deg, cudaStream_t s) {

@@ -1126,6 +1126,7 @@ __global__ void __launch_bounds__(64, 10) raster_bwd4_kernel(RasterArgs a, int64
   const uint32_t* __restrict__ cells = a.cells + cells_offset(rg.x, bin) + cell;
   float* const geo = a.g2d + kG2dGeo * (int64_t)v * a.stride;
   float* const col = a.g2d + kG2dGeo * (int64_t)a.B * a.stride + kG2dCol * (int64_t)v * a.stride;
+  uint8_t* const flags = a.pair_flags ? a.pair_flags + (int64_t)v * a.stride : nullptr;
   const bool odd = lane & 1;
   const uint32_t pair = 3u << (lane & 30);
 
@@ -1154,6 +1155,8 @@ __global__ void __launch_bounds__(64, 10) raster_bwd4_kernel(RasterArgs a, int64
         sm.s0[pn + 1 + lane] = n0;
         sm.s1[pn + 1 + lane] = n1;
         sm.sx[pn + 1 + lane] = make_float2(n2.x, __uint_as_float(g));
+        // (an index at or above n only comes after a capacity overflow)
+        if (flags && (int64_t)g < a.n) flags[g] = 1;
       }
       __syncwarp();
     }
@@ -1341,6 +1344,8 @@ void launch_raster_fwd(const RasterArgs& a, int64_t bins, int ppt, cudaStream_t 
     default: raster_fwd_cells_kernel<1><<<(unsigned)bins, 128, 0, s>>>(a); break;
   }
 }
+
+bool raster_bwd_flags(int ppt) { return ppt == 4; }
 
 void launch_raster_bwd(const RasterArgs& a, int64_t bins, int ppt, cudaStream_t s) {
   if (bins == 0) return;
