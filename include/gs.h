@@ -139,15 +139,16 @@ typedef enum {
                             thread with one block per tile, 8 = one warp per
                             tile.  All variants give the same result up to
                             FP32 rounding. */
-  GS_OPT_RASTER_BWD = 1, /* backward compositing kernel, same values */
-  GS_OPT_BWD_DIRECT = 2, /* backward: a warp whose pixels meet a Gaussian in at
-                            most this many lanes (0..32, default 2) adds the
-                            lanes' gradients with per-lane atomics instead of
-                            a warp reduction.  Same result up to FP32
-                            summation order. */
+  GS_OPT_RASTER_BWD = 1, /* backward compositing kernel, same values (unless
+                            set: 8 for batches of many tiles, 4 otherwise) */
+  GS_OPT_BWD_DIRECT = 2, /* backward with 1 or 2 pixels per thread: a warp whose
+                            pixels meet a Gaussian in at most this many lanes
+                            (0..32, default 2) adds the lanes' gradients with
+                            per-lane atomics instead of a warp reduction.
+                            Same result up to FP32 summation order. */
   GS_OPT_SORT_ITEMS = 3, /* keys per thread of a radix-sort partition: 12, 16
                             (default), 20 or 24 (partitions of 256 x items
-                            keys).  Same result.  Fixed once a training graph
+                            keys; short segments take 4 or 8).  Same result.  Fixed once a training graph
                             is captured (GS_ESTATE). */
   GS_OPT_SORT_WAIT = 4,  /* look-back rounds a radix-sort partition waits for
                             the partitions before it: 1 .. 1048576 (default

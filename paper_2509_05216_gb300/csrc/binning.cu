@@ -28,7 +28,7 @@ namespace gs {
 
 // Exclusive scan of per-(view, block) counts, of one or two kinds (the
 // projection's instances and visible pairs; blockIdx.y): block v of the grid
-// scans view v's nb counts (1024 threads looping over chunks) and writes the
+// scans view v's nb counts (1024 threads, 8,192 counts per round) and writes the
 // view's total.  The last block to finish turns the view totals into segment
 // offsets: seg[v] = first of view v, seg[B] = *total.
 __global__ void __launch_bounds__(1024) scan_block_sums_kernel(ScanArgs a, uint32_t* ticket) {
@@ -42,9 +42,15 @@ __global__ void __launch_bounds__(1024) scan_block_sums_kernel(ScanArgs a, uint3
   if (threadIdx.x == 0) carry = 0;
   __syncthreads();
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  for (int64_t base = 0; base < a.nb; base += 1024) {
-    const int64_t i = base + threadIdx.x;
-    uint64_t x = i < a.nb ? sums[i] : 0;
+  // 8 consecutive counts per thread and round
+  for (int64_t base = 0; base < a.nb; base += 8 * 1024) {
+    const int64_t i0 = base + 8 * threadIdx.x;
+    uint32_t c[8];
+    uint64_t x = 0;
+#pragma unroll
+    for (int q = 0; q < 8; q++) c[q] = i0 + q < a.nb ? sums[i0 + q] : 0u;
+#pragma unroll
+    for (int q = 0; q < 8; q++) x += c[q];
     uint64_t inc = x;
 #pragma unroll
     for (int off = 1; off < 32; off <<= 1) {
@@ -64,10 +70,14 @@ __global__ void __launch_bounds__(1024) scan_block_sums_kernel(ScanArgs a, uint3
       warp_tot[lane] = winc - w;  // exclusive over warps
     }
     __syncthreads();
-    const uint64_t excl = carry + warp_tot[wid] + inc - x;
-    if (i < a.nb) offsets[i] = (uint32_t)excl;
+    uint64_t excl = carry + warp_tot[wid] + inc - x;
+#pragma unroll
+    for (int q = 0; q < 8; q++) {
+      if (i0 + q < a.nb) offsets[i0 + q] = (uint32_t)excl;
+      excl += c[q];
+    }
     __syncthreads();
-    if (threadIdx.x == 1023) carry = excl + x;
+    if (threadIdx.x == 1023) carry = excl;
     __syncthreads();
   }
   if (threadIdx.x == 0) {
@@ -319,11 +329,15 @@ struct SortSmem {
   KeyT buf[kTile];                         // keys, then values, in tile-sorted order
 };
 
-// Lanes that hold the same digit, among the lanes with a key: one vote per
-// digit bit.  (__match_any_sync takes a step per distinct value of the warp,
-// and the digits of a radix pass are nearly all distinct: 64M depth keys, three
-// passes, 1.49 -> 1.20 ms.)
+// Lanes that hold the same digit, among the lanes with a key.
+// __match_any_sync takes a step per distinct value of the warp.  The digits of
+// a pass are nearly all distinct, so one vote per digit bit is faster (64M depth
+// keys, three passes: 1.49 -> 1.20 ms); but the last of several passes sorts by
+// the slowest digit, of which a warp holds few values (102M instances by tile,
+// second pass: 0.51 ms by match, 0.60 ms by votes).
+template <bool FEW>
 __device__ __forceinline__ unsigned digit_peers(uint32_t d, bool ok) {
+  if constexpr (FEW) return __match_any_sync(0xffffffffu, ok ? d : (uint32_t)kRadix);
   unsigned peers = __ballot_sync(0xffffffffu, ok);
 #pragma unroll
   for (int b = 0; b < kRadixBits; b++) {
@@ -334,7 +348,7 @@ __device__ __forceinline__ unsigned digit_peers(uint32_t d, bool ok) {
   return peers;
 }
 
-template <typename KeyT, int ITEMS, int MIN_BLOCKS>
+template <typename KeyT, int ITEMS, int MIN_BLOCKS, bool FEW>
 __global__ void __launch_bounds__(kSortThreads, MIN_BLOCKS) onesweep_pass_kernel(SortArgs a, int pass) {
   constexpr int kSortItems = ITEMS;
   constexpr int kSortTile = kSortThreads * ITEMS;
@@ -400,7 +414,7 @@ __global__ void __launch_bounds__(kSortThreads, MIN_BLOCKS) onesweep_pass_kernel
   for (int i = 0; i < kSortItems; i++) {
     const bool ok = wl + 32 * i < n_here;
     const uint32_t d = ok ? (word[i] >> wsh) & (kRadix - 1) : (uint32_t)kRadix;
-    const unsigned peers = digit_peers(d, ok);
+    const unsigned peers = digit_peers<FEW>(d, ok);
     uint32_t r = 0, before = 0;
     if (ok) {
       before = sm.warp_hist[wid][d];
@@ -540,19 +554,25 @@ __global__ void __launch_bounds__(kSortThreads, MIN_BLOCKS) onesweep_pass_kernel
   }
 }
 
-template <typename KeyT, int ITEMS, int MIN_BLOCKS>
-static void launch_pass(const SortArgs& a, int pass, int64_t grid, cudaStream_t s) {
+template <typename KeyT, int ITEMS, int MIN_BLOCKS, bool FEW>
+static void launch_pass_few(const SortArgs& a, int pass, int64_t grid, cudaStream_t s) {
   const size_t smem = sizeof(SortSmem<KeyT, ITEMS>);
   // once per device (the attribute is per device; not repeated inside a graph capture)
   static bool attr_set[64] = {};
   int dev = 0;
   cudaGetDevice(&dev);
   if (dev < 0 || dev >= 64 || !attr_set[dev]) {
-    cudaFuncSetAttribute(onesweep_pass_kernel<KeyT, ITEMS, MIN_BLOCKS>,
+    cudaFuncSetAttribute(onesweep_pass_kernel<KeyT, ITEMS, MIN_BLOCKS, FEW>,
                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (dev >= 0 && dev < 64) attr_set[dev] = true;
   }
-  onesweep_pass_kernel<KeyT, ITEMS, MIN_BLOCKS><<<(unsigned)grid, kSortThreads, smem, s>>>(a, pass);
+  onesweep_pass_kernel<KeyT, ITEMS, MIN_BLOCKS, FEW><<<(unsigned)grid, kSortThreads, smem, s>>>(a, pass);
+}
+
+template <typename KeyT, int ITEMS, int MIN_BLOCKS>
+static void launch_pass(const SortArgs& a, int pass, int64_t grid, cudaStream_t s) {
+  if (pass > 0 && pass == a.npass - 1) launch_pass_few<KeyT, ITEMS, MIN_BLOCKS, true>(a, pass, grid, s);
+  else launch_pass_few<KeyT, ITEMS, MIN_BLOCKS, false>(a, pass, grid, s);
 }
 
 template <typename KeyT>
@@ -675,9 +695,11 @@ constexpr uint64_t kEmitValue = (1ull << 62) - 1;
 constexpr int kEmitThreads = 256;
 constexpr int kEmitWarps = kEmitThreads / 32;
 
-// Visible pairs per thread: 16, or 4 where partitions of 4,096 pairs would
-// leave SMs without one (37,001 Gaussians in 3 views: 37 -> 17 us).
-constexpr int kEmitMany = 16, kEmitFew = 4;
+// Visible pairs per thread: 12 (64M pairs: 0.92 ms; with 16, fewer blocks per
+// SM for their registers, 0.99 ms; with 8, twice the look-backs, 1.01 ms), or 4
+// where partitions of 3,072 pairs would leave SMs without one (37,001
+// Gaussians in 3 views: 37 -> 17 us).
+constexpr int kEmitMany = 12, kEmitFew = 4;
 static int emit_items(int64_t pairs) {
   return pairs >= (int64_t)kEmitThreads * kEmitMany * sm_count() * 2 ? kEmitMany : kEmitFew;
 }

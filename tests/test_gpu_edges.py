@@ -1,13 +1,17 @@
 """Kernels at the sizes where their partitions can go wrong, against the
 oracles (GPU only): words, blocks and ragged rows of the crossings, blocks and
-sample counts of the densification."""
+sample counts of the densification, strips of the image loss, uneven point
+sets, sort and emission partitions, tiles and pair flags of the compositing
+backwards."""
 import numpy as np
 import pytest
 import torch
 
 from oracle import densify as OD
 from oracle import init as OI
+from oracle import ssim as OS
 from paper_2509_05216_gb300 import gs, inputs
+from tests.gpu_helpers import expected_binning, rel_l2, run_forward
 
 pytestmark = pytest.mark.gpu
 
@@ -85,4 +89,110 @@ def test_densify_blocks_and_sample_counts(n, split_n, opacity):
     np.testing.assert_array_equal(mo, rm)
     np.testing.assert_array_equal(vo, rv)
     assert all(bool(torch.isnan(o[:, nout:]).all()) for o in outs)  # nothing past the outputs
+    ctx.close()
+
+
+# strips of 32 columns and 32 rows: narrower, exact, one more; a batch of ragged views
+@pytest.mark.parametrize("sizes", [[(16, 16)], [(32, 32)], [(33, 31)], [(31, 65), (64, 20)], [(97, 129), (16, 200)]])
+def test_ssim_strips(sizes):
+    cams = [inputs.pinhole(inputs.look_at((0.4, -2.8, 1.0)), w, h) for w, h in sizes]
+    scene = inputs.random_scene(64, 0, 3, extent=0.5)
+    ctx = gs.Context(0)
+    ctx.gs_project(dev(scene["params"]), scene["n"], scene["deg"], cams)
+    rng = np.random.default_rng(len(sizes) + sizes[0][0])
+    xs = [rng.uniform(0, 1, (3, h, w)).astype(np.float32) for w, h in sizes]
+    ys = [np.clip(x + rng.normal(0, 0.1, x.shape), 0, 1).astype(np.float32) for x in xs]
+    x, y = (dev(np.concatenate([a.reshape(-1) for a in v])) for v in (xs, ys))
+    loss, grad = torch.zeros(1, device="cuda"), torch.full_like(x, float("nan"))
+    ctx.gs_ssim_loss(x, y, 0.2, loss, grad)
+    ctx.gs_sync()
+    ref, ref_grads = OS.dssim_loss(xs, ys, 0.2)
+    assert abs(loss.item() - ref) <= 1e-6
+    for g, r in zip(gs.split_images(grad, cams), ref_grads):
+        assert rel_l2(g.cpu().numpy().astype(np.float64), r) <= 1e-5
+    ssim, psnr = ctx.gs_image_metrics(x, y, len(cams))
+    for v in range(len(cams)):
+        assert abs(ssim[v] - OS.ssim(xs[v], ys[v])) <= 2e-6 and abs(psnr[v] - OS.psnr(xs[v], ys[v])) <= 1e-4
+    x[5] = float("inf")  # an infinite pixel makes the sums infinite or NaN, not finite
+    ctx.gs_ssim_loss(x, y, 0.0, loss, None)
+    _, psnr = ctx.gs_image_metrics(x, y, len(cams))
+    assert not np.isfinite(loss.item()) and psnr[0] == -np.inf
+    ctx.close()
+
+
+@pytest.mark.parametrize("kind", ["four", "line", "grid", "cluster_outliers", "duplicates", "uniform"])
+def test_neighbour_scales_of_uneven_sets(kind):
+    rng = np.random.default_rng(17)
+    if kind == "four":
+        pts = rng.uniform(-1, 1, (4, 3))
+    elif kind == "line":  # one axis only
+        pts = np.stack([rng.uniform(-5, 5, 1025), np.zeros(1025), np.zeros(1025)], 1)
+    elif kind == "grid":  # every distance tied, points on cell borders
+        pts = np.stack(np.meshgrid(*[np.arange(16.0)] * 3), -1).reshape(-1, 3)
+    elif kind == "cluster_outliers":  # a cluster in a few of the finest cells, and points that must look far
+        pts = np.concatenate([rng.normal(0, 2e-3, (3000, 3)), rng.uniform(-1, 1, (40, 3)), [[1.0, 1.0, 1.0]]])
+    elif kind == "duplicates":
+        pts = np.repeat(rng.uniform(-1, 1, (700, 3)), 5, axis=0)
+    else:
+        pts = rng.uniform(0, 1, (40001, 3))
+    pts = pts[rng.permutation(pts.shape[0])].astype(np.float32)
+    n = pts.shape[0]
+    nrm = np.tile(np.float32([0, 0, 1]), (n, 1))
+    out = torch.zeros((14, n + (-n) % 4), device="cuda")
+    ctx = gs.Context(0)
+    ctx.gs_init_gaussians(dev(pts), dev(nrm), out, n, 0)
+    ctx.gs_sync()
+    ref = OI.knn_log_scales(pts)
+    # FP32 differences of coordinates up to 5: 3e-7 absolute on each distance
+    near = np.exp(ref)
+    np.testing.assert_allclose(out[3, :n].cpu().numpy(), ref, rtol=0, atol=2e-5 + 6e-7 / near.min() * (kind != "duplicates"))
+    ctx.close()
+
+
+# segments on either side of the sizes at which the sorts and the emission change their keys per thread, one view
+# (partitions in ticket order) and several
+@pytest.mark.parametrize("n,views", [(255, 1), (1025, 3), (66000, 1), (66000, 2), (270001, 1), (700000, 2)])
+def test_binning_sizes(n, views):
+    scene = inputs.random_scene(n, 0, 5, extent=0.9, log_scale=(-6.0, -5.0))
+    cams = [inputs.pinhole(inputs.look_at((0.4 + v, -2.8, 1.0)), 320 - 16 * v, 200) for v in range(views)]
+    ctx = gs.Context(0)
+    run_forward(ctx, scene, cams)
+    bufs = [ctx.gs_get_buffer(b).cpu().numpy() for b in (gs.GS_BUF_REC0, gs.GS_BUF_REC2, gs.GS_BUF_REC3)]
+    keys, vals, ranges, _ = expected_binning(*bufs, cams, n, scene["params"].shape[1])
+    assert np.array_equal(ctx.gs_get_buffer(gs.GS_BUF_KEYS).cpu().numpy().view(np.uint32),
+                          (keys >> np.uint64(32)).astype(np.uint32))
+    assert np.array_equal(ctx.gs_get_buffer(gs.GS_BUF_VALS).cpu().numpy().astype(np.int64), vals)
+    assert np.array_equal(ctx.gs_get_buffer(gs.GS_BUF_RANGES).cpu().numpy().astype(np.int64), ranges)
+    ctx.close()
+
+
+# 16 x 16 tiles cut by the image border, one pixel, an odd tile count; few pixels for the Gaussians (the pairs that
+# take a gradient are flagged) and many
+@pytest.mark.parametrize("n,sizes", [(40, [(16, 16)]), (3000, [(17, 15), (1, 1), (33, 47)]), (20000, [(64, 48), (50, 30)]),
+                                     (500, [(320, 200), (100, 90)])])
+def test_backward_variants_agree(n, sizes):
+    scene = inputs.random_scene(n, 1, 9, extent=0.8)
+    cams = [inputs.pinhole(inputs.look_at((0.4 + v, -2.8, 1.0)), w, h, bg=(0.1, 0.2, 0.3))
+            for v, (w, h) in enumerate(sizes)]
+    _, total = gs.image_offsets(cams)
+    dimg = dev(np.random.default_rng(n).normal(size=total).astype(np.float32))
+    ctx = gs.Context(0)
+    out = {}
+    for fwd, bwd in ((1, 1), (1, 4), (2, 2), (2, 4), (2, 8), (4, 4), (8, 8)):
+        ctx.gs_set_option(gs.GS_OPT_RASTER_FWD, fwd)
+        ctx.gs_set_option(gs.GS_OPT_RASTER_BWD, bwd)
+        stat, count = torch.zeros(n, device="cuda"), torch.zeros(n, device="cuda")
+        ctx.gs_set_densify_stats(stat, count)
+        p, img = run_forward(ctx, scene, cams)
+        grads = torch.full_like(p, float("nan"))
+        for _ in range(2):  # a second backward of the same forward: the same gradients, the statistic again
+            ctx.gs_raster_bwd(p, n, scene["deg"], dimg, grads)
+        ctx.gs_sync()
+        out[fwd, bwd] = [t.cpu().numpy().astype(np.float64) for t in (img, grads, stat, count)]
+        ctx.gs_set_densify_stats(None, None)
+    ref = out[1, 1]
+    for key, got in out.items():
+        assert np.abs(got[0] - ref[0]).max() <= 1e-6, key
+        assert np.isfinite(got[1]).all() and rel_l2(got[1], ref[1]) <= 2e-5, key
+        assert rel_l2(got[2], ref[2]) <= 2e-5 and np.array_equal(got[3], ref[3]), key
     ctx.close()
