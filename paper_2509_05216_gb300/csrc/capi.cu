@@ -63,7 +63,7 @@ struct gs_ctx {
   cudaEvent_t tgt_free[2] = {nullptr, nullptr};
   int64_t host_launches = 0;
   int raster_fwd = 2;  // compositing variants (pixels per thread; 8 = one warp per tile)
-  int raster_bwd = 4;
+  int raster_bwd = 0;  // 0: by the batch's tile count
   int bwd_direct = 2;  // per-lane gradient atomics when at most this many lanes contribute
   int sort_passes = 0;  // LSD passes of the last tile sort
   int sort_items = 16;  // keys per thread of a sort partition
@@ -835,6 +835,8 @@ static gs_status sort_tiles_longest_first(gs_ctx* c) {
   return GS_OK;
 }
 
+static int bwd_variant(const gs_ctx* c) { return c->raster_bwd ? c->raster_bwd : raster_bwd_auto(c->bins); }
+
 static RasterArgs raster_args(gs_ctx* c) {
   RasterArgs r{};
   r.views = P<ViewRec>(c->views);
@@ -935,7 +937,7 @@ gs_status gs_raster_bwd(gs_ctx* c, const gs_params* params, const float* dL_dima
   // views of 2048^2) 0.44 ms saved, 0.15 ms spent; 4M pairs on 8.4M pixels
   // (500,000 Gaussians, 8 views of 1024^2) 16 us saved, 31 us spent; so from
   // three pairs on four pixels.
-  const bool flagged = c->B > 1 && raster_bwd_flags(c->raster_bwd) && 4 * (int64_t)c->B * c->n >= 3 * c->pixels;
+  const bool flagged = c->B > 1 && raster_bwd_flags(bwd_variant(c)) && 4 * (int64_t)c->B * c->n >= 3 * c->pixels;
   if (flagged) {
     const size_t flag_bytes = (size_t)c->B * c->stride;
     GS_TRY(ensure(c, c->pair_flags, flag_bytes));
@@ -945,7 +947,7 @@ gs_status gs_raster_bwd(gs_ctx* c, const gs_params* params, const float* dL_dima
   }
   {
     LaunchScope ls(c, "raster_bwd");
-    launch_raster_bwd(r, c->bins, c->raster_bwd, c->stream);
+    launch_raster_bwd(r, c->bins, bwd_variant(c), c->stream);
   }
   if (flagged) {
     LaunchScope ls(c, "pair_masks");
@@ -1561,7 +1563,7 @@ gs_status gs_get_option(gs_ctx* c, int32_t option, int64_t* value) {
   if (!c || !value) return GS_EINVAL;
   switch (option) {
     case GS_OPT_RASTER_FWD: *value = c->raster_fwd; return GS_OK;
-    case GS_OPT_RASTER_BWD: *value = c->raster_bwd; return GS_OK;
+    case GS_OPT_RASTER_BWD: *value = bwd_variant(c); return GS_OK;
     case GS_OPT_BWD_DIRECT: *value = c->bwd_direct; return GS_OK;
     case GS_OPT_SORT_ITEMS: *value = c->sort_items; return GS_OK;
     case GS_OPT_SORT_WAIT: *value = c->sort_wait; return GS_OK;

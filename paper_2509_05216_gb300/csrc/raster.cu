@@ -1056,34 +1056,45 @@ __global__ void __launch_bounds__(32 * FwdCells<NP>::NW) raster_fwd_cells_kernel
   }
 }
 
-// Backward with 4 pixels per thread: a warp owns the upper or lower 16 x 8
-// pixels of its tile, 16 contribution cells; a pair of lanes owns a cell, each
-// lane one column of 4 pixels (two packed row pairs).  Against 2 pixels per
-// thread, a walked entry's set-up and its reduction (one exchange between the
-// two lanes instead of two levels and a gather over four) serve twice the
-// pixels.
+// Backward by contribution cells, NC columns of a cell per thread: with 1, a
+// warp owns the upper or lower 16 x 8 pixels of its tile and a pair of lanes a
+// cell of 2 x 4 pixels (a lane takes one column, two packed row pairs); with 2,
+// a warp owns the tile and a lane a whole cell.  Against 2 pixels per thread, a
+// walked entry's set-up and its reduction (one exchange between two lanes, or
+// none, instead of two levels and a gather over four) serve more pixels.
 //
-// The warp pays for the pair of lanes with the most entries, so the pairs may
-// run ahead: two batches are staged, a pair that has finished the older one
-// goes on with the newer, and the warp moves on when every pair has finished
-// the older.
-struct Bwd4Smem {
-  // two halves of a neutral record (opacity 0: an idle pair evaluates it
+// Measured (B = 16 views of 2048^2, 4M Gaussians / 8 views of 1024^2, 500,000 /
+// one of 1919 x 1081, 4M / 3 of 517 x 333 and less, 37,001 large ones): 2 pixels
+// per thread 5.61 ms / 1655 us / 617 us / 147 us, 4 pixels 4.40 ms / 1067 us /
+// 417 us / 160 us, 8 pixels 4.15 ms / 1004 us / 391 us / 199 us: the last from
+// the tile count at which one warp per tile fills every SM (raster_bwd_auto).
+//
+// The warp pays for the cell with the most entries, so the cells may run
+// ahead: two batches are staged, a cell that has finished the older one goes
+// on with the newer, and the warp moves on when every cell has finished the
+// older.
+struct BwdCellsSmem {
+  // two halves of a neutral record (opacity 0: an idle cell evaluates it
   // without effect) and 32 records
   float4 s0[2 * 33], s1[2 * 33];
   float2 sx[2 * 33];  // blue, bits of the Gaussian
 };
 
-__global__ void __launch_bounds__(64, 10) raster_bwd4_kernel(RasterArgs a, int64_t bins) {
-  __shared__ Bwd4Smem smem[2];
+template <int NC>
+__global__ void __launch_bounds__(64, NC == 1 ? 10 : 8) raster_bwd_cells_kernel(RasterArgs a, int64_t bins) {
+  constexpr int WPT = NC == 1 ? 2 : 1;  // warps per tile
+  constexpr int NJ = 2 * NC;            // pixel pairs per thread
+  __shared__ BwdCellsSmem smem[2];
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  Bwd4Smem& sm = smem[w];
-  const int64_t bin = a.tile_order ? a.tile_order[blockIdx.x] : (int64_t)blockIdx.x;
+  BwdCellsSmem& sm = smem[w];
+  const int64_t slot0 = NC == 1 ? (int64_t)blockIdx.x : 2 * (int64_t)blockIdx.x + w;
+  if (slot0 >= bins) return;
+  const int64_t bin = a.tile_order ? a.tile_order[slot0] : slot0;
   const int v = view_of_bin(a.views, a.B, (int)bin);
   const ViewRec& V = a.views[v];
   const int tile = (int)bin - V.tile_offset;
-  const int cell = 16 * w + (lane >> 1);
-  const int px = (tile % V.gw) * kTile + 2 * (cell & 7) + (lane & 1);
+  const int cell = WPT == 2 ? 16 * w + (lane >> 1) : lane;
+  const int px = (tile % V.gw) * kTile + 2 * (cell & 7) + (NC == 1 ? (lane & 1) : 0);
   const int py0 = (tile / V.gw) * kTile + 4 * (cell >> 3);
   const uint2 rg = a.ranges[bin];
   const uint32_t* __restrict__ vals = *a.vals;
@@ -1091,30 +1102,30 @@ __global__ void __launch_bounds__(64, 10) raster_bwd4_kernel(RasterArgs a, int64
   const float* dimg = a.dimage + 3 * V.pix_offset;
 
   // per pixel: T (running, from T_final backwards), dL/dC, sum_c dC_c S_c
-  // (S = colour behind), T_final * sum_c dC_c bg_c, and n_last
-  float2 T2[2], dC2[2][3], dCS2[2], bgd2[2];
-  uint32_t nl[4], mymax = 0;
-  {
-    float T[4], dC[4][3], bgd[4];
+  // (S = colour behind), T_final * sum_c dC_c bg_c, and n_last; pair j: column
+  // j / 2, rows 2 (j % 2) and the next
+  float2 T2[NJ], dC2[NJ][3], dCS2[NJ], bgd2[NJ];
+  uint32_t nl[2 * NJ], mymax = 0;
 #pragma unroll
-    for (int k = 0; k < 4; k++) {
-      const bool in = px < V.W && py0 + k < V.H;
-      const int64_t p = (int64_t)(py0 + k) * V.W + px;
+  for (int j = 0; j < NJ; j++) {
+    float T[2], dC[2][3], bgd[2];
+#pragma unroll
+    for (int k = 0; k < 2; k++) {
+      const int x = px + j / 2, y = py0 + 2 * (j % 2) + k;
+      const bool in = x < V.W && y < V.H;
+      const int64_t p = (int64_t)y * V.W + x;
       T[k] = in ? a.tfinal[V.pix_offset + p] : 1.f;
-      nl[k] = in ? a.nlast[V.pix_offset + p] : 0u;
+      nl[2 * j + k] = in ? a.nlast[V.pix_offset + p] : 0u;
 #pragma unroll
       for (int c = 0; c < 3; c++) dC[k][c] = in ? dimg[c * plane + p] : 0.f;
       bgd[k] = T[k] * (dC[k][0] * V.bg[0] + dC[k][1] * V.bg[1] + dC[k][2] * V.bg[2]);
-      mymax = max(mymax, nl[k]);
+      mymax = max(mymax, nl[2 * j + k]);
     }
+    T2[j] = make_float2(T[0], T[1]);
 #pragma unroll
-    for (int j = 0; j < 2; j++) {
-      T2[j] = make_float2(T[2 * j], T[2 * j + 1]);
-#pragma unroll
-      for (int c = 0; c < 3; c++) dC2[j][c] = make_float2(dC[2 * j][c], dC[2 * j + 1][c]);
-      dCS2[j] = bc2(0.f);
-      bgd2[j] = make_float2(bgd[2 * j], bgd[2 * j + 1]);
-    }
+    for (int c = 0; c < 3; c++) dC2[j][c] = make_float2(dC[0][c], dC[1][c]);
+    dCS2[j] = bc2(0.f);
+    bgd2[j] = make_float2(bgd[0], bgd[1]);
   }
   const int total = (int)__reduce_max_sync(0xffffffffu, mymax);
   if (total == 0) return;
@@ -1132,7 +1143,7 @@ __global__ void __launch_bounds__(64, 10) raster_bwd4_kernel(RasterArgs a, int64
 
   int b = ((total - 1) >> 5) << 5;  // next batch to stage
   uint32_t cm_next = cells[b];
-  // the older and the newer staged batch: entries left in the pair's cell,
+  // the older and the newer staged batch: entries left in the lane's cell,
   // list position of the first entry, slot before the first record
   uint32_t mo = 0, mn = 0;
   int so = 0, sn = 0, po = 0, pn = 33;
@@ -1173,43 +1184,60 @@ __global__ void __launch_bounds__(64, 10) raster_bwd4_kernel(RasterArgs a, int64
       const float4 q0 = sm.s0[slot];
       const float4 q1 = sm.s1[slot];
       const float2 qx = sm.sx[slot];
-      const float dx = __fsub_rn(q0.x, fpx);
-      const float dx2 = __fmul_rn(dx, dx);
-      const float a0 = __fmul_rn(q0.z, dx2);
-      const float a1 = __fmul_rn(q0.w, dx);
-      const float2 cC = bc2(q1.x), A1 = bc2(a1), A0 = bc2(a0), op = bc2(q1.y);
+      const float2 cC = bc2(q1.x), op = bc2(q1.y);
       const float2 r = bc2(q1.z), g = bc2(q1.w), bl = bc2(qx.x), qy = bc2(q0.y);
-      float2 racc[3] = {bc2(0.f), bc2(0.f), bc2(0.f)}, oacc = bc2(0.f);
-      float2 S0 = bc2(0.f), S1 = bc2(0.f), S2 = bc2(0.f);
+      float2 racc[3] = {bc2(0.f), bc2(0.f), bc2(0.f)}, oacc = bc2(0.f), S2 = bc2(0.f);
       bool on = false;
+      // moments of dL/dp2: m0 = sum dp, m1 = sum dp dy, and their sums with dx
+      float m1 = 0.f, xm0 = 0.f, g2 = 0.f, g3 = 0.f;
 #pragma unroll
-      for (int jp = 0; jp < 2; jp++) {
-        const float2 ny = make_float2(nfy - (float)(2 * jp), nfy - (float)(2 * jp + 1));
-        on |= bwd_pair2(idx < nl[2 * jp], idx < nl[2 * jp + 1], cC, A1, A0, op, r, g, bl, __fadd2_rn(qy, ny), T2[jp],
-                        dCS2[jp], dC2[jp], bgd2[jp], racc, oacc, S0, S1, S2);
+      for (int c = 0; c < NC; c++) {
+        const float dx = __fsub_rn(q0.x, fpx + (float)c);
+        const float dx2 = __fmul_rn(dx, dx);
+        const float2 A0 = bc2(__fmul_rn(q0.z, dx2)), A1 = bc2(__fmul_rn(q0.w, dx));
+        float2 S0 = bc2(0.f), S1 = bc2(0.f);
+#pragma unroll
+        for (int h = 0; h < 2; h++) {
+          const int jp = 2 * c + h;
+          const float2 ny = make_float2(nfy - (float)(2 * h), nfy - (float)(2 * h + 1));
+          on |= bwd_pair2(idx < nl[2 * jp], idx < nl[2 * jp + 1], cC, A1, A0, op, r, g, bl, __fadd2_rn(qy, ny), T2[jp],
+                          dCS2[jp], dC2[jp], bgd2[jp], racc, oacc, S0, S1, S2);
+        }
+        const float c0 = S0.x + S0.y, c1 = S1.x + S1.y;
+        m1 = c ? m1 + c1 : c1;
+        xm0 = c ? fmaf(dx, c0, xm0) : dx * c0;
+        g2 = c ? fmaf(dx2, c0, g2) : dx2 * c0;
+        g3 = c ? fmaf(dx, c1, g3) : dx * c1;
       }
-      // mean and conic gradients of p2 from the moments of dL/dp2
-      const float m0 = S0.x + S0.y, m1 = S1.x + S1.y;
-      const float g0 = fmaf(q0.w, m1, 2.f * q0.z * dx * m0);  // sum dp (cB dy + 2 cA dx)
-      const float g1 = fmaf(2.f * q1.x, m1, a1 * m0);         // sum dp (2 cC dy + cB dx)
-      const float g2 = dx2 * m0, g3 = dx * m1, g4 = S2.x + S2.y, g5 = oacc.x + oacc.y;
+      // mean and conic gradients of p2 from the moments
+      const float g0 = fmaf(q0.w, m1, 2.f * q0.z * xm0);    // sum dp (cB dy + 2 cA dx)
+      const float g1 = fmaf(2.f * q1.x, m1, q0.w * xm0);    // sum dp (2 cC dy + cB dx)
+      const float g4 = S2.x + S2.y, g5 = oacc.x + oacc.y;
       const float c0 = racc[0].x + racc[0].y, c1 = racc[1].x + racc[1].y, c2 = racc[2].x + racc[2].y;
-      // the pair's sums: the even lane takes the geometry record's first four
-      // values, the odd lane the other five
-      const float x0 = __shfl_xor_sync(0xffffffffu, odd ? g0 : g4, 1);
-      const float x1 = __shfl_xor_sync(0xffffffffu, odd ? g1 : g5, 1);
-      const float x2 = __shfl_xor_sync(0xffffffffu, odd ? g2 : c0, 1);
-      const float x3 = __shfl_xor_sync(0xffffffffu, odd ? g3 : c1, 1);
-      const float x4 = __shfl_xor_sync(0xffffffffu, c2, 1);
-      if (__ballot_sync(0xffffffffu, on) & pair) {
-        const int64_t gi = (int64_t)__float_as_uint(qx.y);
-        const float y0 = x0 + (odd ? g4 : g0), y1 = x1 + (odd ? g5 : g1);
-        const float y2 = x2 + (odd ? c0 : g2), y3 = x3 + (odd ? c1 : g3);
-        if (!odd) {
-          red_v4(geo + kG2dGeo * gi, y0 * grad_scale(0), y1 * grad_scale(1), y2 * grad_scale(2), y3 * grad_scale(3));
-        } else {
-          red_v2(geo + kG2dGeo * gi + 4, y0 * grad_scale(4), y1 * grad_scale(5));
-          red_v4(col + kG2dCol * gi, y2, y3, x4 + c2, 0.f);
+      const int64_t gi = (int64_t)__float_as_uint(qx.y);
+      if constexpr (NC == 2) {
+        if (on) {
+          red_v4(geo + kG2dGeo * gi, g0 * grad_scale(0), g1 * grad_scale(1), g2 * grad_scale(2), g3 * grad_scale(3));
+          red_v2(geo + kG2dGeo * gi + 4, g4 * grad_scale(4), g5 * grad_scale(5));
+          red_v4(col + kG2dCol * gi, c0, c1, c2, 0.f);
+        }
+      } else {
+        // the pair's sums: the even lane takes the geometry record's first
+        // four values, the odd lane the other five
+        const float x0 = __shfl_xor_sync(0xffffffffu, odd ? g0 : g4, 1);
+        const float x1 = __shfl_xor_sync(0xffffffffu, odd ? g1 : g5, 1);
+        const float x2 = __shfl_xor_sync(0xffffffffu, odd ? g2 : c0, 1);
+        const float x3 = __shfl_xor_sync(0xffffffffu, odd ? g3 : c1, 1);
+        const float x4 = __shfl_xor_sync(0xffffffffu, c2, 1);
+        if (__ballot_sync(0xffffffffu, on) & pair) {
+          const float y0 = x0 + (odd ? g4 : g0), y1 = x1 + (odd ? g5 : g1);
+          const float y2 = x2 + (odd ? c0 : g2), y3 = x3 + (odd ? c1 : g3);
+          if (!odd) {
+            red_v4(geo + kG2dGeo * gi, y0 * grad_scale(0), y1 * grad_scale(1), y2 * grad_scale(2), y3 * grad_scale(3));
+          } else {
+            red_v2(geo + kG2dGeo * gi + 4, y0 * grad_scale(4), y1 * grad_scale(5));
+            red_v4(col + kG2dCol * gi, y2, y3, x4 + c2, 0.f);
+          }
         }
       }
     }
@@ -1229,7 +1257,7 @@ void launch_shape(bool fwd, const RasterArgs& a, int64_t bins, cudaStream_t s) {
   using G = Geo<PPT>;
   const unsigned blocks = (unsigned)((bins + G::TPB - 1) / G::TPB);
   if constexpr (PPT != 2 && PPT != 4) if (fwd) raster_fwd_kernel<PPT><<<blocks, G::THREADS, 0, s>>>(a, bins);
-  if constexpr (PPT != 4) if (!fwd) raster_bwd_kernel<PPT><<<blocks, G::THREADS, 0, s>>>(a, bins);
+  if constexpr (PPT != 4 && PPT != 8) if (!fwd) raster_bwd_kernel<PPT><<<blocks, G::THREADS, 0, s>>>(a, bins);
 }
 
 int64_t raster_fwd_warps(int64_t bins, int ppt) {
@@ -1345,14 +1373,24 @@ void launch_raster_fwd(const RasterArgs& a, int64_t bins, int ppt, cudaStream_t 
   }
 }
 
-bool raster_bwd_flags(int ppt) { return ppt == 4; }
+// Pixels per thread of the backward when the caller has chosen none: a warp per
+// tile (8) where those fill every SM's 16 resident warps twice over, two (4)
+// below, and four (2) where only that gives an SM more than 16 warps; with less
+// than 4 tiles per SM the time is that of one tile, shortest with 4 again (256
+// tiles: 51 us against 57 with 2).
+int raster_bwd_auto(int64_t bins) {
+  const int64_t sms = sm_count();
+  return bins >= 32 * sms ? 8 : bins >= 4 * sms && bins < 8 * sms ? 2 : 4;
+}
+
+bool raster_bwd_flags(int ppt) { return ppt == 4 || ppt == 8; }
 
 void launch_raster_bwd(const RasterArgs& a, int64_t bins, int ppt, cudaStream_t s) {
   if (bins == 0) return;
   switch (ppt) {
     case 1: launch_shape<1>(false, a, bins, s); break;
-    case 4: raster_bwd4_kernel<<<(unsigned)bins, 64, 0, s>>>(a, bins); break;
-    case 8: launch_shape<8>(false, a, bins, s); break;
+    case 4: raster_bwd_cells_kernel<1><<<(unsigned)bins, 64, 0, s>>>(a, bins); break;
+    case 8: raster_bwd_cells_kernel<2><<<(unsigned)((bins + 1) / 2), 64, 0, s>>>(a, bins); break;
     default: launch_shape<2>(false, a, bins, s); break;
   }
 }
