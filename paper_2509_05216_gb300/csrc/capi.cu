@@ -1360,9 +1360,9 @@ gs_status gs_init_gaussians(gs_ctx* c, const float* points, const float* normals
   const double cell = emax / (double)(1 << (key_bits / 3));
   k.cell = (float)cell;
   k.inv_cell = (float)(1.0 / cell);
-  // the chosen level has at most n / 2 cells: at most half full
+  // the chosen level has at most n cells: at most 2/3 full
   int tbits = 10;
-  while (((int64_t)1 << tbits) < n) tbits++;
+  while (((int64_t)1 << tbits) < n + n / 2) tbits++;
   k.table_bits = tbits;
   GS_TRY(ensure(c, c->keys0, sizeof(uint32_t) * n));
   GS_TRY(ensure(c, c->keys1, sizeof(uint32_t) * n));
@@ -1370,7 +1370,7 @@ gs_status gs_init_gaussians(gs_ctx* c, const float* points, const float* normals
   GS_TRY(ensure(c, c->vals1, sizeof(uint32_t) * n));
   GS_TRY(ensure(c, c->init_pts, sizeof(float4) * n));
   GS_TRY(ensure(c, c->knn_heads, sizeof(uint32_t) * 16));
-  GS_TRY(ensure(c, c->knn_table, sizeof(uint4) << tbits));
+  GS_TRY(ensure(c, c->knn_table, sizeof(unsigned long long) << tbits));
   GS_TRY(ensure(c, c->init_scales, sizeof(float) * n));
   k.keys[0] = P<uint32_t>(c->keys0);
   k.keys[1] = P<uint32_t>(c->keys1);
@@ -1384,10 +1384,10 @@ gs_status gs_init_gaussians(gs_ctx* c, const float* points, const float* normals
   GS_TRY(sort_pairs(c, n, key_bits, &k.sort_ctrl, &k.sort_passes));
   k.sorted = P<float4>(c->init_pts);
   k.heads = P<uint32_t>(c->knn_heads);
-  k.table = P<uint4>(c->knn_table);
+  k.table = P<unsigned long long>(c->knn_table);
   k.out = P<float>(c->init_scales);
   GS_CUDA(c, cudaMemsetAsync(k.heads, 0, sizeof(uint32_t) * 16, c->stream));
-  GS_CUDA(c, cudaMemsetAsync(k.table, 0xff, sizeof(uint4) << tbits, c->stream));
+  GS_CUDA(c, cudaMemsetAsync(k.table, 0xff, sizeof(unsigned long long) << tbits, c->stream));
   {
     LaunchScope ls(c, "knn_query", 4);
     launch_knn_query(k, c->stream);

@@ -347,23 +347,19 @@ __device__ __forceinline__ uint32_t slot_of(uint32_t key, int bits) {
   return (((key >> 3) * 0x9E3779B1u) >> (35 - bits)) << 3 | (key & 7u);
 }
 
-constexpr uint32_t kEmptySlot = ~0u;
-
-// The run of sorted points of a cell (empty when no point lies in it).
-__device__ __forceinline__ uint2 cell_run(const KnnArgs& a, uint32_t key) {
-  const uint32_t mask = (uint32_t)((1ull << a.table_bits) - 1ull);
-  for (uint32_t s = slot_of(key, a.table_bits), probes = 0; probes <= mask; s = (s + 1) & mask, probes++) {
-    const uint4 e = a.table[s];
-    if (e.x == key) return make_uint2(e.y, e.z);
-    if (e.x == kEmptySlot) break;
-  }
-  return make_uint2(0u, 0u);
+// Table entry of a cell: its code, the first sorted point of its run and the
+// run's length, 7 for longer ones.
+constexpr unsigned long long kEmptySlot = ~0ull;
+__device__ __forceinline__ unsigned long long cell_entry(uint32_t key, int64_t start, int64_t length) {
+  return (unsigned long long)key << 34 | (unsigned long long)start << 3 | (unsigned long long)min(length, (int64_t)7);
 }
 
 // The level whose occupied cells hold kCellPoints points or more on average
 // (the finest such one).  heads[l]: sorted points whose cell at level l, but
 // not at l + 1, differs from their predecessor's; a level has one cell more
-// than the heads at it and above.
+// than the heads at it and above.  (From 1 on the finer level made a surface's
+// look-ups cheaper but left a fifth of a 4M set to the warps of the second
+// kernel: 6.6 ms against 2.0 ms.)
 constexpr int64_t kCellPoints = 2;
 __device__ __forceinline__ int pick_level(const KnnArgs& a) {
   int64_t cells = 1;
@@ -393,6 +389,22 @@ __device__ __forceinline__ int64_t lower_bound(const uint32_t* keys, int64_t lo,
     if ((uint64_t)keys[mid] < key) lo = mid + 1; else hi = mid;
   }
   return lo;
+}
+
+// The run of sorted points of a cell of the given level (empty when no point
+// lies in it).
+__device__ __forceinline__ uint2 cell_run(const KnnArgs& a, const uint32_t* keys, uint32_t cell, int level) {
+  const uint32_t mask = (uint32_t)((1ull << a.table_bits) - 1ull);
+  for (uint32_t s = slot_of(cell, a.table_bits), probes = 0; probes <= mask; s = (s + 1) & mask, probes++) {
+    const unsigned long long e = a.table[s];
+    if (e == kEmptySlot) break;
+    if ((uint32_t)(e >> 34) == cell) {
+      const uint32_t start = (uint32_t)(e >> 3) & 0x7fffffffu, length = (uint32_t)e & 7u;
+      if (length < 7u) return make_uint2(start, start + length);
+      return make_uint2(start, (uint32_t)lower_bound(keys, (int64_t)start + 7, a.n, ((uint64_t)cell + 1) << (3 * level)));
+    }
+  }
+  return make_uint2(0u, 0u);
 }
 
 // Insert the squared distance of sorted point j into the sorted list of the
@@ -463,9 +475,7 @@ __global__ void __launch_bounds__(256) knn_sorted_points_kernel(KnnArgs a) {
   if (threadIdx.x < kMortonBits && s_heads[threadIdx.x]) atomicAdd(a.heads + threadIdx.x, s_heads[threadIdx.x]);
 }
 
-// Insert every cell of the chosen level with its run of sorted points.  The
-// end of a run is found by doubling steps and bisection, so that a cell of
-// many points does not make one thread walk it.
+// Insert every cell of the chosen level with its run of sorted points.
 __global__ void __launch_bounds__(256) knn_table_kernel(KnnArgs a) {
   const int sh = 3 * pick_level(a);
   const uint32_t* keys = sorted_keys(a);
@@ -473,19 +483,11 @@ __global__ void __launch_bounds__(256) knn_table_kernel(KnnArgs a) {
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < a.n; i += (int64_t)gridDim.x * blockDim.x) {
     const uint32_t cell = keys[i] >> sh;
     if (i > 0 && keys[i - 1] >> sh == cell) continue;
-    int64_t step = 1, lo = i + 1;
-    while (i + step < a.n && keys[i + step] >> sh == cell) {
-      lo = i + step + 1;
-      step *= 2;
-    }
-    const int64_t end = lower_bound(keys, lo, min(a.n, i + step), ((uint64_t)cell + 1) << sh);
-    for (uint32_t s = slot_of(cell, a.table_bits), probes = 0; probes <= mask; s = (s + 1) & mask, probes++) {
-      if (atomicCAS(&a.table[s].x, kEmptySlot, cell) == kEmptySlot) {
-        a.table[s].y = (uint32_t)i;
-        a.table[s].z = (uint32_t)end;
-        break;
-      }
-    }
+    int length = 1;
+    while (length < 7 && i + length < a.n && keys[i + length] >> sh == cell) length++;
+    const unsigned long long entry = cell_entry(cell, i, length);
+    for (uint32_t s = slot_of(cell, a.table_bits), probes = 0; probes <= mask; s = (s + 1) & mask, probes++)
+      if (atomicCAS(a.table + s, kEmptySlot, entry) == kEmptySlot) break;
   }
 }
 
@@ -517,55 +519,102 @@ struct CellCube {
   }
 };
 
-// One thread per point, in Morton order: the 3 smallest squared distances to
-// other points, then out[point] = 0.5 log(max(1e-14, mean)).  The points next
-// to it in sorted order bound the third distance; the runs of those of the 3^3
-// cells around it that the bound reaches are listed in shared memory, and one
-// loop goes through all of their points.  (A loop per cell made every warp pay
-// for its fullest cell 27 times.)  A point whose third distance is not inside
-// the cube goes on the list of the next kernel.
+// Distance in cells, along an axis, from a point at f to cell c, less a margin
+// for the rounding of f (1e-4 of a finest cell).
+__device__ __forceinline__ float cell_gap(float f, uint32_t c) {
+  return fmaxf(fmaxf((float)c - f, f - (float)(c + 1u)) - 2e-3f, 0.f);
+}
+
+// A warp takes 32 consecutive points in Morton order: the 3 smallest squared
+// distances of each to other points, then out[point] = 0.5 log(max(1e-14,
+// mean)).  The points next to a point in sorted order bound its third distance.
+// The lanes whose cells are near the first lane's (nearly always all; the rest
+// follow in further rounds, where the Morton order jumps) share a box: its
+// cells, and one more on each side, are looked up 32 at a time, and the points
+// of a cell that some lane's bound reaches are compared by all lanes at once,
+// each read once per warp, so that no lane waits for another's list.  (4M points
+// of a surface, whole initialisation: 8.8 ms with a loop over its own 27 cells
+// per thread and a cell size by the bounding box's volume; 2.85 ms with a list
+// of its cells' runs per thread; 2.03 ms like
+// this.)  A point whose third
+// distance is not inside the cells next to its own goes on the list of the next
+// kernel.
 constexpr int kQueryThreads = 128;
+constexpr int kQuerySpan = 5;  // cells between a lane's and the first lane's, along an axis
 __global__ void __launch_bounds__(kQueryThreads) knn_query_kernel(KnnArgs a) {
-  __shared__ uint2 s_run[27][kQueryThreads];
-  const int64_t i = (int64_t)blockIdx.x * kQueryThreads + threadIdx.x;
-  if (i >= a.n) return;
+  const int lane = threadIdx.x & 31;
+  const int64_t first = (((int64_t)blockIdx.x * kQueryThreads + threadIdx.x) >> 5) * 32;
+  if (first >= a.n) return;
+  const bool mine = first + lane < a.n;
+  const int64_t i = min(first + lane, a.n - 1);
   const int level = pick_level(a);
   const uint32_t* keys = sorted_keys(a);
+  const uint32_t key = keys[i];
   const float4 me = a.sorted[i];
   float best[3] = {3.0e38f, 3.0e38f, 3.0e38f};
   for (int64_t j = max((int64_t)0, i - 4); j < min(a.n, i + 5); j++)
     if (j != i) near_point(a, j, me.x, me.y, me.z, best);
   const float bound = best[2];
-  const CellCube c(a, me, keys[i], level);
-  int runs = 0;
-#pragma unroll
-  for (int q = 0; q < 27; q++) {
-    const int x = q % 3, y = q / 3 % 3, z = q / 9;
-    // (3e38: a cell outside the grid)
-    const float gap2 = c.x.gap2[x] + c.y.gap2[y] + c.z.gap2[z];
-    if (gap2 > bound || gap2 >= 3.0e38f) continue;
-    const uint2 run = cell_run(a, c.x.code[x] | (c.y.code[y] << 1) | (c.z.code[z] << 2));
-    if (run.y > run.x) s_run[runs++][threadIdx.x] = run;
-  }
-  best[0] = best[1] = best[2] = 3.0e38f;  // (the cells hold the neighbours in sorted order too)
-  uint32_t j = 0, end = 0;
-  int r = 0;
-  while (true) {
-    if (j == end) {
-      if (r == runs) break;
-      const uint2 run = s_run[r++][threadIdx.x];
-      j = run.x;
-      end = run.y;
+  best[0] = best[1] = best[2] = 3.0e38f;  // (the cells hold these neighbours too)
+  // the lane's cell and its position in cells; the warp's box
+  const int dim = 1 << (kMortonBits - level);
+  const float scale = a.inv_cell / (float)(1 << level), cell = a.cell * (float)(1 << level);
+  const float fx = (me.x - a.lo[0]) * scale, fy = (me.y - a.lo[1]) * scale, fz = (me.z - a.lo[2]) * scale;
+  const int cx = (int)gather3(key) >> level, cy = (int)gather3(key >> 1) >> level, cz = (int)gather3(key >> 2) >> level;
+  for (uint32_t todo = __ballot_sync(0xffffffffu, mine); todo;) {
+    const int lead = __ffs((int)todo) - 1;
+    // (every lane takes part in the exchanges)
+    const int lx = __shfl_sync(0xffffffffu, cx, lead), ly = __shfl_sync(0xffffffffu, cy, lead);
+    const int lz = __shfl_sync(0xffffffffu, cz, lead);
+    const bool in = ((todo >> lane) & 1u) != 0u && max(abs(cx - lx), max(abs(cy - ly), abs(cz - lz))) <= kQuerySpan;
+    todo &= ~__ballot_sync(0xffffffffu, in);
+    // the box of the lanes taken
+    auto low = [&](int c) { return max(__reduce_min_sync(0xffffffffu, in ? c : 1 << kMortonBits) - 1, 0); };
+    auto high = [&](int c) { return min(__reduce_max_sync(0xffffffffu, in ? c : 0) + 1, dim - 1); };
+    const int x0 = low(cx), y0 = low(cy), z0 = low(cz);
+    const int ex = high(cx) - x0 + 1, exy = ex * (high(cy) - y0 + 1), cells = exy * (high(cz) - z0 + 1);
+    const float cap = in ? 3.0e38f : 0.f, reach = in ? bound : -1.f;  // (the other lanes take nothing)
+    for (int c0 = 0; c0 < cells; c0 += 32) {
+      const int c = c0 + lane;
+      const uint32_t z = (uint32_t)(z0 + c / exy), y = (uint32_t)(y0 + c % exy / ex), x = (uint32_t)(x0 + c % exy % ex);
+      uint2 run = make_uint2(0u, 0u);
+      if (c < cells) run = cell_run(a, keys, spread3(x) | (spread3(y) << 1) | (spread3(z) << 2), level);
+      const uint32_t pos = x | (y << kMortonBits) | (z << (2 * kMortonBits));
+      for (uint32_t m = __ballot_sync(0xffffffffu, run.y > run.x); m; m &= m - 1u) {
+        const int src = __ffs((int)m) - 1;
+        const uint32_t s0 = __shfl_sync(0xffffffffu, run.x, src), s1 = __shfl_sync(0xffffffffu, run.y, src);
+        const uint32_t p = __shfl_sync(0xffffffffu, pos, src);
+        constexpr uint32_t kAxis = (1u << kMortonBits) - 1u;
+        const float gx = cell_gap(fx, p & kAxis), gy = cell_gap(fy, (p >> kMortonBits) & kAxis);
+        const float gz = cell_gap(fz, p >> (2 * kMortonBits));
+        const float gap2 = (gx * gx + gy * gy + gz * gz) * (cell * cell) * 0.999f;
+        if (!__any_sync(0xffffffffu, !(gap2 > fminf(best[2], reach)))) continue;
+#pragma unroll 4
+        for (uint32_t j = s0; j < s1; j++) {
+          const float4 q = __ldg(a.sorted + j);
+          const float dx = q.x - me.x, dy = q.y - me.y, dz = q.z - me.z;
+          float d2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+          // (not the point itself, and nothing at a NaN)
+          d2 = (int64_t)j != i && d2 < cap ? d2 : 3.0e38f;
+          best[2] = fminf(best[2], fmaxf(best[1], d2));
+          best[1] = fminf(best[1], fmaxf(best[0], d2));
+          best[0] = fminf(best[0], d2);
+        }
+      }
     }
-    if ((int64_t)j != i) near_point(a, j, me.x, me.y, me.z, best);
-    j++;
   }
-  if (best[2] <= c.reach2(a, level)) write_scale(a, me, best);
+  // every point within this distance lies in the cells next to the lane's
+  float border = 1.f;
+  border = fminf(border, fminf(fx - (float)cx, 1.f - (fx - (float)cx)));
+  border = fminf(border, fminf(fy - (float)cy, 1.f - (fy - (float)cy)));
+  border = fminf(border, fminf(fz - (float)cz, 1.f - (fz - (float)cz)));
+  const float reach = (1.f + border - 2e-3f) * cell * 0.999f;
+  if (!mine) return;
+  if (best[2] <= reach * reach) write_scale(a, me, best);
   else spare_vals(a)[atomicAdd(a.heads + kTodo, 1u)] = (uint32_t)i;
 }
 
-// The points left over (a few in a thousand on a surface; isolated ones among
-// them need cubes that hold thousands of others): one warp each, over the
+// The points left over (a few in a hundred; isolated ones among them need cubes that hold thousands of others): one warp each, over the
 // cubes of 3^3 cells of coarser and coarser levels until the third distance is
 // inside.  Lanes find the 27 runs by bisection, share the points of the runs,
 // and merge their three best.

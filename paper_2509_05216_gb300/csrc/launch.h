@@ -259,7 +259,7 @@ struct KnnArgs {
   float4* sorted;        // [n] points in sorted order: x, y, z, bits of the point's index
   uint32_t* heads;       // [16], zeroed: sorted points that start a cell, by the coarsest level at which they do;
                          // [12] the points that the first query leaves over
-  uint4* table;          // [2^table_bits] cell, first and one past the last sorted point (cell all ones: empty)
+  unsigned long long* table;  // [2^table_bits] cell, first sorted point and length of its run (all ones: empty)
   int table_bits;
   float* out;            // [n] log-scales
 };
