@@ -8,17 +8,17 @@
 // each pixel's last contributor towards the front, recovering T by division
 // and keeping the colour composited behind.
 //
-// Launch shapes, selected per context (GS_OPT_RASTER_FWD / _BWD): PPT = 1, 2
-// or 4 pixels per thread with 8, 4 or 2 warps per tile (each warp an 8-pixel-
-// wide band), or PPT = 8 with one warp per 16x16 tile.  Every warp walks its
-// tile's list independently (no block barriers).  It stages 32 records at a
-// time, one per lane; each lane tests its record's alpha >= 1/255 ellipse
-// (with a rounding margin) against the warp's pixel rectangle, and the warp
-// walks only the survivors (a ballot mask); with 2 pixels per thread the
-// warp's lanes form groups that each walk the records whose alpha >= 1/255
-// box reaches their own sub-rectangle (see LaneGroups; no ellipse test).
-// This removes only pairs that the per-pixel test would skip, so the result
-// is unchanged.
+// Launch shapes, selected per context (GS_OPT_RASTER_FWD / _BWD) or, for the
+// backward, by the tile count: PPT = 1, 2, 4 or 8 pixels per thread.  Every warp
+// walks its tile's list independently (no block barriers).  It stages 32
+// records at a time, one per lane.  The kernels of 2 and 4 pixels (forward) and
+// 4 and 8 pixels (backward) walk by contribution cells of 2 x 4 pixels: each
+// cell's lanes walk only the records whose alpha >= 1/255 box reaches the cell
+// (forward) or that the forward found to contribute to it (backward).  In the
+// other forwards each lane tests its record's alpha >= 1/255 ellipse (with a
+// rounding margin) against the warp's pixel rectangle, and the warp walks only
+// the survivors (a ballot mask).  This removes only pairs that the per-pixel
+// test would skip, so the result is unchanged.
 #include "gs_internal.cuh"
 #include "launch.h"
 
@@ -108,23 +108,6 @@ __device__ __forceinline__ bool ellipse_hits(const float4& r0, const float4& r1,
                                              float x1, float y0, float y1) {
   if (!box_hits(r0, r2, x0, x1, y0, y1)) return false;
   return ellipse_rect(ellipse_terms(r0, r1), r0, r2, x0, x1, y0, y1);
-}
-
-// Lane-group survivors: the alpha >= 1/255 box against each group's
-// rectangle (bit g: group g).  The box is looser than the ellipse but costs
-// four compares per group; the exact ellipse test against the warp's
-// rectangle on top of it cost the forward more (its per-record terms) than
-// the walk steps it saved.
-template <class Geom>
-__device__ __forceinline__ uint32_t box_group_bits(const float4& r0, const float4& r2, const Geom& geo) {
-  uint32_t bits = 0;
-#pragma unroll
-  for (int g = 0; g < Geom::NG; g++) {
-    float x0, x1, y0, y1;
-    geo.group_rect(g, x0, x1, y0, y1);
-    bits |= box_hits(r0, r2, x0, x1, y0, y1) ? 1u << g : 0u;
-  }
-  return bits;
 }
 
 // p2 at row offset dy = mu_y - y for a lane with column coefficients
@@ -392,10 +375,11 @@ __device__ __forceinline__ bool bwd_pair2(bool livex, bool livey, const float2& 
 
 // ---------------------------------------------------------------- launch shapes
 //
-// PPT = pixels per thread.  A block holds TPB tiles; a warp owns a WR x HR
-// pixel rectangle of its tile (lane l: column l % CW, rows (l / CW) * PPT + k)
-// and walks the tile's list on its own: it stages 32 records at a time into
-// its own shared slots and never waits for the other warps of the block.
+// Of the kernels with one walk per warp (forward 1 and 8 pixels per thread;
+// backward 1 and 2).  A block holds TPB tiles; a warp owns a WR x HR pixel
+// rectangle of its tile (lane l: column l % CW, rows (l / CW) * PPT + k) and
+// walks the tile's list on its own: it stages 32 records at a time into its own
+// shared slots and never waits for the other warps of the block.
 template <int PPT>
 struct Shape;
 template <>
@@ -407,24 +391,16 @@ struct Shape<2> {  // 4 warps per tile, 8 x 8 pixels each
   static constexpr int NW = 4, TPB = 1, CW = 8;
 };
 template <>
-struct Shape<4> {  // 2 warps per tile, 8 x 16 pixels each
-  static constexpr int NW = 2, TPB = 1, CW = 8;
-};
-template <>
 struct Shape<8> {  // 1 warp per tile, 4 tiles per block
   static constexpr int NW = 1, TPB = 4, CW = 16;
 };
 
-// Lane groups: the warp's lanes form NG = 32 / GW groups, each owning a
-// GCW x GRH sub-rectangle of the warp's pixels and walking only the
-// Gaussians whose box reaches it (the warp iterates max over groups; a lane
-// whose group has run out takes no-op steps).  With 2 pixels per thread
-// both kernels use 8 groups of 2 x 4 pixels (one contribution cell each).
+// Lane groups of the backward with 2 pixels per thread: the warp's lanes form
+// NG = 32 / GW groups, each owning a 2 x 4 cell of the warp's pixels and walking
+// only the entries that contributed to it (the warp iterates max over groups; a
+// lane whose group has run out takes no-op steps).
 template <int PPT>
-struct LaneGroups {
-  static constexpr int FWD = PPT == 2 ? 4 : 32;
-  static constexpr int BWD = PPT == 2 ? 4 : 32;
-};
+constexpr int kBwdGroup = PPT == 2 ? 4 : 32;
 
 template <int PPT, int GWv = 32>
 struct Geo {
@@ -437,13 +413,6 @@ struct Geo {
   int64_t bin;
   int v, px, py0, grp;
   float wx0, wx1, wy0, wy1;
-  // rectangle of lane group g
-  __device__ __forceinline__ void group_rect(int g, float& x0, float& x1, float& y0, float& y1) const {
-    x0 = wx0 + (float)((g % NGX) * GCW);
-    x1 = x0 + (float)(GCW - 1);
-    y0 = wy0 + (float)((g / NGX) * GRH);
-    y1 = y0 + (float)(GRH - 1);
-  }
   __device__ bool init(const RasterArgs& a, int64_t bins, int warp, int lane) {
     const int tile_in_block = warp / NW, sub = warp % NW;
     bin = (int64_t)blockIdx.x * TPB + tile_in_block;
@@ -483,7 +452,7 @@ __device__ __forceinline__ int cell_index(int px, int py) {
 }
 template <int PPT>
 __global__ void __launch_bounds__(Geo<PPT>::THREADS) raster_fwd_kernel(RasterArgs a, int64_t bins) {
-  using G = Geo<PPT, LaneGroups<PPT>::FWD>;
+  using G = Geo<PPT>;
   constexpr int NWB = G::NW * G::TPB;  // warps per block
   constexpr int NP = PPT / 2;          // pixel pairs per thread
   __shared__ float4 s0[NWB][32], s1[NWB][32], s2[NWB][32];
@@ -545,42 +514,23 @@ __global__ void __launch_bounds__(Geo<PPT>::THREADS) raster_fwd_kernel(RasterArg
     uint32_t cm[NSL];
 #pragma unroll
     for (int sl = 0; sl < NSL; sl++) cm[sl] = 0u;
-    uint32_t gbits = 0;
     if (i < n) {
       const float4 r0 = p0, r1 = p1, r2 = p2;
       s0[w][lane] = r0;
       s1[w][lane] = r1;
       s2[w][lane] = r2;
-      if constexpr (G::NG > 1) gbits = box_group_bits(r0, r2, geo);
-      else hit = ellipse_hits(r0, r1, r2, geo.wx0, geo.wx1, geo.wy0, geo.wy1);
+      hit = ellipse_hits(r0, r1, r2, geo.wx0, geo.wx1, geo.wy0, geo.wy1);
     }
     {
       const int i1 = i + 32, i2 = i + 64;
       if (i1 < n) stage_one(a, v, g_after, p0, p1, p2);
       g_after = i2 < n ? vals[rg.x + i2] : 0u;
     }
-    // each lane culls its own record; the warp (each lane group) walks the
-    // survivors in order
+    // each lane culls its own record; the warp walks the survivors in order
     uint32_t mask = __ballot_sync(0xffffffffu, hit);
-    int iters = 32;
-    if constexpr (G::NG > 1) {
-#pragma unroll
-      for (int g = 0; g < G::NG; g++) {
-        const uint32_t m = __ballot_sync(0xffffffffu, (gbits >> g) & 1u);
-        mask = g == geo.grp ? m : mask;
-      }
-      // a group whose pixels have all stopped walks nothing more
-      const uint32_t fin = __ballot_sync(0xffffffffu, done == all_done);
-      const uint32_t gm = G::GW == 32 ? 0xffffffffu : ((1u << (G::GW % 32)) - 1u) << (geo.grp * G::GW);
-      if ((fin & gm) == gm) mask = 0u;
-      iters = (int)__reduce_max_sync(0xffffffffu, (uint32_t)__popc(mask));
-    }
     __syncwarp();
-    for (int it = 0; G::NG > 1 ? it < iters : mask != 0u; it++) {
-      const bool act = mask != 0u;
-      // (an idle group evaluates slot 0, which every batch stages: b0 < n)
-      const int j = act ? __ffs(mask) - 1 : 0;
-      mask &= mask - 1u;
+    for (; mask != 0u; mask &= mask - 1u) {
+      const int j = __ffs((int)mask) - 1;
       const float4 q0 = s0[w][j];
       const float4 q2 = s2[w][j];
       const float4 q1 = s1[w][j];
@@ -597,13 +547,10 @@ __global__ void __launch_bounds__(Geo<PPT>::THREADS) raster_fwd_kernel(RasterArg
       } else {
         const float2 cC = bc2(q1.x), A1 = bc2(a1), A0 = bc2(a0), op = bc2(q1.y);
         const float2 r = bc2(q1.z), g = bc2(q1.w), b = bc2(q2.x), qy = bc2(q0.y);
-        // a lane whose group has no survivor left changes nothing
-        uint32_t dn = act ? done : all_done;
 #pragma unroll
         for (int jp = 0; jp < NP; jp++)
           cm[jp / 2 < NSL ? jp / 2 : 0] |= fwd_pair2(cC, A1, A0, op, r, g, b, __fadd2_rn(qy, nfy[jp]), 1u << (2 * jp),
-                                                   idx, dn, T2[jp], C2[jp], last[2 * jp], last[2 * jp + 1]) ? jbit : 0u;
-        done = act ? dn : done;
+                                                   idx, done, T2[jp], C2[jp], last[2 * jp], last[2 * jp + 1]) ? jbit : 0u;
       }
     }
     // the batch's contribution masks: per cell, the OR of its lanes' entry masks
@@ -688,7 +635,7 @@ __global__ void __launch_bounds__(Geo<PPT>::THREADS) raster_fwd_kernel(RasterArg
 
 template <int PPT>
 __global__ void __launch_bounds__(Geo<PPT>::THREADS, PPT == 2 ? 8 : 1) raster_bwd_kernel(RasterArgs a, int64_t bins) {
-  using G = Geo<PPT, LaneGroups<PPT>::BWD>;
+  using G = Geo<PPT, kBwdGroup<PPT>>;
   constexpr int NWB = G::NW * G::TPB;
   constexpr int NP = PPT / 2;  // pixel pairs per thread (0: the scalar one-pixel path)
   constexpr int NS = NP > 0 ? NP : 1;
@@ -887,6 +834,14 @@ __device__ __forceinline__ uint32_t transpose32(uint32_t x, int lane) {
 // lanes each; every cell walks the entries whose alpha >= 1/255 box reaches
 // it (the box test only removes pairs that the per-pixel test would skip; the
 // exact ellipse test on top of it costs more than the walk steps it saves).
+//
+// Bound by issued instructions (1M Gaussians, 4 views of 1024^2: 76 % of the
+// issue slots, 6 % of the DRAM rate).  Measured, NP = 1 / 2: 16 views of 2048^2
+// of 4M Gaussians 4.07 / 3.97 ms, one of 3840 x 2160 0.63 / 0.70 ms (fewer,
+// longer warps leave a tail), 3 small views of 37,001 large ones 97 / 129 us;
+// NP = 1 is the default.  Letting cells run ahead into a second staged batch, as
+// in the backward, costs this shorter step more than it saves (4.07 -> 4.4 ms
+// and more).
 template <int NP>
 struct FwdCells {
   static constexpr int LPC = 4 / NP, NC = 32 / LPC, NCX = NP == 1 ? 4 : 8;  // lanes per cell, cells, cells per row
@@ -1253,20 +1208,24 @@ __global__ void __launch_bounds__(64, NC == 1 ? 10 : 8) raster_bwd_cells_kernel(
 }
 
 template <int PPT>
-void launch_shape(bool fwd, const RasterArgs& a, int64_t bins, cudaStream_t s) {
+static void launch_fwd(const RasterArgs& a, int64_t bins, cudaStream_t s) {
   using G = Geo<PPT>;
-  const unsigned blocks = (unsigned)((bins + G::TPB - 1) / G::TPB);
-  if constexpr (PPT != 2 && PPT != 4) if (fwd) raster_fwd_kernel<PPT><<<blocks, G::THREADS, 0, s>>>(a, bins);
-  if constexpr (PPT != 4 && PPT != 8) if (!fwd) raster_bwd_kernel<PPT><<<blocks, G::THREADS, 0, s>>>(a, bins);
+  raster_fwd_kernel<PPT><<<(unsigned)((bins + G::TPB - 1) / G::TPB), G::THREADS, 0, s>>>(a, bins);
+}
+
+template <int PPT>
+static void launch_bwd(const RasterArgs& a, int64_t bins, cudaStream_t s) {
+  using G = Geo<PPT>;
+  raster_bwd_kernel<PPT><<<(unsigned)((bins + G::TPB - 1) / G::TPB), G::THREADS, 0, s>>>(a, bins);
 }
 
 int64_t raster_fwd_warps(int64_t bins, int ppt) {
   // L1 partial sums of a fused forward: one per warp of each tile
   switch (ppt) {
     case 1: return bins * Geo<1>::NW;
-    case 4: return bins * Geo<4>::NW;
+    case 4: return bins * FwdCells<2>::NW;
     case 8: return bins * Geo<8>::NW;
-    default: return bins * Geo<2>::NW;
+    default: return bins * FwdCells<1>::NW;
   }
 }
 
@@ -1366,9 +1325,9 @@ void launch_pair_stats(const RasterArgs& a, int64_t bins, unsigned long long* ou
 void launch_raster_fwd(const RasterArgs& a, int64_t bins, int ppt, cudaStream_t s) {
   if (bins == 0) return;
   switch (ppt) {
-    case 1: launch_shape<1>(true, a, bins, s); break;
+    case 1: launch_fwd<1>(a, bins, s); break;
     case 4: raster_fwd_cells_kernel<2><<<(unsigned)bins, 64, 0, s>>>(a); break;
-    case 8: launch_shape<8>(true, a, bins, s); break;
+    case 8: launch_fwd<8>(a, bins, s); break;
     default: raster_fwd_cells_kernel<1><<<(unsigned)bins, 128, 0, s>>>(a); break;
   }
 }
@@ -1388,10 +1347,10 @@ bool raster_bwd_flags(int ppt) { return ppt == 4 || ppt == 8; }
 void launch_raster_bwd(const RasterArgs& a, int64_t bins, int ppt, cudaStream_t s) {
   if (bins == 0) return;
   switch (ppt) {
-    case 1: launch_shape<1>(false, a, bins, s); break;
+    case 1: launch_bwd<1>(a, bins, s); break;
     case 4: raster_bwd_cells_kernel<1><<<(unsigned)bins, 64, 0, s>>>(a, bins); break;
     case 8: raster_bwd_cells_kernel<2><<<(unsigned)((bins + 1) / 2), 64, 0, s>>>(a, bins); break;
-    default: launch_shape<2>(false, a, bins, s); break;
+    default: launch_bwd<2>(a, bins, s); break;
   }
 }
 
