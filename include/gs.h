@@ -138,9 +138,9 @@ typedef enum {
   GS_OPT_RASTER_FWD = 0, /* forward compositing kernel: 1, 2 or 4 = pixels per
                             thread with one block per tile, 8 = one warp per
                             tile.  All variants give the same result up to
-                            FP32 rounding. */
-  GS_OPT_RASTER_BWD = 1, /* backward compositing kernel, same values (unless
-                            set: 8 for batches of many tiles, 4 otherwise) */
+                            FP32 rounding.  Unless set, by the batch's tile
+                            count, as the next one and GS_OPT_TILE_ORDER. */
+  GS_OPT_RASTER_BWD = 1, /* backward compositing kernel, same values */
   GS_OPT_BWD_DIRECT = 2, /* backward with 1 or 2 pixels per thread: a warp whose
                             pixels meet a Gaussian in at most this many lanes
                             (0..32, default 2) adds the lanes' gradients with
@@ -159,10 +159,10 @@ typedef enum {
                             path; the blocks return, nothing hangs).  Fixed
                             once a training graph is captured (GS_ESTATE). */
   GS_OPT_TILE_ORDER = 5  /* order in which the compositing kernels take the
-                            batch's tiles: 0 (default) bin order; 1 longest
-                            lists first (tiles bucketed by floor(log2(list
-                            length + 1)), bin order within a bucket; one extra
-                            sort pass over the bins per batch).  Same result
+                            batch's tiles: 0 bin order; 1 longest lists first
+                            (tiles bucketed by floor(log2(list length + 1)),
+                            bin order within a bucket); unless set, 1 for
+                            batches of many tiles.  Same result
                             (the fused L1 loss sums its per-tile partials in
                             bin order either way).  Fixed once a training graph
                             is captured (GS_ESTATE). */

@@ -995,44 +995,116 @@ __global__ void __launch_bounds__(256) tile_ranges_kernel(SortArgs a, uint2* __r
 
 // ---------------------------------------------------------------- tile order
 
-// Keys of the longest-list-first order: tiles bucketed by floor(log2(length
-// + 1)), longest bucket first (a stable sort keeps bin order inside a bucket,
-// so the order is deterministic); block 0 also writes the sort's count and
-// segment bounds.
-__global__ void __launch_bounds__(256) tile_order_keys_kernel(const uint2* __restrict__ ranges, int64_t bins,
-                                                              uint64_t* __restrict__ keys, uint32_t* __restrict__ vals,
-                                                              uint64_t* count, uint32_t* seg) {
-  const int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (b == 0) {
-    *count = (uint64_t)bins;
-    seg[0] = 0u;
-    seg[1] = (uint32_t)bins;
+// Longest-list-first order: tiles bucketed by floor(log2(length + 1)), longest
+// bucket first, bin order inside a bucket (deterministic).  A counting sort in
+// two launches: bucket counts per block of 1,024 tiles, then every block finds
+// its buckets' offsets from all counts and places its tiles.
+constexpr int kOrderTiles = 1024, kOrderWarps = 8, kOrderRounds = kOrderTiles / (32 * kOrderWarps);
+constexpr int kOrderBuckets = 32;
+
+__device__ __forceinline__ int order_bucket(const uint2* ranges, int64_t bins, int64_t t) {
+  if (t >= bins) return -1;
+  const uint2 r = ranges[t];
+  return __clz((int)((r.y > r.x ? r.y - r.x : 0u) + 1u)) & (kOrderBuckets - 1);
+}
+
+__global__ void __launch_bounds__(32 * kOrderWarps) tile_order_count_kernel(const uint2* __restrict__ ranges,
+                                                                            int64_t bins,
+                                                                            uint32_t* __restrict__ counts) {
+  __shared__ uint32_t s_count[kOrderBuckets];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  if (threadIdx.x < kOrderBuckets) s_count[threadIdx.x] = 0;
+  __syncthreads();
+  const int64_t t0 = (int64_t)blockIdx.x * kOrderTiles + wid * (32 * kOrderRounds) + lane;
+#pragma unroll
+  for (int r = 0; r < kOrderRounds; r++) {
+    const int k = order_bucket(ranges, bins, t0 + 32 * r);
+    const uint32_t peers = __match_any_sync(0xffffffffu, k);
+    if (k >= 0 && (peers & ((1u << lane) - 1u)) == 0) atomicAdd(&s_count[k], (uint32_t)__popc(peers));
   }
-  if (b >= bins) return;
-  const uint2 r = ranges[b];
-  const uint32_t len = r.y > r.x ? r.y - r.x : 0u;
-  keys[b] = (uint64_t)(31 - (31 - __clz(len + 1u)));
-  vals[b] = (uint32_t)b;
+  __syncthreads();
+  if (threadIdx.x < kOrderBuckets) counts[(int64_t)blockIdx.x * kOrderBuckets + threadIdx.x] = s_count[threadIdx.x];
 }
 
-__global__ void __launch_bounds__(256) tile_order_finish_kernel(const uint32_t* __restrict__ ctrl, int npass,
-                                                                const uint32_t* __restrict__ v0,
-                                                                const uint32_t* __restrict__ v1, int64_t bins,
-                                                                uint32_t* __restrict__ order) {
-  const uint32_t* src = (ctrl[npass] & kCtrlParity) ? v1 : v0;
-  for (int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; b < bins; b += (int64_t)gridDim.x * blockDim.x)
-    order[b] = src[b];
+__global__ void __launch_bounds__(32 * kOrderWarps) tile_order_place_kernel(const uint2* __restrict__ ranges,
+                                                                            int64_t bins,
+                                                                            const uint32_t* __restrict__ counts,
+                                                                            uint32_t* __restrict__ order) {
+  __shared__ uint32_t s_next[kOrderWarps][kOrderBuckets];  // a warp's next position in each bucket
+  __shared__ uint32_t s_total[kOrderBuckets], s_before[kOrderBuckets];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  (&s_next[0][0])[threadIdx.x] = 0;
+  __syncthreads();
+  const int64_t t0 = (int64_t)blockIdx.x * kOrderTiles + wid * (32 * kOrderRounds) + lane;
+  int bucket[kOrderRounds];
+  uint32_t peers[kOrderRounds];
+#pragma unroll
+  for (int r = 0; r < kOrderRounds; r++) {
+    bucket[r] = order_bucket(ranges, bins, t0 + 32 * r);
+    peers[r] = __match_any_sync(0xffffffffu, bucket[r]);
+    if (bucket[r] >= 0 && (peers[r] & ((1u << lane) - 1u)) == 0) s_next[wid][bucket[r]] += (uint32_t)__popc(peers[r]);
+    __syncwarp();
+  }
+  // per bucket: tiles of all blocks and of the earlier ones (8 lanes each)
+  {
+    const int k = threadIdx.x >> 3;
+    uint32_t total = 0, before = 0;
+    for (int64_t i = threadIdx.x & 7; i < (int64_t)gridDim.x; i += 8) {
+      const uint32_t c = counts[i * kOrderBuckets + k];
+      total += c;
+      before += i < (int64_t)blockIdx.x ? c : 0u;
+    }
+#pragma unroll
+    for (int off = 4; off > 0; off >>= 1) {
+      total += __shfl_xor_sync(0xffffffffu, total, off);
+      before += __shfl_xor_sync(0xffffffffu, before, off);
+    }
+    if ((threadIdx.x & 7) == 0) {
+      s_total[k] = total;
+      s_before[k] = before;
+    }
+  }
+  __syncthreads();
+  if (wid == 0) {
+    // the bucket's first position, then the block's, then each warp's
+    const uint32_t x = s_total[lane];
+    uint32_t inc = x;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, inc, off);
+      if (lane >= off) inc += y;
+    }
+    uint32_t at = inc - x + s_before[lane];
+    for (int w = 0; w < kOrderWarps; w++) {
+      const uint32_t c = s_next[w][lane];
+      s_next[w][lane] = at;
+      at += c;
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int r = 0; r < kOrderRounds; r++) {
+    const int k = bucket[r];
+    const uint32_t lower = peers[r] & ((1u << lane) - 1u);
+    uint32_t at = 0;
+    if (k >= 0) at = s_next[wid][k];
+    __syncwarp();
+    if (k >= 0) {
+      order[at + __popc(lower)] = (uint32_t)(t0 + 32 * r);
+      if (lower == 0) s_next[wid][k] = at + (uint32_t)__popc(peers[r]);
+    }
+    __syncwarp();
+  }
 }
 
-void launch_tile_order_keys(const uint2* ranges, int64_t bins, uint64_t* keys, uint32_t* vals, uint64_t* count,
-                            uint32_t* seg, cudaStream_t s) {
-  tile_order_keys_kernel<<<(unsigned)((bins + 255) / 256), 256, 0, s>>>(ranges, bins, keys, vals, count, seg);
+size_t tile_order_count_bytes(int64_t bins) {
+  return sizeof(uint32_t) * kOrderBuckets * (size_t)((bins + kOrderTiles - 1) / kOrderTiles);
 }
 
-void launch_tile_order_finish(const uint32_t* ctrl, int npass, const uint32_t* v0, const uint32_t* v1, int64_t bins,
-                              uint32_t* order, cudaStream_t s) {
-  const int64_t blocks = std::min<int64_t>((bins + 255) / 256, (int64_t)sm_count() * 8);
-  tile_order_finish_kernel<<<(unsigned)std::max<int64_t>(blocks, 1), 256, 0, s>>>(ctrl, npass, v0, v1, bins, order);
+void launch_tile_order(const uint2* ranges, int64_t bins, uint32_t* counts, uint32_t* order, cudaStream_t s) {
+  const unsigned blocks = (unsigned)((bins + kOrderTiles - 1) / kOrderTiles);
+  tile_order_count_kernel<<<blocks, 32 * kOrderWarps, 0, s>>>(ranges, bins, counts);
+  tile_order_place_kernel<<<blocks, 32 * kOrderWarps, 0, s>>>(ranges, bins, counts, order);
 }
 
 void launch_tile_ranges(const SortArgs& a, int64_t grid_hint, uint2* ranges, cudaStream_t s) {

@@ -62,13 +62,13 @@ struct gs_ctx {
   cudaEvent_t tgt_copied[2] = {nullptr, nullptr};
   cudaEvent_t tgt_free[2] = {nullptr, nullptr};
   int64_t host_launches = 0;
-  int raster_fwd = 2;  // compositing variants (pixels per thread; 8 = one warp per tile)
+  int raster_fwd = 0;  // compositing variants (pixels per thread; 8 = one warp per tile);
   int raster_bwd = 0;  // 0: by the batch's tile count
   int bwd_direct = 2;  // per-lane gradient atomics when at most this many lanes contribute
   int sort_passes = 0;  // LSD passes of the last tile sort
   int sort_items = 16;  // keys per thread of a sort partition
   int sort_wait = 1 << 20;  // look-back rounds before a sort gives up
-  int tile_order_mode = 0;  // 0: composite tiles in bin order; 1: longest lists first
+  int tile_order_mode = -1;  // 0: composite tiles in bin order; 1: longest lists first; -1: by the tile count
   float* dens_grad = nullptr;   // densification statistic accumulated by gs_raster_bwd (caller-owned)
   float* dens_count = nullptr;
   bool tile_order_ready = false;
@@ -86,8 +86,7 @@ struct gs_ctx {
   DevBuf views, rec, rec3, tiles, block_sums, block_offsets, total, keys0, keys1, vals0, vals1,
       zeroed, hist_scan, tfinal, nlast, g2d, l1_partial, sorted_slots, adam_consts,
       target_slot, host_tgt0, host_tgt1, pair_stats, cells, vismask, ssim_table, ssim_partials, ssim_sums,
-      init_pts, init_scales, knn_part, knn_table, knn_heads, ord_keys0, ord_keys1, ord_vals0, ord_vals1, ord_total, ord_hist,
-      ord_hist_scan, ord_lookback, ord_counters, ord_views, tile_order, vis_sums, vis_offsets, dtotal, dkeys0,
+      init_pts, init_scales, knn_part, knn_table, knn_heads, ord_counts, tile_order, vis_sums, vis_offsets, dtotal, dkeys0,
       dkeys1, dvals0, dvals1, dhist_scan, dorder, torder, iso_work, densify_source, pair_flags, contrib;
 
   // launch accounting and optional per-kernel event timing
@@ -394,6 +393,8 @@ gs_status ctx_reserve(gs_ctx* c, int64_t stride, int B, int64_t bins, int64_t pi
   GS_TRY(ensure_exact(c, c->torder, sizeof(uint32_t) * tparts));
   GS_TRY(ensure_exact(c, c->dorder, sizeof(uint32_t) * dparts));
   GS_TRY(ensure_exact(c, c->sorted_slots, 2 * sizeof(void*)));
+  GS_TRY(ensure_exact(c, c->ord_counts, tile_order_count_bytes(bins)));
+  GS_TRY(ensure_exact(c, c->tile_order, sizeof(uint32_t) * bins));
   GS_TRY(ensure_exact(c, c->tfinal, sizeof(float) * pixels));
   GS_TRY(ensure_exact(c, c->nlast, sizeof(uint32_t) * pixels));
   return GS_OK;
@@ -461,9 +462,7 @@ void gs_destroy(gs_ctx* c) {
                     &c->total, &c->keys0, &c->keys1, &c->vals0, &c->vals1, &c->zeroed, &c->hist_scan, &c->tfinal, &c->nlast, &c->g2d, &c->l1_partial,
                     &c->sorted_slots, &c->adam_consts, &c->target_slot, &c->host_tgt0, &c->host_tgt1,
                     &c->pair_stats, &c->cells, &c->vismask, &c->ssim_table, &c->ssim_partials, &c->ssim_sums,
-                    &c->init_pts, &c->init_scales, &c->knn_part, &c->knn_table, &c->knn_heads, &c->ord_keys0, &c->ord_keys1,
-                    &c->ord_vals0, &c->ord_vals1, &c->ord_total, &c->ord_hist, &c->ord_hist_scan, &c->ord_lookback,
-                    &c->ord_counters, &c->ord_views, &c->tile_order, &c->vis_sums, &c->vis_offsets, &c->dtotal,
+                    &c->init_pts, &c->init_scales, &c->knn_part, &c->knn_table, &c->knn_heads, &c->ord_counts, &c->tile_order, &c->vis_sums, &c->vis_offsets, &c->dtotal,
                     &c->dkeys0, &c->dkeys1, &c->dvals0, &c->dvals1, &c->dhist_scan, &c->dorder, &c->torder, &c->iso_work, &c->densify_source, &c->pair_flags, &c->contrib};
   for (DevBuf* b : bufs)
     if (b->p) cudaFree(b->p);
@@ -572,6 +571,7 @@ gs_status gs_project(gs_ctx* c, const gs_params* params, const gs_camera* cams, 
 }
 
 static gs_status sort_tiles_longest_first(gs_ctx* c);
+static int order_mode(const gs_ctx* c);
 
 gs_status gs_bin_sort(gs_ctx* c) {
   if (!c) return GS_EINVAL;
@@ -767,74 +767,34 @@ gs_status gs_bin_sort(gs_ctx* c) {
   }
   GS_CHECK_LAUNCH(c);
   c->tile_order_ready = false;
-  if (c->tile_order_mode == 1) GS_TRY(sort_tiles_longest_first(c));
+  if (order_mode(c) == 1) GS_TRY(sort_tiles_longest_first(c));
   c->sorted = true;
   return GS_OK;
 }
 
-// Longest-list-first order of the batch's tiles (bins bucketed by
-// floor(log2(length + 1)), a one-pass stable sort, bin order inside a
-// bucket) into c->tile_order; every step on the device, so a captured step
-// replays it.
+// Longest-list-first order of the batch's tiles into c->tile_order; every step
+// on the device, so a captured step replays it.
 static gs_status sort_tiles_longest_first(gs_ctx* c) {
-  const int64_t bins = c->bins;
-  const int items = 16;
-  const size_t lb = sort_lookback_bytes(bins, items, 1);
-  GS_TRY(ensure(c, c->ord_keys0, sizeof(uint64_t) * bins));
-  GS_TRY(ensure(c, c->ord_keys1, sizeof(uint64_t) * bins));
-  GS_TRY(ensure(c, c->ord_vals0, sizeof(uint32_t) * bins));
-  GS_TRY(ensure(c, c->ord_vals1, sizeof(uint32_t) * bins));
-  GS_TRY(ensure(c, c->ord_total, sizeof(uint64_t) + sizeof(uint32_t) * (2 + 2 + 16 + 8)));
-  GS_TRY(ensure(c, c->ord_hist, sizeof(uint32_t) * 256));
-  GS_TRY(ensure(c, c->ord_hist_scan, sizeof(uint32_t) * 256));
-  GS_TRY(ensure(c, c->ord_lookback, lb));
-  GS_TRY(ensure(c, c->ord_counters, sizeof(uint32_t) * 8));
-  GS_TRY(ensure(c, c->ord_views, sizeof(ViewRec)));
-  GS_TRY(ensure(c, c->tile_order, sizeof(uint32_t) * bins));
-  uint64_t* count = P<uint64_t>(c->ord_total);
-  uint32_t* seg = reinterpret_cast<uint32_t*>(count + 1);
-  uint32_t* part_off = seg + 2;
-  uint32_t* ctrl = part_off + 2;
-  SortArgs sa{};
-  sa.keys[0] = c->ord_keys0.p;
-  sa.keys[1] = c->ord_keys1.p;
-  sa.key_bytes = 8;
-  sa.view_shift = 32;
-  sa.vals[0] = P<uint32_t>(c->ord_vals0);
-  sa.vals[1] = P<uint32_t>(c->ord_vals1);
-  sa.count = count;
-  sa.capacity = bins;
-  sa.bins = bins;
-  sa.B = 1;
-  sa.views = P<ViewRec>(c->ord_views);
-  sa.seg = seg;
-  sa.part_off = part_off;
-  sa.hist = P<uint32_t>(c->ord_hist);
-  sa.hist_scan = P<uint32_t>(c->ord_hist_scan);
-  sa.ctrl = ctrl;
-  sa.single = ctrl + 16;
-  sa.lookback = P<uint32_t>(c->ord_lookback);
-  sa.lookback_stride = lb / sizeof(uint32_t);
-  sa.counters = P<uint32_t>(c->ord_counters);
-  sa.npass = 1;
-  sa.wait_rounds = c->sort_wait;
-  sa.status = c->status_d;
-  GS_CUDA(c, cudaMemsetAsync(c->ord_views.p, 0, sizeof(ViewRec), c->stream));
-  GS_CUDA(c, cudaMemsetAsync(c->ord_hist.p, 0, sizeof(uint32_t) * 256, c->stream));
-  GS_CUDA(c, cudaMemsetAsync(c->ord_counters.p, 0, sizeof(uint32_t) * 8, c->stream));
-  GS_CUDA(c, cudaMemsetAsync(c->ord_lookback.p, 0, lb, c->stream));
+  GS_TRY(ensure(c, c->ord_counts, tile_order_count_bytes(c->bins)));
+  GS_TRY(ensure(c, c->tile_order, sizeof(uint32_t) * c->bins));
   {
-    LaunchScope ls(c, "tile_order", 5);
-    launch_tile_order_keys(c->ranges, bins, P<uint64_t>(c->ord_keys0), sa.vals[0], count, seg, c->stream);
-    launch_digit_histogram(sa, bins, items, scan_ticket(c), c->stream);
-    launch_onesweep_pass(sa, 0, items, c->stream);
-    launch_tile_order_finish(ctrl, 1, sa.vals[0], sa.vals[1], bins, P<uint32_t>(c->tile_order), c->stream);
+    LaunchScope ls(c, "tile_order", 2);
+    launch_tile_order(c->ranges, c->bins, P<uint32_t>(c->ord_counts), P<uint32_t>(c->tile_order), c->stream);
   }
   GS_CHECK_LAUNCH(c);
   c->tile_order_ready = true;
   return GS_OK;
 }
 
+// (The render server's batches of a few mixed views are too uneven for the
+// longer warps of 4 pixels per thread: a burst of 12 requests 3.64 against 3.38
+// ms with 2.)
+static int fwd_variant(const gs_ctx* c) {
+  return c->raster_fwd ? c->raster_fwd : c->forward_only ? 2 : raster_fwd_auto(c->bins);
+}
+static int order_mode(const gs_ctx* c) {
+  return c->tile_order_mode >= 0 ? c->tile_order_mode : (tile_order_auto(c->bins) ? 1 : 0);
+}
 static int bwd_variant(const gs_ctx* c) { return c->raster_bwd ? c->raster_bwd : raster_bwd_auto(c->bins); }
 
 static RasterArgs raster_args(gs_ctx* c) {
@@ -866,7 +826,7 @@ gs_status gs_raster_fwd(gs_ctx* c, float* images) {
   r.image = images;
   {
     LaunchScope ls(c, "raster_fwd");
-    launch_raster_fwd(r, c->bins, c->raster_fwd, c->stream);
+    launch_raster_fwd(r, c->bins, fwd_variant(c), c->stream);
   }
   GS_CHECK_LAUNCH(c);
   c->rastered = true;
@@ -881,7 +841,7 @@ gs_status gs_raster_fwd_l1(gs_ctx* c, float* images, const float* targets, float
   set_device(c);
   GS_TRY(ensure(c, c->tfinal, sizeof(float) * c->pixels));
   GS_TRY(ensure(c, c->nlast, sizeof(uint32_t) * c->pixels));
-  const int64_t nparts = raster_fwd_warps(c->bins, c->raster_fwd);
+  const int64_t nparts = raster_fwd_warps(c->bins, fwd_variant(c));
   // per-warp partial sums, then the 256 block sums of the finishing reduction
   const size_t part_bytes = (sizeof(float) * std::max<int64_t>(nparts, 1) + 255) / 256 * 256;
   GS_TRY(ensure(c, c->l1_partial, part_bytes + l1_finish_scratch_bytes()));
@@ -896,7 +856,7 @@ gs_status gs_raster_fwd_l1(gs_ctx* c, float* images, const float* targets, float
   r.inv_count = (float)(1.0 / (double)count);
   {
     LaunchScope ls(c, "raster_fwd");
-    launch_raster_fwd(r, c->bins, c->raster_fwd, c->stream);
+    launch_raster_fwd(r, c->bins, fwd_variant(c), c->stream);
   }
   {
     LaunchScope ls(c, "l1_loss", 2);
@@ -1562,12 +1522,12 @@ gs_status gs_set_option(gs_ctx* c, int32_t option, int64_t value) {
 gs_status gs_get_option(gs_ctx* c, int32_t option, int64_t* value) {
   if (!c || !value) return GS_EINVAL;
   switch (option) {
-    case GS_OPT_RASTER_FWD: *value = c->raster_fwd; return GS_OK;
+    case GS_OPT_RASTER_FWD: *value = fwd_variant(c); return GS_OK;
     case GS_OPT_RASTER_BWD: *value = bwd_variant(c); return GS_OK;
     case GS_OPT_BWD_DIRECT: *value = c->bwd_direct; return GS_OK;
     case GS_OPT_SORT_ITEMS: *value = c->sort_items; return GS_OK;
     case GS_OPT_SORT_WAIT: *value = c->sort_wait; return GS_OK;
-    case GS_OPT_TILE_ORDER: *value = c->tile_order_mode; return GS_OK;
+    case GS_OPT_TILE_ORDER: *value = order_mode(c); return GS_OK;
     default: return fail(c, GS_EINVAL, "unknown option %d", option);
   }
 }

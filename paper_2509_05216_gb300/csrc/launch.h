@@ -166,13 +166,9 @@ struct SortArgs {
   const uint32_t** sorted_vals;
 };
 
-// Longest-list-first tile order: key = 31 - floor(log2(list length + 1)),
-// value = bin, for a one-segment stable sort of the bins; the count and the
-// segment bounds of that sort; the sorted values copied into `order`.
-void launch_tile_order_keys(const uint2* ranges, int64_t bins, uint64_t* keys, uint32_t* vals, uint64_t* count,
-                            uint32_t* seg, cudaStream_t s);
-void launch_tile_order_finish(const uint32_t* ctrl, int npass, const uint32_t* v0, const uint32_t* v1, int64_t bins,
-                              uint32_t* order, cudaStream_t s);
+// Longest-list-first tile order (2 kernels; counts: tile_order_count_bytes).
+size_t tile_order_count_bytes(int64_t bins);
+void launch_tile_order(const uint2* ranges, int64_t bins, uint32_t* counts, uint32_t* order, cudaStream_t s);
 
 size_t sort_lookback_bytes(int64_t count, int items, int segments);
 int64_t sort_partitions(int64_t count, int items, int segments);
@@ -197,6 +193,8 @@ void launch_l1_finish(const float* partial, int64_t nparts, double* scratch, dou
 void launch_raster_bwd(const RasterArgs& a, int64_t bins, int ppt, cudaStream_t s);
 bool raster_bwd_flags(int ppt);
 int raster_bwd_auto(int64_t bins);
+int raster_fwd_auto(int64_t bins);
+bool tile_order_auto(int64_t bins);
 // out[0] += list entries up to each pixel's last contributor, out[1] += contributing pairs
 void launch_pair_stats(const RasterArgs& a, int64_t bins, unsigned long long* out, cudaStream_t s);
 

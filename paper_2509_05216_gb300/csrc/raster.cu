@@ -838,8 +838,8 @@ __device__ __forceinline__ uint32_t transpose32(uint32_t x, int lane) {
 // Bound by issued instructions (1M Gaussians, 4 views of 1024^2: 76 % of the
 // issue slots, 6 % of the DRAM rate).  Measured, NP = 1 / 2: 16 views of 2048^2
 // of 4M Gaussians 4.07 / 3.97 ms, one of 3840 x 2160 0.63 / 0.70 ms (fewer,
-// longer warps leave a tail), 3 small views of 37,001 large ones 97 / 129 us;
-// NP = 1 is the default.  Letting cells run ahead into a second staged batch, as
+// longer warps leave a tail), 3 small views of 37,001 large ones 97 / 129 us.
+// Letting cells run ahead into a second staged batch, as
 // in the backward, costs this shorter step more than it saves (4.07 -> 4.4 ms
 // and more).
 template <int NP>
@@ -1021,8 +1021,8 @@ __global__ void __launch_bounds__(32 * FwdCells<NP>::NW) raster_fwd_cells_kernel
 // Measured (B = 16 views of 2048^2, 4M Gaussians / 8 views of 1024^2, 500,000 /
 // one of 1919 x 1081, 4M / 3 of 517 x 333 and less, 37,001 large ones): 2 pixels
 // per thread 5.61 ms / 1655 us / 617 us / 147 us, 4 pixels 4.40 ms / 1067 us /
-// 417 us / 160 us, 8 pixels 4.15 ms / 1004 us / 391 us / 199 us: the last from
-// the tile count at which one warp per tile fills every SM (raster_bwd_auto).
+// 417 us / 160 us, 8 pixels 4.15 ms / 1004 us / 391 us / 199 us (in bin order;
+// raster_bwd_auto chooses).
 //
 // The warp pays for the cell with the most entries, so the cells may run
 // ahead: two batches are staged, a cell that has finished the older one goes
@@ -1332,14 +1332,23 @@ void launch_raster_fwd(const RasterArgs& a, int64_t bins, int ppt, cudaStream_t 
   }
 }
 
-// Pixels per thread of the backward when the caller has chosen none: a warp per
-// tile (8) where those fill every SM's 16 resident warps twice over, two (4)
-// below, and four (2) where only that gives an SM more than 16 warps; with less
-// than 4 tiles per SM the time is that of one tile, shortest with 4 again (256
-// tiles: 51 us against 57 with 2).
+// The variants when the caller has chosen none.  From the tile count at which
+// one warp per tile fills every SM's 16 resident warps twice over, tiles are
+// taken longest lists first, 4 pixels per thread forward and 8 backward: few
+// long-lived warps per tile leave a tail that the order removes (16 views of
+// 2048^2 of 4M Gaussians: forward 4.07 ms with 2 pixels, 3.98 with 4, 3.75 with
+// 4 in order; backward 4.40 with 4 pixels, 4.14 with 8, 3.73 with 8 in order;
+// the order costs 10 to 18 us; one view of 1919 x 1081: 352 / 337 / 311 us and
+// 417 / 386 / 353 us).  Below, bin order, 2 pixels forward, and backward 4
+// pixels -- or 2 where only that gives an SM more than 16 warps (1,049 tiles of
+// large splats: 147 us against 160); with less than 4 tiles per SM the time is
+// that of one tile, shortest with 4 again (256 tiles: 51 us against 57).
+static bool many_tiles(int64_t bins) { return bins >= (int64_t)32 * sm_count(); }
+bool tile_order_auto(int64_t bins) { return many_tiles(bins); }
+int raster_fwd_auto(int64_t bins) { return many_tiles(bins) ? 4 : 2; }
 int raster_bwd_auto(int64_t bins) {
   const int64_t sms = sm_count();
-  return bins >= 32 * sms ? 8 : bins >= 4 * sms && bins < 8 * sms ? 2 : 4;
+  return many_tiles(bins) ? 8 : bins >= 4 * sms && bins < 8 * sms ? 2 : 4;
 }
 
 bool raster_bwd_flags(int ppt) { return ppt == 4 || ppt == 8; }

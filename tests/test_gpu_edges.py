@@ -196,3 +196,29 @@ def test_backward_variants_agree(n, sizes):
         assert np.isfinite(got[1]).all() and rel_l2(got[1], ref[1]) <= 2e-5, key
         assert rel_l2(got[2], ref[2]) <= 2e-5 and np.array_equal(got[3], ref[3]), key
     ctx.close()
+
+
+# enough tiles for the order of longest lists and the kernels of many tiles: several blocks of 1,024 tiles, ragged
+def test_many_tiles_in_order():
+    sizes = [(1111, 703), (640, 480), (1500, 900)]
+    scene = inputs.random_scene(30000, 1, 21, extent=0.9, log_scale=(-6.0, -3.0))
+    cams = [inputs.pinhole(inputs.look_at((0.4 + v, -2.8, 1.0)), w, h) for v, (w, h) in enumerate(sizes)]
+    _, total = gs.image_offsets(cams)
+    dimg = dev(np.random.default_rng(5).normal(size=total).astype(np.float32))
+    tiles = sum(((w + 15) // 16) * ((h + 15) // 16) for w, h in sizes)
+    out = []
+    for plain in (True, False):
+        ctx = gs.Context(0)
+        if plain:
+            for opt, val in ((gs.GS_OPT_RASTER_FWD, 1), (gs.GS_OPT_RASTER_BWD, 1), (gs.GS_OPT_TILE_ORDER, 0)):
+                ctx.gs_set_option(opt, val)
+        p, img = run_forward(ctx, scene, cams)
+        grads = torch.full_like(p, float("nan"))
+        ctx.gs_raster_bwd(p, scene["n"], scene["deg"], dimg, grads)
+        ctx.gs_sync()
+        if not plain and tiles >= 32 * torch.cuda.get_device_properties(0).multi_processor_count:
+            assert ctx.gs_get_option(gs.GS_OPT_TILE_ORDER) == 1 and ctx.gs_get_option(gs.GS_OPT_RASTER_BWD) == 8
+        out.append([t.cpu().numpy().astype(np.float64) for t in (img, grads)])
+        ctx.close()
+    assert np.abs(out[0][0] - out[1][0]).max() <= 1e-6
+    assert np.isfinite(out[1][1]).all() and rel_l2(out[1][1], out[0][1]) <= 2e-5
