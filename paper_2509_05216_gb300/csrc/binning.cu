@@ -253,8 +253,8 @@ __global__ void partition_order_kernel(const uint32_t* __restrict__ part_off, in
 }
 
 // The key base of segment v: its keys' digits are taken from key - base.
-__device__ __forceinline__ uint64_t segment_key_base(const SortArgs& a, int v) {
-  return a.views ? (uint64_t)(uint32_t)a.views[v].tile_offset << a.view_shift : 0ull;
+__device__ __forceinline__ uint32_t segment_key_base(const SortArgs& a, int v) {
+  return a.views ? (uint32_t)a.views[v].tile_offset : 0u;
 }
 
 // Digit counts of every pass of every view in one read of the keys.  hist:
@@ -264,7 +264,6 @@ __device__ __forceinline__ uint64_t segment_key_base(const SortArgs& a, int v) {
 // of instances in emission order, the exponent byte of depths), so their
 // counts are first aggregated over the lanes holding the same digit; the
 // others are added lane by lane.
-template <typename KeyT>
 __global__ void __launch_bounds__(256) digit_histogram_kernel(SortArgs a) {
   __shared__ uint32_t sh[8][kRadix];
   for (int i = threadIdx.x; i < 8 * kRadix; i += blockDim.x) (&sh[0][0])[i] = 0;
@@ -272,16 +271,16 @@ __global__ void __launch_bounds__(256) digit_histogram_kernel(SortArgs a) {
   const int v = blockIdx.y;
   const int64_t count = min((int64_t)*a.count, a.capacity);
   const int64_t lo = min((int64_t)a.seg[v], count), hi = min((int64_t)a.seg[v + 1], count);
-  const KeyT kb = (KeyT)segment_key_base(a, v);
-  const KeyT* __restrict__ keys = static_cast<const KeyT*>(a.keys[0]);
+  const uint32_t kb = segment_key_base(a, v);
+  const uint32_t* __restrict__ keys = a.keys[0];
   const int npass = a.npass, lane = threadIdx.x & 31;
   for (int64_t i0 = lo + (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); i0 < hi;
        i0 += (int64_t)gridDim.x * blockDim.x) {
     const int64_t i = i0 + lane;
     const bool ok = i < hi;
-    const KeyT k = ok ? (KeyT)(keys[i] - kb) : (KeyT)0;
+    const uint32_t k = ok ? keys[i] - kb : 0u;
     for (int p = 0; p < npass; p++) {
-      const uint32_t dg = (uint32_t)(k >> (kRadixBits * p)) & (kRadix - 1);
+      const uint32_t dg = (k >> (kRadixBits * p)) & (kRadix - 1);
       if (p < npass - 2) {
         if (ok) atomicAdd(&sh[p][dg], 1u);
       } else {
@@ -308,12 +307,10 @@ constexpr uint32_t kCtrlParity = 1u, kCtrlTrivial = 2u;
 // one segment; rank its keys by digit of key - segment base (stable), find
 // its offset for each digit by decoupled look-back over the earlier
 // partitions of its segment (bounded waits), then scatter through shared
-// memory so that the global writes are coalesced.  Only the 32-bit word of
-// a key that holds the pass's digit is loaded up front (all loads in flight
-// before ranking; for 64-bit keys, half the registers of whole keys, which
-// spilled); keys and then values go through one shared buffer, and the
+// memory so that the global writes are coalesced.  All key loads are in flight
+// before ranking; keys and then values go through one shared buffer, and the
 // scatter takes each staged key's digit from the key.
-template <typename KeyT, int ITEMS>
+template <int ITEMS>
 struct SortSmem {
   static constexpr int kTile = kSortThreads * ITEMS;
   // per-warp digit counts -> position of the warp's first key of the digit
@@ -324,9 +321,9 @@ struct SortSmem {
   uint32_t global_base[kRadix];
   uint32_t wtot[kSortWarps];
   uint32_t part, seg, seg_lo, seg_hi, first_part;
-  uint64_t key_base;
+  uint32_t key_base;
   int timed_out;
-  KeyT buf[kTile];                         // keys, then values, in tile-sorted order
+  uint32_t buf[kTile];                         // keys, then values, in tile-sorted order
 };
 
 // Lanes that hold the same digit, among the lanes with a key.
@@ -348,21 +345,21 @@ __device__ __forceinline__ unsigned digit_peers(uint32_t d, bool ok) {
   return peers;
 }
 
-template <typename KeyT, int ITEMS, int MIN_BLOCKS, bool FEW>
+template <int ITEMS, int MIN_BLOCKS, bool FEW>
 __global__ void __launch_bounds__(kSortThreads, MIN_BLOCKS) onesweep_pass_kernel(SortArgs a, int pass) {
   constexpr int kSortItems = ITEMS;
   constexpr int kSortTile = kSortThreads * ITEMS;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  SortSmem<KeyT, ITEMS>& sm = *reinterpret_cast<SortSmem<KeyT, ITEMS>*>(smem_raw);
+  SortSmem<ITEMS>& sm = *reinterpret_cast<SortSmem<ITEMS>*>(smem_raw);
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const uint32_t ctrl = a.ctrl[pass];
   if (ctrl & kCtrlTrivial) return;  // whole block: every view has one digit here
   const int par = (int)(ctrl & kCtrlParity);
   // selects, not a dynamically indexed parameter array (which would be
   // copied to local memory)
-  const KeyT* __restrict__ kin = static_cast<const KeyT*>(par ? a.keys[1] : a.keys[0]);
+  const uint32_t* __restrict__ kin = par ? a.keys[1] : a.keys[0];
   const uint32_t* __restrict__ vin = par ? a.vals[1] : a.vals[0];
-  KeyT* __restrict__ kout = static_cast<KeyT*>(par ? a.keys[0] : a.keys[1]);
+  uint32_t* __restrict__ kout = par ? a.keys[0] : a.keys[1];
   uint32_t* __restrict__ vout = par ? a.vals[0] : a.vals[1];
   const int shift = kRadixBits * pass;
   const uint32_t nparts = a.part_off[a.B];
@@ -389,23 +386,16 @@ __global__ void __launch_bounds__(kSortThreads, MIN_BLOCKS) onesweep_pass_kernel
   const uint32_t lp0 = part - sm.first_part;  // partition index inside the segment
   const int64_t base = (int64_t)sm.seg_lo + (int64_t)lp0 * kSortTile;
   const int n_here = (int)min((int64_t)kSortTile, (int64_t)sm.seg_hi - base);
-  const KeyT kb = (KeyT)sm.key_base;
+  const uint32_t kb = sm.key_base;
   const uint32_t* __restrict__ hist_pass = a.hist_scan + ((int64_t)v * a.npass + pass) * kRadix;
   uint32_t* lookback = a.lookback + (size_t)pass * a.lookback_stride;
   const int wl = wid * kSortItems * 32 + lane;  // item i at base + wl + 32 i
 
-  // the 32-bit word of the key that holds the pass's digit (8-bit digits
-  // never straddle the halves of a 64-bit key)
-  constexpr int kWords = (int)(sizeof(KeyT) / 4);
-  const int hw = kWords == 2 && shift >= 32 ? 1 : 0;
-  const int wsh = shift & 31;
-  const uint32_t wsub = (uint32_t)((uint64_t)kb >> (32 * hw));
-  const uint32_t* __restrict__ kin32 = reinterpret_cast<const uint32_t*>(kin) + hw;
   uint32_t word[kSortItems];
 #pragma unroll
   for (int i = 0; i < kSortItems; i++) {
     const int p = wl + 32 * i;
-    word[i] = p < n_here ? kin32[kWords * (base + p)] - wsub : 0u;
+    word[i] = p < n_here ? kin[base + p] - kb : 0u;
   }
   // stable rank inside the warp (warp-striped order), 16-bit per item
   uint32_t rk[kSortItems / 2];
@@ -413,7 +403,7 @@ __global__ void __launch_bounds__(kSortThreads, MIN_BLOCKS) onesweep_pass_kernel
 #pragma unroll
   for (int i = 0; i < kSortItems; i++) {
     const bool ok = wl + 32 * i < n_here;
-    const uint32_t d = ok ? (word[i] >> wsh) & (kRadix - 1) : (uint32_t)kRadix;
+    const uint32_t d = ok ? (word[i] >> shift) & (kRadix - 1) : (uint32_t)kRadix;
     const unsigned peers = digit_peers<FEW>(d, ok);
     uint32_t r = 0, before = 0;
     if (ok) {
@@ -466,9 +456,9 @@ __global__ void __launch_bounds__(kSortThreads, MIN_BLOCKS) onesweep_pass_kernel
     const uint32_t r = (rk[i >> 1] >> ((i & 1) * 16)) & 0xffffu;
     uint32_t lpos = 0xffffu;
     if (ok) {
-      const uint32_t dd = (word[i] >> wsh) & (kRadix - 1);
+      const uint32_t dd = (word[i] >> shift) & (kRadix - 1);
       lpos = sm.warp_hist[wid][dd] + r;
-      sm.buf[lpos] = kWords == 1 ? (KeyT)(word[i] + wsub) : kin[base + wl + 32 * i];
+      sm.buf[lpos] = word[i] + kb;
     }
     if (i & 1) rk[i >> 1] = (rk[i >> 1] & 0xffffu) | (lpos << 16); else rk[i >> 1] = (rk[i >> 1] & 0xffff0000u) | lpos;
   }
@@ -531,15 +521,15 @@ __global__ void __launch_bounds__(kSortThreads, MIN_BLOCKS) onesweep_pass_kernel
     const int q = tid + t * kSortThreads;
     dst[t] = 0xffffffffu;
     if (q < n_here) {
-      const KeyT k = sm.buf[q];
-      const uint32_t dd = (uint32_t)((KeyT)(k - kb) >> shift) & (kRadix - 1);
+      const uint32_t k = sm.buf[q];
+      const uint32_t dd = ((k - kb) >> shift) & (kRadix - 1);
       dst[t] = sm.global_base[dd] + (uint32_t)q;
       if (dst[t] < hi) kout[dst[t]] = k;
     }
   }
   __syncthreads();
   // values through the same buffer
-  uint32_t* vb = reinterpret_cast<uint32_t*>(sm.buf);
+  uint32_t* vb = sm.buf;
 #pragma unroll
   for (int i = 0; i < kSortItems; i++) {
     const int p = wl + 32 * i;
@@ -554,44 +544,38 @@ __global__ void __launch_bounds__(kSortThreads, MIN_BLOCKS) onesweep_pass_kernel
   }
 }
 
-template <typename KeyT, int ITEMS, int MIN_BLOCKS, bool FEW>
+template <int ITEMS, int MIN_BLOCKS, bool FEW>
 static void launch_pass_few(const SortArgs& a, int pass, int64_t grid, cudaStream_t s) {
-  const size_t smem = sizeof(SortSmem<KeyT, ITEMS>);
+  const size_t smem = sizeof(SortSmem<ITEMS>);
   // once per device (the attribute is per device; not repeated inside a graph capture)
   static bool attr_set[64] = {};
   int dev = 0;
   cudaGetDevice(&dev);
   if (dev < 0 || dev >= 64 || !attr_set[dev]) {
-    cudaFuncSetAttribute(onesweep_pass_kernel<KeyT, ITEMS, MIN_BLOCKS, FEW>,
+    cudaFuncSetAttribute(onesweep_pass_kernel<ITEMS, MIN_BLOCKS, FEW>,
                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (dev >= 0 && dev < 64) attr_set[dev] = true;
   }
-  onesweep_pass_kernel<KeyT, ITEMS, MIN_BLOCKS, FEW><<<(unsigned)grid, kSortThreads, smem, s>>>(a, pass);
+  onesweep_pass_kernel<ITEMS, MIN_BLOCKS, FEW><<<(unsigned)grid, kSortThreads, smem, s>>>(a, pass);
 }
 
-template <typename KeyT, int ITEMS, int MIN_BLOCKS>
+template <int ITEMS, int MIN_BLOCKS>
 static void launch_pass(const SortArgs& a, int pass, int64_t grid, cudaStream_t s) {
-  if (pass > 0 && pass == a.npass - 1) launch_pass_few<KeyT, ITEMS, MIN_BLOCKS, true>(a, pass, grid, s);
-  else launch_pass_few<KeyT, ITEMS, MIN_BLOCKS, false>(a, pass, grid, s);
-}
-
-template <typename KeyT>
-static void launch_pass_items(const SortArgs& a, int pass, int items, int64_t grid, cudaStream_t s) {
-  switch (items) {
-    case 4: launch_pass<KeyT, 4, 4>(a, pass, grid, s); break;
-    case 8: launch_pass<KeyT, 8, 4>(a, pass, grid, s); break;
-    case 12: launch_pass<KeyT, 12, 4>(a, pass, grid, s); break;
-    case 20: launch_pass<KeyT, 20, 3>(a, pass, grid, s); break;
-    case 24: launch_pass<KeyT, 24, 2>(a, pass, grid, s); break;
-    default: launch_pass<KeyT, 16, 4>(a, pass, grid, s); break;
-  }
+  if (pass > 0 && pass == a.npass - 1) launch_pass_few<ITEMS, MIN_BLOCKS, true>(a, pass, grid, s);
+  else launch_pass_few<ITEMS, MIN_BLOCKS, false>(a, pass, grid, s);
 }
 
 void launch_onesweep_pass(const SortArgs& a, int pass, int items, cudaStream_t s) {
   const int64_t grid = sort_partitions(a.capacity, items, a.B);
   if (grid <= 0) return;
-  if (a.key_bytes == 4) launch_pass_items<uint32_t>(a, pass, items, grid, s);
-  else launch_pass_items<uint64_t>(a, pass, items, grid, s);
+  switch (items) {
+    case 4: launch_pass<4, 4>(a, pass, grid, s); break;
+    case 8: launch_pass<8, 4>(a, pass, grid, s); break;
+    case 12: launch_pass<12, 4>(a, pass, grid, s); break;
+    case 20: launch_pass<20, 3>(a, pass, grid, s); break;
+    case 24: launch_pass<24, 2>(a, pass, grid, s); break;
+    default: launch_pass<16, 4>(a, pass, grid, s); break;
+  }
 }
 
 // Exclusive scan of each (view, pass)'s 256 digit counts (block v of the
@@ -678,8 +662,7 @@ void launch_digit_histogram(const SortArgs& a, int64_t grid_hint, int items, uin
   int64_t want = (grid_hint + 511) / 512;
   want = want < 1 ? 1 : (want > (int64_t)sms * 8 ? (int64_t)sms * 8 : want);
   const unsigned per_view = (unsigned)std::max<int64_t>(1, want / a.B);
-  if (a.key_bytes == 4) digit_histogram_kernel<uint32_t><<<dim3(per_view, a.B), 256, 0, s>>>(a);
-  else digit_histogram_kernel<uint64_t><<<dim3(per_view, a.B), 256, 0, s>>>(a);
+  digit_histogram_kernel<<<dim3(per_view, a.B), 256, 0, s>>>(a);
   launch_digit_scan(a, items, ticket, s);
 }
 
@@ -956,7 +939,7 @@ size_t emit_lookback_reserve(int64_t pair_capacity, int segments) {
 __global__ void __launch_bounds__(256) tile_ranges_kernel(SortArgs a, uint2* __restrict__ ranges) {
   const int64_t count = min((int64_t)*a.count, a.capacity);
   const int par = (int)(a.ctrl[a.npass] & kCtrlParity);
-  const uint32_t* __restrict__ keys = static_cast<const uint32_t*>(par ? a.keys[1] : a.keys[0]);
+  const uint32_t* __restrict__ keys = par ? a.keys[1] : a.keys[0];
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     *a.sorted_keys = keys;
     *a.sorted_vals = par ? a.vals[1] : a.vals[0];

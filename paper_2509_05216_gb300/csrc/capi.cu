@@ -659,12 +659,10 @@ gs_status gs_bin_sort(gs_ctx* c) {
 
   // 2. stable sort of each view's pairs by depth
   SortArgs ds{};
-  ds.keys[0] = c->dkeys0.p;
-  ds.keys[1] = c->dkeys1.p;
+  ds.keys[0] = P<uint32_t>(c->dkeys0);
+  ds.keys[1] = P<uint32_t>(c->dkeys1);
   ds.vals[0] = P<uint32_t>(c->dvals0);
   ds.vals[1] = P<uint32_t>(c->dvals1);
-  ds.key_bytes = 4;
-  ds.view_shift = 0;
   ds.views = nullptr;
   ds.count = dw.total;
   ds.capacity = pc;
@@ -724,12 +722,10 @@ gs_status gs_bin_sort(gs_ctx* c) {
 
   // 4. stable sort of each view's instances by tile
   SortArgs sa{};
-  sa.keys[0] = c->keys0.p;
-  sa.keys[1] = c->keys1.p;
+  sa.keys[0] = P<uint32_t>(c->keys0);
+  sa.keys[1] = P<uint32_t>(c->keys1);
   sa.vals[0] = P<uint32_t>(c->vals0);
   sa.vals[1] = P<uint32_t>(c->vals1);
-  sa.key_bytes = 4;
-  sa.view_shift = 0;
   sa.views = P<ViewRec>(c->views);
   sa.count = iw.total;
   sa.capacity = cap;
@@ -1153,10 +1149,8 @@ static gs_status sort_pairs(gs_ctx* c, int64_t n, int bits, const uint32_t** ctr
   GS_CUDA(c, cudaMemcpyAsync(total, &cnt, sizeof(cnt), cudaMemcpyHostToDevice, c->stream));
   GS_CUDA(c, cudaMemcpyAsync(seg, segs, sizeof(segs), cudaMemcpyHostToDevice, c->stream));
   SortArgs sa{};
-  sa.keys[0] = c->keys0.p;
-  sa.keys[1] = c->keys1.p;
-  sa.key_bytes = 4;
-  sa.view_shift = 0;
+  sa.keys[0] = P<uint32_t>(c->keys0);
+  sa.keys[1] = P<uint32_t>(c->keys1);
   sa.vals[0] = P<uint32_t>(c->vals0);
   sa.vals[1] = P<uint32_t>(c->vals1);
   sa.count = total;

@@ -139,15 +139,13 @@ size_t emit_lookback_reserve(int64_t pair_capacity, int segments);
 // sorted) is decided on the device, so the sequence can be captured in a
 // CUDA graph.
 struct SortArgs {
-  void* keys[2];             // uint32 or uint64 keys (key_bytes)
+  uint32_t* keys[2];
   uint32_t* vals[2];
-  int key_bytes;             // 4 or 8
-  int view_shift;            // a segment's key base: views[v].tile_offset << view_shift
   const uint64_t* count;     // device: number of pairs (clamped to capacity)
   int64_t capacity;          // pairs the buffers hold
   int64_t bins;              // valid bin ids are [0, bins)
   int B;                     // views: one segment each
-  const ViewRec* views;      // NULL: key base 0 for every segment
+  const ViewRec* views;      // a segment's key base is its view's first tile (NULL: 0)
   const uint32_t* seg;       // [B + 1] segment offsets
   uint32_t* part_off;        // [B + 1] first partition of each segment
   uint32_t* part_order;      // [partitions] status slot of the partition each ticket takes
