@@ -1018,25 +1018,36 @@ __global__ void __launch_bounds__(32 * FwdCells<NP>::NW) raster_fwd_cells_kernel
 // walked entry's set-up and its reduction (one exchange between two lanes, or
 // none, instead of two levels and a gather over four) serve more pixels.
 //
-// Measured (B = 16 views of 2048^2, 4M Gaussians / 8 views of 1024^2, 500,000 /
-// one of 1919 x 1081, 4M / 3 of 517 x 333 and less, 37,001 large ones): 2 pixels
-// per thread 5.61 ms / 1655 us / 617 us / 147 us, 4 pixels 4.40 ms / 1067 us /
-// 417 us / 160 us, 8 pixels 4.15 ms / 1004 us / 391 us / 199 us (in bin order;
-// raster_bwd_auto chooses).
+// Bound by issued instructions and, at 14 to 20 warps per SM, their latencies.
+// Measured in order of list length (16 views of 2048^2, 4M Gaussians / 8 views of
+// 1024^2, 500,000 / one of 1919 x 1081, 4M): 4 pixels 3.62 ms / 970 us / 359 us,
+// 8 pixels 3.27 ms / 851 us / 326 us; 2 pixels with a walk per lane group, in bin
+// order: 5.61 ms / 1655 us / 617 us.
 //
 // The warp pays for the cell with the most entries, so the cells may run
 // ahead: two batches are staged, a cell that has finished the older one goes
 // on with the newer, and the warp moves on when every cell has finished the
-// older.
+// older.  The records of the batch after those two are copied asynchronously
+// meanwhile (8 pixels per thread, staged before the walk instead: 38 % of the
+// issue slots, 3.7 stalls per instruction on those loads, and 3.73 ms / 903 us /
+// 353 us for the above; asking for 8 resident blocks instead of 7 spills 34 bytes
+// instead of 8: 3.45 ms).
 struct BwdCellsSmem {
-  // two halves of a neutral record (opacity 0: an idle cell evaluates it
-  // without effect) and 32 records
-  float4 s0[2 * 33], s1[2 * 33];
-  float2 sx[2 * 33];  // blue, bits of the Gaussian
+  // three parts of a neutral record (opacity 0: an idle cell evaluates it
+  // without effect) and 32 records: the older and the newer batch, and the one
+  // whose records are on their way
+  float4 s0[3 * 33], s1[3 * 33];
+  float2 sx[3 * 33];  // blue, bits of the Gaussian
 };
 
+template <int BYTES>
+__device__ __forceinline__ void copy_async(void* dst, const void* src) {
+  const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(d), "l"(src), "n"(BYTES) : "memory");
+}
+
 template <int NC>
-__global__ void __launch_bounds__(64, NC == 1 ? 10 : 8) raster_bwd_cells_kernel(RasterArgs a, int64_t bins) {
+__global__ void __launch_bounds__(64, NC == 1 ? 10 : 7) raster_bwd_cells_kernel(RasterArgs a, int64_t bins) {
   constexpr int WPT = NC == 1 ? 2 : 1;  // warps per tile
   constexpr int NJ = 2 * NC;            // pixel pairs per thread
   __shared__ BwdCellsSmem smem[2];
@@ -1084,7 +1095,7 @@ __global__ void __launch_bounds__(64, NC == 1 ? 10 : 8) raster_bwd_cells_kernel(
   }
   const int total = (int)__reduce_max_sync(0xffffffffu, mymax);
   if (total == 0) return;
-  if (lane < 2) {
+  if (lane < 3) {
     sm.s0[33 * lane] = sm.s1[33 * lane] = make_float4(0.f, 0.f, 0.f, 0.f);
     sm.sx[33 * lane] = make_float2(0.f, 0.f);
   }
@@ -1096,36 +1107,62 @@ __global__ void __launch_bounds__(64, NC == 1 ? 10 : 8) raster_bwd_cells_kernel(
   const bool odd = lane & 1;
   const uint32_t pair = 3u << (lane & 30);
 
-  int b = ((total - 1) >> 5) << 5;  // next batch to stage
+  // next batch to fetch; its masks and indices are loaded a step ahead
+  int b = ((total - 1) >> 5) << 5;
   uint32_t cm_next = cells[b];
-  // the older and the newer staged batch: entries left in the lane's cell,
-  // list position of the first entry, slot before the first record
-  uint32_t mo = 0, mn = 0;
-  int so = 0, sn = 0, po = 0, pn = 33;
+  uint32_t g_next = b + lane < total ? vals[rg.x + b + lane] : 0u;
+  // the older, the newer and the coming batch: entries left in the lane's
+  // cell, list position of the first entry, slot before the first record
+  uint32_t mo = 0, mn = 0, mp = 0;
+  int so = 0, sn = 0, sp = 0, po = 0, pn = 33, pp = 66;
+  bool any_n = false, any_p = false;
   while (true) {
-    // the next batch in which an entry contributed to a pixel of the warp
-    uint32_t any = 0;
-    mn = 0;
+    // the coming batch becomes the newer, the newer the older; the older's
+    // part takes the records of the next batch in which an entry contributed
+    // to a pixel of the warp, asynchronously, while the other two are walked
+    const int free_part = po;
+    mo = mn;
+    so = sn;
+    po = pn;
+    mn = mp;
+    sn = sp;
+    pn = pp;
+    pp = free_part;
+    const bool any_o = any_n;
+    any_n = any_p;
+    uint32_t any = 0, g = 0;
+    mp = 0;
     for (; b >= 0 && any == 0u; b -= 32) {
       const int nb = total - b;
-      mn = nb >= 32 ? cm_next : cm_next & ((1u << nb) - 1u);
-      if (b >= 32) cm_next = cells[b - 32];
-      any = __reduce_or_sync(0xffffffffu, mn);
-      sn = b;
-    }
-    if (any) {
-      if ((any >> lane) & 1u) {
-        const uint32_t g = vals[rg.x + sn + lane];
-        float4 n0, n1, n2;
-        stage_one(a, v, g, n0, n1, n2);
-        sm.s0[pn + 1 + lane] = n0;
-        sm.s1[pn + 1 + lane] = n1;
-        sm.sx[pn + 1 + lane] = make_float2(n2.x, __uint_as_float(g));
-        // (an index at or above n only comes after a capacity overflow)
-        if (flags && (int64_t)g < a.n) flags[g] = 1;
+      mp = nb >= 32 ? cm_next : cm_next & ((1u << nb) - 1u);
+      g = g_next;
+      if (b >= 32) {
+        cm_next = cells[b - 32];
+        g_next = vals[rg.x + b - 32 + lane];
       }
-      __syncwarp();
+      any = __reduce_or_sync(0xffffffffu, mp);
+      sp = b;
     }
+    any_p = any != 0u;
+    if ((any >> lane) & 1u) {
+      const int slot = pp + 1 + lane;
+      if ((int64_t)g < a.n) {
+        const int64_t o = kRecStride * ((int64_t)v * a.stride + g);
+        copy_async<16>(&sm.s0[slot], a.rec0 + o);
+        copy_async<16>(&sm.s1[slot], a.rec1 + o);
+        copy_async<4>(&sm.sx[slot].x, a.rec2 + o);
+        sm.sx[slot].y = __uint_as_float(g);
+        if (flags) flags[g] = 1;
+      } else {  // only after a capacity overflow: a record without effect
+        sm.s0[slot] = sm.s1[slot] = make_float4(0.f, 0.f, 0.f, 0.f);
+        sm.sx[slot] = make_float2(0.f, 0.f);
+      }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    if (!(any_o || any_n || any_p)) break;
+    // all but the coming batch's records have arrived, and every lane sees them
+    asm volatile("cp.async.wait_group 1;" ::: "memory");
+    __syncwarp();
     const int iters = (int)__reduce_max_sync(0xffffffffu, (uint32_t)__popc(mo));
     for (int it = 0; it < iters; it++) {  // back to front
       const bool older = mo != 0u;
@@ -1196,15 +1233,9 @@ __global__ void __launch_bounds__(64, NC == 1 ? 10 : 8) raster_bwd_cells_kernel(
         }
       }
     }
-    if (!any) break;
-    // the newer batch becomes the older; its half is kept, the other is free
-    mo = mn;
-    so = sn;
-    const int t = po;
-    po = pn;
-    pn = t;
-    __syncwarp();
+    __syncwarp();  // (the older batch's part is overwritten next)
   }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
 }
 
 template <int PPT>
@@ -1333,23 +1364,18 @@ void launch_raster_fwd(const RasterArgs& a, int64_t bins, int ppt, cudaStream_t 
 }
 
 // The variants when the caller has chosen none.  From the tile count at which
-// one warp per tile fills every SM's 16 resident warps twice over, tiles are
-// taken longest lists first, 4 pixels per thread forward and 8 backward: few
+// one warp per tile fills every SM's 14 to 16 resident warps twice over, tiles
+// are taken longest lists first, 4 pixels per thread forward and 8 backward: few
 // long-lived warps per tile leave a tail that the order removes (16 views of
 // 2048^2 of 4M Gaussians: forward 4.07 ms with 2 pixels, 3.98 with 4, 3.75 with
-// 4 in order; backward 4.40 with 4 pixels, 4.14 with 8, 3.73 with 8 in order;
-// the order costs 10 to 18 us; one view of 1919 x 1081: 352 / 337 / 311 us and
-// 417 / 386 / 353 us).  Below, bin order, 2 pixels forward, and backward 4
-// pixels -- or 2 where only that gives an SM more than 16 warps (1,049 tiles of
-// large splats: 147 us against 160); with less than 4 tiles per SM the time is
-// that of one tile, shortest with 4 again (256 tiles: 51 us against 57).
+// 4 in order; backward 3.62 with 4 pixels in order, 3.27 with 8; the order costs
+// 10 to 18 us; one view of 1919 x 1081: 352 / 337 / 311 us and 359 / 326 us).
+// Below, bin order, 2 pixels forward and 4 backward (256 tiles: 47 us against 58
+// with 8; 1,049 tiles of large splats: 137 to 150 us against 161, and 147 with 2).
 static bool many_tiles(int64_t bins) { return bins >= (int64_t)32 * sm_count(); }
 bool tile_order_auto(int64_t bins) { return many_tiles(bins); }
 int raster_fwd_auto(int64_t bins) { return many_tiles(bins) ? 4 : 2; }
-int raster_bwd_auto(int64_t bins) {
-  const int64_t sms = sm_count();
-  return many_tiles(bins) ? 8 : bins >= 4 * sms && bins < 8 * sms ? 2 : 4;
-}
+int raster_bwd_auto(int64_t bins) { return many_tiles(bins) ? 8 : 4; }
 
 bool raster_bwd_flags(int ppt) { return ppt == 4 || ppt == 8; }
 
