@@ -401,7 +401,10 @@ gs_status gs_adam(gs_ctx* ctx, gs_params* p, const gs_params* g, gs_params* m, g
  * parameter update) to size every workspace; the capture itself uses a
  * private stream.  Every pointer (parameters, gradients, moments, targets,
  * images, dL/dimages, loss: device) is baked into the graph and must stay
- * valid, except the targets, which each launch names.
+ * valid, except the targets, which each launch names.  The context takes any
+ * other work between replays: a workspace of the step that it outgrows is kept
+ * for the graph beside the larger one, until the next capture; only when
+ * memory runs out is the graph given up for it (GS_ESTATE from then on).
  * Errors: GS_EINVAL, GS_ENOMEM, GS_ECUDA, and those of the steps. */
 gs_status gs_train_graph_capture(gs_ctx* ctx, gs_params* params, gs_params* grads, gs_params* m, gs_params* v,
                                  const gs_adam_hp* hp, const gs_camera* cams, int32_t B, const float* targets,
@@ -412,7 +415,9 @@ gs_status gs_train_graph_capture(gs_ctx* ctx, gs_params* params, gs_params* grad
  * and Adam step number `step` (>= 1).  Cameras, Adam constants and the
  * targets pointer go through a pinned staging area that the graph copies at
  * its start; the call waits (host) until the previous replay has made that
- * copy.  Capacity overflow is reported by gs_sync.
+ * copy.  Capacity overflow is reported by gs_sync.  The captured batch is then
+ * the context's current one (gs_get_buffer, gs_raster_bwd and the others that
+ * follow gs_project), whatever batch came before.
  * Errors: GS_ESTATE (nothing captured), GS_EINVAL (cameras differ, NULL
  * targets), GS_ECUDA. */
 gs_status gs_train_graph_launch(gs_ctx* ctx, const gs_camera* cams, int32_t B, const float* targets, int64_t step);

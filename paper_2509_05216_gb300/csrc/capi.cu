@@ -27,9 +27,26 @@ struct DevBuf {
   size_t cap = 0;
 };
 
+// A batch as the steps after gs_project find it.
+struct BatchState {
+  int B = 0, deg = 0;
+  int64_t n = 0, stride = 0, bins = 0, pixels = 0, nblocks = 0;
+  int sort_passes = 0;      // LSD passes of the tile sort
+  uint2* ranges = nullptr;  // tile ranges (in `zeroed`)
+  bool tile_order_ready = false;
+};
+
+// A workspace of the captured step: the allocation that the graph's kernels
+// hold.  A batch that needs a larger one gets its own, kept as the spare while
+// the graph's is in place.
+struct GraphBuf {
+  DevBuf* buf;
+  DevBuf own, spare;
+};
+
 }  // namespace
 
-struct gs_ctx {
+struct gs_ctx : BatchState {  // (the last batch)
   int device = 0;
   cudaStream_t stream = nullptr;
   gs_config cfg{};
@@ -43,6 +60,8 @@ struct gs_ctx {
   bool capturing = false;
   cudaStream_t graph_stream = nullptr;
   cudaGraphExec_t gexec = nullptr;
+  BatchState graph_batch;            // the captured batch, restored by every replay
+  std::vector<GraphBuf> graph_bufs;  // its workspaces
   cudaEvent_t staged_ev = nullptr;  // the graph's staging copies have run
   // a captured step clears the 2D-gradient records on a side branch that
   // runs beside the forward compositing (fork and join events)
@@ -65,23 +84,19 @@ struct gs_ctx {
   int raster_fwd = 0;  // compositing variants (pixels per thread; 8 = one warp per tile);
   int raster_bwd = 0;  // 0: by the batch's tile count
   int bwd_direct = 2;  // per-lane gradient atomics when at most this many lanes contribute
-  int sort_passes = 0;  // LSD passes of the last tile sort
   int sort_items = 16;  // keys per thread of a sort partition
   int sort_wait = 1 << 20;  // look-back rounds before a sort gives up
   int tile_order_mode = -1;  // 0: composite tiles in bin order; 1: longest lists first; -1: by the tile count
   float* dens_grad = nullptr;   // densification statistic accumulated by gs_raster_bwd (caller-owned)
   float* dens_count = nullptr;
-  bool tile_order_ready = false;
   int64_t batch_cap = 0;    // instance capacity of the next sorts (0: cfg.instance_capacity)
   bool forward_only = false;  // no contribution cells: gs_raster_bwd unavailable (render server)
   bool cells_ready = false;   // the last forward recorded contribution cells
 
-  // last batch
-  int B = 0, deg = 0;
-  int64_t n = 0, stride = 0, bins = 0, pixels = 0, instances = 0, nblocks = 0;
+  // the last batch's progress and views
   bool projected = false, sorted = false, rastered = false;
+  int64_t instances = 0;
   std::vector<ViewRec> views_h;
-  uint2* ranges = nullptr;  // tile ranges of the last sort (in `zeroed`)
 
   DevBuf views, rec, rec3, tiles, block_sums, block_offsets, total, keys0, keys1, vals0, vals1,
       zeroed, hist_scan, tfinal, nlast, g2d, l1_partial, sorted_slots, adam_consts,
@@ -135,17 +150,59 @@ gs_status fail(gs_ctx* c, gs_status st, const char* fmt, ...) {
                   __LINE__);                                                                    \
   } while (0)
 
+// Workspaces that a captured step works on (the others belong to single calls).
+std::vector<DevBuf*> step_bufs(gs_ctx* c) {
+  return {&c->views,       &c->rec,        &c->rec3,       &c->tiles,       &c->block_sums,   &c->block_offsets,
+          &c->total,       &c->keys0,      &c->keys1,      &c->vals0,       &c->vals1,        &c->zeroed,
+          &c->hist_scan,   &c->tfinal,     &c->nlast,      &c->g2d,         &c->l1_partial,   &c->sorted_slots,
+          &c->adam_consts, &c->target_slot, &c->cells,     &c->vismask,     &c->ord_counts,   &c->tile_order,
+          &c->vis_sums,    &c->vis_offsets, &c->dtotal,    &c->dkeys0,      &c->dkeys1,       &c->dvals0,
+          &c->dvals1,      &c->dhist_scan, &c->dorder,     &c->torder,      &c->pair_flags,   &c->contrib};
+}
+
+// Free the captured step and the workspaces that only it, or only other batches
+// beside it, hold.
+void drop_graph(gs_ctx* c) {
+  if (!c->gexec) return;
+  cudaStreamSynchronize(c->stream);
+  cudaGraphExecDestroy(c->gexec);
+  c->gexec = nullptr;
+  for (GraphBuf& g : c->graph_bufs) {
+    if (g.buf->p != g.own.p) cudaFree(g.own.p);
+    if (g.spare.p) cudaFree(g.spare.p);
+  }
+  c->graph_bufs.clear();
+}
+
 gs_status ensure(gs_ctx* c, DevBuf& b, size_t bytes, bool exact = false) {
   if (bytes == 0) bytes = 16;
   if (b.cap >= bytes) return GS_OK;
   size_t want = exact ? bytes : bytes + bytes / 8;
   if (b.p) {
-    GS_CUDA(c, cudaStreamSynchronize(c->stream));
-    GS_CUDA(c, cudaFree(b.p));
-    b.p = nullptr;
-    b.cap = 0;
+    // an allocation that a captured step works on stays for its replays
+    GraphBuf* held = nullptr;
+    for (GraphBuf& g : c->graph_bufs)
+      if (g.own.p == b.p) held = &g;
+    if (held && held->spare.cap >= bytes) {
+      b = held->spare;
+      held->spare = DevBuf{};
+      return GS_OK;
+    }
+    DevBuf& old = held ? held->spare : b;
+    if (old.p) {
+      GS_CUDA(c, cudaStreamSynchronize(c->stream));
+      GS_CUDA(c, cudaFree(old.p));
+    }
+    old = DevBuf{};
+    b = DevBuf{};
   }
   cudaError_t e = cudaMalloc(&b.p, want);
+  if (e != cudaSuccess && c->gexec && !c->capturing) {
+    // rather the new batch than the captured step (GS_ESTATE until the next capture)
+    (void)cudaGetLastError();
+    drop_graph(c);
+    e = cudaMalloc(&b.p, want);
+  }
   if (e != cudaSuccess) {
     (void)cudaGetLastError();
     b.p = nullptr;
@@ -458,6 +515,7 @@ void gs_destroy(gs_ctx* c) {
   cudaSetDevice(c->device);
   if (c->stream) cudaStreamSynchronize(c->stream);
   else cudaDeviceSynchronize();
+  drop_graph(c);
   DevBuf* bufs[] = {&c->views, &c->rec, &c->rec3, &c->tiles, &c->block_sums, &c->block_offsets,
                     &c->total, &c->keys0, &c->keys1, &c->vals0, &c->vals1, &c->zeroed, &c->hist_scan, &c->tfinal, &c->nlast, &c->g2d, &c->l1_partial,
                     &c->sorted_slots, &c->adam_consts, &c->target_slot, &c->host_tgt0, &c->host_tgt1,
@@ -475,7 +533,6 @@ void gs_destroy(gs_ctx* c) {
   if (c->status_h) cudaFreeHost(c->status_h);
   if (c->pinned) cudaFreeHost(c->pinned);
   if (c->staging) cudaFreeHost(c->staging);
-  if (c->gexec) cudaGraphExecDestroy(c->gexec);
   if (c->graph_stream) cudaStreamDestroy(c->graph_stream);
   if (c->staged_ev) cudaEventDestroy(c->staged_ev);
   if (c->side_stream) cudaStreamDestroy(c->side_stream);
@@ -1550,10 +1607,7 @@ gs_status gs_train_graph_capture(gs_ctx* c, gs_params* p, gs_params* g, gs_param
   if (!c->join_ev) GS_CUDA(c, cudaEventCreateWithFlags(&c->join_ev, cudaEventDisableTiming));
   const size_t g2d_bytes = sizeof(float) * (kG2dGeo + kG2dCol) * (size_t)B * c->stride;
   if (c->g2d.cap < g2d_bytes) return fail(c, GS_ESTATE, "2D-gradient records not sized by the warm-up pass");
-  if (c->gexec) {
-    GS_CUDA(c, cudaGraphExecDestroy(c->gexec));
-    c->gexec = nullptr;
-  }
+  drop_graph(c);
   cudaStream_t user = c->stream;
   c->stream = c->graph_stream;
   c->capturing = true;
@@ -1611,6 +1665,9 @@ gs_status gs_train_graph_capture(gs_ctx* c, gs_params* p, gs_params* g, gs_param
   c->graph_planes = n_planes(p->sh_degree);
   c->graph_loss = loss;
   c->graph_count = 3 * c->pixels;
+  c->graph_batch = *c;
+  for (DevBuf* b : step_bufs(c))
+    if (b->p) c->graph_bufs.push_back(GraphBuf{b, *b, DevBuf{}});
   return GS_OK;
 }
 
@@ -1635,6 +1692,14 @@ gs_status gs_train_graph_launch(gs_ctx* c, const gs_camera* cams, int32_t B, con
     LaunchScope ls(c, "train_graph", (int)c->graph_kernels);
     GS_CUDA(c, cudaGraphLaunch(c->gexec, c->stream));
   }
+  // the captured batch is the context's current one again, in the workspaces
+  // that the graph holds
+  for (GraphBuf& g : c->graph_bufs)
+    if (g.buf->p != g.own.p) {
+      g.spare = *g.buf;
+      *g.buf = g.own;
+    }
+  static_cast<BatchState&>(*c) = c->graph_batch;
   c->projected = c->sorted = c->rastered = true;
   c->cells_ready = !c->forward_only;
   return GS_OK;
