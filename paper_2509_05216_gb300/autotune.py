@@ -3,8 +3,8 @@
 For a workload key (Gaussian count, resolution mix, views per batch, GPU name)
 it times the real training step under every candidate value of each option
 (CUDA events on the current stream, after a warm-up step) and keeps the
-fastest.  Results are cached as JSON so a later run with the same key skips
-the search.
+fastest.  Results are cached as JSON so a later run with the same key and the
+same kernel sources skips the search.
 """
 from __future__ import annotations
 
@@ -13,7 +13,7 @@ import os
 
 import torch
 
-from . import gs
+from . import build, gs
 
 CANDIDATES = {gs.GS_OPT_RASTER_FWD: [2, 8, 4, 1], gs.GS_OPT_RASTER_BWD: [2, 4, 8, 1],
               gs.GS_OPT_BWD_DIRECT: [2, 0, 4, 8], gs.GS_OPT_SORT_ITEMS: [16, 12, 20, 24],
@@ -51,6 +51,12 @@ def _save(db):
         pass
 
 
+def _cached(db, key):
+    """The entry of `key`, if it was timed with the present kernels."""
+    entry = db.get(key)
+    return entry if entry and entry.get("kernels") == build.digest() else None
+
+
 def time_step(step, reps=3):
     """Shortest of `reps` single-step times (ms) after one warm-up step: the
     minimum is the least disturbed by clock or power-state drift."""
@@ -70,7 +76,7 @@ def time_step(step, reps=3):
 def report(key):
     """The timings (ms per step, "option=value") of the cached search for
     `key`, or None."""
-    entry = _load().get(key)
+    entry = _cached(_load(), key)
     return entry.get("ms") if entry else None
 
 
@@ -82,8 +88,9 @@ def tune(ctxs, step, key, candidates=None, reps=3, rounds=2, use_cache=True):
     Returns {option: value} and leaves the chosen values set."""
     candidates = candidates or CANDIDATES
     db = _load() if use_cache else {}
-    if key in db:
-        chosen = {int(k): v for k, v in db[key]["options"].items()}
+    entry = _cached(db, key)
+    if entry:
+        chosen = {int(k): v for k, v in entry["options"].items()}
     else:
         chosen, report = {}, {}
         for opt, values in candidates.items():
@@ -99,7 +106,8 @@ def tune(ctxs, step, key, candidates=None, reps=3, rounds=2, use_cache=True):
             for c in ctxs:
                 c.gs_set_option(opt, best)
             chosen[opt] = best
-        db[key] = {"options": {str(k): v for k, v in chosen.items()}, "ms": report}
+        db[key] = {"options": {str(k): v for k, v in chosen.items()}, "ms": report,
+                   "kernels": build.digest()}
         if use_cache:
             _save(db)
     for opt, v in chosen.items():

@@ -7,7 +7,9 @@ header is newer than the library.
 from __future__ import annotations
 
 import concurrent.futures as cf
+import functools
 import glob
+import hashlib
 import os
 import shutil
 import subprocess
@@ -37,6 +39,16 @@ def sources():
 def _deps():
     return sources() + glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(CSRC, "*.h")) + \
         [os.path.join(ROOT, "include", "gs.h")]
+
+
+@functools.lru_cache(maxsize=1)
+def digest() -> str:
+    """Digest of the kernel sources and the C header."""
+    h = hashlib.sha256()
+    for p in sorted(_deps(), key=os.path.basename):
+        with open(p, "rb") as f:
+            h.update(os.path.basename(p).encode() + b"\0" + f.read())
+    return h.hexdigest()[:16]
 
 
 def up_to_date() -> bool:
