@@ -476,7 +476,7 @@ def gpu_arm(args):
         clk_max = float(peaks.get("sm_max_mhz", 2070.0))
         peak = sms * 128 * 2 * clk_max * 1e6 / 1e12  # FP32 TFLOP/s, FMA = 2
         achieved = work / (avg_ms / 1e3) / 1e12
-        variant = tuned.get(gs.GS_OPT_RASTER_BWD if dom["name"] == "raster_bwd" else gs.GS_OPT_RASTER_FWD, 2)
+        variant = ctx.gs_get_option(gs.GS_OPT_RASTER_BWD if dom["name"] == "raster_bwd" else gs.GS_OPT_RASTER_FWD)
         roof = {"bound": "alu", "achieved": round(achieved, 2), "peak": round(peak, 1), "unit": "TFLOP/s",
                 "frac": round(achieved / peak, 4), "traffic": None,
                 "kernel": "%s<%d>" % (dom["name"], variant),

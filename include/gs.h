@@ -138,8 +138,9 @@ typedef enum {
   GS_OPT_RASTER_FWD = 0, /* forward compositing kernel: 1, 2 or 4 = pixels per
                             thread with one block per tile, 8 = one warp per
                             tile.  All variants give the same result up to
-                            FP32 rounding.  Unless set, by the batch's tile
-                            count, as the next one and GS_OPT_TILE_ORDER. */
+                            FP32 rounding.  GS_OPT_AUTO (default, as of the
+                            next one and GS_OPT_TILE_ORDER): by each batch's
+                            tile count. */
   GS_OPT_RASTER_BWD = 1, /* backward compositing kernel, same values */
   GS_OPT_BWD_DIRECT = 2, /* backward with 1 or 2 pixels per thread: a warp whose
                             pixels meet a Gaussian in at most this many lanes
@@ -148,8 +149,9 @@ typedef enum {
                             Same result up to FP32 summation order. */
   GS_OPT_SORT_ITEMS = 3, /* keys per thread of a radix-sort partition: 12, 16
                             (default), 20 or 24 (partitions of 256 x items
-                            keys; short segments take 4 or 8).  Same result.  Fixed once a training graph
-                            is captured (GS_ESTATE). */
+                            keys; segments of up to 65,536 keys take 4, of up
+                            to 262,144 8).  Same result.  Fixed once a training
+                            graph is captured (GS_ESTATE). */
   GS_OPT_SORT_WAIT = 4,  /* look-back rounds a radix-sort partition waits for
                             the partitions before it: 1 .. 1048576 (default
                             1048576, about a second), after which the sort
@@ -161,14 +163,21 @@ typedef enum {
   GS_OPT_TILE_ORDER = 5  /* order in which the compositing kernels take the
                             batch's tiles: 0 bin order; 1 longest lists first
                             (tiles bucketed by floor(log2(list length + 1)),
-                            bin order within a bucket); unless set, 1 for
-                            batches of many tiles.  Same result
+                            bin order within a bucket); GS_OPT_AUTO (default):
+                            1 for batches of many tiles.  Same result
                             (the fused L1 loss sums its per-tile partials in
                             bin order either way).  Fixed once a training graph
                             is captured (GS_ESTATE). */
 } gs_option;
 
-/* Set / read an option.  Errors: GS_EINVAL (unknown option, bad value). */
+/* Value of GS_OPT_RASTER_FWD, GS_OPT_RASTER_BWD and GS_OPT_TILE_ORDER: chosen
+ * for each batch. */
+#define GS_OPT_AUTO (-1)
+
+/* Set / read an option.  While a variant or the tile order is GS_OPT_AUTO,
+ * gs_get_option gives what the last projected batch takes; setting that value
+ * keeps it for every later batch, setting GS_OPT_AUTO returns to the choice by
+ * batch.  Errors: GS_EINVAL (unknown option, bad value). */
 gs_status gs_set_option(gs_ctx* ctx, int32_t option, int64_t value);
 gs_status gs_get_option(gs_ctx* ctx, int32_t option, int64_t* value);
 

@@ -15,9 +15,9 @@ import torch
 
 from . import build, gs
 
-CANDIDATES = {gs.GS_OPT_RASTER_FWD: [2, 8, 4, 1], gs.GS_OPT_RASTER_BWD: [2, 4, 8, 1],
+CANDIDATES = {gs.GS_OPT_RASTER_FWD: [gs.GS_OPT_AUTO, 2, 8, 4, 1], gs.GS_OPT_RASTER_BWD: [gs.GS_OPT_AUTO, 2, 4, 8, 1],
               gs.GS_OPT_BWD_DIRECT: [2, 0, 4, 8], gs.GS_OPT_SORT_ITEMS: [16, 12, 20, 24],
-              gs.GS_OPT_TILE_ORDER: [0, 1]}
+              gs.GS_OPT_TILE_ORDER: [gs.GS_OPT_AUTO, 0, 1]}
 
 
 def workload_key(n, cams, batch):

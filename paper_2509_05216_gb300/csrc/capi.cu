@@ -81,12 +81,13 @@ struct gs_ctx : BatchState {  // (the last batch)
   cudaEvent_t tgt_copied[2] = {nullptr, nullptr};
   cudaEvent_t tgt_free[2] = {nullptr, nullptr};
   int64_t host_launches = 0;
-  int raster_fwd = 0;  // compositing variants (pixels per thread; 8 = one warp per tile);
-  int raster_bwd = 0;  // 0: by the batch's tile count
+  // compositing variants (pixels per thread; 8 = one warp per tile)
+  int raster_fwd = GS_OPT_AUTO;  // GS_OPT_AUTO: by the batch's tile count
+  int raster_bwd = GS_OPT_AUTO;
   int bwd_direct = 2;  // per-lane gradient atomics when at most this many lanes contribute
   int sort_items = 16;  // keys per thread of a sort partition
   int sort_wait = 1 << 20;  // look-back rounds before a sort gives up
-  int tile_order_mode = -1;  // 0: composite tiles in bin order; 1: longest lists first; -1: by the tile count
+  int tile_order_mode = GS_OPT_AUTO;  // 0: composite tiles in bin order; 1: longest lists first; GS_OPT_AUTO: by the tile count
   float* dens_grad = nullptr;   // densification statistic accumulated by gs_raster_bwd (caller-owned)
   float* dens_count = nullptr;
   int64_t batch_cap = 0;    // instance capacity of the next sorts (0: cfg.instance_capacity)
@@ -843,12 +844,12 @@ static gs_status sort_tiles_longest_first(gs_ctx* c) {
 // longer warps of 4 pixels per thread: a burst of 12 requests 3.64 against 3.38
 // ms with 2.)
 static int fwd_variant(const gs_ctx* c) {
-  return c->raster_fwd ? c->raster_fwd : c->forward_only ? 2 : raster_fwd_auto(c->bins);
+  return c->raster_fwd != GS_OPT_AUTO ? c->raster_fwd : c->forward_only ? 2 : raster_fwd_auto(c->bins);
 }
 static int order_mode(const gs_ctx* c) {
-  return c->tile_order_mode >= 0 ? c->tile_order_mode : (tile_order_auto(c->bins) ? 1 : 0);
+  return c->tile_order_mode != GS_OPT_AUTO ? c->tile_order_mode : (tile_order_auto(c->bins) ? 1 : 0);
 }
-static int bwd_variant(const gs_ctx* c) { return c->raster_bwd ? c->raster_bwd : raster_bwd_auto(c->bins); }
+static int bwd_variant(const gs_ctx* c) { return c->raster_bwd != GS_OPT_AUTO ? c->raster_bwd : raster_bwd_auto(c->bins); }
 
 static RasterArgs raster_args(gs_ctx* c) {
   RasterArgs r{};
@@ -1541,8 +1542,8 @@ gs_status gs_set_option(gs_ctx* c, int32_t option, int64_t value) {
   switch (option) {
     case GS_OPT_RASTER_FWD:
     case GS_OPT_RASTER_BWD:
-      if (value != 1 && value != 2 && value != 4 && value != 8)
-        return fail(c, GS_EINVAL, "raster variant must be 1, 2, 4 or 8");
+      if (value != 1 && value != 2 && value != 4 && value != 8 && value != GS_OPT_AUTO)
+        return fail(c, GS_EINVAL, "raster variant must be 1, 2, 4, 8 or automatic (-1)");
       (option == GS_OPT_RASTER_FWD ? c->raster_fwd : c->raster_bwd) = (int)value;
       return GS_OK;
     case GS_OPT_BWD_DIRECT:
@@ -1556,7 +1557,8 @@ gs_status gs_set_option(gs_ctx* c, int32_t option, int64_t value) {
       c->sort_items = (int)value;
       return GS_OK;
     case GS_OPT_TILE_ORDER:
-      if (value != 0 && value != 1) return fail(c, GS_EINVAL, "tile order must be 0 or 1");
+      if (value != 0 && value != 1 && value != GS_OPT_AUTO)
+        return fail(c, GS_EINVAL, "tile order must be 0, 1 or automatic (-1)");
       if (c->capturing || c->gexec) return fail(c, GS_ESTATE, "tile order is fixed once a graph is captured");
       c->tile_order_mode = (int)value;
       return GS_OK;

@@ -82,6 +82,8 @@ class gs_kernel_stat(ctypes.Structure):
 
 GS_OPT_RASTER_FWD, GS_OPT_RASTER_BWD, GS_OPT_BWD_DIRECT, GS_OPT_SORT_ITEMS, GS_OPT_SORT_WAIT, GS_OPT_TILE_ORDER = \
     0, 1, 2, 3, 4, 5
+GS_OPT_AUTO = -1  # of the two variants and the tile order: by each batch's tile count
+
 
 class gs_serve_cfg(ctypes.Structure):
     _fields_ = [("slots", ctypes.c_int32), ("max_batch_views", ctypes.c_int32), ("max_queue", ctypes.c_int32),
