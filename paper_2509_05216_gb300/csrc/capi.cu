@@ -947,11 +947,15 @@ gs_status gs_raster_bwd(gs_ctx* c, const gs_params* params, const float* dL_dima
   // The compositing backward can flag the (view, Gaussian) pairs that it adds a
   // gradient to, so that the projection backward reads only their records.
   // The reads saved grow with the pairs, the flags' cost with the entries
-  // walked, roughly the pixels: 64M pairs on 67M pixels (4M Gaussians, 16
-  // views of 2048^2) 0.44 ms saved, 0.15 ms spent; 4M pairs on 8.4M pixels
-  // (500,000 Gaussians, 8 views of 1024^2) 16 us saved, 31 us spent; so from
-  // three pairs on four pixels.
-  const bool flagged = c->B > 1 && raster_bwd_flags(bwd_variant(c)) && 4 * (int64_t)c->B * c->n >= 3 * c->pixels;
+  // walked, roughly the pixels, on top of a clear and a launch.  gs_raster_bwd
+  // with flags against without, by pairs (pairs per pixel): 64M (0.95) -333 us of
+  // 5197; 16M (0.95) -77 and -50; 4M (0.95) -7, (1.9) -11, (0.48) +2; 2.4M (0.57) 0;
+  // 3.2M in 64 views (3.1) +4; 1.6M (0.76) +1; 0.4M (0.76 and 1.5) +8; 0.1M (0.56 and
+  // 2.3) +7 and +12 of 140 and 171.  So from three pairs on four pixels and 3.5M
+  // pairs.
+  const int64_t pairs = (int64_t)c->B * c->n;
+  const bool flagged =
+      c->B > 1 && raster_bwd_flags(bwd_variant(c)) && 4 * pairs >= 3 * c->pixels && pairs >= 3500000;
   if (flagged) {
     const size_t flag_bytes = (size_t)c->B * c->stride;
     GS_TRY(ensure(c, c->pair_flags, flag_bytes));

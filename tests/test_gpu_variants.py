@@ -83,3 +83,48 @@ def test_backward_kernels_agree_in_every_element():
     for bwd in (2, 4, 8):
         assert torch.isfinite(out[bwd]).all()
         assert ((out[bwd] - out[1]).abs() / largest).max().item() <= 1e-4, bwd
+
+
+# enough (view, Gaussian) pairs for the flags of those that took a gradient: one word of views, three with a last one
+# that is not whole, all 64; ragged tiles
+@pytest.mark.parametrize("n,views", [(1200001, 3), (200003, 18), (60001, 64)])
+@pytest.mark.parametrize("bwd", [4, 8])
+def test_backward_of_flagged_pairs(n, views, bwd):
+    scene = inputs.random_scene(n, 0, 6, extent=0.8, log_scale=(-5.5, -4.0))
+    cams = [inputs.pinhole(inputs.look_at((2.8 * np.cos(0.1 * v), 2.8 * np.sin(0.1 * v), 0.5)), 47 + v % 3, 50)
+            for v in range(views)]
+    assert n * views >= 3500000 and 4 * n * views >= 3 * sum(c["width"] * c["height"] for c in cams)
+    _, total = gs.image_offsets(cams)
+    dimg = torch.from_numpy(np.random.default_rng(7).normal(size=total).astype(np.float32)).cuda()
+    out = {}
+    for kernel in (1, bwd):  # (the one-pixel kernel keeps no flags)
+        ctx = gs.Context(0)
+        ctx.gs_set_option(gs.GS_OPT_RASTER_BWD, kernel)
+        stat, count = torch.zeros(n, device="cuda"), torch.zeros(n, device="cuda")
+        ctx.gs_set_densify_stats(stat, count)
+        p, _ = run_forward(ctx, scene, cams)
+        grads = torch.full_like(p, float("nan"))
+        ctx.profile_reset()
+        ctx.gs_raster_bwd(p, n, 0, dimg, grads)
+        ctx.gs_sync()
+        launched = {k["name"] for k in ctx.profile_read() if k["launches"]}
+        assert ("pair_masks" in launched) == (kernel != 1)
+        out[kernel] = [t.cpu().numpy().astype(np.float64) for t in (grads, stat, count)]
+        ctx.gs_set_densify_stats(None, None)
+        ctx.close()
+    assert np.isfinite(out[bwd][0]).all() and rel_l2(out[bwd][0], out[1][0]) <= 2e-5
+    assert rel_l2(out[bwd][1], out[1][1]) <= 2e-5 and np.array_equal(out[bwd][2], out[1][2])
+
+
+def test_small_batches_keep_no_flags():
+    """Below 3.5M pairs the flags' clear and launch cost more than they save, however few the pixels."""
+    scene, _ = mixed()
+    cams = [inputs.pinhole(inputs.look_at((0.4 + v, -2.8, 1.0)), 48, 32) for v in range(2)]
+    _, total = gs.image_offsets(cams)
+    ctx = gs.Context(0)
+    p, _ = run_forward(ctx, scene, cams)
+    ctx.profile_reset()
+    ctx.gs_raster_bwd(p, scene["n"], scene["deg"], torch.ones(total, device="cuda"), torch.zeros_like(p))
+    ctx.gs_sync()
+    assert not any(k["name"] == "pair_masks" and k["launches"] for k in ctx.profile_read())
+    ctx.close()
