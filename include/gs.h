@@ -346,7 +346,8 @@ gs_status gs_iso_emit(gs_ctx* ctx, const float* volume, int32_t nx, int32_t ny, 
  * normalised; (0, 1, 0, 0) for n = -z), opacity logit as given, SH DC
  * 2 sqrt(pi) (c - 1/2) with the Lambertian grey c = 0.1 + 0.9 max(0,
  * n . (1,1,1)/sqrt 3), higher SH 0.  The neighbours are found on the GPU with
- * a uniform grid (points sorted by cell with the binning's radix sort).
+ * a grid of cubes, sorted by Morton code with the binning's radix sort, whose
+ * size is picked on the device by the points per occupied cell.
  * Synchronises the stream; ends the context's current batch.  Errors:
  * GS_EINVAL (n < 4, n != out->n, m < n, flatten <= 0, points spanning no
  * box), GS_ENOMEM, GS_ECUDA. */

@@ -1367,15 +1367,9 @@ gs_status gs_init_gaussians(gs_ctx* c, const float* points, const float* normals
   k.sel = select;
   k.n = n;
   double emax = 0.0;
-  for (int d = 0; d < 3; d++) {
-    emax = std::max(emax, (double)bounds[3 + d] - (double)bounds[d]);
-    k.lo[d] = bounds[d];
-  }
+  for (int d = 0; d < 3; d++) emax = std::max(emax, (double)bounds[3 + d] - (double)bounds[d]);
   if (!(emax > 0.0) || !std::isfinite(emax)) return fail(c, GS_EINVAL, "points must span a finite, nonzero box");
-  const int key_bits = knn_key_bits();
-  const double cell = emax / (double)(1 << (key_bits / 3));
-  k.cell = (float)cell;
-  k.inv_cell = (float)(1.0 / cell);
+  const int key_bits = knn_grid(bounds, bounds + 3, &k);
   // the chosen level has at most n cells: at most 2/3 full
   int tbits = 10;
   while (((int64_t)1 << tbits) < n + n / 2) tbits++;
@@ -1385,7 +1379,7 @@ gs_status gs_init_gaussians(gs_ctx* c, const float* points, const float* normals
   GS_TRY(ensure(c, c->vals0, sizeof(uint32_t) * n));
   GS_TRY(ensure(c, c->vals1, sizeof(uint32_t) * n));
   GS_TRY(ensure(c, c->init_pts, sizeof(float4) * n));
-  GS_TRY(ensure(c, c->knn_heads, sizeof(uint32_t) * 16));
+  GS_TRY(ensure(c, c->knn_heads, sizeof(uint32_t) * kKnnWords));
   GS_TRY(ensure(c, c->knn_table, sizeof(unsigned long long) << tbits));
   GS_TRY(ensure(c, c->init_scales, sizeof(float) * n));
   k.keys[0] = P<uint32_t>(c->keys0);
@@ -1402,7 +1396,7 @@ gs_status gs_init_gaussians(gs_ctx* c, const float* points, const float* normals
   k.heads = P<uint32_t>(c->knn_heads);
   k.table = P<unsigned long long>(c->knn_table);
   k.out = P<float>(c->init_scales);
-  GS_CUDA(c, cudaMemsetAsync(k.heads, 0, sizeof(uint32_t) * 16, c->stream));
+  GS_CUDA(c, cudaMemsetAsync(k.heads, 0, sizeof(uint32_t) * kKnnWords, c->stream));
   GS_CUDA(c, cudaMemsetAsync(k.table, 0xff, sizeof(unsigned long long) << tbits, c->stream));
   {
     LaunchScope ls(c, "knn_query", 4);

@@ -314,13 +314,31 @@ __global__ void __launch_bounds__(192) knn_bounds_finish_kernel(const float* __r
 
 namespace {
 
-// The finest grid has 2^10 cells along the longest side of the bounding box;
-// a point's key is the Morton code of its finest cell, so that one sort orders
-// the points by cell at every level l (cells of 2^l finest ones: the key
-// without its low 3 l bits), and a cell of any level is a run of the sorted
-// points.
-constexpr int kMortonBits = 10;
+// A point's key is the Morton code of its finest cell, so that one sort orders
+// the points by cell at every level l (cubes of 2^l finest cells along each
+// axis), and a cell of any level is a run of the sorted points.  The finest
+// cells are cubes too, 2^10 to 2^16 along the longest side of the bounding
+// box: as many as 30 key bits allow, for a side of the box takes only the bits
+// that its cells need.  A box with three long sides has 2^10, a flat one up to
+// 2^15, a line 2^16 (a position's rounding, in finest cells, allows no more).
+// With 2^10 for every box a line's finest cells hold thousands of points: 4M
+// points on a line, whole call 21.5 ms (1.1 ms like this), on a ribbon 7.0 ms
+// (1.2 ms).
+//
+// Bit order of a key: with a <= b <= c bits along the axes, the low a bits of
+// all three interleaved, the next b - a of the two longer, the last of the
+// longest; the bits of a level's cell are the key without its low
+// min(l, a) + min(l, b) + min(l, c) ones.
+constexpr int kMaxLevels = 16, kKeyBits = 30;
+constexpr float kKnnMargin = 2e-3f;  // of a position in finest cells, 2^10 along the longest side
 
+__device__ __forceinline__ uint32_t spread2(uint32_t x) {  // bit i -> bit 2 i
+  x = (x | (x << 8)) & 0x00ff00ffu;
+  x = (x | (x << 4)) & 0x0f0f0f0fu;
+  x = (x | (x << 2)) & 0x33333333u;
+  x = (x | (x << 1)) & 0x55555555u;
+  return x;
+}
 __device__ __forceinline__ uint32_t spread3(uint32_t x) {  // bit i -> bit 3 i
   x &= 0x3ffu;
   x = (x | (x << 16)) & 0x030000ffu;
@@ -329,17 +347,64 @@ __device__ __forceinline__ uint32_t spread3(uint32_t x) {  // bit i -> bit 3 i
   x = (x | (x << 2)) & 0x09249249u;
   return x;
 }
-__device__ __forceinline__ uint32_t gather3(uint32_t x) {  // bit 3 i -> bit i
-  x &= 0x09249249u;
-  x = (x | (x >> 2)) & 0x030c30c3u;
-  x = (x | (x >> 4)) & 0x0300f00fu;
-  x = (x | (x >> 8)) & 0x030000ffu;
-  x = (x | (x >> 16)) & 0x3ffu;
-  return x;
+
+// Key of the cell (x, y, z) of a level (coordinates in the order of a.bits).
+// EVEN, here and below: the same bits along every axis, which are 10 then (the
+// common box; by the general code the query takes 5 % longer there).
+template <bool EVEN = false>
+__device__ __forceinline__ uint32_t cell_key(const KnnArgs& a, uint32_t x, uint32_t y, uint32_t z, int level) {
+  if constexpr (EVEN) return spread3(x) | (spread3(y) << 1) | (spread3(z) << 2);
+  const int ba = max(a.bits[0] - level, 0), bb = max(a.bits[1] - level, 0);
+  const uint32_t low = (1u << ba) - 1u;
+  uint32_t k = spread3(x) | (spread3(y & low) << 1) | (spread3(z & low) << 2);
+  if (a.bits[0] != a.bits[2]) {
+    y >>= ba;
+    z >>= ba;
+    k |= (spread2(y) | (spread2(z & ((1u << (bb - ba)) - 1u)) << 1)) << (3 * ba);
+    k |= (z >> (bb - ba)) << (ba + 2 * bb);
+  }
+  return k;
 }
 
-__device__ __forceinline__ uint32_t fine_cell(float x, float lo, float inv) {
-  return (uint32_t)min(max((int)((x - lo) * inv), 0), (1 << kMortonBits) - 1);
+// Low bits of a key that a level's cells leave out.
+__device__ __forceinline__ int level_shift(const KnnArgs& a, int level) {
+  return min(level, a.bits[0]) + min(level, a.bits[1]) + min(level, a.bits[2]);
+}
+
+// The coarsest level at which two keys whose highest different bit is `bit` are
+// of different cells.
+__device__ __forceinline__ int level_of_bit(const KnnArgs& a, int bit) {
+  const int ba = a.bits[0], bb = a.bits[1];
+  return bit < 3 * ba ? bit / 3 : bit < ba + 2 * bb ? ba + (bit - 3 * ba) / 2 : bit - ba - bb;
+}
+
+template <bool EVEN = false>
+__device__ __forceinline__ int cells_along(const KnnArgs& a, int k, int level) {
+  return 1 << (EVEN ? kKeyBits / 3 - level : max(a.bits[k] - level, 0));
+}
+
+// A point's position in cells of a level, and its cell.
+template <bool EVEN = false>
+struct CellPos {
+  float f[3];
+  int c[3];
+  __device__ __forceinline__ CellPos(const KnnArgs& a, float x, float y, float z, int level) {
+    const float scale = 1.f / (float)(1 << level);
+#pragma unroll
+    for (int k = 0; k < 3; k++) {
+      const int axis = EVEN ? k : a.axis[k];
+      const float v = axis == 0 ? x : axis == 1 ? y : z;
+      const float u = (v - a.lo[k]) * a.inv_cell;
+      c[k] = min(max((int)u, 0), (1 << (EVEN ? kKeyBits / 3 : a.bits[k])) - 1) >> level;
+      f[k] = u * scale;
+    }
+  }
+};
+
+// Margin of a position in cells of a level.
+template <bool EVEN = false>
+__device__ __forceinline__ float cell_margin(const KnnArgs& a, int level) {
+  return EVEN ? kKnnMargin : fmaxf(kKnnMargin, a.margin / (float)(1 << level));
 }
 
 // First slot of a cell: the 8 cells of a cube of the next level share a line.
@@ -362,13 +427,19 @@ __device__ __forceinline__ unsigned long long cell_entry(uint32_t key, int64_t s
 // kernel: 6.6 ms against 2.0 ms.)
 constexpr int64_t kCellPoints = 2;
 __device__ __forceinline__ int pick_level(const KnnArgs& a) {
+  // (all words in flight at once; they are 0 from the coarsest level up)
+  uint4 h[kMaxLevels / 4];
+#pragma unroll
+  for (int i = 0; i < kMaxLevels / 4; i++) h[i] = *reinterpret_cast<const uint4*>(a.heads + 4 * i);
   int64_t cells = 1;
-  int level = kMortonBits;
-  for (int l = kMortonBits - 1; l >= 0; l--) {
-    cells += a.heads[l];
-    if (cells * kCellPoints <= a.n) level = l; else break;
+  int level = kMaxLevels;
+#pragma unroll
+  for (int l = kMaxLevels - 1; l >= 0; l--) {
+    const uint4 q = h[l / 4];
+    cells += l % 4 == 0 ? q.x : l % 4 == 1 ? q.y : l % 4 == 2 ? q.z : q.w;
+    level -= cells * kCellPoints <= a.n ? 1 : 0;  // (grows with every level: those that fit come first)
   }
-  return level;
+  return min(level, a.bits[2]);
 }
 
 __device__ __forceinline__ const uint32_t* sorted_keys(const KnnArgs& a) {
@@ -379,7 +450,8 @@ __device__ __forceinline__ const uint32_t* sorted_keys(const KnnArgs& a) {
 __device__ __forceinline__ uint32_t* spare_vals(const KnnArgs& a) {
   return (a.sort_ctrl[a.sort_passes] & 1u) ? a.vals[0] : a.vals[1];
 }
-constexpr int kTodo = 12;  // word of `heads` that counts the points left to the warps
+constexpr int kTodo = kKnnWords - 1;  // word of `heads` that counts the points left to the warps
+static_assert(kTodo >= kMaxLevels, "a word per level before it");
 
 // First sorted position in [lo, n) whose key is at least `key`.
 __device__ __forceinline__ int64_t lower_bound(const uint32_t* keys, int64_t lo, int64_t n, uint64_t key) {
@@ -401,7 +473,7 @@ __device__ __forceinline__ uint2 cell_run(const KnnArgs& a, const uint32_t* keys
     if ((uint32_t)(e >> 34) == cell) {
       const uint32_t start = (uint32_t)(e >> 3) & 0x7fffffffu, length = (uint32_t)e & 7u;
       if (length < 7u) return make_uint2(start, start + length);
-      return make_uint2(start, (uint32_t)lower_bound(keys, (int64_t)start + 7, a.n, ((uint64_t)cell + 1) << (3 * level)));
+      return make_uint2(start, (uint32_t)lower_bound(keys, (int64_t)start + 7, a.n, ((uint64_t)cell + 1) << level_shift(a, level)));
     }
   }
   return make_uint2(0u, 0u);
@@ -422,19 +494,17 @@ __device__ __forceinline__ void near_point(const KnnArgs& a, int64_t j, float px
 }
 
 // One axis of the 3^3 cells around a point's cell c (of dim cells; f: the
-// point's fraction of it): per neighbour the spread coordinate and the squared
-// distance to it (3e38 outside the grid), less a margin for the rounding of f
-// (1e-4 of a finest cell).  *border: distance to the nearer side of the cell.
+// point's fraction of it): per neighbour the squared distance to it (3e38
+// outside the grid), less a margin for the rounding of f.  *border: distance to
+// the nearer side of the cell.
 struct CellAxis {
-  uint32_t code[3];
+  int c;
   float gap2[3];
 };
-__device__ __forceinline__ CellAxis cell_axis(int c, int dim, float f, float cell, float* border) {
+__device__ __forceinline__ CellAxis cell_axis(int c, int dim, float f, float margin, float cell, float* border) {
   CellAxis x;
-  const float lo = fmaxf(f - 2e-3f, 0.f) * cell, hi = fmaxf(1.f - f - 2e-3f, 0.f) * cell;
-  x.code[0] = spread3((uint32_t)(c - 1));
-  x.code[1] = spread3((uint32_t)c);
-  x.code[2] = spread3((uint32_t)(c + 1));
+  const float lo = fmaxf(f - margin, 0.f) * cell, hi = fmaxf(1.f - f - margin, 0.f) * cell;
+  x.c = c;
   x.gap2[0] = c > 0 ? lo * lo * 0.999f : 3.0e38f;
   x.gap2[1] = 0.f;
   x.gap2[2] = c + 1 < dim ? hi * hi * 0.999f : 3.0e38f;
@@ -447,10 +517,8 @@ __device__ __forceinline__ CellAxis cell_axis(int c, int dim, float f, float cel
 __global__ void __launch_bounds__(256) knn_keys_kernel(KnnArgs a) {
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < a.n; i += (int64_t)gridDim.x * blockDim.x) {
     const int64_t src = a.sel ? a.sel[i] : i;
-    const uint32_t x = fine_cell(a.pts[3 * src], a.lo[0], a.inv_cell);
-    const uint32_t y = fine_cell(a.pts[3 * src + 1], a.lo[1], a.inv_cell);
-    const uint32_t z = fine_cell(a.pts[3 * src + 2], a.lo[2], a.inv_cell);
-    a.keys[0][i] = spread3(x) | (spread3(y) << 1) | (spread3(z) << 2);
+    const CellPos<> p(a, a.pts[3 * src], a.pts[3 * src + 1], a.pts[3 * src + 2], 0);
+    a.keys[0][i] = cell_key(a, (uint32_t)p.c[0], (uint32_t)p.c[1], (uint32_t)p.c[2], 0);
     a.vals[0][i] = (uint32_t)i;
   }
 }
@@ -458,8 +526,8 @@ __global__ void __launch_bounds__(256) knn_keys_kernel(KnnArgs a) {
 // The points in sorted order (position and output index in one float4), and
 // the heads per level.
 __global__ void __launch_bounds__(256) knn_sorted_points_kernel(KnnArgs a) {
-  __shared__ uint32_t s_heads[kMortonBits];
-  if (threadIdx.x < kMortonBits) s_heads[threadIdx.x] = 0;
+  __shared__ uint32_t s_heads[kMaxLevels];
+  if (threadIdx.x < kMaxLevels) s_heads[threadIdx.x] = 0;
   __syncthreads();
   const uint32_t* keys = sorted_keys(a);
   const uint32_t* vals = keys == a.keys[1] ? a.vals[1] : a.vals[0];
@@ -469,15 +537,15 @@ __global__ void __launch_bounds__(256) knn_sorted_points_kernel(KnnArgs a) {
     const int64_t src = a.sel ? a.sel[o] : (int64_t)o;
     a.sorted[i] = make_float4(a.pts[3 * src], a.pts[3 * src + 1], a.pts[3 * src + 2], __uint_as_float(o));
     const uint32_t diff = i > 0 ? keys[i] ^ keys[i - 1] : 0u;
-    if (diff) atomicAdd(&s_heads[min((31 - __clz(diff)) / 3, kMortonBits - 1)], 1u);
+    if (diff) atomicAdd(&s_heads[min(level_of_bit(a, 31 - __clz(diff)), kMaxLevels - 1)], 1u);
   }
   __syncthreads();
-  if (threadIdx.x < kMortonBits && s_heads[threadIdx.x]) atomicAdd(a.heads + threadIdx.x, s_heads[threadIdx.x]);
+  if (threadIdx.x < kMaxLevels && s_heads[threadIdx.x]) atomicAdd(a.heads + threadIdx.x, s_heads[threadIdx.x]);
 }
 
 // Insert every cell of the chosen level with its run of sorted points.
 __global__ void __launch_bounds__(256) knn_table_kernel(KnnArgs a) {
-  const int sh = 3 * pick_level(a);
+  const int sh = level_shift(a, pick_level(a));
   const uint32_t* keys = sorted_keys(a);
   const uint32_t mask = (uint32_t)((1ull << a.table_bits) - 1ull);
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < a.n; i += (int64_t)gridDim.x * blockDim.x) {
@@ -502,27 +570,27 @@ __device__ __forceinline__ void write_scale(const KnnArgs& a, const float4& me, 
 // The cells around a sorted point at one level.
 struct CellCube {
   CellAxis x, y, z;
-  float border;
-  __device__ __forceinline__ CellCube(const KnnArgs& a, const float4& me, uint32_t key, int l) {
-    const int dim = 1 << (kMortonBits - l);
-    const float scale = 1.f / (float)(1 << l), cell = a.cell * (float)(1 << l);
-    const int cx = (int)gather3(key) >> l, cy = (int)gather3(key >> 1) >> l, cz = (int)gather3(key >> 2) >> l;
+  float border, margin;
+  __device__ __forceinline__ CellCube(const KnnArgs& a, const float4& me, int l) {
+    const float cell = a.cell * (float)(1 << l);
+    const CellPos<> p(a, me.x, me.y, me.z, l);
     border = 1.f;
-    x = cell_axis(cx, dim, (me.x - a.lo[0]) * a.inv_cell * scale - (float)cx, cell, &border);
-    y = cell_axis(cy, dim, (me.y - a.lo[1]) * a.inv_cell * scale - (float)cy, cell, &border);
-    z = cell_axis(cz, dim, (me.z - a.lo[2]) * a.inv_cell * scale - (float)cz, cell, &border);
+    margin = cell_margin(a, l);
+    x = cell_axis(p.c[0], cells_along(a, 0, l), p.f[0] - (float)p.c[0], margin, cell, &border);
+    y = cell_axis(p.c[1], cells_along(a, 1, l), p.f[1] - (float)p.c[1], margin, cell, &border);
+    z = cell_axis(p.c[2], cells_along(a, 2, l), p.f[2] - (float)p.c[2], margin, cell, &border);
   }
   // squared distance within which every point lies in the cube
   __device__ __forceinline__ float reach2(const KnnArgs& a, int l) const {
-    const float r = (1.f + border - 2e-3f) * a.cell * (float)(1 << l) * 0.999f;
+    const float r = (1.f + border - margin) * a.cell * (float)(1 << l) * 0.999f;
     return r * r;
   }
 };
 
 // Distance in cells, along an axis, from a point at f to cell c, less a margin
-// for the rounding of f (1e-4 of a finest cell).
-__device__ __forceinline__ float cell_gap(float f, uint32_t c) {
-  return fmaxf(fmaxf((float)c - f, f - (float)(c + 1u)) - 2e-3f, 0.f);
+// for the rounding of f.
+__device__ __forceinline__ float cell_gap(float f, int c, float margin) {
+  return fmaxf(fmaxf((float)c - f, f - (float)(c + 1)) - margin, 0.f);
 }
 
 // A warp takes 32 consecutive points in Morton order: the 3 smallest squared
@@ -541,6 +609,7 @@ __device__ __forceinline__ float cell_gap(float f, uint32_t c) {
 // kernel.
 constexpr int kQueryThreads = 128;
 constexpr int kQuerySpan = 5;  // cells between a lane's and the first lane's, along an axis
+template <bool EVEN>
 __global__ void __launch_bounds__(kQueryThreads) knn_query_kernel(KnnArgs a) {
   const int lane = threadIdx.x & 31;
   const int64_t first = (((int64_t)blockIdx.x * kQueryThreads + threadIdx.x) >> 5) * 32;
@@ -549,7 +618,6 @@ __global__ void __launch_bounds__(kQueryThreads) knn_query_kernel(KnnArgs a) {
   const int64_t i = min(first + lane, a.n - 1);
   const int level = pick_level(a);
   const uint32_t* keys = sorted_keys(a);
-  const uint32_t key = keys[i];
   const float4 me = a.sorted[i];
   float best[3] = {3.0e38f, 3.0e38f, 3.0e38f};
   for (int64_t j = max((int64_t)0, i - 4); j < min(a.n, i + 5); j++)
@@ -557,10 +625,10 @@ __global__ void __launch_bounds__(kQueryThreads) knn_query_kernel(KnnArgs a) {
   const float bound = best[2];
   best[0] = best[1] = best[2] = 3.0e38f;  // (the cells hold these neighbours too)
   // the lane's cell and its position in cells; the warp's box
-  const int dim = 1 << (kMortonBits - level);
-  const float scale = a.inv_cell / (float)(1 << level), cell = a.cell * (float)(1 << level);
-  const float fx = (me.x - a.lo[0]) * scale, fy = (me.y - a.lo[1]) * scale, fz = (me.z - a.lo[2]) * scale;
-  const int cx = (int)gather3(key) >> level, cy = (int)gather3(key >> 1) >> level, cz = (int)gather3(key >> 2) >> level;
+  const CellPos<EVEN> at(a, me.x, me.y, me.z, level);
+  const float cell = a.cell * (float)(1 << level), margin = cell_margin<EVEN>(a, level);
+  const float fx = at.f[0], fy = at.f[1], fz = at.f[2];
+  const int cx = at.c[0], cy = at.c[1], cz = at.c[2];
   for (uint32_t todo = __ballot_sync(0xffffffffu, mine); todo;) {
     const int lead = __ffs((int)todo) - 1;
     // (every lane takes part in the exchanges)
@@ -569,24 +637,27 @@ __global__ void __launch_bounds__(kQueryThreads) knn_query_kernel(KnnArgs a) {
     const bool in = ((todo >> lane) & 1u) != 0u && max(abs(cx - lx), max(abs(cy - ly), abs(cz - lz))) <= kQuerySpan;
     todo &= ~__ballot_sync(0xffffffffu, in);
     // the box of the lanes taken
-    auto low = [&](int c) { return max(__reduce_min_sync(0xffffffffu, in ? c : 1 << kMortonBits) - 1, 0); };
-    auto high = [&](int c) { return min(__reduce_max_sync(0xffffffffu, in ? c : 0) + 1, dim - 1); };
+    auto low = [&](int c) { return max(__reduce_min_sync(0xffffffffu, in ? c : 1 << kMaxLevels) - 1, 0); };
+    auto high = [&](int c, int k) {
+      return min(__reduce_max_sync(0xffffffffu, in ? c : 0) + 1, cells_along<EVEN>(a, k, level) - 1);
+    };
     const int x0 = low(cx), y0 = low(cy), z0 = low(cz);
-    const int ex = high(cx) - x0 + 1, exy = ex * (high(cy) - y0 + 1), cells = exy * (high(cz) - z0 + 1);
+    const int ex = high(cx, 0) - x0 + 1, exy = ex * (high(cy, 1) - y0 + 1), cells = exy * (high(cz, 2) - z0 + 1);
     const float cap = in ? 3.0e38f : 0.f, reach = in ? bound : -1.f;  // (the other lanes take nothing)
     for (int c0 = 0; c0 < cells; c0 += 32) {
       const int c = c0 + lane;
-      const uint32_t z = (uint32_t)(z0 + c / exy), y = (uint32_t)(y0 + c % exy / ex), x = (uint32_t)(x0 + c % exy % ex);
+      const int z = z0 + c / exy, y = y0 + c % exy / ex, x = x0 + c % exy % ex;
       uint2 run = make_uint2(0u, 0u);
-      if (c < cells) run = cell_run(a, keys, spread3(x) | (spread3(y) << 1) | (spread3(z) << 2), level);
-      const uint32_t pos = x | (y << kMortonBits) | (z << (2 * kMortonBits));
+      if (c < cells) run = cell_run(a, keys, cell_key<EVEN>(a, (uint32_t)x, (uint32_t)y, (uint32_t)z, level), level);
+      // the cell in 10 bits per axis: in the grid, or, where that may take more, in the box
+      const int bx = EVEN ? 0 : x0, by = EVEN ? 0 : y0, bz = EVEN ? 0 : z0;
+      const uint32_t pos = (uint32_t)((x - bx) | ((y - by) << 10) | ((z - bz) << 20));
       for (uint32_t m = __ballot_sync(0xffffffffu, run.y > run.x); m; m &= m - 1u) {
         const int src = __ffs((int)m) - 1;
         const uint32_t s0 = __shfl_sync(0xffffffffu, run.x, src), s1 = __shfl_sync(0xffffffffu, run.y, src);
         const uint32_t p = __shfl_sync(0xffffffffu, pos, src);
-        constexpr uint32_t kAxis = (1u << kMortonBits) - 1u;
-        const float gx = cell_gap(fx, p & kAxis), gy = cell_gap(fy, (p >> kMortonBits) & kAxis);
-        const float gz = cell_gap(fz, p >> (2 * kMortonBits));
+        const float gx = cell_gap(fx, bx + (int)(p & 0x3ffu), margin), gy = cell_gap(fy, by + (int)((p >> 10) & 0x3ffu), margin);
+        const float gz = cell_gap(fz, bz + (int)(p >> 20), margin);
         const float gap2 = (gx * gx + gy * gy + gz * gz) * (cell * cell) * 0.999f;
         if (!__any_sync(0xffffffffu, !(gap2 > fminf(best[2], reach)))) continue;
 #pragma unroll 4
@@ -608,7 +679,7 @@ __global__ void __launch_bounds__(kQueryThreads) knn_query_kernel(KnnArgs a) {
   border = fminf(border, fminf(fx - (float)cx, 1.f - (fx - (float)cx)));
   border = fminf(border, fminf(fy - (float)cy, 1.f - (fy - (float)cy)));
   border = fminf(border, fminf(fz - (float)cz, 1.f - (fz - (float)cz)));
-  const float reach = (1.f + border - 2e-3f) * cell * 0.999f;
+  const float reach = (1.f + border - margin) * cell * 0.999f;
   if (!mine) return;
   if (best[2] <= reach * reach) write_scale(a, me, best);
   else spare_vals(a)[atomicAdd(a.heads + kTodo, 1u)] = (uint32_t)i;
@@ -627,18 +698,18 @@ __global__ void __launch_bounds__(256) knn_far_kernel(KnnArgs a) {
     const int64_t i = spare_vals(a)[t];
     const float4 me = a.sorted[i];
     float third[3] = {3.0e38f, 3.0e38f, 3.0e38f};
-    for (int l = min(level + 1, kMortonBits); l <= kMortonBits; l++) {
-      const CellCube c(a, me, keys[i], l);
+    for (int l = min(level + 1, a.bits[2]); l <= a.bits[2]; l++) {
+      const CellCube c(a, me, l);
+      const int shift = level_shift(a, l);
       const int x = lane % 3, y = lane / 3 % 3, z = lane / 9;
       uint32_t lo = 0, hi = 0;
       auto pick = [](const float (&g)[3], int k) { return k == 0 ? g[0] : k == 1 ? g[1] : g[2]; };
-      auto code = [](const uint32_t (&g)[3], int k) { return k == 0 ? g[0] : k == 1 ? g[1] : g[2]; };
       if (lane < 27) {
         const float gap2 = pick(c.x.gap2, x) + pick(c.y.gap2, y) + pick(c.z.gap2, z);
         if (!(gap2 > third[2]) && gap2 < 3.0e38f) {
-          const uint64_t k = code(c.x.code, x) | (code(c.y.code, y) << 1) | (code(c.z.code, z) << 2);
-          lo = (uint32_t)lower_bound(keys, 0, a.n, k << (3 * l));
-          hi = (uint32_t)lower_bound(keys, lo, a.n, (k + 1) << (3 * l));
+          const uint64_t k = cell_key(a, (uint32_t)(c.x.c + x - 1), (uint32_t)(c.y.c + y - 1), (uint32_t)(c.z.c + z - 1), l);
+          lo = (uint32_t)lower_bound(keys, 0, a.n, k << shift);
+          hi = (uint32_t)lower_bound(keys, lo, a.n, (k + 1) << shift);
         }
       }
       float best[3] = {3.0e38f, 3.0e38f, 3.0e38f};
@@ -677,12 +748,41 @@ static unsigned knn_blocks(int64_t n) {
 
 void launch_knn_keys(const KnnArgs& a, cudaStream_t s) { knn_keys_kernel<<<knn_blocks(a.n), 256, 0, s>>>(a); }
 
-int knn_key_bits() { return 3 * kMortonBits; }
+int knn_grid(const float* lo, const float* hi, KnnArgs* a) {
+  double ext[3], longest = 0.0;
+  for (int d = 0; d < 3; d++) longest = std::max(longest, ext[d] = std::max((double)hi[d] - (double)lo[d], 0.0));
+  // (at 2^10 the bits never exceed 30)
+  for (int levels = kMaxLevels; levels >= kKeyBits / 3; levels--) {
+    const double cell = longest / (double)(1 << levels);
+    int bits[3], total = 0;
+    for (int d = 0; d < 3; d++) {
+      // bits of the last cell along the axis (the end of the longest side falls on the next one's border)
+      const int last = (int)(ext[d] / cell * (1.0 + 1e-6));
+      for (bits[d] = 0; bits[d] < levels && (last >> bits[d]) != 0;) bits[d]++;
+      total += bits[d];
+    }
+    if (total > kKeyBits) continue;
+    for (int k = 0; k < 3; k++) a->axis[k] = k;
+    std::stable_sort(a->axis, a->axis + 3, [&](int x, int y) { return bits[x] < bits[y]; });
+    for (int k = 0; k < 3; k++) {
+      a->bits[k] = bits[a->axis[k]];
+      a->lo[k] = lo[a->axis[k]];
+    }
+    a->cell = (float)cell;
+    a->inv_cell = (float)(1.0 / cell);
+    // ten times the rounding of a position at the far end (a difference and two roundings of the product)
+    a->margin = kKnnMargin * (float)(1 << (levels - kKeyBits / 3));
+    return total;
+  }
+  return 0;
+}
 
 void launch_knn_query(const KnnArgs& a, cudaStream_t s) {
   knn_sorted_points_kernel<<<knn_blocks(a.n), 256, 0, s>>>(a);
   knn_table_kernel<<<knn_blocks(a.n), 256, 0, s>>>(a);
-  knn_query_kernel<<<(unsigned)((a.n + kQueryThreads - 1) / kQueryThreads), kQueryThreads, 0, s>>>(a);
+  const unsigned queries = (unsigned)((a.n + kQueryThreads - 1) / kQueryThreads);
+  if (a.bits[0] == a.bits[2]) knn_query_kernel<true><<<queries, kQueryThreads, 0, s>>>(a);
+  else knn_query_kernel<false><<<queries, kQueryThreads, 0, s>>>(a);
   knn_far_kernel<<<knn_blocks(a.n), 256, 0, s>>>(a);
 }
 

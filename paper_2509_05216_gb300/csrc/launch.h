@@ -247,14 +247,17 @@ struct KnnArgs {
   const float* pts;      // [m][3]
   const int64_t* sel;    // [n] the points searched (NULL: the first n)
   int64_t n;
-  float lo[3], cell, inv_cell;  // finest cells
+  // finest cells: the axes by their number of index bits, least first, the box's corner along them
+  int axis[3], bits[3];
+  float lo[3], cell, inv_cell;
+  float margin;          // of a position in finest cells, for its rounding
   uint32_t* keys[2];     // [n] Morton codes of the finest cells; the sort's buffers
   uint32_t* vals[2];     // [n] points
   const uint32_t* sort_ctrl;  // sort_ctrl[sort_passes] bit 0: which buffer is sorted
   int sort_passes;
   float4* sorted;        // [n] points in sorted order: x, y, z, bits of the point's index
-  uint32_t* heads;       // [16], zeroed: sorted points that start a cell, by the coarsest level at which they do;
-                         // [12] the points that the first query leaves over
+  uint32_t* heads;       // [kKnnWords], zeroed: sorted points that start a cell, by the coarsest level at which they
+                         // do; the last word: the points that the first query leaves over
   unsigned long long* table;  // [2^table_bits] cell, first sorted point and length of its run (all ones: empty)
   int table_bits;
   float* out;            // [n] log-scales
@@ -262,7 +265,9 @@ struct KnnArgs {
 // out: min xyz, max xyz of the points
 void launch_knn_bounds(const float* pts, const int64_t* sel, int64_t n, float* part, int nparts, float* out,
                        cudaStream_t s);
-int knn_key_bits();
+constexpr int kKnnWords = 32;
+// axis, bits, lo, cell, inv_cell and margin for points in [lo, hi]; key bits
+int knn_grid(const float* lo, const float* hi, KnnArgs* a);
 void launch_knn_keys(const KnnArgs& a, cudaStream_t s);
 void launch_knn_query(const KnnArgs& a, cudaStream_t s);
 
