@@ -128,3 +128,72 @@ def test_small_batches_keep_no_flags():
     ctx.gs_sync()
     assert not any(k["name"] == "pair_masks" and k["launches"] for k in ctx.profile_read())
     ctx.close()
+
+
+def test_crossings_emitted_into_too_small_outputs():
+    """gs_iso_emit with a capacity below the count: the first crossings, nothing past them, GS_ECAPACITY by gs_sync."""
+    import ctypes
+    rng = np.random.default_rng(2)
+    vol = torch.from_numpy(rng.uniform(-1.0, 1.0, (33, 40, 70)).astype(np.float32)).cuda()
+    nz, ny, nx = vol.shape
+    ctx = gs.Context(0)
+    pts, nrm = ctx.gs_iso_crossings(vol, 0.1, (0.0, 0.0, 0.0), (1.0, 1.0, 1.0))
+    m = pts.shape[0]
+    work = torch.empty(ctx.L.gs_iso_workspace_bytes(nx, ny, nz), device="cuda", dtype=torch.uint8)
+    zero, one = (ctypes.c_float * 3)(0, 0, 0), (ctypes.c_float * 3)(1, 1, 1)
+    count = ctypes.c_int64()
+    v, w = ctypes.c_void_p(vol.data_ptr()), ctypes.c_void_p(work.data_ptr())
+    for cap in (0, 1, m // 2, m - 1, m):
+        p = torch.full((m, 3), float("nan"), device="cuda")
+        q = torch.full((m, 3), float("nan"), device="cuda")
+        assert ctx.L.gs_iso_count(ctx.h, v, nx, ny, nz, ctypes.c_float(0.1), w, ctypes.byref(count)) == gs.GS_OK
+        assert count.value == m
+        assert ctx.L.gs_iso_emit(ctx.h, v, nx, ny, nz, ctypes.c_float(0.1), zero, one, w, ctypes.c_void_p(p.data_ptr()),
+                                 ctypes.c_void_p(q.data_ptr()), cap) == gs.GS_OK
+        if cap < m:
+            with pytest.raises(gs.GsError):
+                ctx.gs_sync()
+        else:
+            ctx.gs_sync()
+        assert torch.equal(p[:cap], pts[:cap]) and torch.equal(q[:cap], nrm[:cap])
+        assert torch.isnan(p[cap:]).all() and torch.isnan(q[cap:]).all()
+    ctx.gs_sync()
+    ctx.close()
+
+
+def test_captured_step_of_many_tiles():
+    """The automatic variants and tile order of a batch of many tiles, captured, against the one-pixel kernels in bin
+    order call by call."""
+    scene = inputs.random_scene(20000, 1, 21, extent=0.9, log_scale=(-6.0, -3.0))
+    start = inputs.perturb(scene, 3)
+    cams = [inputs.pinhole(inputs.look_at((0.4 + v, -2.8, 1.0)), w, h)
+            for v, (w, h) in enumerate([(1511, 903), (640, 480)])]
+    n, deg = start["n"], start["deg"]
+    _, total = gs.image_offsets(cams)
+    plain = gs.Context(0)
+    for opt, val in ((gs.GS_OPT_RASTER_FWD, 1), (gs.GS_OPT_RASTER_BWD, 1), (gs.GS_OPT_TILE_ORDER, 0)):
+        plain.gs_set_option(opt, val)
+    _, target = run_forward(plain, scene, cams)
+    inst = plain.gs_get_counts()[0]
+    hp = dict(lr_mean=1e-3, lr_scale=5e-3, lr_quat=1e-3, lr_opacity=0.05, lr_sh_dc=2.5e-3, lr_sh_rest=1e-4)
+    p = torch.from_numpy(start["params"]).cuda()
+    g, m, v = (torch.zeros_like(p) for _ in range(3))
+    img, d, loss = torch.empty(total, device="cuda"), torch.empty(total, device="cuda"), torch.zeros(1, device="cuda")
+    ctx = gs.Context(0, instance_capacity=2 * inst + 65536)
+    ctx.gs_train_graph_capture(p, g, m, v, n, deg, hp, cams, target, img, d, loss)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    assert sum(((c["width"] + 15) // 16) * ((c["height"] + 15) // 16) for c in cams) >= 32 * sms
+    assert [ctx.gs_get_option(o) for o in (gs.GS_OPT_RASTER_FWD, gs.GS_OPT_RASTER_BWD, gs.GS_OPT_TILE_ORDER)] == [4, 8, 1]
+    ctx.gs_train_graph_launch(cams, target, 1)
+    ctx.gs_sync()
+    q, ref = run_forward(plain, start, cams)
+    assert (img - ref).abs().max().item() <= 1e-6
+    # (dL/dimage from the captured step's image, so that no sign of image - target differs)
+    grads = torch.full_like(q, float("nan"))
+    plain.gs_raster_bwd(q, n, deg, d, grads)
+    plain.gs_sync()
+    a, b = (t.cpu().numpy().astype(np.float64) for t in (g, grads))
+    assert rel_l2(a, b) <= 2e-5
+    assert torch.isfinite(p).all()
+    ctx.close()
+    plain.close()
