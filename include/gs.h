@@ -461,7 +461,10 @@ gs_status gs_train_graph_launch_host(gs_ctx* ctx, const gs_camera* cams, int32_t
  * bytes per resident Gaussian (stride), 20 bytes per pixel and 8 bytes per
  * 16x16 tile (max_view_pixels / 128 + 64 tiles) -- and the rest of its share
  * of the budget (memory_budget_bytes / slots, less 1 MiB) as room for tile
- * instances at 26 bytes each (at most 2^30 - 2).  Nothing is allocated or
+ * instances at 26 bytes each (at most 2^30 - 2).  Of the 26 the instance sort
+ * takes 17; the depth sort (17 bytes per resident Gaussian and view) and the
+ * tile order (4 bytes per tile) are reserved beside the account, and exceed it
+ * where the room for instances is short.  Nothing is allocated or
  * waited for while batches are launched.  A batch is admitted into a slot by
  * that room: each request is charged an instance estimate (1.25 x the most a
  * view of its pixel count has needed so far; for a size not seen yet, two

@@ -157,8 +157,8 @@ void launch_compact(const CompactArgs& a, cudaStream_t s) {
 constexpr int kRadixBits = 8;
 constexpr int kRadix = 1 << kRadixBits;
 constexpr int kSortThreads = 256;
-// keys per thread (12, 16, 20 or 24; a context option, autotuned): a
-// partition holds 256 x items keys
+// keys per thread: 12, 16, 20 or 24 (a context option, autotuned), 4 or 8 in
+// short segments (sort_items_for); a partition holds 256 x items keys
 constexpr int kSortWarps = kSortThreads / 32;
 constexpr uint32_t kFlagAggregate = 1u << 30;
 constexpr uint32_t kFlagPrefix = 2u << 30;

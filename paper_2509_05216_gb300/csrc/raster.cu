@@ -8,8 +8,8 @@
 // each pixel's last contributor towards the front, recovering T by division
 // and keeping the colour composited behind.
 //
-// Launch shapes, selected per context (GS_OPT_RASTER_FWD / _BWD) or, for the
-// backward, by the tile count: PPT = 1, 2, 4 or 8 pixels per thread.  Every warp
+// Launch shapes, by the batch's tile count or set per context
+// (GS_OPT_RASTER_FWD / _BWD): PPT = 1, 2, 4 or 8 pixels per thread.  Every warp
 // walks its tile's list independently (no block barriers).  It stages 32
 // records at a time, one per lane.  The kernels of 2 and 4 pixels (forward) and
 // 4 and 8 pixels (backward) walk by contribution cells of 2 x 4 pixels: each
@@ -836,9 +836,10 @@ __device__ __forceinline__ uint32_t transpose32(uint32_t x, int lane) {
 // exact ellipse test on top of it costs more than the walk steps it saves).
 //
 // Bound by issued instructions (1M Gaussians, 4 views of 1024^2: 76 % of the
-// issue slots, 6 % of the DRAM rate).  Measured, NP = 1 / 2: 16 views of 2048^2
-// of 4M Gaussians 4.07 / 3.97 ms, one of 3840 x 2160 0.63 / 0.70 ms (fewer,
-// longer warps leave a tail), 3 small views of 37,001 large ones 97 / 129 us.
+// issue slots, 6 % of the DRAM rate).  Measured in bin order, NP = 1 / 2: 16
+// views of 2048^2 of 4M Gaussians 4.07 / 3.97 ms, one of 3840 x 2160 0.63 / 0.70
+// ms (fewer, longer warps leave a tail, which the tile order removes: the rule at
+// the end of this file), 3 small views of 37,001 large ones 97 / 129 us.
 // Letting cells run ahead into a second staged batch, as
 // in the backward, costs this shorter step more than it saves (4.07 -> 4.4 ms
 // and more).
@@ -1372,6 +1373,12 @@ void launch_raster_fwd(const RasterArgs& a, int64_t bins, int ppt, cudaStream_t 
 // 10 to 18 us; one view of 1919 x 1081: 352 / 337 / 311 us and 359 / 326 us).
 // Below, bin order, 2 pixels forward and 4 backward (256 tiles: 47 us against 58
 // with 8; 1,049 tiles of large splats: 137 to 150 us against 161, and 147 with 2).
+// Around the line (one view of 4M Gaussians; projection, binning and forward
+// with 2 pixels in bin order / 4 in list order, then gs_raster_bwd with 4 in bin /
+// 8 in list order): 2,560 tiles 1243 / 1350 and 725 / 804 us; 4,000 tiles 1149 / 1204 and 616 /
+// 679; 4,992 tiles 978 / 992 and 578 / 623; 8,160 tiles 994 / 919 and 607 / 575;
+// 14,400 tiles 1030 / 962 and 664 / 606; 32,400 tiles 1212 / 1149 and 840 / 739;
+// from close by, 4,992 tiles 827 / 777 and 508 / 467.
 static bool many_tiles(int64_t bins) { return bins >= (int64_t)32 * sm_count(); }
 bool tile_order_auto(int64_t bins) { return many_tiles(bins); }
 int raster_fwd_auto(int64_t bins) { return many_tiles(bins) ? 4 : 2; }

@@ -43,8 +43,10 @@ constexpr int kMaxRetries = 4;      // capacity retries of one request
 constexpr int32_t kDefaultViewPixels = 3840 * 2160;
 // reservation per slot (documented with gs_serve_cfg): per view 72 bytes per
 // Gaussian (records, tile rect, tile count), 20 bytes per pixel (T_final,
-// n_last, batch image) and 8 per tile (ranges); 26 bytes per tile instance
-// (keys and values double-buffered, sort look-back)
+// n_last, batch image) and 8 per tile (ranges); 26 bytes per tile instance.  An
+// instance takes 17 (keys and values double-buffered, sort look-back); the other
+// 9 are what the account has for the depth sort's pairs (17 bytes per Gaussian
+// and view) and the tile order (4 per tile), which are reserved beside it
 constexpr int64_t kGaussBytes = 72, kPixelBytes = 20, kTileBytes = 8, kInstanceBytes = 26;
 constexpr int64_t kSlackBytes = 1 << 20;
 constexpr int64_t kMaxInstances = ((int64_t)1 << 30) - 2;
