@@ -175,6 +175,30 @@ void drop_graph(gs_ctx* c) {
   c->graph_bufs.clear();
 }
 
+// Room for an allocation of `want` bytes that failed, from what a captured step
+// keeps beside the current workspaces, if that can be enough: the spares first,
+// then the step itself (GS_ESTATE until the next capture).  false: nothing freed.
+bool make_room(gs_ctx* c, size_t want) {
+  if (!c->gexec || c->capturing) return false;
+  size_t spare = 0, held = 0, free_bytes = 0, total = 0;
+  for (const GraphBuf& g : c->graph_bufs) {
+    spare += g.spare.cap;
+    held += g.buf->p != g.own.p ? g.own.cap : 0;
+  }
+  if (cudaMemGetInfo(&free_bytes, &total) != cudaSuccess || spare + held == 0 || free_bytes + spare + held < want)
+    return false;
+  if (spare == 0) {
+    drop_graph(c);
+    return true;
+  }
+  cudaStreamSynchronize(c->stream);
+  for (GraphBuf& g : c->graph_bufs) {
+    if (g.spare.p) cudaFree(g.spare.p);
+    g.spare = DevBuf{};
+  }
+  return true;
+}
+
 gs_status ensure(gs_ctx* c, DevBuf& b, size_t bytes, bool exact = false) {
   if (bytes == 0) bytes = 16;
   if (b.cap >= bytes) return GS_OK;
@@ -198,10 +222,9 @@ gs_status ensure(gs_ctx* c, DevBuf& b, size_t bytes, bool exact = false) {
     b = DevBuf{};
   }
   cudaError_t e = cudaMalloc(&b.p, want);
-  if (e != cudaSuccess && c->gexec && !c->capturing) {
-    // rather the new batch than the captured step (GS_ESTATE until the next capture)
+  while (e != cudaSuccess) {
     (void)cudaGetLastError();
-    drop_graph(c);
+    if (!make_room(c, want)) break;
     e = cudaMalloc(&b.p, want);
   }
   if (e != cudaSuccess) {

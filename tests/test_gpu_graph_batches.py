@@ -101,3 +101,31 @@ def test_a_larger_set_is_captured_anew():
     assert torch.isfinite(st.p).all() and loss.item() <= 0.2
     ctx.close()
     plain.close()
+
+
+def test_an_impossible_request_leaves_the_graph():
+    """A workspace that no memory could hold is refused (GS_ENOMEM), and the captured step goes on."""
+    ref, cur, cams = setup()
+    n, deg = cur["n"], cur["deg"]
+    plain = gs.Context(0)
+    targets = render(plain, ref, cams)
+    inst, _, _ = plain.gs_get_counts()
+    _, total = gs.image_offsets(cams)
+    images = []
+    for disturbed in (False, True):
+        st = State(cur)
+        img, d, loss = torch.empty(total, device="cuda"), torch.empty(total, device="cuda"), torch.zeros(1, device="cuda")
+        ctx = gs.Context(0, instance_capacity=2 * inst + 1024)
+        ctx.gs_train_graph_capture(st.p, st.g, st.m, st.v, n, deg, HP, cams, targets, img, d, loss)
+        if disturbed:
+            # 64 views of 65,536^2 projected (no pixel buffer is touched); the image loss's partials would take 9 TB
+            huge = [inputs.pinhole(inputs.look_at((0.4, -2.8, 1.0)), 65536, 65536)] * 64
+            ctx.gs_project(torch.from_numpy(ref["params"]).cuda(), n, deg, huge)
+            with pytest.raises(gs.GsError, match="cudaMalloc"):
+                ctx.gs_ssim_loss(img, targets, 0.2, loss, d)
+        ctx.gs_train_graph_launch(cams, targets, 1)
+        ctx.gs_sync()
+        images.append(img.clone())
+        ctx.close()
+    assert torch.equal(images[0], images[1])
+    plain.close()
