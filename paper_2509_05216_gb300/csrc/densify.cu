@@ -9,10 +9,11 @@
 // of its own distribution (scales shrunk by 0.8 N) when large; Gaussians
 // whose opacity is below the minimum are removed.  New Gaussians start with
 // zero Adam moments.  The output keeps the input order, a Gaussian's outputs
-// together: a counting pass (outputs per block of 1,024 Gaussians), the
+// together: a counting pass (outputs per block of 256 or 1,024 Gaussians), the
 // binning's block-sum scan, a pass that writes the source of every output
 // (and the means of the split samples), and a copy of every plane that
 // gathers by source and writes whole coalesced lines.
+#include <algorithm>
 #include <cmath>
 
 #include "gs_internal.cuh"
@@ -60,22 +61,29 @@ __device__ __forceinline__ uint32_t block_prefix(uint32_t c, uint32_t* warp_tot,
 
 }  // namespace
 
-constexpr int kDensifyItems = 4;  // Gaussians per thread of the counting and source passes
-constexpr int kDensifyBlock = 256 * kDensifyItems;
+// Gaussians per thread of the counting and source passes: 4, or 1 below 5 blocks
+// of 1,024 per SM (a thread's splits are a chain).  Whole call, 1 / 4 per thread:
+// 5,000 Gaussians of degree 0 51 / 63 us, 160,000 of degree 3 92 / 98, 700,000 231 /
+// 235, 1M 313 / 305, 4M 1120 / 1080.
+constexpr int kDensifyMany = 4, kDensifyFew = 1;
+static int densify_items(int64_t n) {
+  return n >= (int64_t)5 * 256 * kDensifyMany * sm_count() ? kDensifyMany : kDensifyFew;
+}
 // Source word of an output: its input Gaussian (n below 2^31), and the top
 // bit when its moments start at zero.  A clone's copy follows its original,
 // whose word is the bare Gaussian; a fresh output that does not is a split
 // sample.
 constexpr uint32_t kSrcFresh = 1u << 31;
 
-// Thread t takes Gaussians 4 t .. 4 t + 3 of the block's 1,024, so that one
-// block scan of the threads' sums keeps the input order.
+// Thread t takes ITEMS consecutive Gaussians of the block's 256 ITEMS, so that
+// one block scan of the threads' sums keeps the input order.
+template <int ITEMS>
 __global__ void __launch_bounds__(256) densify_count_kernel(DensifyArgs a) {
   __shared__ uint32_t warp_tot[8];
   uint32_t c = 0;
 #pragma unroll
-  for (int i = 0; i < kDensifyItems; i++) {
-    const int64_t g = (int64_t)blockIdx.x * kDensifyBlock + threadIdx.x * kDensifyItems + i;
+  for (int i = 0; i < ITEMS; i++) {
+    const int64_t g = (int64_t)blockIdx.x * (256 * ITEMS) + threadIdx.x * ITEMS + i;
     if (g < a.n) c += (uint32_t)outputs(decide(a, g), a.split_n);
   }
   uint32_t tot;
@@ -83,13 +91,14 @@ __global__ void __launch_bounds__(256) densify_count_kernel(DensifyArgs a) {
   if (threadIdx.x == 0) a.block_counts[blockIdx.x] = tot;
 }
 
+template <int ITEMS>
 __global__ void __launch_bounds__(256) densify_source_kernel(DensifyArgs a) {
   __shared__ uint32_t warp_tot[8];
-  const int64_t g0 = (int64_t)blockIdx.x * kDensifyBlock + threadIdx.x * kDensifyItems;
-  int kind[kDensifyItems];
+  const int64_t g0 = (int64_t)blockIdx.x * (256 * ITEMS) + threadIdx.x * ITEMS;
+  int kind[ITEMS];
   uint32_t c = 0;
 #pragma unroll
-  for (int i = 0; i < kDensifyItems; i++) {
+  for (int i = 0; i < ITEMS; i++) {
     kind[i] = g0 + i < a.n ? decide(a, g0 + i) : kPrune;
     c += (uint32_t)outputs(kind[i], a.split_n);
   }
@@ -98,7 +107,7 @@ __global__ void __launch_bounds__(256) densify_source_kernel(DensifyArgs a) {
   o += a.block_offsets[blockIdx.x];
   const int64_t S = a.stride, OS = a.out_stride;
 #pragma unroll
-  for (int i = 0; i < kDensifyItems; i++) {
+  for (int i = 0; i < ITEMS; i++) {
     const int64_t g = g0 + i;
     if (kind[i] == kKeep || kind[i] == kClone) {
       a.source[o++] = (uint32_t)g;
@@ -169,18 +178,28 @@ __global__ void __launch_bounds__(256) densify_copy_kernel(DensifyArgs a, int64_
   }
 }
 
-int64_t densify_blocks(int64_t n) { return (n + kDensifyBlock - 1) / kDensifyBlock; }
+int64_t densify_blocks(int64_t n) {
+  const int block = 256 * densify_items(n);
+  return (n + block - 1) / block;
+}
 
 void launch_densify_count(const DensifyArgs& a, cudaStream_t s) {
-  densify_count_kernel<<<(unsigned)densify_blocks(a.n), 256, 0, s>>>(a);
+  const unsigned blocks = (unsigned)densify_blocks(a.n);
+  if (densify_items(a.n) == kDensifyMany) densify_count_kernel<kDensifyMany><<<blocks, 256, 0, s>>>(a);
+  else densify_count_kernel<kDensifyFew><<<blocks, 256, 0, s>>>(a);
 }
 
 void launch_densify_emit(const DensifyArgs& a, int64_t n_out, cudaStream_t s) {
   if (n_out <= 0) return;
-  densify_source_kernel<<<(unsigned)densify_blocks(a.n), 256, 0, s>>>(a);
-  constexpr int kPlanes = 15;  // planes per block: a quarter of degree 3's 59
-  densify_copy_kernel<<<dim3((unsigned)((n_out + 1023) / 1024), (a.planes + kPlanes - 1) / kPlanes), 256, 0, s>>>(
-      a, n_out, kPlanes);
+  const unsigned in_blocks = (unsigned)densify_blocks(a.n);
+  if (densify_items(a.n) == kDensifyMany) densify_source_kernel<kDensifyMany><<<in_blocks, 256, 0, s>>>(a);
+  else densify_source_kernel<kDensifyFew><<<in_blocks, 256, 0, s>>>(a);
+  // planes per block: a quarter of degree 3's 59, fewer where that leaves less
+  // than 4 blocks per SM (a block's planes are a chain of load latencies: 5,000
+  // Gaussians, whole call, 63 us with 15 planes, 55 with 1)
+  const int64_t blocks = (n_out + 1023) / 1024;
+  const int planes = (int)std::clamp<int64_t>(a.planes * blocks / ((int64_t)sm_count() * 4), 1, 15);
+  densify_copy_kernel<<<dim3((unsigned)blocks, (a.planes + planes - 1) / planes), 256, 0, s>>>(a, n_out, planes);
 }
 
 }  // namespace gs
