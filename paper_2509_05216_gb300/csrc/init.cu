@@ -47,8 +47,12 @@ __device__ __forceinline__ float3 vol_grad(const IsoArgs& a, int x, int y, int z
 }
 
 constexpr int kIsoThreads = 256;
-constexpr int kIsoWords = 4;                           // words per thread of the counting and emitting passes
-constexpr int kIsoBlockWords = kIsoThreads * kIsoWords;  // 32,768 vertices per block
+// Words per block of the counting and emitting passes: 1,024 (32,768 vertices), or
+// 64 below 256 blocks of those, whose threads would take a block's crossings in a
+// long chain of rounds.  Whole call with 64 / 1,024: 33^3 75 / 122 us, 33 x 512 x 40 74 / 121, 128^3
+// 72 / 96, 200^3 90 / 92, 256^3 110 / 99, 512^3 491 / 245.
+constexpr int kIsoMany = 1024, kIsoFew = 64;
+constexpr int64_t kIsoFewBelow = 256 * kIsoMany;
 
 // Exclusive prefix of `c` over the block (256 threads); *total = block sum.
 __device__ __forceinline__ uint32_t block_excl_scan(uint32_t c, uint32_t* warp_tot, uint32_t* total) {
@@ -146,13 +150,14 @@ __global__ void __launch_bounds__(256) iso_sides_kernel(IsoArgs a) {
   if (w0 + lane < a.nwords) a.sides[w0 + lane] = mine;
 }
 
-// Crossings per block of 1,024 words, from the side bits alone.
+// Crossings per block of WORDS words, from the side bits alone.
+template <int WORDS>
 __global__ void __launch_bounds__(kIsoThreads) iso_count_kernel(IsoArgs a) {
   __shared__ uint32_t warp_tot[kIsoThreads / 32];
   uint32_t c = 0;
 #pragma unroll
-  for (int i = 0; i < kIsoWords; i++) {
-    const int64_t w = (int64_t)blockIdx.x * kIsoBlockWords + i * kIsoThreads + threadIdx.x;
+  for (int k = threadIdx.x; k < WORDS; k += kIsoThreads) {
+    const int64_t w = (int64_t)blockIdx.x * WORDS + k;
     if (w < a.nwords) {
       uint32_t ex, ey, ez;
       crossing_masks(a, w, ex, ey, ez);
@@ -169,28 +174,32 @@ __global__ void __launch_bounds__(kIsoThreads) iso_count_kernel(IsoArgs a) {
 // memory and its threads take the crossings one by one: crossing o finds its
 // word by bisection over the first crossings and its vertex by bisection
 // over the word's bits, so that no lane waits for words without crossings.
+template <int WORDS>
 __global__ void __launch_bounds__(kIsoThreads) iso_emit_kernel(IsoArgs a) {
+  constexpr int kItems = WORDS > kIsoThreads ? WORDS / kIsoThreads : 1;  // words per thread (of the first WORDS threads)
   __shared__ uint32_t warp_tot[kIsoThreads / 32];
-  __shared__ uint32_t s_first[kIsoBlockWords];
-  __shared__ uint32_t s_mask[3][kIsoBlockWords];
-  const int64_t word0 = (int64_t)blockIdx.x * kIsoBlockWords;
-  uint32_t c[kIsoWords], sum = 0;
+  __shared__ uint32_t s_first[WORDS];
+  __shared__ uint32_t s_mask[3][WORDS];
+  const int64_t word0 = (int64_t)blockIdx.x * WORDS;
+  uint32_t c[kItems], sum = 0;
 #pragma unroll
-  for (int i = 0; i < kIsoWords; i++) {
-    const int k = threadIdx.x * kIsoWords + i;
+  for (int i = 0; i < kItems; i++) {
+    const int k = threadIdx.x * kItems + i;
     uint32_t ex = 0, ey = 0, ez = 0;
-    if (word0 + k < a.nwords) crossing_masks(a, word0 + k, ex, ey, ez);
-    s_mask[0][k] = ex;
-    s_mask[1][k] = ey;
-    s_mask[2][k] = ez;
+    if (k < WORDS && word0 + k < a.nwords) crossing_masks(a, word0 + k, ex, ey, ez);
+    if (k < WORDS) {
+      s_mask[0][k] = ex;
+      s_mask[1][k] = ey;
+      s_mask[2][k] = ez;
+    }
     c[i] = __popc(ex) + __popc(ey) + __popc(ez);
     sum += c[i];
   }
   uint32_t total;
   uint32_t run = block_excl_scan(sum, warp_tot, &total);
 #pragma unroll
-  for (int i = 0; i < kIsoWords; i++) {
-    s_first[threadIdx.x * kIsoWords + i] = run;
+  for (int i = 0; i < kItems; i++) {
+    if (threadIdx.x * kItems + i < WORDS) s_first[threadIdx.x * kItems + i] = run;
     run += c[i];
   }
   __syncthreads();
@@ -201,7 +210,7 @@ __global__ void __launch_bounds__(kIsoThreads) iso_emit_kernel(IsoArgs a) {
     // crossings share their successor's first crossing and are passed over)
     int k = 0;
 #pragma unroll
-    for (int step = kIsoBlockWords / 2; step > 0; step >>= 1)
+    for (int step = WORDS / 2; step > 0; step >>= 1)
       if (s_first[k + step] <= q) k += step;
     const uint32_t ex = s_mask[0][k], ey = s_mask[1][k], ez = s_mask[2][k];
     uint32_t r = q - s_first[k];
@@ -251,16 +260,24 @@ __global__ void __launch_bounds__(kIsoThreads) iso_emit_kernel(IsoArgs a) {
 }
 
 int64_t iso_words(int64_t nverts) { return (nverts + 31) / 32; }
-int64_t iso_blocks(int64_t nverts) { return (iso_words(nverts) + kIsoBlockWords - 1) / kIsoBlockWords; }
+static int iso_block_words(int64_t nverts) { return iso_words(nverts) < kIsoFewBelow ? kIsoFew : kIsoMany; }
+int64_t iso_blocks(int64_t nverts) {
+  const int words = iso_block_words(nverts);
+  return (iso_words(nverts) + words - 1) / words;
+}
 
 void launch_iso_count(const IsoArgs& a, cudaStream_t s) {
   const int64_t warps = (a.nwords + 31) / 32;
   iso_sides_kernel<<<(unsigned)((warps + 7) / 8), 256, 0, s>>>(a);
-  iso_count_kernel<<<(unsigned)iso_blocks(a.nverts), kIsoThreads, 0, s>>>(a);
+  const unsigned blocks = (unsigned)iso_blocks(a.nverts);
+  if (iso_block_words(a.nverts) == kIsoMany) iso_count_kernel<kIsoMany><<<blocks, kIsoThreads, 0, s>>>(a);
+  else iso_count_kernel<kIsoFew><<<blocks, kIsoThreads, 0, s>>>(a);
 }
 
 void launch_iso_emit(const IsoArgs& a, cudaStream_t s) {
-  iso_emit_kernel<<<(unsigned)iso_blocks(a.nverts), kIsoThreads, 0, s>>>(a);
+  const unsigned blocks = (unsigned)iso_blocks(a.nverts);
+  if (iso_block_words(a.nverts) == kIsoMany) iso_emit_kernel<kIsoMany><<<blocks, kIsoThreads, 0, s>>>(a);
+  else iso_emit_kernel<kIsoFew><<<blocks, kIsoThreads, 0, s>>>(a);
 }
 
 // ---------------------------------------------------------------- k nearest neighbours

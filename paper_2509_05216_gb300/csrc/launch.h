@@ -231,7 +231,7 @@ struct IsoArgs {
   float iso;
   float origin[3], h[3];
   uint32_t* sides;                // [nwords] bit b of word w: sample 32 w + b >= iso
-  uint32_t* block_counts;         // [iso_blocks] crossings per block of 1,024 words
+  uint32_t* block_counts;         // [iso_blocks] crossings per block of words
   const uint32_t* block_offsets;  // emit pass: exclusive scan of block_counts
   float* points;                  // [capacity][3]
   float* normals;                 // [capacity][3]
