@@ -211,6 +211,7 @@ struct SsimArgs {
   float* partials;         // per pixel dSSIM/d(mx), dSSIM/dE[x^2]: [count][2], then dSSIM/dE[xy]: [count]
   int rows;                // rows per strip (ssim_strip_rows)
   double* block_sums;      // [strips][3]: sums of the SSIM map, |x - y|, (x - y)^2
+  uint32_t* ticket;        // device word, 0 between launches
   float* grad;             // dL/dx (backward)
   float2 win[11];          // normalised Gaussian window (sigma 1.5), each weight twice
   float w_l1, w_ssim, inv_count;

@@ -77,3 +77,31 @@ def test_ssim_map_is_the_ieee_quotient(scale):
         got, _ = ctx.gs_image_metrics(dx, dy, views)
         assert np.all(np.abs(np.array(got) - ref) <= np.spacing(np.abs(ref)) * (1 + 1e-6))
     ctx.close()
+
+
+# every number of rows per strip (4 to 128, by the batch's pixels) and both block sizes, with ragged last strips
+@pytest.mark.parametrize("sizes", [[(61, 67)], [(301, 299)], [(515, 511)], [(701, 763)], [(1027, 1001)], [(1919, 1081)],
+                                   [(1451, 1449), (1453, 1447)], [(97, 131)] * 5 + [(300, 20)]])
+def test_strips_of_every_length(sizes):
+    cams = [inputs.pinhole(inputs.look_at((0.4, -2.8, 1.0)), w, h) for w, h in sizes]
+    scene = inputs.random_scene(64, 0, 3, extent=0.5)
+    ctx = gs.Context(0)
+    ctx.gs_project(torch.from_numpy(scene["params"]).cuda(), scene["n"], scene["deg"], cams)
+    rng = np.random.default_rng(sizes[0][0])
+    xs = [rng.uniform(0, 1, (3, h, w)).astype(np.float32) for w, h in sizes]
+    ys = [np.clip(x + rng.normal(0, 0.1, x.shape), 0, 1).astype(np.float32) for x in xs]
+    x, y = (torch.from_numpy(np.concatenate([a.reshape(-1) for a in v])).cuda() for v in (xs, ys))
+    loss, grad = torch.zeros(1, device="cuda"), torch.full_like(x, float("nan"))
+    for _ in range(2):  # (the second call finds the first one's state)
+        ctx.gs_ssim_loss(x, y, 0.2, loss, grad)
+    ctx.gs_sync()
+    ref, ref_grads = OS.dssim_loss(xs, ys, 0.2)
+    # the tolerances of the strips' small batches: FP32 window sums, means over thousands of pixels
+    assert abs(loss.item() - ref) <= 1e-6
+    for g, r in zip(gs.split_images(grad, cams), ref_grads):
+        g = g.cpu().numpy().astype(np.float64)
+        assert np.linalg.norm(g - r) <= 1e-5 * np.linalg.norm(r)
+    ssim, psnr = ctx.gs_image_metrics(x, y, len(cams))
+    for v in range(len(cams)):
+        assert abs(ssim[v] - OS.ssim(xs[v], ys[v])) <= 2e-6 and abs(psnr[v] - OS.psnr(xs[v], ys[v])) <= 1e-4
+    ctx.close()
