@@ -872,7 +872,9 @@ static int fwd_variant(const gs_ctx* c) {
 static int order_mode(const gs_ctx* c) {
   return c->tile_order_mode != GS_OPT_AUTO ? c->tile_order_mode : (tile_order_auto(c->bins) ? 1 : 0);
 }
-static int bwd_variant(const gs_ctx* c) { return c->raster_bwd != GS_OPT_AUTO ? c->raster_bwd : raster_bwd_auto(c->bins); }
+static int bwd_variant(const gs_ctx* c) {
+  return c->raster_bwd != GS_OPT_AUTO ? c->raster_bwd : raster_bwd_auto(c->bins, (int64_t)c->B * c->n);
+}
 
 static RasterArgs raster_args(gs_ctx* c) {
   RasterArgs r{};

@@ -1364,7 +1364,7 @@ void launch_raster_fwd(const RasterArgs& a, int64_t bins, int ppt, cudaStream_t 
   }
 }
 
-// The variants when the caller has chosen none.  From the tile count at which
+// The variants when the caller has chosen none (GS_OPT_AUTO).  From the tile count at which
 // one warp per tile fills every SM's 14 to 16 resident warps twice over, tiles
 // are taken longest lists first, 4 pixels per thread forward and 8 backward: few
 // long-lived warps per tile leave a tail that the order removes (16 views of
@@ -1382,7 +1382,23 @@ void launch_raster_fwd(const RasterArgs& a, int64_t bins, int ppt, cudaStream_t 
 static bool many_tiles(int64_t bins) { return bins >= (int64_t)32 * sm_count(); }
 bool tile_order_auto(int64_t bins) { return many_tiles(bins); }
 int raster_fwd_auto(int64_t bins) { return many_tiles(bins) ? 4 : 2; }
-int raster_bwd_auto(int64_t bins) { return many_tiles(bins) ? 8 : 4; }
+
+// Backward of a few tiles with long lists: their chains are the time, and more
+// warps per tile, each with the entries of fewer pixels, shorten them.  Up to a
+// tile per SM, 1 pixel per thread (8 warps per tile); up to 4 tiles per SM, 2
+// pixels, or 1 where the lists are very long; both from 160 (view, Gaussian) pairs
+// per tile.  gs_raster_bwd with 1 / 2 / 4 pixels: 64 tiles and 625 pairs per tile 145 / 149 /
+// 183 us; 123 and 325 187 / 189 / 242; 330 and 182 184 / 182 / 208; 475 and 421 200 / 202 / 237;
+// 256 and 3,125 350 / 431 / 499; on the other side 256 and 39 77 / 77 / 63; 427 and 94 163 / 164 / 168; 1,000 and 40
+// 124 / 101 / 71; 800 and 1,250 438 / 471 / 482.  (Over 280 batches of 16 to 1,280 tiles
+// it takes 2 % more than the best of the three, always 4 pixels 5 %; batches whose
+// pixels stop early lose up to a quarter by it.)
+int raster_bwd_auto(int64_t bins, int64_t pairs) {
+  if (many_tiles(bins)) return 8;
+  const int64_t sms = sm_count();
+  if (bins > 4 * sms || pairs < 160 * bins) return 4;
+  return bins <= sms || pairs >= 1024 * bins ? 1 : 2;
+}
 
 bool raster_bwd_flags(int ppt) { return ppt == 4 || ppt == 8; }
 

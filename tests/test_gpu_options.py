@@ -39,3 +39,25 @@ def test_automatic_options_come_back():
     with pytest.raises(gs.GsError):
         ctx.gs_set_option(gs.GS_OPT_TILE_ORDER, -2)
     ctx.close()
+
+
+# (tiles per SM, pairs per tile) on both sides of the lines between the backward kernels; 152 SMs
+@pytest.mark.parametrize("w,h,n,kernel", [(192, 192, 23039, 4), (192, 192, 23040, 1), (208, 192, 25000, 2), (208, 192, 160000, 1),
+                                          (608, 256, 98000, 2), (624, 256, 110000, 4), (2048, 2048, 30000, 8)])
+def test_backward_kernel_by_tiles_and_pairs(w, h, n, kernel):
+    scene = inputs.random_scene(n, 0, 4, extent=0.8, log_scale=(-6.0, -5.0))
+    cams = [inputs.pinhole(inputs.look_at((0.4, -2.8, 1.0)), w, h)]
+    ctx = gs.Context(0)
+    p, img = run_forward(ctx, scene, cams)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    if sms == 152:
+        assert ctx.gs_get_option(gs.GS_OPT_RASTER_BWD) == kernel
+    dimg = torch.randn(img.shape, generator=torch.Generator(device="cuda").manual_seed(1), device="cuda")
+    grads = [torch.full_like(p, float("nan")) for _ in range(2)]
+    ctx.gs_raster_bwd(p, n, 0, dimg, grads[0])
+    ctx.gs_set_option(gs.GS_OPT_RASTER_BWD, 4)
+    ctx.gs_raster_bwd(p, n, 0, dimg, grads[1])
+    ctx.gs_sync()
+    a, b = (g[:, :n].double() for g in grads)
+    assert torch.isfinite(a).all() and ((a - b).norm() / b.norm()).item() <= 2e-5
+    ctx.close()
