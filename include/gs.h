@@ -140,8 +140,7 @@ typedef enum {
                             tile.  All variants give the same result up to
                             FP32 rounding.  GS_OPT_AUTO (default, as of the
                             next one and GS_OPT_TILE_ORDER): by each batch's
-                            tile count (the backward's also by its (view,
-                            Gaussian) pairs). */
+                            tiles and (view, Gaussian) pairs. */
   GS_OPT_RASTER_BWD = 1, /* backward compositing kernel, same values */
   GS_OPT_BWD_DIRECT = 2, /* backward with 1 or 2 pixels per thread: a warp whose
                             pixels meet a Gaussian in at most this many lanes

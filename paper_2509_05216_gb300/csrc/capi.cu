@@ -867,7 +867,7 @@ static gs_status sort_tiles_longest_first(gs_ctx* c) {
 // longer warps of 4 pixels per thread: a burst of 12 requests 3.64 against 3.38
 // ms with 2.)
 static int fwd_variant(const gs_ctx* c) {
-  return c->raster_fwd != GS_OPT_AUTO ? c->raster_fwd : c->forward_only ? 2 : raster_fwd_auto(c->bins);
+  return c->raster_fwd != GS_OPT_AUTO ? c->raster_fwd : c->forward_only ? 2 : raster_fwd_auto(c->bins, (int64_t)c->B * c->n);
 }
 static int order_mode(const gs_ctx* c) {
   return c->tile_order_mode != GS_OPT_AUTO ? c->tile_order_mode : (tile_order_auto(c->bins) ? 1 : 0);

@@ -191,7 +191,7 @@ void launch_l1_finish(const float* partial, int64_t nparts, double* scratch, dou
 void launch_raster_bwd(const RasterArgs& a, int64_t bins, int ppt, cudaStream_t s);
 bool raster_bwd_flags(int ppt);
 int raster_bwd_auto(int64_t bins, int64_t pairs);
-int raster_fwd_auto(int64_t bins);
+int raster_fwd_auto(int64_t bins, int64_t pairs);
 bool tile_order_auto(int64_t bins);
 // out[0] += list entries up to each pixel's last contributor, out[1] += contributing pairs
 void launch_pair_stats(const RasterArgs& a, int64_t bins, unsigned long long* out, cudaStream_t s);

@@ -1379,9 +1379,17 @@ void launch_raster_fwd(const RasterArgs& a, int64_t bins, int ppt, cudaStream_t 
 // 679; 4,992 tiles 978 / 992 and 578 / 623; 8,160 tiles 994 / 919 and 607 / 575;
 // 14,400 tiles 1030 / 962 and 664 / 606; 32,400 tiles 1212 / 1149 and 840 / 739;
 // from close by, 4,992 tiles 827 / 777 and 508 / 467.
+//
+// Many tiles with 512 (view, Gaussian) pairs each or more are mostly empty ones
+// around a few with long lists: those keep 2 pixels forward and 4 backward, in
+// list order.  Forward, then gs_raster_bwd, with 2 and 4 / 4 and 8 pixels: 4M Gaussians,
+// 8 views of 236 x 1625 6.50 / 6.82 and 3.71 / 4.57 ms; 2M, 8 views of 512^2 1010 / 1112
+// and 1035 / 1224 us; 1M, 16 of 400^2 1237 / 1407 and 1179 / 1359; on a surface that fills
+// the view, 6M, one of 1300 x 1000 264 / 255 and 693 / 672.
 static bool many_tiles(int64_t bins) { return bins >= (int64_t)32 * sm_count(); }
+static bool long_lists(int64_t bins, int64_t pairs) { return pairs >= 512 * bins; }
 bool tile_order_auto(int64_t bins) { return many_tiles(bins); }
-int raster_fwd_auto(int64_t bins) { return many_tiles(bins) ? 4 : 2; }
+int raster_fwd_auto(int64_t bins, int64_t pairs) { return many_tiles(bins) && !long_lists(bins, pairs) ? 4 : 2; }
 
 // Backward of a few tiles with long lists: their chains are the time, and more
 // warps per tile, each with the entries of fewer pixels, shorten them.  Up to a
@@ -1394,7 +1402,7 @@ int raster_fwd_auto(int64_t bins) { return many_tiles(bins) ? 4 : 2; }
 // it takes 2 % more than the best of the three, always 4 pixels 5 %; batches whose
 // pixels stop early lose up to a quarter by it.)
 int raster_bwd_auto(int64_t bins, int64_t pairs) {
-  if (many_tiles(bins)) return 8;
+  if (many_tiles(bins)) return long_lists(bins, pairs) ? 4 : 8;
   const int64_t sms = sm_count();
   if (bins > 4 * sms || pairs < 160 * bins) return 4;
   return bins <= sms || pairs >= 1024 * bins ? 1 : 2;

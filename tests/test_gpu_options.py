@@ -1,5 +1,7 @@
 """Options that follow the batch until set, and again once set to automatic
 (GPU only)."""
+import math
+
 import pytest
 import torch
 
@@ -39,6 +41,22 @@ def test_automatic_options_come_back():
     with pytest.raises(gs.GsError):
         ctx.gs_set_option(gs.GS_OPT_TILE_ORDER, -2)
     ctx.close()
+
+
+def test_many_tiles_of_long_lists():
+    """Many tiles with 512 pairs each or more: list order, but the kernels of fewer pixels per thread."""
+    cams = [inputs.pinhole(inputs.look_at((2.8 * math.cos(0.2 * v), 2.8 * math.sin(0.2 * v), 0.5)), 208, 192) for v in range(32)]
+    for n, kernels in ((79000, (4, 8, 1)), (81000, (2, 4, 1))):  # 32 n / 4,992 tiles: 506 and 519
+        scene = inputs.random_scene(n, 0, 4, extent=0.8, log_scale=(-6.0, -5.0))
+        ctx = gs.Context(0)
+        _, img = run_forward(ctx, scene, cams)
+        got = tuple(ctx.gs_get_option(o) for o in AUTOMATIC)
+        if torch.cuda.get_device_properties(0).multi_processor_count == 152:
+            assert got == kernels
+        for opt, value in zip(AUTOMATIC, (1, 1, 0)):
+            ctx.gs_set_option(opt, value)
+        assert (run_forward(ctx, scene, cams)[1] - img).abs().max().item() <= 1e-6
+        ctx.close()
 
 
 # (tiles per SM, pairs per tile) on both sides of the lines between the backward kernels; 152 SMs
