@@ -31,6 +31,7 @@ struct DevBuf {
 struct BatchState {
   int B = 0, deg = 0;
   int64_t n = 0, stride = 0, bins = 0, pixels = 0, nblocks = 0;
+  int64_t filled = 0;       // tiles that the scene may fill: those within about 49 degrees of the axis in x and y
   int sort_passes = 0;      // LSD passes of the tile sort
   uint2* ranges = nullptr;  // tile ranges (in `zeroed`)
   bool tile_order_ready = false;
@@ -645,6 +646,11 @@ gs_status gs_project(gs_ctx* c, const gs_params* params, const gs_camera* cams, 
   c->stride = stride;
   c->deg = params->sh_degree;
   c->bins = tile_off;
+  c->filled = 0;
+  for (const ViewRec& r : c->views_h) {
+    const double w = std::min((double)r.W, 2.3 * r.fx), h = std::min((double)r.H, 2.3 * r.fy);
+    c->filled += std::max<int64_t>(1, (int64_t)std::ceil(w / kTile) * (int64_t)std::ceil(h / kTile));
+  }
   c->pixels = pix_off;
   c->nblocks = nb;
   c->projected = true;
@@ -867,13 +873,13 @@ static gs_status sort_tiles_longest_first(gs_ctx* c) {
 // longer warps of 4 pixels per thread: a burst of 12 requests 3.64 against 3.38
 // ms with 2.)
 static int fwd_variant(const gs_ctx* c) {
-  return c->raster_fwd != GS_OPT_AUTO ? c->raster_fwd : c->forward_only ? 2 : raster_fwd_auto(c->bins, (int64_t)c->B * c->n);
+  return c->raster_fwd != GS_OPT_AUTO ? c->raster_fwd : c->forward_only ? 2 : raster_fwd_auto(c->filled, (int64_t)c->B * c->n);
 }
 static int order_mode(const gs_ctx* c) {
-  return c->tile_order_mode != GS_OPT_AUTO ? c->tile_order_mode : (tile_order_auto(c->bins) ? 1 : 0);
+  return c->tile_order_mode != GS_OPT_AUTO ? c->tile_order_mode : (tile_order_auto(c->filled) ? 1 : 0);
 }
 static int bwd_variant(const gs_ctx* c) {
-  return c->raster_bwd != GS_OPT_AUTO ? c->raster_bwd : raster_bwd_auto(c->bins, (int64_t)c->B * c->n);
+  return c->raster_bwd != GS_OPT_AUTO ? c->raster_bwd : raster_bwd_auto(c->filled, (int64_t)c->B * c->n);
 }
 
 static RasterArgs raster_args(gs_ctx* c) {

@@ -190,9 +190,9 @@ void launch_l1_finish(const float* partial, int64_t nparts, double* scratch, dou
                       cudaStream_t s);
 void launch_raster_bwd(const RasterArgs& a, int64_t bins, int ppt, cudaStream_t s);
 bool raster_bwd_flags(int ppt);
-int raster_bwd_auto(int64_t bins, int64_t pairs);
-int raster_fwd_auto(int64_t bins, int64_t pairs);
-bool tile_order_auto(int64_t bins);
+int raster_bwd_auto(int64_t tiles, int64_t pairs);
+int raster_fwd_auto(int64_t tiles, int64_t pairs);
+bool tile_order_auto(int64_t tiles);
 // out[0] += list entries up to each pixel's last contributor, out[1] += contributing pairs
 void launch_pair_stats(const RasterArgs& a, int64_t bins, unsigned long long* out, cudaStream_t s);
 

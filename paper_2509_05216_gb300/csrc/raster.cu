@@ -1364,7 +1364,10 @@ void launch_raster_fwd(const RasterArgs& a, int64_t bins, int ppt, cudaStream_t 
   }
 }
 
-// The variants when the caller has chosen none (GS_OPT_AUTO).  From the tile count at which
+// The variants when the caller has chosen none (GS_OPT_AUTO), by the tiles that
+// the scene may fill: not those beyond 2.3 focal lengths of image width or height (9
+// views of 219 x 1937 with 60 degrees across, 160,867 Gaussians, whole step 1267 us by
+// all 15,372 tiles, 1121 by 4,032).  From the tile count at which
 // one warp per tile fills every SM's 14 to 16 resident warps twice over, tiles
 // are taken longest lists first, 4 pixels per thread forward and 8 backward: few
 // long-lived warps per tile leave a tail that the order removes (16 views of
@@ -1380,16 +1383,16 @@ void launch_raster_fwd(const RasterArgs& a, int64_t bins, int ppt, cudaStream_t 
 // 14,400 tiles 1030 / 962 and 664 / 606; 32,400 tiles 1212 / 1149 and 840 / 739;
 // from close by, 4,992 tiles 827 / 777 and 508 / 467.
 //
-// Many tiles with 512 (view, Gaussian) pairs each or more are mostly empty ones
-// around a few with long lists: those keep 2 pixels forward and 4 backward, in
-// list order.  Forward, then gs_raster_bwd, with 2 and 4 / 4 and 8 pixels: 4M Gaussians,
-// 8 views of 236 x 1625 6.50 / 6.82 and 3.71 / 4.57 ms; 2M, 8 views of 512^2 1010 / 1112
-// and 1035 / 1224 us; 1M, 16 of 400^2 1237 / 1407 and 1179 / 1359; on a surface that fills
-// the view, 6M, one of 1300 x 1000 264 / 255 and 693 / 672.
-static bool many_tiles(int64_t bins) { return bins >= (int64_t)32 * sm_count(); }
-static bool long_lists(int64_t bins, int64_t pairs) { return pairs >= 512 * bins; }
-bool tile_order_auto(int64_t bins) { return many_tiles(bins); }
-int raster_fwd_auto(int64_t bins, int64_t pairs) { return many_tiles(bins) && !long_lists(bins, pairs) ? 4 : 2; }
+// Many tiles with 2,048 (view, Gaussian) pairs each or more keep 2 pixels forward
+// and 4 backward, in list order: their lists are long and, around an object, few.
+// Forward, then gs_raster_bwd, with 2 and 4 / 4 and 8 pixels: 4M Gaussians, 8 views of 236 x
+// 1625 (2,614 pairs per tile) 6.50 / 6.82 and 3.71 / 4.57 ms, 8 of 300 x 1200 (2,807) 5.92 /
+// 6.84 and 4.10 / 4.90 ms; surfaces that fill the view, with fewer pairs per tile: one of 1300 x 1000 (1,161)
+// 264 / 255 and 693 / 672 us, 4 of 2048 x 300 (1,645) 360 / 347 and 775 / 766 us.
+static bool many_tiles(int64_t tiles) { return tiles >= (int64_t)32 * sm_count(); }
+static bool long_lists(int64_t tiles, int64_t pairs) { return pairs >= 2048 * tiles; }
+bool tile_order_auto(int64_t tiles) { return many_tiles(tiles); }
+int raster_fwd_auto(int64_t tiles, int64_t pairs) { return many_tiles(tiles) && !long_lists(tiles, pairs) ? 4 : 2; }
 
 // Backward of a few tiles with long lists: their chains are the time, and more
 // warps per tile, each with the entries of fewer pixels, shorten them.  Up to a
@@ -1401,11 +1404,11 @@ int raster_fwd_auto(int64_t bins, int64_t pairs) { return many_tiles(bins) && !l
 // 124 / 101 / 71; 800 and 1,250 438 / 471 / 482.  (Over 280 batches of 16 to 1,280 tiles
 // it takes 2 % more than the best of the three, always 4 pixels 5 %; batches whose
 // pixels stop early lose up to a quarter by it.)
-int raster_bwd_auto(int64_t bins, int64_t pairs) {
-  if (many_tiles(bins)) return long_lists(bins, pairs) ? 4 : 8;
+int raster_bwd_auto(int64_t tiles, int64_t pairs) {
+  if (many_tiles(tiles)) return long_lists(tiles, pairs) ? 4 : 8;
   const int64_t sms = sm_count();
-  if (bins > 4 * sms || pairs < 160 * bins) return 4;
-  return bins <= sms || pairs >= 1024 * bins ? 1 : 2;
+  if (tiles > 4 * sms || pairs < 160 * tiles) return 4;
+  return tiles <= sms || pairs >= 1024 * tiles ? 1 : 2;
 }
 
 bool raster_bwd_flags(int ppt) { return ppt == 4 || ppt == 8; }

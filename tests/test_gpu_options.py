@@ -44,10 +44,10 @@ def test_automatic_options_come_back():
 
 
 def test_many_tiles_of_long_lists():
-    """Many tiles with 512 pairs each or more: list order, but the kernels of fewer pixels per thread."""
-    cams = [inputs.pinhole(inputs.look_at((2.8 * math.cos(0.2 * v), 2.8 * math.sin(0.2 * v), 0.5)), 208, 192) for v in range(32)]
-    for n, kernels in ((79000, (4, 8, 1)), (81000, (2, 4, 1))):  # 32 n / 4,992 tiles: 506 and 519
-        scene = inputs.random_scene(n, 0, 4, extent=0.8, log_scale=(-6.0, -5.0))
+    """Many tiles with 2,048 pairs each or more: list order, but the kernels of fewer pixels per thread."""
+    cams = [inputs.pinhole(inputs.look_at((2.8 * math.cos(0.1 * v), 2.8 * math.sin(0.1 * v), 0.5)), 208, 96) for v in range(63)]
+    for n, kernels in ((159000, (4, 8, 1)), (161000, (2, 4, 1))):  # 63 n / 4,914 tiles: 2,038 and 2,064
+        scene = inputs.random_scene(n, 0, 4, extent=0.8, log_scale=(-6.5, -5.5))
         ctx = gs.Context(0)
         _, img = run_forward(ctx, scene, cams)
         got = tuple(ctx.gs_get_option(o) for o in AUTOMATIC)
@@ -59,9 +59,11 @@ def test_many_tiles_of_long_lists():
         ctx.close()
 
 
-# (tiles per SM, pairs per tile) on both sides of the lines between the backward kernels; 152 SMs
+# (tiles per SM, pairs per tile) on both sides of the lines between the backward kernels; 152 SMs; tall views count as
+# 2.3 focal lengths (30 tiles of 500), wide ones whole
 @pytest.mark.parametrize("w,h,n,kernel", [(192, 192, 23039, 4), (192, 192, 23040, 1), (208, 192, 25000, 2), (208, 192, 160000, 1),
-                                          (608, 256, 98000, 2), (624, 256, 110000, 4), (2048, 2048, 30000, 8)])
+                                          (400, 384, 98000, 2), (416, 384, 110000, 4), (2048, 2048, 30000, 8),
+                                          (240, 8000, 30000, 4), (8000, 240, 30000, 8), (240, 8000, 90000, 2)])
 def test_backward_kernel_by_tiles_and_pairs(w, h, n, kernel):
     scene = inputs.random_scene(n, 0, 4, extent=0.8, log_scale=(-6.0, -5.0))
     cams = [inputs.pinhole(inputs.look_at((0.4, -2.8, 1.0)), w, h)]
