@@ -1407,7 +1407,7 @@ int raster_fwd_auto(int64_t tiles, int64_t pairs) { return many_tiles(tiles) && 
 int raster_bwd_auto(int64_t tiles, int64_t pairs) {
   if (many_tiles(tiles)) return long_lists(tiles, pairs) ? 4 : 8;
   const int64_t sms = sm_count();
-  if (tiles > 4 * sms || pairs < 160 * tiles) return 4;
+  if (tiles == 0 || tiles > 4 * sms || pairs < 160 * tiles) return 4;
   return tiles <= sms || pairs >= 1024 * tiles ? 1 : 2;
 }
 

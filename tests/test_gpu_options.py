@@ -18,6 +18,7 @@ def test_automatic_options_come_back():
     few = [inputs.pinhole(inputs.look_at((0.4, -2.8, 1.0)), 100, 80)]
     many = [inputs.pinhole(inputs.look_at((0.4, -2.8, 1.0)), 2048, 2048)]  # 16,384 tiles, 100 per SM
     ctx = gs.Context(0)
+    assert [ctx.gs_get_option(o) for o in AUTOMATIC] == [2, 4, 0]  # (nothing projected yet)
 
     def read(cams):
         _, img = run_forward(ctx, scene, cams)
